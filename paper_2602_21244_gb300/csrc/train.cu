@@ -8,20 +8,21 @@
 //             y, u = y/|y|, v_r' = |v_r| u, centre-of-mass update, moment
 //             matching over pseudo-cells of 16 pairs (32 particles), loss
 //   backward  dL/dv_new -> closed-form moment-matching and projection
-//             backward -> dz4 = dL/dy; the activations recomputed: the low
-//             bf16 terms of h1 and h2 regenerated by running layers 1 and 2
-//             again from the saved input and high terms, then for l = 3, 2,
-//             1: z_l by an MMA from exactly the forward's operands, so every
-//             recomputed z_l equals the forward's bit for bit (the stored
-//             variant reads back the copy the forward wrote to global
-//             memory instead),
+//             backward -> dz4 = dL/dy; z_3 is still in the accumulator that
+//             the forward left it in (the output layer has columns of its
+//             own), z_2 and z_1 are recomputed by an MMA from exactly the
+//             forward's operands (h1's low bf16 terms stay in tensor memory, so
+//             nothing else has to be regenerated), so every z_l equals the
+//             forward's bit for bit (the stored variant reads back the copy
+//             the forward wrote to global memory instead),
 //             dz_l = dh_l * act'(z_l), dW_l += dz_l^T h_{l-1} (MN-major
 //             operands, accumulated in TMEM across the CTA's tiles),
 //             dh_{l-1} = dz_l W_l (W_l read MN-major from the forward tile)
 //   flush     per-CTA partial gradients to global memory; a second kernel
 //             sums them over CTAs in a fixed order (deterministic)
 // TMEM columns: 0..127 scratch, 128..255 dW2, 256..383 dW3, 384..415 dW1
-// (hi|lo input columns), 416..431 dW4^T.
+// (hi|lo input columns), 416..431 dW4^T, 432..447 output layer, 448..511 the
+// low terms of h1 (A operand).
 #include <cuda_bf16.h>
 
 #include "internal.cuh"
@@ -48,8 +49,8 @@ constexpr uint32_t S_WKLO = S_WK + kT * kH * 2;
 constexpr uint32_t S_DZ4 = S_WKLO + kT * kH * 2;       // [128 x 16] dz of the output layer (bf16)
 constexpr uint32_t S_DZ4F = S_DZ4 + kT * 16 * 2;       // [128 x 3] FP32
 constexpr uint32_t S_BIAS = S_DZ4F + kT * 4 * 4;       // 3*128 + 16 floats
-constexpr uint32_t S_DB = S_BIAS + (3 * kH + 16) * 4;  // 3*128 + 16 floats (bias gradients)
-constexpr uint32_t S_MISC = S_DB + (3 * kH + 16) * 4;  // mbarrier, tmem ptr, flag, loss
+constexpr uint32_t S_WO32 = S_BIAS + (3 * kH + 16) * 4;  // output weights in FP32 [3 x 128]
+constexpr uint32_t S_MISC = S_WO32 + 3 * kH * 4;       // mbarrier, tmem ptr, flag
 constexpr uint32_t S_TOTAL = S_MISC + 64;
 // per-CTA partial: dW1 [128 x 32], dW2, dW3 [128 x 128], dW4^T [128 x 16], then the bias
 // gradients of each of the 4 TMEM lane groups [4 x 400], then the loss of each lane group
@@ -58,7 +59,7 @@ constexpr int kPLOSS = kPDB + 4 * 400;
 constexpr int kPartial = kPLOSS + 16;
 constexpr int kNW = kH * 8 + 2 * kH * kH + 3 * kH;   // weights (d_in 8)
 constexpr int kNB = 3 * kH + 3;                      // biases
-constexpr uint32_t TM_DW2 = 128, TM_DW3 = 256, TM_DW1 = 384, TM_DW4 = 416;
+constexpr uint32_t TM_DW2 = 128, TM_DW3 = 256, TM_DW1 = 384, TM_DW4 = 416, TM_OUT = 432, TM_H1LO = 448;
 }  // namespace
 
 struct TrainArgs {
@@ -84,13 +85,6 @@ __device__ __forceinline__ float act_grad(int act, float z) {
   if (act == 1) return z > 0.f ? 1.f : 0.f;
   const float s = __fdividef(1.f, 1.f + __expf(-z));
   return s * (1.f + z * (1.f - s));
-}
-
-// sum over the 16 lanes of this half-warp (groups are 16 consecutive rows)
-__device__ __forceinline__ double half_sum(double v) {
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
 }
 
 // v[32] per lane -> lane l returns the sum over the warp's lanes of v[l]
@@ -125,6 +119,53 @@ __device__ __forceinline__ uint64_t kdesc(uint32_t a, int K) { return tc::sdesc(
 // MN-major view of a [rows x F] tile: MN = F (features), K = rows
 __device__ __forceinline__ uint64_t mdesc(uint32_t a, int F) { return tc::sdesc(a, (uint32_t)(F / 8) * 128, 128); }
 
+// ---- FP64 helpers of the row stage.  GB300's FP64 pipe (about 1/64 of the
+// FP32 rate; a warp instruction costs the same however few lanes need it)
+// bounds that stage, so square roots and reciprocals start from the
+// special-function unit's FP64 approximations (relative error below 2^-19
+// over the whole range) and take two Newton steps (2^-38, then FP64 rounding)
+// instead of the general routines: about 10 FP64 instructions against 20 to 30.
+__device__ __forceinline__ double rsqrt64(double x) {   // x > 0, normal
+  double r;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double h = 0.5 * x;
+  r = fma(r, fma(-h * r, r, 0.5), r);
+  return fma(r, fma(-h * r, r, 0.5), r);
+}
+// the smallest x that rsqrt64 takes (its products stay normal): below it the
+// general routines run
+constexpr double kTiny64 = 1e-280, kHuge64 = 1e280;
+__device__ __forceinline__ bool plain64(double x) { return x > kTiny64 && x < kHuge64; }
+__device__ __forceinline__ double sqrt64(double x) {
+  if (!plain64(x)) return sqrt(x);
+  const double r = rsqrt64(x), y = x * r;
+  return fma(0.5 * r, fma(-y, y, x), y);
+}
+
+// sums over the 16 lanes of this half-warp (groups are 16 consecutive rows)
+// of K values at once, K a power of two up to 8: each step halves the values a lane still adds (the
+// other half goes to its partner), so K values take K + log2(16/K) - 1 or so FP64
+// additions instead of 4 K; the totals come back by shuffles alone.
+template <int K>
+__device__ __forceinline__ void half_sums(double* v) {
+  const int lane = threadIdx.x & 31;
+  int w = 8;
+#pragma unroll
+  for (int k = K / 2; k >= 1; k >>= 1, w >>= 1) {
+    const bool up = lane & w;
+#pragma unroll
+    for (int q = 0; q < k; ++q) {
+      const double send = up ? v[q] : v[q + k], keep = up ? v[q + k] : v[q];
+      v[q] = keep + __shfl_xor_sync(0xffffffffu, send, w);
+    }
+  }
+  double t = v[0];
+  for (; w >= 1; w >>= 1) t += __shfl_xor_sync(0xffffffffu, t, w);
+  // value q sits in the lanes whose upper bits of the half-warp index spell q
+#pragma unroll
+  for (int q = 0; q < K; ++q) v[q] = __shfl_sync(0xffffffffu, t, (lane & 16) | (q * (16 / K)));
+}
+
 __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
   extern __shared__ __align__(1024) char sm[];
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
@@ -134,36 +175,48 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
   uint32_t* tptr = (uint32_t*)(sm + S_MISC + 8);
   volatile int* flag = (volatile int*)(sm + S_MISC + 12);
   float* bias = (float*)(sm + S_BIAS);
+  const float* wo32 = (const float*)(sm + S_WO32);
   // bias gradients and loss accumulate in registers of fixed threads (no atomics,
   // so the result does not depend on warp scheduling)
   float dbacc[3] = {0.f, 0.f, 0.f};  // layer l, column c0 + lane
   float dbo[3] = {0.f, 0.f, 0.f};    // output bias (lane 0 of warps 0..3)
   double lossw = 0.0;                // loss of this warp's rows (lane 0 of warps 0..3)
   float* dz4f = (float*)(sm + S_DZ4F);
-  // ---- weights into K-major tiles, biases
+  // ---- weights into K-major tiles (eight columns, one 16-byte store, at a
+  // time: a mini-batch of one tile per CTA pays this once per step), biases
   {
     uint32_t* z = (uint32_t*)(sm + S_WOUT);
-    for (int q = t; q < (16 * kH * 2 + kH * kXin * 2) / 4; q += kNT) z[q] = 0u;
+    for (int q = t; q < (16 * kH * 2) / 4; q += kNT) z[q] = 0u;
     const float* bsrc = a.theta + kNW;
     for (int q = t; q < 3 * kH + 16; q += kNT) bias[q] = q < 3 * kH + 3 ? bsrc[q] : 0.f;
     __syncthreads();
-    for (int e = t; e < kH * 8; e += kNT) {
-      const int n = e >> 3, k = e & 7;
-      const uint16_t wb = to_bf16(a.theta[e]);
-      *(uint16_t*)(sm + S_WIN + tc::kmajor_offset(n, k, kXin)) = wb;
-      *(uint16_t*)(sm + S_WIN + tc::kmajor_offset(n, 16 + k, kXin)) = wb;
+    auto put8 = [&](uint32_t dst, const float* w8) {
+      uint32_t r[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) r[q] = tc::pack_bf16x2(w8[2 * q], w8[2 * q + 1]);
+      tc::st_shared_v4(sb + dst, r[0], r[1], r[2], r[3]);
+    };
+    if (t < kH) {   // W1's eight columns, in columns 0..7 (hi) and 16..23 (lo) of its tile
+      put8(S_WIN + tc::kmajor_offset(t, 0, kXin), a.theta + 8 * t);
+      put8(S_WIN + tc::kmajor_offset(t, 16, kXin), a.theta + 8 * t);
+      tc::st_shared_v4(sb + S_WIN + tc::kmajor_offset(t, 8, kXin), 0u, 0u, 0u, 0u);
+      tc::st_shared_v4(sb + S_WIN + tc::kmajor_offset(t, 24, kXin), 0u, 0u, 0u, 0u);
     }
     const float* w2 = a.theta + kH * 8;
-    for (int e = t; e < kH * kH; e += kNT) {
-      *(uint16_t*)(sm + S_W2 + tc::kmajor_offset(e >> 7, e & 127, kH)) = to_bf16(w2[e]);
-      *(uint16_t*)(sm + S_W3 + tc::kmajor_offset(e >> 7, e & 127, kH)) = to_bf16(w2[kH * kH + e]);
+    for (int e = t; e < kH * kH / 8; e += kNT) {
+      const int n = e >> 4, k = (e & 15) * 8;
+      put8(S_W2 + tc::kmajor_offset(n, k, kH), w2 + n * kH + k);
+      put8(S_W3 + tc::kmajor_offset(n, k, kH), w2 + kH * kH + n * kH + k);
     }
     const float* w4 = w2 + 2 * kH * kH;
-    for (int e = t; e < 3 * kH; e += kNT)
-      *(uint16_t*)(sm + S_WOUT + tc::kmajor_offset(e >> 7, e & 127, kH)) = to_bf16(w4[e]);
+    for (int e = t; e < 3 * kH; e += kNT) {
+      const uint16_t b = to_bf16(w4[e]);
+      *(uint16_t*)(sm + S_WOUT + tc::kmajor_offset(e >> 7, e & 127, kH)) = b;
+      ((float*)(sm + S_WO32))[e] = __uint_as_float((uint32_t)b << 16);
+    }
   }
   if (warp == 0) { tc::tmem_alloc(tptr, 512); tc::tmem_relinquish(); }
-  if (t == 0) { tc::mbar_init(mbar, 1); tc::mbar_fence_init(); }
+  if (t == 0) { tc::mbar_init(mbar, 1); tc::mbar_fence_init(); *flag = 1; }
   tc::fence_async_smem();
   tc::fence_before();
   __syncthreads();
@@ -171,43 +224,48 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
   const uint32_t tm = *(volatile uint32_t*)tptr;
   const uint32_t lane_tm = tm + ((uint32_t)((warp & 3) * 32) << 16);
   uint32_t phase = 0;
-  bool alive = true;
   int tiles_done = 0;
 
-  // one elected thread commits the issued MMAs and waits; everyone syncs
-  auto sync_mma = [&]() -> bool {
-    if (t == 0) {
-      tc::commit(mbar);
-      *flag = tc::mbar_wait(mbar, phase, a.status, kBarrierLimitNs) ? 1 : 0;
-    }
-    __syncthreads();
+  // Every thread waits for the committed MMAs itself (each then reads TMEM
+  // and reuses the operands' shared memory without a barrier); a timeout
+  // clears the flag, read after the next barrier so that all threads leave together.
+  auto wait_mma = [&]() {
+    if (!tc::mbar_wait(mbar, phase, a.status, kBarrierLimitNs)) *flag = 0;
     phase ^= 1u;
     tc::fence_after();
-    return *flag != 0;
   };
-  auto to_mma = [&]() {  // make shared-memory writes and TMEM reads visible before an MMA
+  // make shared-memory writes and TMEM accesses visible before an MMA; false after a timeout
+  auto to_mma = [&]() -> bool {
     tc::fence_async_smem();
     tc::fence_before();
     __syncthreads();
+    return *flag != 0;
   };
 
+  // z1 from x (hi + lo): two K steps (thread 0)
+  auto input_mma = [&]() {
+    const uint32_t id = tc::idesc_bf16(kT, kH);
+    for (int s = 0; s < 2; ++s)
+      tc::mma_bf16(tm, kdesc(sb + S_X + 256u * s, kXin), kdesc(sb + S_WIN + 256u * s, kXin), id, s > 0);
+  };
   // The MMA of hidden layer l + 1 (l = 1, 2) on its input as hi + lo terms:
-  // h1 = S_H1 + S_WKLO, h2 = S_H2 + S_WK (thread 0)
+  // h1 = S_H1 + TM_H1LO (tensor memory), h2 = S_H2 + S_WK (thread 0)
   auto hidden_mma = [&](int l) {
     const uint32_t id = tc::idesc_bf16(kT, kH);
-    const uint32_t wl = l == 1 ? S_W2 : S_W3, hhi = l == 1 ? S_H1 : S_H2, hlo = l == 1 ? S_WKLO : S_WK;
+    const uint32_t wl = l == 1 ? S_W2 : S_W3, hhi = l == 1 ? S_H1 : S_H2;
     for (int s = 0; s < 8; ++s)
       tc::mma_bf16(tm, kdesc(sb + hhi + 256u * s, kH), kdesc(sb + wl + 256u * s, kH), id, s > 0);
-    for (int s = 0; s < 8; ++s)
-      tc::mma_bf16(tm, kdesc(sb + hlo + 256u * s, kH), kdesc(sb + wl + 256u * s, kH), id, 1);
+    for (int s = 0; s < 8; ++s) {
+      if (l == 1) tc::mma_bf16_ta(tm, tm + TM_H1LO + 8u * s, kdesc(sb + wl + 256u * s, kH), id, 1);
+      else tc::mma_bf16(tm, kdesc(sb + S_WK + 256u * s, kH), kdesc(sb + wl + 256u * s, kH), id, 1);
+    }
   };
   // Epilogue of hidden layer l from this thread's 32 accumulator values v:
   // bias, activation (SiLU four values at a time on the paired FP32 pipe, as
-  // in the collide kernel's epilogue), the hi + lo split; hi and lo stored as
-  // the next layer's input (l = 0: S_H1, S_WKLO; l = 1: S_H2, S_WK; l = 2,
-  // the output layer's: S_WK, S_WKLO).  with_hi false: only the lo term
-  // (the backward's regeneration; the hi terms are still in S_H1, S_H2).
-  auto hidden_epilogue = [&](int l, const float* v, bool with_hi) {
+  // in the collide kernel's epilogue), the hi + lo split; stored as the next
+  // layer's input (l = 0: S_H1 and, the low terms, tensor memory; l = 1:
+  // S_H2, S_WK; l = 2, the output layer's: S_WK, S_WKLO).
+  auto hidden_epilogue = [&](int l, const float* v) {
     uint32_t pk[16], lo[16];
     const float2* b2 = (const float2*)(bias + l * kH + c0);
 #pragma unroll
@@ -233,134 +291,161 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const uint32_t off = tc::kmajor_offset(row, c0 + 8 * j, kH);
-      if (with_hi) tc::st_shared_v4(sb + dhi + off, pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
-      tc::st_shared_v4(sb + dlo + off, lo[4 * j], lo[4 * j + 1], lo[4 * j + 2], lo[4 * j + 3]);
+      tc::st_shared_v4(sb + dhi + off, pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
+      if (l > 0) tc::st_shared_v4(sb + dlo + off, lo[4 * j], lo[4 * j + 1], lo[4 * j + 2], lo[4 * j + 3]);
+    }
+    if (l == 0) {   // row m in lane m, two bf16 per column
+      tc::st16_async(lane_tm + TM_H1LO + (uint32_t)(c0 >> 1), lo);
+      tc::wait_st();
+    }
+  };
+  // The input row of pair p as its nonzero packed words: columns 0..7 of the
+  // hi term in x[0..3], of the lo term in x[4..7].  Warps 4..7 form the next
+  // tile's rows while warps 0..3 run the row stage.
+  auto features = [&](int64_t p, uint32_t* x) {
+    float f[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) f[q] = 0.f;
+    if (p < a.n) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) f[c] = (float)((a.vi[3 * p + c] - a.vj[3 * p + c]) * a.sigma_v_inv);
+      f[3] = (float)(a.T[p] * a.T_ref_inv);
+      const u32x4 wa = draw(a.seed, (uint32_t)p, 0u, a.t, TAG_NOISE, 0);
+      const u32x4 wb = draw(a.seed, (uint32_t)p, 0u, a.t, TAG_NOISE, 1);
+      box_muller2(u53(wa.x, wa.y), u53(wa.z, wa.w), &f[4], &f[5]);
+      box_muller2(u53(wb.x, wb.y), u53(wb.z, wb.w), &f[6], &f[7]);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      x[q] = tc::pack_bf16x2(f[2 * q], f[2 * q + 1]);
+      x[4 + q] = tc::pack_bf16x2(f[2 * q] - __uint_as_float(x[q] << 16), f[2 * q + 1] - __uint_as_float(x[q] & 0xFFFF0000u));
+    }
+  };
+  // act'(z + bias) of this thread's 32 values of layer l
+  auto act_slopes = [&](int l, const float* z, float* g) {
+#pragma unroll
+    for (int q = 0; q < 32; ++q) g[q] = act_grad(a.act, z[q] + bias[l * kH + c0 + q]);
+  };
+  // this tile's z_l of the stored variant, row-major [128 x 128]
+  auto stored_z = [&](int64_t tile, int l) { return (float4*)(a.zst + (((size_t)tile * 3 + l) * kT + row) * kH + c0); };
+  auto load_z = [&](int64_t tile, int l, float* z) {
+    if (a.zst) {
+      const float4* src = stored_z(tile, l);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const float4 f = src[q];
+        z[4 * q] = f.x; z[4 * q + 1] = f.y; z[4 * q + 2] = f.z; z[4 * q + 3] = f.w;
+      }
+    } else {
+      tc::ld32(lane_tm + (uint32_t)c0, z);
     }
   };
 
   const int64_t ntiles = (a.n + kT - 1) / kT;
+  const bool rowthr = t < kT, xthr = cg == 1;
+  uint32_t xw[8];   // warps 4..7: the coming tile's input row
+  if (xthr) features((int64_t)blockIdx.x * kT + row, xw);
+  bool alive = true, busy = false;   // busy: the last tile's final MMAs are not waited for yet
   for (int64_t tile = blockIdx.x; tile < ntiles && alive; tile += gridDim.x) {
     const int64_t p = tile * kT + row;
-    const bool rowthr = t < kT;
     const bool valid = rowthr && p < a.n;
-    double vi[3] = {0, 0, 0}, vj[3] = {0, 0, 0};
-    // ---------------- features (rows)
-    if (rowthr) {
-      float f[16];
-#pragma unroll
-      for (int q = 0; q < 16; ++q) f[q] = 0.f;
-      if (valid) {
-        for (int c = 0; c < 3; ++c) { vi[c] = a.vi[3 * p + c]; vj[c] = a.vj[3 * p + c]; }
-        f[0] = (float)((vi[0] - vj[0]) * a.sigma_v_inv);
-        f[1] = (float)((vi[1] - vj[1]) * a.sigma_v_inv);
-        f[2] = (float)((vi[2] - vj[2]) * a.sigma_v_inv);
-        f[3] = (float)(a.T[p] * a.T_ref_inv);
-        const u32x4 wa = draw(a.seed, (uint32_t)p, 0u, a.t, TAG_NOISE, 0);
-        const u32x4 wb = draw(a.seed, (uint32_t)p, 0u, a.t, TAG_NOISE, 1);
-        box_muller2(u53(wa.x, wa.y), u53(wa.z, wa.w), &f[4], &f[5]);
-        box_muller2(u53(wb.x, wb.y), u53(wb.z, wb.w), &f[6], &f[7]);
-      }
-      uint32_t hi[8], lo[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        hi[q] = tc::pack_bf16x2(f[2 * q], f[2 * q + 1]);
-        lo[q] = tc::pack_bf16x2(f[2 * q] - __uint_as_float(hi[q] << 16), f[2 * q + 1] - __uint_as_float(hi[q] & 0xFFFF0000u));
-      }
-      tc::st_shared_v4(sb + S_X + tc::kmajor_offset(row, 0, kXin), hi[0], hi[1], hi[2], hi[3]);
-      tc::st_shared_v4(sb + S_X + tc::kmajor_offset(row, 8, kXin), hi[4], hi[5], hi[6], hi[7]);
-      tc::st_shared_v4(sb + S_X + tc::kmajor_offset(row, 16, kXin), lo[0], lo[1], lo[2], lo[3]);
-      tc::st_shared_v4(sb + S_X + tc::kmajor_offset(row, 24, kXin), lo[4], lo[5], lo[6], lo[7]);
+    if (busy) wait_mma();   // dW1 of the last tile reads the input tile
+    if (xthr) {
+      tc::st_shared_v4(sb + S_X + tc::kmajor_offset(row, 0, kXin), xw[0], xw[1], xw[2], xw[3]);
+      tc::st_shared_v4(sb + S_X + tc::kmajor_offset(row, 8, kXin), 0u, 0u, 0u, 0u);
+      tc::st_shared_v4(sb + S_X + tc::kmajor_offset(row, 16, kXin), xw[4], xw[5], xw[6], xw[7]);
+      tc::st_shared_v4(sb + S_X + tc::kmajor_offset(row, 24, kXin), 0u, 0u, 0u, 0u);
     }
-    to_mma();
+    if (!(alive = to_mma())) break;
     // ---------------- forward, layers 1..3 (scratch accumulator at TMEM column 0)
-    for (int l = 0; l < 3 && alive; ++l) {
+    for (int l = 0; l < 3; ++l) {
       if (t == 0) {
         tc::fence_after();
-        const uint32_t id = tc::idesc_bf16(kT, kH);
-        if (l == 0) {
-          for (int s = 0; s < 2; ++s)
-            tc::mma_bf16(tm, kdesc(sb + S_X + 256u * s, kXin), kdesc(sb + S_WIN + 256u * s, kXin), id, s > 0);
-        } else {
-          hidden_mma(l);
-        }
+        if (l == 0) input_mma();
+        else hidden_mma(l);
+        tc::commit(mbar);
       }
-      if (!sync_mma()) { alive = false; break; }
+      wait_mma();
       float v[32];
       tc::ld32(lane_tm + (uint32_t)c0, v);
-      if (a.zst && a.mode != 0) {   // stored variant: this tile's z_l, row-major [128 x 128]
-        float4* dst = (float4*)(a.zst + (((size_t)tile * 3 + l) * kT + row) * kH + c0);
+      if (a.zst && a.mode != 0) {
+        float4* dst = stored_z(tile, l);
 #pragma unroll
         for (int q = 0; q < 8; ++q) dst[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
       }
-      hidden_epilogue(l, v, true);
-      to_mma();
+      hidden_epilogue(l, v);
+      if (!(alive = to_mma())) break;
     }
     if (!alive) break;
-    // ---------------- output layer
+    // ---------------- output layer, into columns of its own: z3 stays in the
+    // scratch accumulator for the backward
     if (t == 0) {
       tc::fence_after();
       const uint32_t id = tc::idesc_bf16(kT, 16);
       for (int s = 0; s < 8; ++s)
-        tc::mma_bf16(tm, kdesc(sb + S_WK + 256u * s, kH), kdesc(sb + S_WOUT + 256u * s, kH), id, s > 0);
+        tc::mma_bf16(tm + TM_OUT, kdesc(sb + S_WK + 256u * s, kH), kdesc(sb + S_WOUT + 256u * s, kH), id, s > 0);
       for (int s = 0; s < 8; ++s)
-        tc::mma_bf16(tm, kdesc(sb + S_WKLO + 256u * s, kH), kdesc(sb + S_WOUT + 256u * s, kH), id, 1);
-    }
-    if (!sync_mma()) { alive = false; break; }
-    float y[3] = {0.f, 0.f, 0.f};
-    if (cg == 0) {
-      float v[16];
-      tc::ld16(lane_tm, v);
-      y[0] = v[0] + bias[3 * kH]; y[1] = v[1] + bias[3 * kH + 1]; y[2] = v[2] + bias[3 * kH + 2];
+        tc::mma_bf16(tm + TM_OUT, kdesc(sb + S_WKLO + 256u * s, kH), kdesc(sb + S_WOUT + 256u * s, kH), id, 1);
+      tc::commit(mbar);
     }
     // ---------------- shell projection, pair update, moment matching, loss (rows)
     if (rowthr) {
-      double ur[3], g = 0.0, ny = 0.0, u[3], pi[3], pj[3];
-      for (int c = 0; c < 3; ++c) ur[c] = vi[c] - vj[c];
-      g = sqrt(ur[0] * ur[0] + ur[1] * ur[1] + ur[2] * ur[2]);
-      const double yd[3] = {y[0], y[1], y[2]};
-      ny = sqrt(yd[0] * yd[0] + yd[1] * yd[1] + yd[2] * yd[2]);
-      const double iny = valid && ny > 0.0 ? 1.0 / ny : 0.0;
+      double vi[3] = {0, 0, 0}, vj[3] = {0, 0, 0};
+      if (valid)
+        for (int c = 0; c < 3; ++c) { vi[c] = a.vi[3 * p + c]; vj[c] = a.vj[3 * p + c]; }
+      double ur[3], g = 0.0, u[3], cm[3];
+      for (int c = 0; c < 3; ++c) { ur[c] = vi[c] - vj[c]; cm[c] = 0.5 * (vi[c] + vj[c]); }
+      g = sqrt64(ur[0] * ur[0] + ur[1] * ur[1] + ur[2] * ur[2]);
+      wait_mma();
+      float v[16];
+      tc::ld16(lane_tm + TM_OUT, v);
+      const double yd[3] = {v[0] + bias[3 * kH], v[1] + bias[3 * kH + 1], v[2] + bias[3 * kH + 2]};
+      const double ny2 = yd[0] * yd[0] + yd[1] * yd[1] + yd[2] * yd[2];
+      // 1/|y| (0 for y = 0)
+      const double iny = !valid ? 0.0 : plain64(ny2) ? rsqrt64(ny2) : ny2 > 0.0 ? 1.0 / sqrt(ny2) : 0.0;
+      double pi[3], pj[3];
       for (int c = 0; c < 3; ++c) {
         u[c] = yd[c] * iny;
-        const double cm = 0.5 * (vi[c] + vj[c]);
-        pi[c] = cm + 0.5 * g * u[c];
-        pj[c] = cm - 0.5 * g * u[c];
+        const double h = 0.5 * g * u[c];
+        pi[c] = cm[c] + h;
+        pj[c] = cm[c] - h;
       }
       // group moments over the 32 particles of the pseudo-cell (two passes)
-      double upre[3], upost[3], thpre = 0.0, thpost = 0.0;
+      double us[8];
+      for (int c = 0; c < 3; ++c) { us[c] = vi[c] + vj[c]; us[4 + c] = pi[c] + pj[c]; }
+      us[3] = us[7] = 0.0;
+      half_sums<8>(us);
+      double upre[3], dpi[3], dpj[3], th[2] = {0.0, 0.0};
       for (int c = 0; c < 3; ++c) {
-        upre[c] = half_sum(vi[c] + vj[c]) * (1.0 / (2 * kGroup));
-        upost[c] = half_sum(pi[c] + pj[c]) * (1.0 / (2 * kGroup));
-      }
-      double dpi[3], dpj[3], tpre = 0.0, tpost = 0.0;
-      for (int c = 0; c < 3; ++c) {
+        upre[c] = us[c] * (1.0 / (2 * kGroup));
+        const double upost = us[4 + c] * (1.0 / (2 * kGroup));
         const double a1 = vi[c] - upre[c], a2 = vj[c] - upre[c];
-        tpre += a1 * a1 + a2 * a2;
-        dpi[c] = pi[c] - upost[c];
-        dpj[c] = pj[c] - upost[c];
-        tpost += dpi[c] * dpi[c] + dpj[c] * dpj[c];
+        th[0] = fma(a1, a1, fma(a2, a2, th[0]));
+        dpi[c] = pi[c] - upost;
+        dpj[c] = pj[c] - upost;
+        th[1] = fma(dpi[c], dpi[c], fma(dpj[c], dpj[c], th[1]));
       }
-      thpre = half_sum(tpre);
-      thpost = half_sum(tpost);
-      const double alpha = thpost > 0.0 ? sqrt(thpre / thpost) : 1.0;
+      half_sums<2>(th);
+      // alpha = sqrt(Theta_pre / Theta_post)
+      const double thp = th[0] * th[1];
+      const double alpha = plain64(thp) ? th[0] * rsqrt64(thp) : th[1] > 0.0 ? sqrt(th[0] / th[1]) : 1.0;
       double ni[3], nj[3];
-      for (int c = 0; c < 3; ++c) { ni[c] = upre[c] + alpha * dpi[c]; nj[c] = upre[c] + alpha * dpj[c]; }
+      for (int c = 0; c < 3; ++c) { ni[c] = fma(alpha, dpi[c], upre[c]); nj[c] = fma(alpha, dpj[c], upre[c]); }
       if (a.mode == 0) {
         if (valid) for (int c = 0; c < 3; ++c) { a.oi[3 * p + c] = ni[c]; a.oj[3 * p + c] = nj[c]; }
       } else {
-        double Gi[3] = {0, 0, 0}, Gj[3] = {0, 0, 0};
+        double Gd[3] = {0, 0, 0};   // G_i - G_j
         double l2 = 0.0;
         if (valid) {
           if (a.mode == 2) {
             const double sc = a.sigma_v_inv * a.sigma_v_inv / (double)a.n;
             for (int c = 0; c < 3; ++c) {
               const double ri = ni[c] - a.ti[3 * p + c], rj = nj[c] - a.tj[3 * p + c];
-              l2 += ri * ri + rj * rj;
-              Gi[c] = ri * sc;
-              Gj[c] = rj * sc;
+              l2 = fma(ri, ri, fma(rj, rj, l2));
+              Gd[c] = (ri - rj) * sc;
             }
           } else {
-            for (int c = 0; c < 3; ++c) { Gi[c] = a.gi[3 * p + c]; Gj[c] = a.gj[3 * p + c]; }
+            for (int c = 0; c < 3; ++c) Gd[c] = a.gi[3 * p + c] - a.gj[3 * p + c];
           }
         }
         if (a.mode == 2) {  // loss = sum |v_new - v_target|^2 / sigma_v^2 / (2 n)
@@ -369,42 +454,52 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
           for (int o = 16; o > 0; o >>= 1) lw += __shfl_xor_sync(0xffffffffu, lw, o);
           lossw += lw;
         }
-        // moment-matching backward: dL/dv = alpha (G - Gbar) - (alpha S / Theta_post) (v - u_post)
-        double gbar[3], S = 0.0;
-        for (int c = 0; c < 3; ++c) gbar[c] = half_sum(Gi[c] + Gj[c]) * (1.0 / (2 * kGroup));
-        double sl = 0.0;
-        for (int c = 0; c < 3; ++c) sl += Gi[c] * dpi[c] + Gj[c] * dpj[c];
-        S = half_sum(sl);
-        const double k2 = thpost > 0.0 ? alpha * S / thpost : 0.0;
+        // Backward of moment matching, dL/dv = alpha (G - Gbar) - (alpha S /
+        // Theta_post) (v - u_post), then of the centre-of-mass update (v_r'
+        // enters as +1/2 for i, -1/2 for j) and of the projection, dy =
+        // (g/|y|)(I - u u^T) dv_r'.  In dv_r' = (dL/dv_i - dL/dv_j)/2 the mean
+        // Gbar cancels, and the last term, (v_i - v_j)/2 = g u / 2 along u,
+        // is what (I - u u^T) removes: dv_r' = alpha (G_i - G_j)/2 gives the same dy.
         double dvr[3], ud = 0.0;
         for (int c = 0; c < 3; ++c) {
-          const double di = alpha * (Gi[c] - gbar[c]) - k2 * dpi[c];
-          const double dj = alpha * (Gj[c] - gbar[c]) - k2 * dpj[c];
-          dvr[c] = 0.5 * (di - dj);   // v_r' enters as +1/2 for i, -1/2 for j
-          ud += u[c] * dvr[c];
+          dvr[c] = 0.5 * alpha * Gd[c];
+          ud = fma(u[c], dvr[c], ud);
         }
-        // projection backward: dy = (g/|y|)(I - u u^T) dv_r'
         const double s = valid ? g * iny : 0.0;
-        for (int c = 0; c < 3; ++c) dz4f[4 * row + c] = valid ? (float)(s * (dvr[c] - u[c] * ud)) : 0.f;
+        for (int c = 0; c < 3; ++c) {
+          const float d = valid ? (float)(s * fma(-u[c], ud, dvr[c])) : 0.f;
+          dz4f[4 * row + c] = d;
+          // bias gradient of the output layer
+          float s3 = d;
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) s3 += __shfl_xor_sync(0xffffffffu, s3, o);
+          dbo[c] += s3;
+        }
         uint32_t d0 = tc::pack_bf16x2(dz4f[4 * row], dz4f[4 * row + 1]);
         uint32_t d1 = tc::pack_bf16x2(dz4f[4 * row + 2], 0.f);
         tc::st_shared_v4(sb + S_DZ4 + tc::kmajor_offset(row, 0, 16), d0, d1, 0u, 0u);
         tc::st_shared_v4(sb + S_DZ4 + tc::kmajor_offset(row, 8, 16), 0u, 0u, 0u, 0u);
       }
+    } else {
+      phase ^= 1u;   // the output layer's MMAs, which only the row threads wait for
+      if (xthr && tile + gridDim.x < ntiles) features((tile + gridDim.x) * kT + row, xw);
     }
-    if (a.mode == 0) { tc::fence_before(); __syncthreads(); tc::fence_after(); continue; }
-    // bias gradient of the output layer
-    if (t < kT) {
-      float v3[3] = {dz4f[4 * row], dz4f[4 * row + 1], dz4f[4 * row + 2]};
-      for (int c = 0; c < 3; ++c) {
-        float s3 = v3[c];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s3 += __shfl_xor_sync(0xffffffffu, s3, o);
-        dbo[c] += s3;
-      }
+    if (a.mode == 0) {
+      tc::fence_before();
+      __syncthreads();
+      tc::fence_after();
+      alive = *flag != 0;
+      continue;
     }
-    to_mma();
-    // ---------------- dW4^T += h3^T dz4 (hi and lo), and z3 recomputed from h2
+    // ---------------- layers 3, 2, 1: z3 is still in the scratch accumulator
+    float dh[32];
+    {
+      float z[32];
+      load_z(tile, 2, z);
+      act_slopes(2, z, dh);
+    }
+    if (!(alive = to_mma())) break;
+    // dW4^T += h3^T dz4 (hi and lo)
     const uint32_t acc0 = tiles_done > 0 ? 1u : 0u;
     if (t == 0) {
       tc::fence_after();
@@ -414,114 +509,84 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
                      (acc0 | (s > 0)) ? 1u : 0u);
       for (int s = 0; s < 8; ++s)
         tc::mma_bf16(tm + TM_DW4, mdesc(sb + S_WKLO + 2u * 2048u * s, kH), mdesc(sb + S_DZ4 + 2u * 256u * s, 16), id4, 1);
-      if (!a.zst) {   // regeneration starts with z1 from x (hi + lo)
-        const uint32_t id = tc::idesc_bf16(kT, kH);
-        for (int s = 0; s < 2; ++s)
-          tc::mma_bf16(tm, kdesc(sb + S_X + 256u * s, kXin), kdesc(sb + S_WIN + 256u * s, kXin), id, s > 0);
-      }
+      tc::commit(mbar);
     }
-    if (!sync_mma()) { alive = false; break; }
-    if (!a.zst) {
-      // h1 and h2 low terms regenerated (the forward's arithmetic on the same
-      // accumulators), then z3 = W3 (h2 hi + lo): all equal to the forward's
-      for (int l = 0; l < 2 && alive; ++l) {
-        float v[32];
-        tc::ld32(lane_tm + (uint32_t)c0, v);
-        hidden_epilogue(l, v, false);
-        to_mma();
-        if (t == 0) {
-          tc::fence_after();
-          hidden_mma(l + 1);
-        }
-        if (!sync_mma()) alive = false;
-      }
-      if (!alive) break;
-    }
-    // dh3 = dz4 W4 on CUDA cores (K = 3), dz3 = dh3 * act'(z3)
-    float dh[32];
+    // dz3 = dh3 act'(z3) with dh3 = dz4 W4 on CUDA cores (K = 3)
     {
-#pragma unroll
-      for (int q = 0; q < 32; ++q) dh[q] = 0.f;
       const float d0 = dz4f[4 * row], d1 = dz4f[4 * row + 1], d2 = dz4f[4 * row + 2];
-      for (int q = 0; q < 32; ++q) {
-        const int k = c0 + q;
-        const float w0 = __uint_as_float((uint32_t)(*(const uint16_t*)(sm + S_WOUT + tc::kmajor_offset(0, k, kH))) << 16);
-        const float w1 = __uint_as_float((uint32_t)(*(const uint16_t*)(sm + S_WOUT + tc::kmajor_offset(1, k, kH))) << 16);
-        const float w2 = __uint_as_float((uint32_t)(*(const uint16_t*)(sm + S_WOUT + tc::kmajor_offset(2, k, kH))) << 16);
-        dh[q] = d0 * w0 + d1 * w1 + d2 * w2;
-      }
+#pragma unroll
+      for (int q = 0; q < 32; ++q)
+        dh[q] = (d0 * wo32[c0 + q] + d1 * wo32[kH + c0 + q] + d2 * wo32[2 * kH + c0 + q]) * dh[q];
     }
-    // layers 3, 2, 1
-    for (int l = 2; l >= 0 && alive; --l) {
-      float z[32];
-      if (a.zst) {
-        const float4* src = (const float4*)(a.zst + (((size_t)tile * 3 + l) * kT + row) * kH + c0);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const float4 f = src[q];
-          z[4 * q] = f.x; z[4 * q + 1] = f.y; z[4 * q + 2] = f.z; z[4 * q + 3] = f.w;
-        }
-      } else {
-        tc::ld32(lane_tm + (uint32_t)c0, z);
-      }
-      float dz[32];
-#pragma unroll
-      for (int q = 0; q < 32; ++q) dz[q] = dh[q] * act_grad(a.act, z[q] + bias[l * kH + c0 + q]);
+    for (int l = 2;; --l) {
+      // dh holds dz_l: stored as the operand of dW_l and dh_{l-1} once the
+      // MMAs that read the last one (h3's high terms for l = 2) are done
       uint32_t pk[16];
 #pragma unroll
-      for (int q = 0; q < 16; ++q) pk[q] = tc::pack_bf16x2(dz[2 * q], dz[2 * q + 1]);
+      for (int q = 0; q < 16; ++q) pk[q] = tc::pack_bf16x2(dh[2 * q], dh[2 * q + 1]);
+      if (l == 2) wait_mma();
 #pragma unroll
       for (int j = 0; j < 4; ++j)
         tc::st_shared_v4(sb + S_WK + tc::kmajor_offset(row, c0 + 8 * j, kH), pk[4 * j], pk[4 * j + 1], pk[4 * j + 2],
                          pk[4 * j + 3]);
-      dbacc[l] += warp_colsum32(dz);
-      to_mma();
-      // dW_l += dz^T h_{l-1}; dh_{l-1} = dz W_l (not needed for l = 0)
+      if (!(alive = to_mma())) break;
+      // dh_{l-1} = dz W_l (not needed for l = 0), then dW_l += dz^T h_{l-1},
+      // which runs on while dh_{l-1} is read back
       if (t == 0) {
         tc::fence_after();
         if (l > 0) {
           const uint32_t hprev = l == 2 ? S_H2 : S_H1;
           const uint32_t wl = l == 2 ? S_W3 : S_W2;
           const uint32_t dw = l == 2 ? TM_DW3 : TM_DW2;
+          const uint32_t idh = tc::idesc_bf16(kT, kH) | (1u << 16);
+          for (int s = 0; s < 8; ++s)
+            tc::mma_bf16(tm, kdesc(sb + S_WK + 256u * s, kH), mdesc(sb + wl + 2u * 2048u * s, kH), idh, s > 0);
+          tc::commit(mbar);
           const uint32_t idw = tc::idesc_bf16(kH, kH) | (1u << 15) | (1u << 16);
           for (int s = 0; s < 8; ++s)
             tc::mma_bf16(tm + dw, mdesc(sb + S_WK + 2u * 2048u * s, kH), mdesc(sb + hprev + 2u * 2048u * s, kH), idw,
                          (acc0 | (s > 0)) ? 1u : 0u);
-          const uint32_t idh = tc::idesc_bf16(kT, kH) | (1u << 16);
-          for (int s = 0; s < 8; ++s)
-            tc::mma_bf16(tm, kdesc(sb + S_WK + 256u * s, kH), mdesc(sb + wl + 2u * 2048u * s, kH), idh, s > 0);
         } else {
           const uint32_t idw = tc::idesc_bf16(kH, kXin) | (1u << 15) | (1u << 16);
           for (int s = 0; s < 8; ++s)
             tc::mma_bf16(tm + TM_DW1, mdesc(sb + S_WK + 2u * 2048u * s, kH), mdesc(sb + S_X + 2u * 512u * s, kXin), idw,
                          (acc0 | (s > 0)) ? 1u : 0u);
+          tc::commit(mbar);
         }
       }
-      if (!sync_mma()) { alive = false; break; }
+      dbacc[l] += warp_colsum32(dh);   // (the column sums; dh is not used after)
       if (l == 0) break;
+      wait_mma();
       tc::ld32(lane_tm + (uint32_t)c0, dh);
-      tc::fence_before();
-      __syncthreads();
-      if (a.zst) continue;   // the stored variant reads z_{l-1} back
-      // z_{l-1} recomputed from the forward's own operands: h1 (hi + lo, the
-      // low terms regenerated above and still in S_WKLO) for layer 2, x (hi
-      // + lo) for layer 1
+      if (!(alive = to_mma())) break;
+      // z_{l-1} recomputed from the forward's own operands (h1 hi + lo, then
+      // x hi + lo) into the scratch accumulator; its commit covers dW_l too
       if (t == 0) {
         tc::fence_after();
-        const uint32_t id = tc::idesc_bf16(kT, kH);
-        if (l == 2) {
-          hidden_mma(1);
-        } else {
-          for (int s = 0; s < 2; ++s)
-            tc::mma_bf16(tm, kdesc(sb + S_X + 256u * s, kXin), kdesc(sb + S_WIN + 256u * s, kXin), id, s > 0);
+        if (!a.zst) {
+          if (l == 2) hidden_mma(1);
+          else input_mma();
         }
+        tc::commit(mbar);
       }
-      if (!sync_mma()) { alive = false; break; }
+      wait_mma();
+      {
+        float z[32], g[32];
+        load_z(tile, l - 1, z);
+        act_slopes(l - 1, z, g);
+#pragma unroll
+        for (int q = 0; q < 32; ++q) dh[q] *= g[q];
+      }
     }
+    if (!alive) break;
+    busy = true;
     ++tiles_done;
-    tc::fence_before();
-    __syncthreads();
   }
+  if (busy && alive) wait_mma();
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  alive = alive && *flag != 0;
   // ---------------- flush this CTA's partial gradients
   if (alive && a.mode != 0) {
     float* P = a.partial + (size_t)blockIdx.x * kPartial;
@@ -529,17 +594,20 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
       for (int q = t; q < kPartial; q += kNT) P[q] = 0.f;
     } else {
       float v[32];
+      auto put = [&](float* dst, int k) {   // k consecutive values of this thread (16-byte aligned)
+        for (int q = 0; q < k; q += 4) *(float4*)(dst + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
+      };
       // dW2, dW3: [128 out x 128 in]
       tc::ld32(lane_tm + TM_DW2 + (uint32_t)c0, v);
-      for (int q = 0; q < 32; ++q) P[kH * kXin + row * kH + c0 + q] = v[q];
+      put(P + kH * kXin + row * kH + c0, 32);
       tc::ld32(lane_tm + TM_DW3 + (uint32_t)c0, v);
-      for (int q = 0; q < 32; ++q) P[kH * kXin + kH * kH + row * kH + c0 + q] = v[q];
+      put(P + kH * kXin + kH * kH + row * kH + c0, 32);
       if (cg == 0) {
         tc::ld32(lane_tm + TM_DW1, v);  // [128 out x 32 (hi | lo)]
-        for (int q = 0; q < 32; ++q) P[row * kXin + q] = v[q];
-        float w4[16];
-        tc::ld16(lane_tm + TM_DW4, w4);  // [128 in x 16 out]
-        for (int q = 0; q < 16; ++q) P[kH * kXin + 2 * kH * kH + row * 16 + q] = w4[q];
+        put(P + row * kXin, 32);
+      } else if (cg == 1) {
+        tc::ld16(lane_tm + TM_DW4, v);  // [128 in x 16 out]
+        put(P + kH * kXin + 2 * kH * kH + row * 16, 16);
       }
       const int g = warp & 3;
       for (int l = 0; l < 3; ++l) P[kPDB + g * 400 + l * kH + c0 + lane] = dbacc[l];
@@ -557,36 +625,74 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
   if (warp == 0) tc::tmem_dealloc(tm, 512);
 }
 
+// s plus n values `stride` floats apart, added in order; sixteen loads are
+// in flight at a time (the sum is a chain of FP32 additions, the loads are not:
+// one at a time, the 152 partials cost as many round trips to L2).
+__device__ __forceinline__ float ordered_sum(float s, const float* __restrict__ p, int n, size_t stride) {
+  constexpr int kFly = 16;
+  float v[kFly];
+  for (int b = 0; b < n; b += kFly) {
+#pragma unroll
+    for (int q = 0; q < kFly; ++q) v[q] = b + q < n ? p[(size_t)(b + q) * stride] : 0.f;
+#pragma unroll
+    for (int q = 0; q < kFly; ++q)
+      if (b + q < n) s += v[q];
+  }
+  return s;
+}
+
 // Sum the per-CTA partials in CTA order; write gradients in the weight layout
-// (row-major per layer, then biases) and the loss.
-__global__ void k_train_reduce(const float* __restrict__ partial, int nblk, int d_in, float* __restrict__ grad,
-                               double* loss) {
+// (row-major per layer, then biases) and the loss.  One output per thread, a
+// warp for the loss; 16,384 threads with one load in flight each took 81 us
+// for 34,563 outputs of 128 CTAs.
+constexpr int kReduceThreads = 128;
+__global__ void __launch_bounds__(kReduceThreads) k_train_reduce(const float* __restrict__ partial, int nblk, int d_in,
+                                                                 float* __restrict__ grad, double* loss) {
   const int nw = kH * d_in + 2 * kH * kH + 3 * kH;
   const int nb = kNB;
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nw + nb + 1; q += gridDim.x * blockDim.x) {
-    float s = 0.f;
-    if (q < kH * d_in) {                       // W1[o][k] = hi column k + lo column 16 + k
-      const int o = q / d_in, k = q % d_in;
-      for (int b = 0; b < nblk; ++b) s += partial[(size_t)b * kPartial + o * kXin + k] + partial[(size_t)b * kPartial + o * kXin + 16 + k];
-    } else if (q < kH * d_in + 2 * kH * kH) {  // W2, W3
-      const int r = q - kH * d_in;
-      for (int b = 0; b < nblk; ++b) s += partial[(size_t)b * kPartial + kH * kXin + r];
-    } else if (q < nw) {                       // W4[o][k] = dW4^T[k][o]
-      const int r = q - kH * d_in - 2 * kH * kH, o = r / kH, k = r % kH;
-      for (int b = 0; b < nblk; ++b) s += partial[(size_t)b * kPartial + kH * kXin + 2 * kH * kH + k * 16 + o];
-    } else if (q < nw + nb) {                  // biases: lane groups 0..3 of every CTA, in order
-      const int r = q - nw;
-      for (int b = 0; b < nblk; ++b)
-        for (int g = 0; g < 4; ++g) s += partial[(size_t)b * kPartial + kPDB + g * 400 + r];
-    } else {
+  if (blockIdx.x == 0) {   // the loss: lane l the values l, l + 32, ... of [CTA][lane group], then a tree
+    if (threadIdx.x < 32) {
       double l = 0.0;
-      for (int b = 0; b < nblk; ++b)
-        for (int g = 0; g < 4; ++g) l += partial[(size_t)b * kPartial + kPLOSS + g];
-      if (loss) *loss = l;
-      continue;
+      for (int q = threadIdx.x; q < 4 * nblk; q += 32) l += partial[(size_t)(q >> 2) * kPartial + kPLOSS + (q & 3)];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+      if (threadIdx.x == 0 && loss) *loss = l;
     }
-    grad[q] = s;
+    return;
   }
+  const int q = (blockIdx.x - 1) * kReduceThreads + threadIdx.x;
+  if (q >= nw + nb) return;
+  float s = 0.f;
+  if (q < kH * d_in) {                       // W1[o][k] = hi column k + lo column 16 + k
+    const float* p = partial + (q / d_in) * kXin + q % d_in;
+    for (int b = 0; b < nblk; b += 8) {
+      float v[16];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        v[2 * r] = b + r < nblk ? p[(size_t)(b + r) * kPartial] : 0.f;
+        v[2 * r + 1] = b + r < nblk ? p[(size_t)(b + r) * kPartial + 16] : 0.f;
+      }
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+        if (b + r < nblk) s += v[2 * r] + v[2 * r + 1];
+    }
+  } else if (q < kH * d_in + 2 * kH * kH) {  // W2, W3
+    s = ordered_sum(s, partial + kH * kXin + (q - kH * d_in), nblk, kPartial);
+  } else if (q < nw) {                       // W4[o][k] = dW4^T[k][o]
+    const int r = q - kH * d_in - 2 * kH * kH, o = r / kH, k = r % kH;
+    s = ordered_sum(s, partial + kH * kXin + 2 * kH * kH + k * 16 + o, nblk, kPartial);
+  } else {                                   // biases: lane groups 0..3 of every CTA, in order
+    const float* p = partial + kPDB + (q - nw);
+    for (int b = 0; b < nblk; b += 4) {
+      float v[16];
+#pragma unroll
+      for (int r = 0; r < 16; ++r) v[r] = b + r / 4 < nblk ? p[(size_t)(b + r / 4) * kPartial + (r & 3) * 400] : 0.f;
+#pragma unroll
+      for (int r = 0; r < 16; ++r)
+        if (b + r / 4 < nblk) s += v[r];
+    }
+  }
+  grad[q] = s;
 }
 
 // Adam (Kingma & Ba 2015, Algorithm 1) on FP32 parameters theta = [weights, biases];
@@ -633,7 +739,9 @@ int launch_train(Ctx* c, const dsmc_mlp_t& mlp, int mode, uint64_t seed, uint64_
   k_train<<<blocks, kNT, S_TOTAL, s>>>(a);
   count_launches(c, 1);
   if (mode != 0) {
-    k_train_reduce<<<64, 256, 0, s>>>((const float*)ws, blocks, mlp.d_in, grad, loss);
+    const int outs = kH * mlp.d_in + 2 * kH * kH + 3 * kH + kNB;
+    k_train_reduce<<<1 + (outs + kReduceThreads - 1) / kReduceThreads, kReduceThreads, 0, s>>>(
+        (const float*)ws, blocks, mlp.d_in, grad, loss);
     count_launches(c, 1);
   }
   return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
