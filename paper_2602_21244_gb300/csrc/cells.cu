@@ -786,9 +786,94 @@ k_cells(int32_t n_cells, const int32_t* __restrict__ cs, double* vx, double* vy,
   }
 }
 
+// The same moments and matching for few cells: one group of 32 / SEG cells per
+// warp, SEG lanes each, without claims, and each lane's first kOnceHold
+// particles held in registers from the one read that serves the exponent, the
+// sums and the update.
+constexpr int kOnceHold = 4;
+
+template <bool MATCH, int SEG>
+__global__ void __launch_bounds__(kCwWarps * 32)
+k_cells_once(int32_t n_cells, const int32_t* __restrict__ cs, double* vx, double* vy, double* vz, double* mom,
+             int* status) {
+  const int lane = threadIdx.x & 31, sl = lane & (SEG - 1);
+  const int64_t k = ((int64_t)blockIdx.x * kCwWarps + (threadIdx.x >> 5)) * (32 / SEG) + lane / SEG;
+  const bool act = k < n_cells;
+  const int32_t a = act ? cs[k] : 0, b = act ? cs[k + 1] : 0, n = b - a;
+  double* mk = mom + 5 * (act ? k : 0);
+  double x[kOnceHold], y[kOnceHold], z[kOnceHold];
+  int E = 0;
+#pragma unroll
+  for (int u = 0; u < kOnceHold; ++u) {
+    const int32_t i = a + u * SEG + sl;
+    x[u] = y[u] = z[u] = 0.0;   // adds nothing to the sums
+    if (i < b) { x[u] = vx[i]; y[u] = vy[i]; z[u] = vz[i]; }
+  }
+#pragma unroll
+  for (int u = 0; u < kOnceHold; ++u) E = max(E, max(dexp(x[u]), max(dexp(y[u]), dexp(z[u]))));
+  for (int32_t i = a + kOnceHold * SEG + sl; i < b; i += SEG) E = max(E, max(dexp(vx[i]), max(dexp(vy[i]), dexp(vz[i]))));
+  E = seg_max_i<SEG>(E);
+  const int Ec = E + cell_scale(E, n).c, sp = fix_split(n);
+  FixAcc q{0, 0, 0, 0ull, 0ull, 0ull};
+#pragma unroll
+  for (int u = 0; u < kOnceHold; ++u) {
+    fix_add(q, q.sx, x[u], Ec, sp);
+    fix_add(q, q.sy, y[u], Ec, sp);
+    fix_add(q, q.sz, z[u], Ec, sp);
+  }
+  for (int32_t i = a + kOnceHold * SEG + sl; i < b; i += SEG) {
+    fix_add(q, q.sx, vx[i], Ec, sp);
+    fix_add(q, q.sy, vy[i], Ec, sp);
+    fix_add(q, q.sz, vz[i], Ec, sp);
+  }
+  const CellFix C = cellfix_from(E, n, seg_sum_acc<SEG>(q));
+  if (!MATCH) {
+    if (act && sl < 5) moment_store(C, n, sl, mk, status);
+  } else {
+    double alpha, o;
+    match_coeffs(C, n, sl, mk, &alpha, &o);
+    const int l0 = lane & ~(SEG - 1);
+    const double ox = __shfl_sync(0xffffffffu, o, l0), oy = __shfl_sync(0xffffffffu, o, l0 + 1),
+                 oz = __shfl_sync(0xffffffffu, o, l0 + 2);
+#pragma unroll
+    for (int u = 0; u < kOnceHold; ++u) {
+      const int32_t i = a + u * SEG + sl;
+      if (i < b) { vx[i] = fma(alpha, x[u], ox); vy[i] = fma(alpha, y[u], oy); vz[i] = fma(alpha, z[u], oz); }
+    }
+    for (int32_t i = a + kOnceHold * SEG + sl; i < b; i += SEG) {
+      vx[i] = fma(alpha, vx[i], ox);
+      vy[i] = fma(alpha, vy[i], oy);
+      vz[i] = fma(alpha, vz[i], oz);
+    }
+  }
+}
+
+// Which kernel: the claiming kernel's chain of two claims, two passes over
+// memory and the batched remainder takes 18 us (moments) and 25 to 29 us
+// (matching) however few cells there are; one group per warp takes 9 and 9 to
+// 10 us (launch overhead included) at 100 to 2,867 cells, 22.7 against 26.2 us
+// (moments) at 40,000 cells of 20 particles and 40.5 against 46.4 us at 37,500 of 61, but from then on its FP64
+// remainder, paid per group of 4 cells instead of 16, costs more (matching
+// 18.5 against 25.2 us at 10,000 cells, 43.2 against 39.1 us at 40,000; at
+// 150,000 cells 113 against 100 us and 240 against 175 us).  32 lanes per
+// cell for up to 8 cells per SM (1,000 cells of 50: 9.5 against 12.3 us).
 static int launch_cells(Ctx* c, bool match, int32_t n_cells, const int32_t* cs, double* vx, double* vy,
                         double* vz, double* mom, cudaStream_t s) {
   if (n_cells <= 0) return 0;
+  if (n_cells <= (match ? 128 : 320) * sm_count(c)) {
+    const int seg = n_cells <= 8 * sm_count(c) ? 32 : 8;
+    const unsigned gb = grid_for(n_cells, kCwWarps * 32 / seg, INT_MAX);
+    int* st = status_ptr(c);
+    if (match) {
+      if (seg == 32) k_cells_once<true, 32><<<gb, kCwWarps * 32, 0, s>>>(n_cells, cs, vx, vy, vz, mom, st);
+      else k_cells_once<true, 8><<<gb, kCwWarps * 32, 0, s>>>(n_cells, cs, vx, vy, vz, mom, st);
+    } else {
+      if (seg == 32) k_cells_once<false, 32><<<gb, kCwWarps * 32, 0, s>>>(n_cells, cs, vx, vy, vz, mom, st);
+      else k_cells_once<false, 8><<<gb, kCwWarps * 32, 0, s>>>(n_cells, cs, vx, vy, vz, mom, st);
+    }
+    count_launches(c, 1);
+    return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
+  }
   const Shape sh = shape_or_default(c, match ? DSMC_TUNE_MOMENT_MATCH : DSMC_TUNE_MOMENTS);
   const int64_t runs = ((int64_t)n_cells + kCwRun - 1) / kCwRun;
   const unsigned g = grid_for(runs, kCwWarps * kCwClaims, sm_count(c) * sh.blocks_per_sm);
