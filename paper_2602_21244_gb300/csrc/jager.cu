@@ -19,6 +19,7 @@
 //     (1 - u^k = s^2 (1 + u + ... + u^(k-1)), expm1) so that it keeps FP32
 //     relative accuracy as r -> r_min.
 #include <cmath>
+#include <cstring>
 #include <mutex>
 #include <vector>
 
@@ -319,6 +320,9 @@ struct Turn {
 // times, and the warp is reconverged before the FP64 steps, which then run
 // for all lanes as long as any lane still refines (GB300's FP64 pipe costs a
 // warp instruction however few lanes are active).
+constexpr int kScanSteps = 4000;   // a multiple of 32
+constexpr int kScanShared = 20;    // fine scans a warp shares (more run side by side)
+
 template <bool kWarp>
 __device__ Turn rmin_device(const PotDev& P, float b, float E) {
   Turn T = {};
@@ -332,14 +336,52 @@ __device__ Turn rmin_device(const PotDev& P, float b, float E) {
   float r_hi;
   if (P.kind == 0) r_hi = fmaxf(b, P.sigma0) * 1.000001f;
   else r_hi = fmaxf(b, __powf(P.fkappa / E, 1.f / P.fp)) * 2.f;
-  const float q = (P.kind == 0 && E < P.orbit_E) ? 0.995f : 0.9f;
+  const bool fine = P.kind == 0 && E < P.orbit_E;
+  const float q = fine ? 0.995f : 0.9f;
   float r_lo = r_hi;
   bool found = false;
-  for (int t = 0; t < 4000; ++t) {
-    r_lo = r_hi * q;
-    if (F32(P, b2, E, r_lo, &dF) < 0.f) { found = true; break; }
-    r_hi = r_lo;
-    if (r_hi < 1e-3f) break;
+  auto scan = [&]() {
+    for (int t = 0; t < kScanSteps; ++t) {
+      r_lo = r_hi * q;
+      if (F32(P, b2, E, r_lo, &dF) < 0.f) { found = true; break; }
+      r_hi = r_lo;
+      if (r_hi < 1e-3f) break;
+    }
+  };
+  if (!kWarp) {
+    scan();
+  } else {
+    // the lanes with coarse steps scan side by side; a fine scan, up to a few
+    // hundred steps that most lanes do not need, is shared by the warp while
+    // few lanes need it: 32 steps at a time, one per lane
+    const unsigned fm = __ballot_sync(0xffffffffu, fine);
+    const bool shared = __popc(fm) <= kScanShared;
+    if (!fine || !shared) scan();
+    __syncwarp();
+    for (unsigned left = shared ? fm : 0u; left; left &= left - 1u) {
+      const int owner = __ffs(left) - 1, lane = threadIdx.x & 31;
+      const float ob2 = __shfl_sync(0xffffffffu, b2, owner), oE = __shfl_sync(0xffffffffu, E, owner);
+      float r = __shfl_sync(0xffffffffu, r_hi, owner), olo = r, ohi = r;
+      bool neg = false;
+      for (int t = 0; t < kScanSteps; t += 32) {
+        // lane k: the end points of step t + k, the products formed one after
+        // another as the scan forms them
+        float prev = r, mine = r;
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+          if (i <= lane) { prev = mine; mine = mine * 0.995f; }
+        float dFx;
+        const bool n = F32(P, ob2, oE, mine, &dFx) < 0.f;
+        const unsigned stop = __ballot_sync(0xffffffffu, n || mine < 1e-3f);
+        const int at = stop ? __ffs(stop) - 1 : 31;
+        neg = stop && __shfl_sync(0xffffffffu, (int)n, at);
+        olo = __shfl_sync(0xffffffffu, mine, at);
+        ohi = neg ? __shfl_sync(0xffffffffu, prev, at) : olo;
+        if (stop) break;
+        r = olo;
+      }
+      if (lane == owner) { found = neg; r_lo = olo; r_hi = ohi; }
+    }
   }
   const float r_nf = r_hi;   // the result when no sign change was found
   if (!kWarp && !found) {
@@ -422,9 +464,102 @@ __device__ Turn rmin_device(const PotDev& P, float b, float E) {
 }
 
 // ---------------------------------------------------------------- chi
-// kWarp: see rmin_device (every lane of the warp calls it together).
+// What the integrand needs of a quadrature node alone: s, w = 1 - u = s^2,
+// u, the weight factor 2 w_q s, and G_k = 1 + u + ... + u^(k-1) for k =
+// 1..16 (r^-k - r0^-k = -r0^-k w G_k).  Formed once per block in shared
+// memory; forming the G_k of every node for every pair was a fifth of the
+// quadrature's instructions.
+constexpr int kRowWords = 20;
+
+// A block's shared memory: the rows of both node sets (n_nodes, then n_low),
+// then per warp the parameters and the integrand of up to kOwners pairs whose
+// nodes the warp shares.
+constexpr int kOwners = 8, kParWords = 32, kTermStride = kMaxNodes + 4;
+constexpr int kWarpWords = kOwners * (kParWords + kTermStride);
+constexpr size_t chi_smem(int threads) {
+  return sizeof(float) * (size_t)(2 * kMaxNodes * kRowWords + threads / 32 * kWarpWords);
+}
+
+struct ChiShared {
+  const float* rows;
+  float *par, *term;   // this warp's
+};
+
+// Called by the whole block (with a barrier) before the first chi_device<true>.
+__device__ __forceinline__ ChiShared chi_shared(const PotDev& P, float* sm) {
+  for (int i = threadIdx.x; i < P.n_nodes + P.n_low; i += blockDim.x) {
+    const int q = i < P.n_nodes ? i : kMaxNodes + i - P.n_nodes;
+    const float s = P.s_node[q];
+    const float w = s * s;          // 1 - u, exact
+    const float u = 1.f - w;
+    float* row = sm + i * kRowWords;
+    row[0] = s; row[1] = w; row[2] = u; row[3] = P.w_node[q] * 2.f * s;
+    float Gk = 0.f, uk = 1.f;
+#pragma unroll
+    for (int k = 1; k <= 16; ++k) {
+      Gk += uk;
+      uk *= u;
+      row[3 + k] = Gk;
+    }
+  }
+  __syncthreads();
+  float* mine = sm + 2 * kMaxNodes * kRowWords + (threadIdx.x >> 5) * kWarpWords;
+  return ChiShared{sm, mine, mine + kOwners * kParWords};
+}
+
+// The pair's coefficients about its turning point (Jager form).
+struct PairCoef {
+  float d[17], qn[6], r0, Rep0, e0, P0, bt2, iE, F0;
+};
+
+// The integrand at one node, without the weight factor.
+__device__ __forceinline__ float node_term(const PotDev& P, const PairCoef& c, const float* rowp) {
+  const float4* row = (const float4*)rowp;
+  const float4 h = row[0];
+  const float w = h.y, u = h.z;
+  float G16[16];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float4 g = row[1 + k];
+    G16[4 * k] = g.x; G16[4 * k + 1] = g.y; G16[4 * k + 2] = g.z; G16[4 * k + 3] = g.w;
+  }
+  const float r0 = c.r0;
+  const float dr = r0 * w / u;    // r - r0
+  const float r = r0 + dr;
+  // repulsion: Rep0 * expm1(poly(r) - poly(r0))
+  const float dpoly = dr * (P.fa1 + P.fa2 * (r + r0) - P.fam1 / (r * r0) -
+                            P.fam2 * (r + r0) / (r * r * r0 * r0));
+  const float drep = c.Rep0 * expm1f(dpoly);
+  float dQ = 0.f, dP = 0.f;
+#pragma unroll
+  for (int k = 1; k <= 16; ++k) {
+    dP += c.d[k] * G16[k - 1];
+    if ((k & 1) == 0 && k >= 6) dQ += c.qn[(k - 6) >> 1] * G16[k - 1];
+  }
+  dQ *= -w;                     // sum_n C (r^-2n - r0^-2n)
+  dP *= -w;                     // P(r) - P(r0)
+  const float dh = c.e0 * (expm1f(-P.fbeta * dr) * (c.P0 + dP) + dP);
+  const float dV = drep - dQ + dh;
+  const float G0 = c.bt2 * w * (1.f + u);
+  const float dG = dV * c.iE - c.F0;
+  const float G = fmaxf(G0 - dG, 1e-30f);
+  const float rG = rsqrtf(G), rG0 = rsqrtf(G0);
+  return dG * rG * rG0 / (G * rG + G0 * rG0);
+}
+
+constexpr int kLongShared = 28;   // pairs with the long rule that a warp shares (more run side by side)
+
+// kWarp: see rmin_device (every lane of the warp calls it together, with the
+// block's ChiShared).  Then the pairs with the short rule run side by side,
+// and the nodes of a pair with the long rule (below orbit_E) are spread over
+// the warp's lanes, four each, the integrand summed by the pair's own lane in
+// the order of the nodes: one such pair in a warp used to hold the other lanes
+// for the long rule's 128 nodes (of the chi batch's pairs, a twelfth of them with the
+// long rule, 95 % of the warps did).  2^22 pairs of that batch: 4.00 -> 2.55
+// ms, bit-identical; what is left is the FP64 refinement (111 FP64
+// instructions per warp at 19 cycles: 0.9 ms) and the FP32 instructions.
 template <bool kWarp = false>
-__device__ float chi_device(const PotDev& P, float b_in, float E) {
+__device__ float chi_device(const PotDev& P, float b_in, float E, ChiShared S = ChiShared{}) {
   if (!kWarp && !(b_in > 0.f)) return (float)DSMC_PI;
   const float b = b_in > 0.f ? b_in : 1.f;   // b = 0: head-on, chi = pi (set at the end)
   const Turn Tp = rmin_device<kWarp>(P, b, E);
@@ -437,7 +572,14 @@ __device__ float chi_device(const PotDev& P, float b_in, float E) {
   if (P.kind == 1) F0 = 1.f - bt2;
   // per-pair coefficients about the FP64 turning point (Jager form), so that
   // the integrand's F(r_min) = 0 holds to FP64 rather than to FP32 rounding
-  float d[17], qn[6], Rep0 = 0.f, e0 = 0.f, P0 = 0.f, Vc0 = 0.f, powk = 0.f;
+  PairCoef cf;
+  float (&d)[17] = cf.d, (&qn)[6] = cf.qn;
+  float& Rep0 = cf.Rep0;
+  float& e0 = cf.e0;
+  float& P0 = cf.P0;
+  Rep0 = e0 = P0 = 0.f;
+  cf.r0 = r0; cf.bt2 = bt2; cf.iE = iE; cf.F0 = F0;
+  float Vc0 = 0.f, powk = 0.f;
   const bool core = P.kind == 0 && r0 < P.frc;
   if (P.kind == 0 && !core) {
     // d_p = D_p r0^-p and the dispersion coefficients C_2n r0^-2n, each the
@@ -464,6 +606,52 @@ __device__ float chi_device(const PotDev& P, float b_in, float E) {
   if (core) { double dd; V0d = V64(P, rd, &dd); }
   float I = 0.f;
   const bool low = P.kind == 0 && E < P.orbit_E;
+  if (kWarp && P.kind == 0) {
+    const int lane = threadIdx.x & 31;
+    unsigned lm = __ballot_sync(0xffffffffu, low && !core);
+    const bool shared = __popc(lm) <= kLongShared;
+    if (!core && !(low && shared)) {
+      const float* row = S.rows + (low ? P.n_nodes * kRowWords : 0);
+      for (int q = low ? P.n_low : P.n_nodes; q > 0; --q, row += kRowWords) I += row[3] * node_term(P, cf, row);
+    }
+    __syncwarp();
+    if (!shared) lm = 0u;
+    while (lm) {
+      const int cnt = min(kOwners, __popc(lm)), rank = __popc(lm & ((1u << lane) - 1u));
+      const bool mine = ((lm >> lane) & 1u) && rank < cnt;
+      if (mine) {
+        float4* o = (float4*)(S.par + rank * kParWords);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) o[k] = make_float4(d[4 * k + 1], d[4 * k + 2], d[4 * k + 3], d[4 * k + 4]);
+        o[4] = make_float4(qn[0], qn[1], qn[2], qn[3]);
+        o[5] = make_float4(qn[4], qn[5], r0, Rep0);
+        o[6] = make_float4(e0, P0, bt2, iE);
+      }
+      __syncwarp();
+      const float* lrows = S.rows + P.n_nodes * kRowWords;
+      for (int o = 0; o < cnt; ++o) {
+        const float4* v = (const float4*)(S.par + o * kParWords);
+        PairCoef c;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float4 x = v[k];
+          c.d[4 * k + 1] = x.x; c.d[4 * k + 2] = x.y; c.d[4 * k + 3] = x.z; c.d[4 * k + 4] = x.w;
+        }
+        const float4 x4 = v[4], x5 = v[5], x6 = v[6];
+        c.qn[0] = x4.x; c.qn[1] = x4.y; c.qn[2] = x4.z; c.qn[3] = x4.w;
+        c.qn[4] = x5.x; c.qn[5] = x5.y; c.r0 = x5.z; c.Rep0 = x5.w;
+        c.e0 = x6.x; c.P0 = x6.y; c.bt2 = x6.z; c.iE = x6.w;
+        c.F0 = F0;   // 0 for the Jager form
+        for (int q = lane; q < P.n_low; q += 32) S.term[o * kTermStride + q] = node_term(P, c, lrows + q * kRowWords);
+      }
+      __syncwarp();
+      if (mine)
+        for (int q = 0; q < P.n_low; ++q) I += lrows[q * kRowWords + 3] * S.term[rank * kTermStride + q];
+      __syncwarp();
+      for (int o = 0; o < cnt; ++o) lm &= lm - 1u;
+    }
+    if (!core) return b_in > 0.f ? -2.f * bt * I : (float)DSMC_PI;
+  }
   const int q0 = low ? kMaxNodes : 0, q1 = q0 + (low ? P.n_low : P.n_nodes);
   for (int q = q0; q < q1; ++q) {
     const float s = P.s_node[q];
@@ -530,7 +718,7 @@ static void gauss_legendre01(int n, double* x, double* w) {
   }
 }
 
-static PotDev make_pot(const dsmc_gas_t& gas, const dsmc_potential_t& p, int n_nodes) {
+static PotDev build_pot(double mass, const dsmc_potential_t& p, int n_nodes) {
   PotDev P = {};
   P.kind = p.kind;
   P.n_nodes = n_nodes;
@@ -541,7 +729,7 @@ static PotDev make_pot(const dsmc_gas_t& gas, const dsmc_potential_t& p, int n_n
   P.fam2 = (float)p.am2; P.fbeta = (float)p.beta; P.frc = (float)P.rc; P.fAt = (float)p.At;
   P.fat = (float)p.at;
   P.d_hs = p.d_hs; P.kappa = p.kappa; P.p = p.p; P.fkappa = (float)p.kappa; P.fp = (float)p.p;
-  P.mass_over_4k = (float)(gas.mass / (4.0 * DSMC_KB));
+  P.mass_over_4k = (float)(mass / (4.0 * DSMC_KB));
   P.ex64 = make_exp64();
   // D_p = sum_{n: 2n >= p} C_2n beta^(2n-p) / (2n-p)!
   for (int pp = 0; pp <= 16; ++pp) {
@@ -587,11 +775,41 @@ static PotDev make_pot(const dsmc_gas_t& gas, const dsmc_potential_t& p, int n_n
   return P;
 }
 
+// The constants above of a (mass, potential, node count).  Building them (the
+// Gauss-Legendre rules, the zero and the depth of V) takes the host about 0.4
+// ms, so the last few are kept, found by the values they were built from.
+static PotDev make_pot(const dsmc_gas_t& gas, const dsmc_potential_t& p, int n_nodes) {
+  struct Kept {
+    double mass;
+    dsmc_potential_t p;
+    int n_nodes = 0;
+    PotDev P;
+  };
+  constexpr int kKept = 8;
+  static std::mutex mu;
+  static Kept kept[kKept];
+  static int next = 0;
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    for (const Kept& k : kept)
+      if (k.n_nodes == n_nodes && memcmp(&k.mass, &gas.mass, sizeof(double)) == 0 && memcmp(&k.p, &p, sizeof(p)) == 0)
+        return k.P;
+  }
+  const PotDev P = build_pot(gas.mass, p, n_nodes);
+  std::lock_guard<std::mutex> lock(mu);
+  Kept& k = kept[next];
+  next = (next + 1) % kKept;
+  k.mass = gas.mass; k.p = p; k.n_nodes = n_nodes; k.P = P;
+  return P;
+}
+
 // ---------------------------------------------------------------- kernels
 // Warp-uniform loop: every lane of a warp computes chi together (a lane past
 // the end, or with g = 0, on harmless inputs whose result is not kept).
-__global__ void __launch_bounds__(128) k_jager_chi(PotDev P, int64_t n, const float* __restrict__ b,
-                                                   const float* __restrict__ g, float* __restrict__ chi) {
+__global__ void __launch_bounds__(128, 4) k_jager_chi(PotDev P, int64_t n, const float* __restrict__ b,
+                                                      const float* __restrict__ g, float* __restrict__ chi) {
+  extern __shared__ float4 chi_sm[];
+  const ChiShared S = chi_shared(P, (float*)chi_sm);
   const int lane = threadIdx.x & 31;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
@@ -599,7 +817,7 @@ __global__ void __launch_bounds__(128) k_jager_chi(PotDev P, int64_t n, const fl
     const bool valid = q < n;
     const float gg = valid ? g[q] : 0.f;
     const bool use = valid && gg > 0.f;
-    const float c = chi_device<true>(P, use ? b[q] : 1.f, use ? P.mass_over_4k * gg * gg : 1.0e4f);
+    const float c = chi_device<true>(P, use ? b[q] : 1.f, use ? P.mass_over_4k * gg * gg : 1.0e4f, S);
     if (valid) chi[q] = use ? c : 0.f;
   }
 }
@@ -661,7 +879,8 @@ struct JagerArgs {
 // it together (live false: a lane with no pair, or whose dependency wait
 // failed, computes on harmless inputs and stores nothing), so that chi's FP64
 // refinement and the FP64 rotation run with the warp converged.
-__device__ __forceinline__ void collide_pair(const PotDev& P, const JagerArgs& a, int64_t p, int4 q, bool live) {
+__device__ __forceinline__ void collide_pair(const PotDev& P, const ChiShared& S, const JagerArgs& a, int64_t p,
+                                             int4 q, bool live) {
   double xi = 0.0, yi = 0.0, zi = 0.0, xj = 0.0, yj = 0.0, zj = 0.0;
   if (live) {
     xi = __ldcg(a.vx + q.x); yi = __ldcg(a.vy + q.x); zi = __ldcg(a.vz + q.x);
@@ -673,7 +892,7 @@ __device__ __forceinline__ void collide_pair(const PotDev& P, const JagerArgs& a
   const u32x4 w = draw(a.seed, (uint32_t)q.w, (uint32_t)q.z, a.step, TAG_JAGER);
   const float b = use ? f64_to_f32(a.bmax_A * sqrt64(u53_int(w.x, w.y))) : 1.f;
   const float E = use ? P.mass_over_4k * f64_to_f32(g2) : 1.0e4f;
-  const float chi_c = chi_device<true>(P, b, E);
+  const float chi_c = chi_device<true>(P, b, E, S);
   const float chi = use ? chi_c : 0.f;
   if (live && a.chi_out) a.chi_out[p] = chi;
   __syncwarp();
@@ -701,6 +920,8 @@ __device__ __forceinline__ void collide_pair(const PotDev& P, const JagerArgs& a
 // pair does not change its result.
 __global__ void __launch_bounds__(128, 4) k_collide_jager(PotDev P, JagerArgs a) {
   if (a.step_dev) a.step = *a.step_dev;
+  extern __shared__ float4 chi_sm[];
+  const ChiShared S = chi_shared(P, (float*)chi_sm);
   const int R = a.info->n_rounds;
   const int lane = threadIdx.x & 31;
   int r = 0;
@@ -720,7 +941,7 @@ __global__ void __launch_bounds__(128, 4) k_collide_jager(PotDev P, JagerArgs a)
       ok = wait_deps(a.done, q.x, q.y, a.deps[p], a.bar + 2, a.status);
     }
     __syncwarp();
-    collide_pair(P, a, p, q, valid && ok);
+    collide_pair(P, S, a, p, q, valid && ok);
     if (valid && ok) release_pair(a.done, q.x, q.y, (unsigned)(r + 1));
     if (!__all_sync(0xffffffffu, ok)) break;
   }
@@ -870,7 +1091,8 @@ int launch_jager_chi(Ctx* c, const dsmc_gas_t& gas, const dsmc_potential_t& pot,
   if (n == 0) return 0;
   const PotDev P = make_pot(gas, pot, n_nodes);
   const Shape sh = shape_or_default(c, DSMC_TUNE_JAGER_CHI);
-  k_jager_chi<<<blocks_n(n, sh.threads, sm_count(c) * sh.blocks_per_sm), sh.threads, 0, s>>>(P, n, b, g, chi);
+  k_jager_chi<<<blocks_n(n, sh.threads, sm_count(c) * sh.blocks_per_sm), sh.threads, chi_smem(sh.threads), s>>>(
+      P, n, b, g, chi);
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
 }
@@ -878,7 +1100,8 @@ int launch_jager_chi(Ctx* c, const dsmc_gas_t& gas, const dsmc_potential_t& pot,
 // resident blocks per SM of the Jager collide at a block size (0 on failure)
 int occupancy_collide_jager(int threads) {
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)k_collide_jager, threads, 0) != cudaSuccess)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)k_collide_jager, threads,
+                                                    chi_smem(threads)) != cudaSuccess)
     return 0;
   return per_sm;
 }
@@ -898,7 +1121,7 @@ int launch_collide_jager(Ctx* c, const dsmc_gas_t& gas, const dsmc_potential_t& 
   if (cudaMemsetAsync(a.bar, 0, 4 * sizeof(unsigned), s) != cudaSuccess ||
       cudaMemsetAsync(a.done, 0, sizeof(unsigned) * (size_t)(n > 0 ? n : 1), s) != cudaSuccess)
     return DSMC_ERR_CUDA;
-  k_collide_jager<<<blocks, sh.threads, 0, s>>>(P, a);
+  k_collide_jager<<<blocks, sh.threads, chi_smem(sh.threads), s>>>(P, a);
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : record(c, DSMC_ERR_CUDA, "collide_jager: launch failed");
 }

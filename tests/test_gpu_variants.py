@@ -50,3 +50,32 @@ def test_one_group_per_warp_moments_report_nonfinite():
     v[1][3] = np.nan
     C.cell_moments(cuda(cs), *[cuda(c) for c in v])
     assert C.sync_status() == D.DSMC_ERR_NONFINITE
+
+
+@pytest.mark.parametrize("n_nodes", [8, 33, 128])
+def test_chi_does_not_depend_on_the_warp_it_runs_in(n_nodes):
+    """The chi batch shares the bracket scan and the nodes of a warp's low-energy pairs between its lanes
+    while few of them are low; the sums keep the order of the nodes, so a pair's chi is the same bits in
+    warps of any mix (0, 1, 8, 9, 20, 21, 28, 29 and 32 low pairs), with head-on, motionless and
+    core-penetrating pairs among them, and in a batch that ends inside a warp."""
+    from paper_2602_21244_gb300 import dsmc as D
+    from paper_2602_21244_gb300 import workloads as W
+    C = ctx()
+    gas = D.make_gas(dict(mass=W.M_AR, fn_over_vc=1.0, dt=1.0, model=1, b_max=1.2e-9))
+    pot = D.make_potential(W.JAGER_SYNTHETIC_AR)
+    rng = np.random.default_rng(n_nodes)
+    g, b = [], []
+    for low in (0, 1, 8, 9, 20, 21, 28, 29, 32, 3):
+        gg = np.where(rng.permutation(32) < low, rng.uniform(100, 400, 32), rng.uniform(500, 15000, 32))
+        g.append(gg)
+        b.append(12.0 * np.sqrt(rng.random(32)))
+    g, b = (np.concatenate(a).astype(np.float32)[:-5] for a in (g, b))
+    g[40], g[41], b[42], g[70], b[70] = 0.0, 9.0e4, 0.0, 9.0e4, 0.5
+    whole = host(C.jager_chi(gas, pot, cuda(b), cuda(g), n_nodes=n_nodes))
+    assert C.sync_status() == 0 and np.isfinite(whole).all() and whole[42] == np.float32(np.pi) and whole[40] == 0
+    for order in (np.argsort(g), rng.permutation(len(g))):
+        again = host(C.jager_chi(gas, pot, cuda(b[order]), cuda(g[order]), n_nodes=n_nodes))
+        assert np.array_equal(again, whole[order])
+    one = [float(host(C.jager_chi(gas, pot, cuda(b[q:q + 1]), cuda(g[q:q + 1]), n_nodes=n_nodes))[0])
+           for q in range(0, len(g), 7)]
+    assert np.array_equal(np.float32(one), whole[::7])
