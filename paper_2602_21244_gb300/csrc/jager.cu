@@ -177,12 +177,13 @@ __host__ __device__ inline double V64(const PotDev& P, double r, double* dV, dou
 // *ex receive A e^{poly} and e^{-beta r}, *Pr the damping polynomial P(r)
 // (Jager form), from which the quadrature's coefficients are carried to the
 // root, *dPr P'(r) and *dpoly poly'(r) in FP32 for that carry.
+template <int KIND>
 __device__ __forceinline__ double V64n(const PotDev& P, double r, double ir, float* dV, double* rep_out,
                                        double* ex_out, double* Pr_out, float* dPr_out, float* dpoly_out) {
   const double ir2 = ir * ir;
   *dPr_out = 0.f;
   *dpoly_out = 0.f;
-  if (P.kind == 2) {
+  if ((KIND >= 0 ? KIND : P.kind) == 2) {
     const double v = P.kappa * pow(r, -P.p);
     *dV = f64_to_f32(-P.p * v * ir);
     return v;
@@ -252,9 +253,11 @@ __device__ __forceinline__ double sqrt64(double x) {
 
 // ---------------------------------------------------------------- FP32 potential
 // V = A e^{poly} - sum_n C_2n r^-2n + e^{-beta r} sum_p D_p r^-p  (r >= rc)
+template <int KIND>
 __device__ __forceinline__ float V32(const PotDev& P, float r, float* dV) {
-  if (P.kind == 1) { *dV = 0.f; return 0.f; }
-  if (P.kind == 2) {
+  const int kind = KIND >= 0 ? KIND : P.kind;
+  if (kind == 1) { *dV = 0.f; return 0.f; }
+  if (kind == 2) {
     const float v = P.fkappa * __powf(r, -P.fp);
     *dV = -P.fp * v / r;
     return v;
@@ -287,9 +290,10 @@ __device__ __forceinline__ float V32(const PotDev& P, float r, float* dV) {
   return rep - q + eb * Pr;
 }
 
+template <int KIND>
 __device__ __forceinline__ float F32(const PotDev& P, float b2, float E, float r, float* dF) {
   float dV;
-  const float V = V32(P, r, &dV);
+  const float V = V32<KIND>(P, r, &dV);
   const float ir2 = 1.f / (r * r);
   *dF = 2.f * b2 * ir2 / r - dV / E;
   return 1.f - b2 * ir2 - V / E;
@@ -323,10 +327,14 @@ struct Turn {
 constexpr int kScanSteps = 4000;   // a multiple of 32
 constexpr int kScanShared = 20;    // fine scans a warp shares (more run side by side)
 
-template <bool kWarp>
+// KIND: the potential's kind when the kernel is compiled for it (the other
+// kinds' code, FP64 pow among it, then does not spread the hot loops over the
+// instruction cache), or -1.
+template <bool kWarp, int KIND>
 __device__ Turn rmin_device(const PotDev& P, float b, float E) {
   Turn T = {};
-  if (P.kind == 1) {   // the same kind for every lane
+  const int kind = KIND >= 0 ? KIND : P.kind;
+  if (kind == 1) {   // the same kind for every lane
     T.r = (double)fmaxf(b, (float)P.d_hs);
     T.ir = rcp64(T.r);
     return T;
@@ -334,16 +342,16 @@ __device__ Turn rmin_device(const PotDev& P, float b, float E) {
   const float b2 = b * b;
   float dF;
   float r_hi;
-  if (P.kind == 0) r_hi = fmaxf(b, P.sigma0) * 1.000001f;
+  if (kind == 0) r_hi = fmaxf(b, P.sigma0) * 1.000001f;
   else r_hi = fmaxf(b, __powf(P.fkappa / E, 1.f / P.fp)) * 2.f;
-  const bool fine = P.kind == 0 && E < P.orbit_E;
+  const bool fine = kind == 0 && E < P.orbit_E;
   const float q = fine ? 0.995f : 0.9f;
   float r_lo = r_hi;
   bool found = false;
   auto scan = [&]() {
     for (int t = 0; t < kScanSteps; ++t) {
       r_lo = r_hi * q;
-      if (F32(P, b2, E, r_lo, &dF) < 0.f) { found = true; break; }
+      if (F32<KIND>(P, b2, E, r_lo, &dF) < 0.f) { found = true; break; }
       r_hi = r_lo;
       if (r_hi < 1e-3f) break;
     }
@@ -367,11 +375,11 @@ __device__ Turn rmin_device(const PotDev& P, float b, float E) {
         // lane k: the end points of step t + k, the products formed one after
         // another as the scan forms them
         float prev = r, mine = r;
-#pragma unroll
+#pragma unroll 8
         for (int i = 0; i < 32; ++i)
           if (i <= lane) { prev = mine; mine = mine * 0.995f; }
         float dFx;
-        const bool n = F32(P, ob2, oE, mine, &dFx) < 0.f;
+        const bool n = F32<KIND>(P, ob2, oE, mine, &dFx) < 0.f;
         const unsigned stop = __ballot_sync(0xffffffffu, n || mine < 1e-3f);
         const int at = stop ? __ffs(stop) - 1 : 31;
         neg = stop && __shfl_sync(0xffffffffu, (int)n, at);
@@ -394,7 +402,7 @@ __device__ Turn rmin_device(const PotDev& P, float b, float E) {
   // ends the iteration even when it lands on a bracket end.
   float r = r_hi;
   for (int it = 0; it < 24 && found; ++it) {
-    const float f = F32(P, b2, E, r, &dF);
+    const float f = F32<KIND>(P, b2, E, r, &dF);
     if (f == 0.f) break;
     if (f < 0.f) r_lo = r; else r_hi = r;
     float rn = r - f / dF;
@@ -416,7 +424,7 @@ __device__ Turn rmin_device(const PotDev& P, float b, float E) {
     if (kWarp ? !__any_sync(0xffffffffu, act) : !act) break;
     float dV, ppf;
     const double ir2 = ir * ir;
-    const double V = V64n(P, rd, ir, &dV, &rep0, &ex0, &Pr0, &dPr0, &ppf);
+    const double V = V64n<KIND>(P, rd, ir, &dV, &rep0, &ex0, &Pr0, &dPr0, &ppf);
     const double f = 1.0 - bd2 * ir2 - V * iEd;
     // F'(r) in FP32 (see V64n)
     const float irf = f64_to_f32(ir);
@@ -449,7 +457,7 @@ __device__ Turn rmin_device(const PotDev& P, float b, float E) {
   }
   T.r = rd;
   T.ir = ir;
-  if (P.kind == 0 && rd >= P.rc) {
+  if (kind == 0 && rd >= P.rc) {
     if (fabs(dr) <= 1e-4 * rd) {
       const double eb = -P.beta * dr;
       T.rep = rep0 * (1.0 + dpoly * (1.0 + 0.5 * dpoly));
@@ -457,14 +465,14 @@ __device__ Turn rmin_device(const PotDev& P, float b, float E) {
       T.Pr = fma(f32_to_f64(dPr0), dr, Pr0);
     } else {  // a long last step (not converged): evaluate at rd
       float dV, dPr, ppf;
-      V64n(P, rd, ir, &dV, &T.rep, &T.ex, &T.Pr, &dPr, &ppf);
+      V64n<KIND>(P, rd, ir, &dV, &T.rep, &T.ex, &T.Pr, &dPr, &ppf);
     }
   }
   return T;
 }
 
 // ---------------------------------------------------------------- chi
-// What the integrand needs of a quadrature node alone: s, w = 1 - u = s^2,
+// What the integrand needs of a quadrature node alone: 1/u, w = 1 - u = s^2,
 // u, the weight factor 2 w_q s, and G_k = 1 + u + ... + u^(k-1) for k =
 // 1..16 (r^-k - r0^-k = -r0^-k w G_k).  Formed once per block in shared
 // memory; forming the G_k of every node for every pair was a fifth of the
@@ -472,12 +480,12 @@ __device__ Turn rmin_device(const PotDev& P, float b, float E) {
 constexpr int kRowWords = 20;
 
 // A block's shared memory: the rows of both node sets (n_nodes, then n_low),
-// then per warp the parameters and the integrand of up to kOwners pairs whose
-// nodes the warp shares.
-constexpr int kOwners = 8, kParWords = 32, kTermStride = kMaxNodes + 4;
-constexpr int kWarpWords = kOwners * (kParWords + kTermStride);
-constexpr size_t chi_smem(int threads) {
-  return sizeof(float) * (size_t)(2 * kMaxNodes * kRowWords + threads / 32 * kWarpWords);
+// then per warp its lanes' parameters and the integrand of up to kOwners pairs
+// whose nodes the warp shares.
+constexpr int kOwners = 8, kParWords = 28, kTermStride = kMaxNodes + 4;
+constexpr int kWarpWords = 32 * kParWords + kOwners * kTermStride;
+constexpr size_t chi_smem(int threads, int rows = 2 * kMaxNodes) {
+  return sizeof(float) * (size_t)(rows * kRowWords + threads / 32 * kWarpWords);
 }
 
 struct ChiShared {
@@ -493,7 +501,7 @@ __device__ __forceinline__ ChiShared chi_shared(const PotDev& P, float* sm) {
     const float w = s * s;          // 1 - u, exact
     const float u = 1.f - w;
     float* row = sm + i * kRowWords;
-    row[0] = s; row[1] = w; row[2] = u; row[3] = P.w_node[q] * 2.f * s;
+    row[0] = __frcp_rn(u); row[1] = w; row[2] = u; row[3] = P.w_node[q] * 2.f * s;
     float Gk = 0.f, uk = 1.f;
 #pragma unroll
     for (int k = 1; k <= 16; ++k) {
@@ -503,8 +511,8 @@ __device__ __forceinline__ ChiShared chi_shared(const PotDev& P, float* sm) {
     }
   }
   __syncthreads();
-  float* mine = sm + 2 * kMaxNodes * kRowWords + (threadIdx.x >> 5) * kWarpWords;
-  return ChiShared{sm, mine, mine + kOwners * kParWords};
+  float* mine = sm + (P.n_nodes + P.n_low) * kRowWords + (threadIdx.x >> 5) * kWarpWords;
+  return ChiShared{sm, mine, mine + 32 * kParWords};
 }
 
 // The pair's coefficients about its turning point (Jager form).
@@ -524,7 +532,13 @@ __device__ __forceinline__ float node_term(const PotDev& P, const PairCoef& c, c
     G16[4 * k] = g.x; G16[4 * k + 1] = g.y; G16[4 * k + 2] = g.z; G16[4 * k + 3] = g.w;
   }
   const float r0 = c.r0;
-  const float dr = r0 * w / u;    // r - r0
+  // r - r0 = r0 w / u, correctly rounded: a quotient from the rounded 1/u and
+  // two corrections by its exact remainder (Markstein 1990; r0 w and u are
+  // far from the ends of the FP32 range)
+  const float rw = r0 * w;
+  float dr = rw * h.x;
+  dr = fmaf(fmaf(-dr, u, rw), h.x, dr);
+  dr = fmaf(fmaf(-dr, u, rw), h.x, dr);
   const float r = r0 + dr;
   // repulsion: Rep0 * expm1(poly(r) - poly(r0))
   const float dpoly = dr * (P.fa1 + P.fa2 * (r + r0) - P.fam1 / (r * r0) -
@@ -547,7 +561,10 @@ __device__ __forceinline__ float node_term(const PotDev& P, const PairCoef& c, c
   return dG * rG * rG0 / (G * rG + G0 * rG0);
 }
 
-constexpr int kLongShared = 28;   // pairs with the long rule that a warp shares (more run side by side)
+// pairs with the long and with the short rule that a warp shares (more run
+// side by side: a shared pair costs the warp n/32 nodes and about a node's
+// instructions to hand over and sum, pairs side by side cost all n nodes)
+constexpr int kLongShared = 28, kShortShared = 16;
 
 // kWarp: see rmin_device (every lane of the warp calls it together, with the
 // block's ChiShared).  Then the pairs with the short rule run side by side,
@@ -556,20 +573,23 @@ constexpr int kLongShared = 28;   // pairs with the long rule that a warp shares
 // the order of the nodes: one such pair in a warp used to hold the other lanes
 // for the long rule's 128 nodes (of the chi batch's pairs, a twelfth of them with the
 // long rule, 95 % of the warps did).  2^22 pairs of that batch: 4.00 -> 2.55
-// ms, bit-identical; what is left is the FP64 refinement (111 FP64
-// instructions per warp at 19 cycles: 0.9 ms) and the FP32 instructions.
-template <bool kWarp = false>
-__device__ float chi_device(const PotDev& P, float b_in, float E, ChiShared S = ChiShared{}) {
+// ms, and 1.90 ms with one copy of the node's code for both ways and the other
+// potentials' code compiled apart (a fifth of the warps' stalls were
+// instruction fetches), bit-identical; what is left is the FP64 refinement
+// (111 FP64 instructions per warp at 19 cycles: 0.9 ms) and the FP32 instructions.
+template <bool kWarp = false, int KIND = -1>
+__device__ float chi_device(const PotDev& P, float b_in, float E, ChiShared S = ChiShared{}, bool use = true) {
+  const int kind = KIND >= 0 ? KIND : P.kind;
   if (!kWarp && !(b_in > 0.f)) return (float)DSMC_PI;
   const float b = b_in > 0.f ? b_in : 1.f;   // b = 0: head-on, chi = pi (set at the end)
-  const Turn Tp = rmin_device<kWarp>(P, b, E);
+  const Turn Tp = rmin_device<kWarp, KIND>(P, b, E);
   const double rd = Tp.r, ird = Tp.ir;
   const float r0 = f64_to_f32(rd);
   const float bt = f64_to_f32(f32_to_f64(b) * ird);
   const float bt2 = bt * bt;
   const float iE = 1.f / E;
   float F0 = 0.f;
-  if (P.kind == 1) F0 = 1.f - bt2;
+  if (kind == 1) F0 = 1.f - bt2;
   // per-pair coefficients about the FP64 turning point (Jager form), so that
   // the integrand's F(r_min) = 0 holds to FP64 rather than to FP32 rounding
   PairCoef cf;
@@ -580,8 +600,8 @@ __device__ float chi_device(const PotDev& P, float b_in, float E, ChiShared S = 
   Rep0 = e0 = P0 = 0.f;
   cf.r0 = r0; cf.bt2 = bt2; cf.iE = iE; cf.F0 = F0;
   float Vc0 = 0.f, powk = 0.f;
-  const bool core = P.kind == 0 && r0 < P.frc;
-  if (P.kind == 0 && !core) {
+  const bool core = kind == 0 && r0 < P.frc;
+  if (kind == 0 && !core) {
     // d_p = D_p r0^-p and the dispersion coefficients C_2n r0^-2n, each the
     // FP32 rounding of a product formed with about 44 bits: the powers of
     // 1/r0 as FP32 pairs (1/r0 split from its FP64 value), the coefficients
@@ -598,57 +618,71 @@ __device__ float chi_device(const PotDev& P, float b_in, float E, ChiShared S = 
     P0 = f64_to_f32(Tp.Pr);   // P(r0), carried from the last FP64 evaluation
     Rep0 = f64_to_f32(Tp.rep);
     e0 = f64_to_f32(Tp.ex);
-  } else if (P.kind == 2) {
+  } else if (kind == 2) {
     Vc0 = (float)(P.kappa * pow(rd, -P.p));
     powk = P.fp;
   }
   double V0d = 0.0;
   if (core) { double dd; V0d = V64(P, rd, &dd); }
   float I = 0.f;
-  const bool low = P.kind == 0 && E < P.orbit_E;
-  if (kWarp && P.kind == 0) {
+  const bool low = kind == 0 && E < P.orbit_E;
+  if (kWarp && kind == 0) {
     const int lane = threadIdx.x & 31;
-    unsigned lm = __ballot_sync(0xffffffffu, low && !core);
-    const bool shared = __popc(lm) <= kLongShared;
-    if (!core && !(low && shared)) {
-      const float* row = S.rows + (low ? P.n_nodes * kRowWords : 0);
-      for (int q = low ? P.n_low : P.n_nodes; q > 0; --q, row += kRowWords) I += row[3] * node_term(P, cf, row);
+    const unsigned lowm = __ballot_sync(0xffffffffu, use && low && !core);
+    const unsigned highm = __ballot_sync(0xffffffffu, use && !low && !core);
+    const unsigned shm = (__popc(lowm) <= kLongShared ? lowm : 0u) | (__popc(highm) <= kShortShared ? highm : 0u);
+    const bool shared = (shm >> lane) & 1u;
+    if (shared) {
+      float4* o = (float4*)(S.par + lane * kParWords);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) o[k] = make_float4(d[4 * k + 1], d[4 * k + 2], d[4 * k + 3], d[4 * k + 4]);
+      o[4] = make_float4(qn[0], qn[1], qn[2], qn[3]);
+      o[5] = make_float4(qn[4], qn[5], r0, Rep0);
+      o[6] = make_float4(e0, P0, bt2, iE);
     }
     __syncwarp();
-    if (!shared) lm = 0u;
-    while (lm) {
-      const int cnt = min(kOwners, __popc(lm)), rank = __popc(lm & ((1u << lane) - 1u));
-      const bool mine = ((lm >> lane) & 1u) && rank < cnt;
-      if (mine) {
-        float4* o = (float4*)(S.par + rank * kParWords);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) o[k] = make_float4(d[4 * k + 1], d[4 * k + 2], d[4 * k + 3], d[4 * k + 4]);
-        o[4] = make_float4(qn[0], qn[1], qn[2], qn[3]);
-        o[5] = make_float4(qn[4], qn[5], r0, Rep0);
-        o[6] = make_float4(e0, P0, bt2, iE);
+    // one loop over nodes for both ways: first every lane its own pair's (slot
+    // -1), then pair by pair the warp's lanes the nodes of a shared one, up
+    // to kOwners of them before their lanes sum
+    const float* rows = S.rows + (low ? P.n_nodes * kRowWords : 0);
+    int slot = -1, mine = -1, q = 0, step = 1, nq = use && !core && !shared ? (low ? P.n_low : P.n_nodes) : 0;
+    for (unsigned left = shm;;) {
+#pragma unroll 1
+      for (; q < nq; q += step) {
+        const float* row = rows + q * kRowWords;
+        const float x = node_term(P, cf, row);
+        if (slot < 0) I += row[3] * x;
+        else S.term[slot * kTermStride + q] = x;
       }
-      __syncwarp();
-      const float* lrows = S.rows + P.n_nodes * kRowWords;
-      for (int o = 0; o < cnt; ++o) {
-        const float4* v = (const float4*)(S.par + o * kParWords);
-        PairCoef c;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const float4 x = v[k];
-          c.d[4 * k + 1] = x.x; c.d[4 * k + 2] = x.y; c.d[4 * k + 3] = x.z; c.d[4 * k + 4] = x.w;
+      if (slot == kOwners - 1 || (slot >= 0 && !left)) {
+        __syncwarp();
+        if (mine >= 0) {
+          const float* mrows = S.rows + (low ? P.n_nodes * kRowWords : 0);
+          const int n = low ? P.n_low : P.n_nodes;
+          for (int k = 0; k < n; ++k) I += mrows[k * kRowWords + 3] * S.term[mine * kTermStride + k];
         }
-        const float4 x4 = v[4], x5 = v[5], x6 = v[6];
-        c.qn[0] = x4.x; c.qn[1] = x4.y; c.qn[2] = x4.z; c.qn[3] = x4.w;
-        c.qn[4] = x5.x; c.qn[5] = x5.y; c.r0 = x5.z; c.Rep0 = x5.w;
-        c.e0 = x6.x; c.P0 = x6.y; c.bt2 = x6.z; c.iE = x6.w;
-        c.F0 = F0;   // 0 for the Jager form
-        for (int q = lane; q < P.n_low; q += 32) S.term[o * kTermStride + q] = node_term(P, c, lrows + q * kRowWords);
+        mine = slot = -1;
+        __syncwarp();
       }
-      __syncwarp();
-      if (mine)
-        for (int q = 0; q < P.n_low; ++q) I += lrows[q * kRowWords + 3] * S.term[rank * kTermStride + q];
-      __syncwarp();
-      for (int o = 0; o < cnt; ++o) lm &= lm - 1u;
+      if (!left) break;
+      const int owner = __ffs(left) - 1;
+      left &= left - 1u;
+      ++slot;
+      if (lane == owner) mine = slot;
+      const float4* v = (const float4*)(S.par + owner * kParWords);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float4 x = v[k];
+        d[4 * k + 1] = x.x; d[4 * k + 2] = x.y; d[4 * k + 3] = x.z; d[4 * k + 4] = x.w;
+      }
+      const float4 x4 = v[4], x5 = v[5], x6 = v[6];
+      qn[0] = x4.x; qn[1] = x4.y; qn[2] = x4.z; qn[3] = x4.w;
+      qn[4] = x5.x; qn[5] = x5.y; cf.r0 = x5.z; Rep0 = x5.w;
+      e0 = x6.x; P0 = x6.y; cf.bt2 = x6.z; cf.iE = x6.w;
+      const bool olow = (lowm >> owner) & 1u;
+      rows = S.rows + (olow ? P.n_nodes * kRowWords : 0);
+      nq = olow ? P.n_low : P.n_nodes;
+      q = lane; step = 32;
     }
     if (!core) return b_in > 0.f ? -2.f * bt * I : (float)DSMC_PI;
   }
@@ -659,7 +693,7 @@ __device__ float chi_device(const PotDev& P, float b_in, float E, ChiShared S = 
     const float u = 1.f - w;
     const float dr = r0 * w / u;    // r - r0
     float dV = 0.f;
-    if (P.kind == 0 && !core) {
+    if (!kWarp && kind == 0 && !core) {   // (a warp's are done above)
       const float r = r0 + dr;
       // repulsion: Rep0 * expm1(poly(r) - poly(r0))
       const float dpoly = dr * (P.fa1 + P.fa2 * (r + r0) - P.fam1 / (r * r0) -
@@ -678,7 +712,7 @@ __device__ float chi_device(const PotDev& P, float b_in, float E, ChiShared S = 
       dP *= -w;                     // P(r) - P(r0)
       const float dh = e0 * (expm1f(-P.fbeta * dr) * (P0 + dP) + dP);
       dV = drep - dQ + dh;
-    } else if (P.kind == 2) {
+    } else if (kind == 2) {
       dV = Vc0 * expm1f(powk * log1pf(-w));  // kappa (r^-p - r0^-p)
     } else if (core) {
       double dd;
@@ -806,6 +840,7 @@ static PotDev make_pot(const dsmc_gas_t& gas, const dsmc_potential_t& p, int n_n
 // ---------------------------------------------------------------- kernels
 // Warp-uniform loop: every lane of a warp computes chi together (a lane past
 // the end, or with g = 0, on harmless inputs whose result is not kept).
+template <int KIND>
 __global__ void __launch_bounds__(128, 4) k_jager_chi(PotDev P, int64_t n, const float* __restrict__ b,
                                                       const float* __restrict__ g, float* __restrict__ chi) {
   extern __shared__ float4 chi_sm[];
@@ -817,7 +852,7 @@ __global__ void __launch_bounds__(128, 4) k_jager_chi(PotDev P, int64_t n, const
     const bool valid = q < n;
     const float gg = valid ? g[q] : 0.f;
     const bool use = valid && gg > 0.f;
-    const float c = chi_device<true>(P, use ? b[q] : 1.f, use ? P.mass_over_4k * gg * gg : 1.0e4f, S);
+    const float c = chi_device<true, KIND>(P, use ? b[q] : 1.f, use ? P.mass_over_4k * gg * gg : 1.0e4f, S, use);
     if (valid) chi[q] = use ? c : 0.f;
   }
 }
@@ -879,6 +914,7 @@ struct JagerArgs {
 // it together (live false: a lane with no pair, or whose dependency wait
 // failed, computes on harmless inputs and stores nothing), so that chi's FP64
 // refinement and the FP64 rotation run with the warp converged.
+template <int KIND>
 __device__ __forceinline__ void collide_pair(const PotDev& P, const ChiShared& S, const JagerArgs& a, int64_t p,
                                              int4 q, bool live) {
   double xi = 0.0, yi = 0.0, zi = 0.0, xj = 0.0, yj = 0.0, zj = 0.0;
@@ -892,7 +928,7 @@ __device__ __forceinline__ void collide_pair(const PotDev& P, const ChiShared& S
   const u32x4 w = draw(a.seed, (uint32_t)q.w, (uint32_t)q.z, a.step, TAG_JAGER);
   const float b = use ? f64_to_f32(a.bmax_A * sqrt64(u53_int(w.x, w.y))) : 1.f;
   const float E = use ? P.mass_over_4k * f64_to_f32(g2) : 1.0e4f;
-  const float chi_c = chi_device<true>(P, b, E, S);
+  const float chi_c = chi_device<true, KIND>(P, b, E, S, use);
   const float chi = use ? chi_c : 0.f;
   if (live && a.chi_out) a.chi_out[p] = chi;
   __syncwarp();
@@ -918,6 +954,7 @@ __device__ __forceinline__ void collide_pair(const PotDev& P, const ChiShared& S
 // magnitude (bracket scan, Newton iterations), so no warp waits for a round
 // to end: only true dependencies order the work.  Which thread handles a
 // pair does not change its result.
+template <int KIND>
 __global__ void __launch_bounds__(128, 4) k_collide_jager(PotDev P, JagerArgs a) {
   if (a.step_dev) a.step = *a.step_dev;
   extern __shared__ float4 chi_sm[];
@@ -941,7 +978,7 @@ __global__ void __launch_bounds__(128, 4) k_collide_jager(PotDev P, JagerArgs a)
       ok = wait_deps(a.done, q.x, q.y, a.deps[p], a.bar + 2, a.status);
     }
     __syncwarp();
-    collide_pair(P, S, a, p, q, valid && ok);
+    collide_pair<KIND>(P, S, a, p, q, valid && ok);
     if (valid && ok) release_pair(a.done, q.x, q.y, (unsigned)(r + 1));
     if (!__all_sync(0xffffffffu, ok)) break;
   }
@@ -1072,6 +1109,8 @@ __global__ void k_selftest_math(Exp64 E, int which, int64_t n, const double* __r
   }
 }
 
+constexpr size_t kDefaultSmem = 48 * 1024;   // dynamic shared memory a kernel may have without asking
+
 static unsigned blocks_n(int64_t n, int threads, int cap) {
   int64_t b = (n + threads - 1) / threads;
   if (b < 1) b = 1;
@@ -1091,19 +1130,27 @@ int launch_jager_chi(Ctx* c, const dsmc_gas_t& gas, const dsmc_potential_t& pot,
   if (n == 0) return 0;
   const PotDev P = make_pot(gas, pot, n_nodes);
   const Shape sh = shape_or_default(c, DSMC_TUNE_JAGER_CHI);
-  k_jager_chi<<<blocks_n(n, sh.threads, sm_count(c) * sh.blocks_per_sm), sh.threads, chi_smem(sh.threads), s>>>(
-      P, n, b, g, chi);
+  const size_t sm = chi_smem(sh.threads, P.n_nodes + P.n_low);
+  const auto k = P.kind == 0 ? k_jager_chi<0> : k_jager_chi<-1>;
+  if (sm > kDefaultSmem &&
+      cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
+    return record(c, DSMC_ERR_CUDA, "jager_chi: shared-memory attribute");
+  k<<<blocks_n(n, sh.threads, sm_count(c) * sh.blocks_per_sm), sh.threads, sm, s>>>(P, n, b, g, chi);
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
 }
 
 // resident blocks per SM of the Jager collide at a block size (0 on failure)
-int occupancy_collide_jager(int threads) {
+static int occupancy_jager(const void* k, int threads, size_t sm) {
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)k_collide_jager, threads,
-                                                    chi_smem(threads)) != cudaSuccess)
+  if (sm > kDefaultSmem &&
+      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
     return 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, sm) != cudaSuccess) return 0;
   return per_sm;
+}
+int occupancy_collide_jager(int threads) {
+  return occupancy_jager((const void*)k_collide_jager<0>, threads, chi_smem(threads));
 }
 
 int launch_collide_jager(Ctx* c, const dsmc_gas_t& gas, const dsmc_potential_t& pot,
@@ -1112,16 +1159,18 @@ int launch_collide_jager(Ctx* c, const dsmc_gas_t& gas, const dsmc_potential_t& 
                          double* vz, float* chi_out, void* ws, size_t ws_bytes, cudaStream_t s) {
   if (ws_bytes < collide_ws(n)) return record(c, DSMC_ERR_ARG, "collide_jager: workspace too small");
   const Shape sh = shape_or_default(c, DSMC_TUNE_COLLIDE_JAGER);
-  const int occ = occupancy_collide_jager(sh.threads);
+  const PotDev P = make_pot(gas, pot, n_nodes);
+  const size_t sm = chi_smem(sh.threads, P.n_nodes + P.n_low);
+  const auto k = P.kind == 0 ? k_collide_jager<0> : k_collide_jager<-1>;
+  const int occ = occupancy_jager((const void*)k, sh.threads, sm);
   if (occ < 1) return record(c, DSMC_ERR_CUDA, "collide_jager: occupancy query failed");
   const int blocks = sm_count(c) * (sh.blocks_per_sm > 0 && sh.blocks_per_sm < occ ? sh.blocks_per_sm : occ);
-  PotDev P = make_pot(gas, pot, n_nodes);
   JagerArgs a{gas.seed, step, graph_step_ptr(c), gas.b_max * 1e10, (const int4*)pairs, deps, ro, info, vx, vy, vz,
               chi_out, (unsigned*)ws, barrier_ptr(c), status_ptr(c)};
   if (cudaMemsetAsync(a.bar, 0, 4 * sizeof(unsigned), s) != cudaSuccess ||
       cudaMemsetAsync(a.done, 0, sizeof(unsigned) * (size_t)(n > 0 ? n : 1), s) != cudaSuccess)
     return DSMC_ERR_CUDA;
-  k_collide_jager<<<blocks, sh.threads, chi_smem(sh.threads), s>>>(P, a);
+  k<<<blocks, sh.threads, sm, s>>>(P, a);
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : record(c, DSMC_ERR_CUDA, "collide_jager: launch failed");
 }
