@@ -629,7 +629,9 @@ int dsmc_step(dsmc_ctx_t* c, const dsmc_gas_t* gas, const dsmc_path_t* path,
 
 // the step from the sorted velocities on: moments (on the context's side
 // stream, beside the selection: both only read the sorted velocities),
-// selection, pair update, moment matching (after the moments have joined)
+// selection, then, once the moments have joined, the pair update (which
+// changes the velocities they read, and on the neural path reads them) and
+// moment matching
 static int step_after_sort(dsmc_ctx_t* c, const dsmc_gas_t* gas, const dsmc_path_t* path,
                            const dsmc_step_buffers_t* B, uint64_t step, void* stream) {
   cudaStream_t s = S(stream);
@@ -642,10 +644,10 @@ static int step_after_sort(dsmc_ctx_t* c, const dsmc_gas_t* gas, const dsmc_path
     rc = dsmc_select_pairs_ordered(c, gas, B->n, B->n_cells, B->cell_start, B->svx, B->svy, B->svz,
                                    B->sigma_g_max, step, B->capacity, B->pairs, B->deps, B->round_offsets,
                                    B->info, step_order(path), B->ws, B->ws_bytes, stream);
-  if (!rc) rc = collide_step(c, gas, path, B, step, stream);
   const bool joined = joined_ev && cudaStreamWaitEvent(s, c->f_ev[1], 0) == cudaSuccess;
   if (rc) return rc;
   if (!joined) return dsmc::record(c, DSMC_ERR_CUDA, "step: join of the moments stream failed");
+  if ((rc = collide_step(c, gas, path, B, step, stream))) return rc;
   return dsmc_moment_match(c, B->n_cells, B->cell_start, B->mom, B->svx, B->svy, B->svz, stream);
 }
 
