@@ -19,9 +19,17 @@ namespace dsmc {
 constexpr int kScanThreads = 256;
 constexpr int kScanPer = 16;
 constexpr int kScanItems = kScanThreads * kScanPer;
+// up to here one block scans alone (tile after tile), in one launch (40,000
+// counts took one block 34 us, two launches 10 us)
+constexpr int kScanOnePer = 4;
+constexpr int64_t kScanOne = 2 * 1024 * kScanOnePer;
+// up to here every block of the second launch sums the blocks before it
+// itself, and the pass over the block sums is not launched
+constexpr int64_t kScanBlocks = 2048;
 
+template <int THREADS = kScanThreads>
 __device__ __forceinline__ int block_exclusive_scan(int v, int* total) {
-  __shared__ int wsum[kScanThreads / 32];
+  __shared__ int wsum[THREADS / 32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   int x = v;
 #pragma unroll
@@ -32,17 +40,17 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* total) {
   if (lane == 31) wsum[wid] = x;
   __syncthreads();
   if (wid == 0) {
-    int s = lane < kScanThreads / 32 ? wsum[lane] : 0;
+    int s = lane < THREADS / 32 ? wsum[lane] : 0;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int y = __shfl_up_sync(0xffffffffu, s, o);
       if (lane >= o) s += y;
     }
-    if (lane < kScanThreads / 32) wsum[lane] = s;
+    if (lane < THREADS / 32) wsum[lane] = s;
   }
   __syncthreads();
   const int before = (wid ? wsum[wid - 1] : 0) + x - v;
-  *total = wsum[kScanThreads / 32 - 1];
+  *total = wsum[THREADS / 32 - 1];
   __syncthreads();
   return before;
 }
@@ -71,8 +79,17 @@ __global__ void k_scan_blocks(int32_t* bsum, int64_t nb) {
   }
 }
 
-__global__ void k_scan_apply(const int32_t* __restrict__ in, int64_t n, const int32_t* bsum,
+// bsum: the blocks' sums (scanned false) or their exclusive scan
+__global__ void k_scan_apply(const int32_t* __restrict__ in, int64_t n, const int32_t* bsum, int scanned,
                              int32_t* __restrict__ out) {
+  int first;
+  if (scanned) {
+    first = bsum[blockIdx.x];
+  } else {
+    int v = 0;
+    for (unsigned q = threadIdx.x; q < blockIdx.x; q += kScanThreads) v += bsum[q];
+    block_exclusive_scan(v, &first);
+  }
   const int64_t base = (int64_t)blockIdx.x * kScanItems + (int64_t)threadIdx.x * kScanPer;
   int v[kScanPer];
   int s = 0;
@@ -82,7 +99,7 @@ __global__ void k_scan_apply(const int32_t* __restrict__ in, int64_t n, const in
     s += v[q];
   }
   int total;
-  int run = bsum[blockIdx.x] + block_exclusive_scan(s, &total);
+  int run = first + block_exclusive_scan(s, &total);
 #pragma unroll
   for (int q = 0; q < kScanPer; ++q) {
     if (base + q < n) out[base + q] = run;
@@ -91,18 +108,47 @@ __global__ void k_scan_apply(const int32_t* __restrict__ in, int64_t n, const in
   if (base <= n - 1 && n - 1 < base + kScanPer) out[n] = run;  // total after the last element
 }
 
+__global__ void __launch_bounds__(1024) k_scan_one(const int32_t* __restrict__ in, int64_t n,
+                                                   int32_t* __restrict__ out) {
+  int run = 0;
+  for (int64_t t0 = 0; t0 < n; t0 += 1024 * kScanOnePer) {
+    const int64_t base = t0 + (int64_t)threadIdx.x * kScanOnePer;
+    int v[kScanOnePer], s = 0;
+#pragma unroll
+    for (int q = 0; q < kScanOnePer; ++q) {
+      v[q] = base + q < n ? in[base + q] : 0;
+      s += v[q];
+    }
+    int total;
+    int at = run + block_exclusive_scan<1024>(s, &total);
+    run += total;
+#pragma unroll
+    for (int q = 0; q < kScanOnePer; ++q) {
+      if (base + q < n) out[base + q] = at;
+      at += v[q];
+    }
+  }
+  if (threadIdx.x == 0) out[n] = run;
+}
+
 size_t scan_ws(int64_t n) { return align256(sizeof(int32_t) * (size_t)((n + kScanItems - 1) / kScanItems + 1)); }
 
 int launch_scan(Ctx* c, const int32_t* in, int32_t* out, int64_t n, void* ws, cudaStream_t s) {
   if (n <= 0) {
     return cudaMemsetAsync(out, 0, sizeof(int32_t), s) == cudaSuccess ? 0 : DSMC_ERR_CUDA;
   }
+  if (n <= kScanOne) {
+    k_scan_one<<<1, 1024, 0, s>>>(in, n, out);
+    if (c) count_launches(c, 1);
+    return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
+  }
   const int64_t nb = (n + kScanItems - 1) / kScanItems;
   int32_t* bsum = (int32_t*)ws;
+  const bool scan_sums = nb > kScanBlocks;
   k_scan_reduce<<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, bsum);
-  k_scan_blocks<<<1, kScanThreads, 0, s>>>(bsum, nb);
-  k_scan_apply<<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, bsum, out);
-  if (c) count_launches(c, 3);
+  if (scan_sums) k_scan_blocks<<<1, kScanThreads, 0, s>>>(bsum, nb);
+  k_scan_apply<<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, bsum, scan_sums, out);
+  if (c) count_launches(c, 2 + scan_sums);
   return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
 }
 
@@ -396,6 +442,10 @@ k_rs_rowscan(const int32_t* __restrict__ cnt, int32_t chunks, int32_t* __restric
 // write consecutive addresses of each digit's run (its global start from
 // the scan), so the stores coalesce.
 // Values: the input index (first pass) or vals.
+// base null: few chunks (kRsDirect), each block sums the counts of the earlier
+// chunks and the digit's total from tot = k_rs_count's table itself, and the
+// scan of that table is not launched.
+constexpr int32_t kRsDirect = 16;
 constexpr int kRsPer = kRsChunk / kRsWarps / 32;
 static_assert(kRsWarps * 32 == kRadix, "one thread per digit in the offset step");
 
@@ -459,7 +509,17 @@ k_rs_scatter(const int32_t* __restrict__ cell_id, const uint32_t* __restrict__ k
     int ct = 0;
 #pragma unroll
     for (int q = 0; q < kRsWarps; ++q) ct += sm.wh[q][d];
-    const int gt = tot[d];
+    int gt = 0, before = 0;
+    if (base) {
+      gt = tot[d];
+      before = base[(size_t)d * chunks + blockIdx.x];
+    } else {
+      for (int32_t q = 0; q < chunks; ++q) {
+        const int v = tot[(size_t)d * chunks + q];
+        gt += v;
+        if (q < (int32_t)blockIdx.x) before += v;
+      }
+    }
     int x = ct, xg = gt;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -480,7 +540,7 @@ k_rs_scatter(const int32_t* __restrict__ cell_id, const uint32_t* __restrict__ k
     __syncthreads();
     const int ls = (w ? wt[w - 1] : 0) + x - ct;    // chunk-local start of digit d
     const int gs = (w ? wg[w - 1] : 0) + xg - gt;   // global start of digit d
-    gdelta[d] = gs + base[(size_t)d * chunks + blockIdx.x] - ls;
+    gdelta[d] = gs + before - ls;
     int acc = ls;
 #pragma unroll
     for (int q = 0; q < kRsWarps; ++q) { const int c = sm.wh[q][d]; sm.wh[q][d] = acc; acc += c; }
@@ -594,11 +654,11 @@ int launch_sort_keys(Ctx* c, int32_t n, int32_t n_cells, const int32_t* cell_id,
     int32_t* vout = last ? perm : ((q & 1) ? vb : va);
     k_rs_count<<<chunks, 256, 0, s>>>(cell_id, kin, n, n_cells, q * kRadixBits, chunks, cnt,
                                       q == 0 ? status_ptr(c) : nullptr);
-    count_launches(c, 1);
-    k_rs_rowscan<<<kRadix, 256, 0, s>>>(cnt, chunks, off, dtot);
-    k_rs_scatter<<<chunks, kRsWarps * 32, 0, s>>>(cell_id, kin, vin, n, n_cells, q * kRadixBits, chunks, off,
-                                                  dtot, kout, vout);
-    count_launches(c, 2);
+    const bool direct = chunks <= kRsDirect;
+    if (!direct) k_rs_rowscan<<<kRadix, 256, 0, s>>>(cnt, chunks, off, dtot);
+    k_rs_scatter<<<chunks, kRsWarps * 32, 0, s>>>(cell_id, kin, vin, n, n_cells, q * kRadixBits, chunks,
+                                                  direct ? nullptr : off, direct ? cnt : dtot, kout, vout);
+    count_launches(c, 3 - direct);
     kin = kout;
     vin = vout;
   }
@@ -618,12 +678,21 @@ int launch_gather_one(Ctx* c, int32_t n, int32_t n_cells, const int32_t* cell_st
   return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
 }
 
+// All three components in one launch while they fit in L2 together (24 B per
+// particle: half of its 129 MB); beyond that one component at a time.
+constexpr int32_t kGatherAll = 2500000;
+
 int launch_gather(Ctx* c, int32_t n, int32_t n_cells, const int32_t* cell_start, const int32_t* perm,
                   const double* vx, const double* vy, const double* vz, double* svx, double* svy,
                   double* svz, cudaStream_t s) {
   if (n <= 0) return 0;
   const Shape sh = shape_or_default(c, DSMC_TUNE_GATHER);
   const unsigned g = grid_for(n, sh.threads, sm_count(c) * sh.blocks_per_sm);
+  if (n <= kGatherAll) {
+    k_gather<<<g, sh.threads, 0, s>>>(n, cell_start, n_cells, perm, vx, vy, vz, svx, svy, svz);
+    count_launches(c, 1);
+    return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
+  }
   k_gather1<<<g, sh.threads, 0, s>>>(n, cell_start, n_cells, perm, vx, svx);
   k_gather1<<<g, sh.threads, 0, s>>>(n, cell_start, n_cells, perm, vy, svy);
   k_gather1<<<g, sh.threads, 0, s>>>(n, cell_start, n_cells, perm, vz, svz);

@@ -87,6 +87,26 @@ int occupancy_collide_vhs(int threads) {
   return per_sm;
 }
 
+// The done stamps and the barrier words (abort, unit cursor) of a collide call
+// start at zero: one launch for both.
+__global__ void k_clear_stamps(unsigned* __restrict__ done, int32_t n, unsigned* bar) {
+  if (blockIdx.x == 0 && threadIdx.x < 4) bar[threadIdx.x] = 0u;
+  const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+  // 16 bytes at a time from an aligned workspace, word by word otherwise and at the end
+  const int64_t n4 = ((uintptr_t)done & 15u) ? 0 : n / 4;
+  for (int64_t q = first; q < n4; q += stride) ((uint4*)done)[q] = make_uint4(0u, 0u, 0u, 0u);
+  for (int64_t q = 4 * n4 + first; q < n; q += stride) done[q] = 0u;
+}
+
+int launch_clear_stamps(Ctx* c, unsigned* done, int32_t n, unsigned* bar, cudaStream_t s) {
+  int64_t b = ((int64_t)n + 4095) / 4096;
+  if (b < 1) b = 1;
+  if (b > 8 * sm_count(c)) b = 8 * sm_count(c);
+  k_clear_stamps<<<(unsigned)b, 256, 0, s>>>(done, n, bar);
+  count_launches(c, 1);
+  return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
+}
+
 size_t collide_ws(int32_t n) { return align256(sizeof(unsigned) * (size_t)(n > 0 ? n : 1)); }
 
 int launch_collide_vhs(Ctx* c, const dsmc_gas_t& gas, uint64_t step, int32_t n, const int32_t* pairs,
@@ -99,9 +119,7 @@ int launch_collide_vhs(Ctx* c, const dsmc_gas_t& gas, uint64_t step, int32_t n, 
   const int blocks = sm_count(c) * (sh.blocks_per_sm > 0 && sh.blocks_per_sm < occ ? sh.blocks_per_sm : occ);
   VhsArgs a{gas.seed, step, graph_step_ptr(c), (const int4*)pairs, deps, ro, info, vx, vy, vz,
             (unsigned*)ws, barrier_ptr(c), status_ptr(c)};
-  if (cudaMemsetAsync(a.bar, 0, 4 * sizeof(unsigned), s) != cudaSuccess ||
-      cudaMemsetAsync(a.done, 0, sizeof(unsigned) * (size_t)(n > 0 ? n : 1), s) != cudaSuccess)
-    return DSMC_ERR_CUDA;
+  if (int rc = launch_clear_stamps(c, a.done, n, a.bar, s)) return rc;
   k_collide_vhs<<<blocks, sh.threads, 0, s>>>(a);
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : record(c, DSMC_ERR_CUDA, "collide_vhs: launch failed");

@@ -309,6 +309,7 @@ int launch_sgmax_init(Ctx* c, const dsmc_gas_t& gas, int32_t n_cells, const doub
                       double factor, double* sgmax, cudaStream_t s);
 // per-particle done stamps of the collide kernels
 size_t collide_ws(int32_t n);
+int launch_clear_stamps(Ctx* c, unsigned* done, int32_t n, unsigned* bar, cudaStream_t s);
 int launch_collide_vhs(Ctx* c, const dsmc_gas_t& gas, uint64_t step, int32_t n, const int32_t* pairs,
                        const uint32_t* deps, const int32_t* ro, const dsmc_select_info_t* info, double* vx,
                        double* vy, double* vz, void* ws, size_t ws_bytes, cudaStream_t s);

@@ -1167,9 +1167,7 @@ int launch_collide_jager(Ctx* c, const dsmc_gas_t& gas, const dsmc_potential_t& 
   const int blocks = sm_count(c) * (sh.blocks_per_sm > 0 && sh.blocks_per_sm < occ ? sh.blocks_per_sm : occ);
   JagerArgs a{gas.seed, step, graph_step_ptr(c), gas.b_max * 1e10, (const int4*)pairs, deps, ro, info, vx, vy, vz,
               chi_out, (unsigned*)ws, barrier_ptr(c), status_ptr(c)};
-  if (cudaMemsetAsync(a.bar, 0, 4 * sizeof(unsigned), s) != cudaSuccess ||
-      cudaMemsetAsync(a.done, 0, sizeof(unsigned) * (size_t)(n > 0 ? n : 1), s) != cudaSuccess)
-    return DSMC_ERR_CUDA;
+  if (int rc = launch_clear_stamps(c, a.done, n, a.bar, s)) return rc;
   k<<<blocks, sh.threads, sm, s>>>(P, a);
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : record(c, DSMC_ERR_CUDA, "collide_jager: launch failed");
@@ -1207,9 +1205,7 @@ int launch_collide_table(Ctx* c, const dsmc_gas_t& gas, const dsmc_chi_table_t& 
   a.pairs = (const int4*)pairs; a.deps = deps; a.ro = ro; a.info = info;
   a.vx = vx; a.vy = vy; a.vz = vz; a.chi_out = chi_out;
   a.done = (unsigned*)ws; a.bar = barrier_ptr(c); a.status = status_ptr(c);
-  if (cudaMemsetAsync(a.bar, 0, 4 * sizeof(unsigned), s) != cudaSuccess ||
-      cudaMemsetAsync(a.done, 0, sizeof(unsigned) * (size_t)(n > 0 ? n : 1), s) != cudaSuccess)
-    return DSMC_ERR_CUDA;
+  if (int rc = launch_clear_stamps(c, a.done, n, a.bar, s)) return rc;
   k_collide_table<<<blocks, sh.threads, 0, s>>>(a);
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : record(c, DSMC_ERR_CUDA, "collide_table: launch failed");

@@ -925,9 +925,7 @@ int launch_collide_neural(Ctx* c, const dsmc_gas_t& gas, const dsmc_mlp_t& mlp,
   a.T_feat_f = (float)(a.m_over_3k * a.T_ref_inv);
   a.mom = mom; a.u_out = u_out; a.pairs = (const int4*)pairs; a.deps = deps; a.ro = ro; a.info = info;
   a.vx = vx; a.vy = vy; a.vz = vz; a.done = (unsigned*)ws; a.bar = barrier_ptr(c); a.status = status_ptr(c);
-  if (cudaMemsetAsync(a.bar, 0, 4 * sizeof(unsigned), s) != cudaSuccess ||
-      cudaMemsetAsync(a.done, 0, sizeof(unsigned) * (size_t)(n > 0 ? n : 1), s) != cudaSuccess)
-    return DSMC_ERR_CUDA;
+  if (int rc = launch_clear_stamps(c, a.done, n, a.bar, s)) return rc;
   k_collide_neural<<<sm_count(c) * per_sm, kPipeThreads, P.total, s>>>(sh, w, bias, a);
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : record(c, DSMC_ERR_CUDA, "collide_neural: launch failed");

@@ -1,8 +1,11 @@
 // No-Time-Counter pair selection (Sec. 2.2) and the conflict-free round
 // schedule of the accepted pairs.
 //
-//   k_sel_count   warp per cell: M = floor(1/2 N(N-1) F_N/V_c (sg)max dt + U),
-//                 evaluate every candidate, count acceptances, new (sg)max
+//   k_sel_nwords  M = floor(1/2 N(N-1) F_N/V_c (sg)max dt + U) of every cell
+//   scan          accept-bit words -> each cell's first word (the two in one
+//                 launch for few cells)
+//   k_sel_count   warp per cell: evaluate every candidate, count acceptances,
+//                 new (sg)max
 //   scan          counts -> per-cell pair offsets
 //   k_sel_emit    warp per cell: the accepted candidates (from the count
 //                 pass's accept bits) compacted in candidate order and their
@@ -13,6 +16,11 @@
 //                 of the pairs (cell-major candidate order inside a round),
 //                 each with the rounds of the previous pairs of its particles
 //
+// A gas of a few thousand particles is bound by its launches, about 3 us each:
+// the zeroing, *info and the scans' middle pass ride on other kernels (a
+// 100-cell gas's selection took 13 launches and two memsets, now 8; its whole
+// step 128 -> 82 us).
+//
 // The accept decision and M are taken in FP64 with explicitly rounded
 // operations (no contraction into FMA), in the operation order of the
 // definition, so that they agree exactly with any other correctly rounded
@@ -22,25 +30,67 @@
 namespace dsmc {
 
 constexpr int kSelWarps = 8;
+constexpr int kTotalsWords = 2 * DSMC_MAX_ROUNDS + 64;   // round counts, round count, candidate count (SelWs)
 
-// Words of accept bits per cell: ceil(M/32) for the cell's candidate count M.
-__global__ void k_sel_nwords(SelArgs a) {
+// The NTC candidate count M of a cell, and its words of accept bits: ceil(M/32).
+__device__ __forceinline__ int32_t cell_words(const SelArgs& a, int32_t k) {
+  const int32_t N = a.cs[k + 1] - a.cs[k];
+  int bad = 0;
+  const int32_t M = N < 2 ? 0 : ntc_count(a, k, N, &bad);
+  if (bad) set_status(a.status, DSMC_ERR_CAPACITY);
+  a.ncand[k] = M;
+  const int64_t words = ((int64_t)M + 31) / 32;
+  return (int32_t)(words <= a.words_cap ? words : 0);  // too many: never kept
+}
+
+// What the later kernels add to starts at zero: the round counts, the round
+// count and the candidate count (together in the workspace), and the
+// caller's round offsets (the whole list, for a step without pairs).
+__device__ __forceinline__ void clear_totals(const SelArgs& a, int32_t* round_off, int t, int nt) {
+  for (int q = t; q < kTotalsWords; q += nt) a.round_count[q] = 0;
+  for (int q = t; q <= DSMC_MAX_ROUNDS; q += nt) round_off[q] = 0;
+}
+
+__global__ void k_sel_nwords(SelArgs a, int32_t* round_off) {
   if (a.step_dev) a.step = *a.step_dev;
-  unsigned long long total = 0;
-  for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < a.n_cells; k += gridDim.x * blockDim.x) {
-    const int32_t N = a.cs[k + 1] - a.cs[k];
-    int bad = 0;
-    const int32_t M = N < 2 ? 0 : ntc_count(a, k, N, &bad);
-    if (bad) set_status(a.status, DSMC_ERR_CAPACITY);
-    a.ncand[k] = M;
-    total += (unsigned long long)M;
-    const int64_t words = ((int64_t)M + 31) / 32;
-    a.wcnt[k] = (int32_t)(words <= a.words_cap ? words : 0);  // too many: never kept
-  }
-  // one atomic per warp for the step's candidate count
+  if (blockIdx.x == 0) clear_totals(a, round_off, threadIdx.x, blockDim.x);
+  for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < a.n_cells; k += gridDim.x * blockDim.x)
+    a.wcnt[k] = cell_words(a, k);
+}
+
+// The same and the exclusive scan of the words in one block, for few cells:
+// one launch instead of two.
+constexpr int kWordsThreads = 1024;
+constexpr int32_t kWordsOne = 4 * kWordsThreads;
+__global__ void __launch_bounds__(kWordsThreads) k_sel_nwords_one(SelArgs a, int32_t* round_off, int32_t* wofs) {
+  if (a.step_dev) a.step = *a.step_dev;
+  __shared__ int wsum[kWordsThreads / 32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  clear_totals(a, round_off, threadIdx.x, kWordsThreads);
+  int run = 0;
+  for (int32_t t0 = 0; t0 < a.n_cells; t0 += kWordsThreads) {
+    const int32_t k = t0 + threadIdx.x;
+    const int v = k < a.n_cells ? cell_words(a, k) : 0;
+    int x = v;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
-  if ((threadIdx.x & 31) == 0 && total) atomicAdd(a.n_cand, total);
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[w] = x;
+    __syncthreads();
+    int tot = wsum[lane];   // 32 warps
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, tot, o);
+      if (lane >= o) tot += y;
+    }
+    const int before = w ? __shfl_sync(0xffffffffu, tot, w - 1) : 0;
+    if (k < a.n_cells) wofs[k] = run + before + x - v;
+    run += __shfl_sync(0xffffffffu, tot, 31);
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) wofs[a.n_cells] = run;
 }
 
 // Stage the cell's velocities (FP32) in this warp's shared-memory slice
@@ -166,14 +216,16 @@ __global__ void __launch_bounds__(kSelWarps * 32, 4) k_sel_count(SelArgs a) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int32_t warps = gridDim.x * kSelWarps;
   const int32_t npairs = (a.n_cells + 1) / 2;
+  unsigned long long cands = 0;
   for (int32_t kp = blockIdx.x * kSelWarps + wid; kp < npairs; kp += warps) {
     const int32_t kk[2] = {2 * kp, 2 * kp + 1 < a.n_cells ? 2 * kp + 1 : a.n_cells};
     bool small = true;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       if (kk[h] >= a.n_cells) continue;
-      const int32_t N = a.cs[kk[h] + 1] - a.cs[kk[h]];
-      if (N >= 2 && (N > kStage / 2 || a.ncand[kk[h]] > 16)) small = false;
+      const int32_t N = a.cs[kk[h] + 1] - a.cs[kk[h]], M = a.ncand[kk[h]];   // (0 for N < 2)
+      cands += (unsigned long long)M;
+      if (N >= 2 && (N > kStage / 2 || M > 16)) small = false;
     }
     if (small) {
       count_pair(a, stage[wid], kk, lane);
@@ -182,6 +234,7 @@ __global__ void __launch_bounds__(kSelWarps * 32, 4) k_sel_count(SelArgs a) {
       if (kk[1] < a.n_cells) count_cell(a, stage[wid], kk[1], lane);
     }
   }
+  if (lane == 0 && cands) atomicAdd(a.n_cand, cands);   // the step's candidate count
 }
 
 constexpr int kEmitWarps = 8;
@@ -443,8 +496,8 @@ k_sel_rcount(const int32_t* __restrict__ tmp_round, const int32_t* __restrict__ 
   }
 }
 
-// Block r: exclusive scan of cnt[r][0..chunks) + the offset of round r (in
-// place).  The round offsets (exclusive scan of the per-round counts) are
+// For every round r: exclusive scan of cnt[r][0..chunks) + the offset of round r (in
+// place).  Block 0 also writes *info.  The round offsets (exclusive scan of the per-round counts) are
 // formed here too: block r sums the counts of rounds < r, and block 0
 // writes the whole list.
 __device__ __forceinline__ int block_sum_256(int v, int* red) {
@@ -462,12 +515,20 @@ __device__ __forceinline__ int block_sum_256(int v, int* red) {
 __global__ void __launch_bounds__(256)
 k_sel_rscan(const int32_t* __restrict__ offs, int32_t n_cells, int64_t capacity,
             const int32_t* __restrict__ n_rounds, const int32_t* __restrict__ round_count,
-            int32_t* __restrict__ round_off, int32_t n_chunks, int32_t* __restrict__ cnt) {
+            int32_t* __restrict__ round_off, int32_t n_chunks, int32_t* __restrict__ cnt,
+            const unsigned long long* __restrict__ n_cand, dsmc_select_info_t* info) {
   __shared__ int warp_tot[8];
   __shared__ int red[8];
   __shared__ int carry;
   const int64_t total = offs[n_cells];
-  if (total > capacity || (int)blockIdx.x >= *n_rounds) return;
+  const int R = total > capacity ? 0 : *n_rounds;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    info->n_pairs = total;
+    info->n_candidates = (int64_t)*n_cand;
+    info->n_rounds = R;
+    info->pad_ = 0;
+  }
+  if ((int)blockIdx.x >= R) return;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (blockIdx.x == 0) {
     // round_off[0..DSMC_MAX_ROUNDS]: kPer consecutive counts per thread
@@ -498,30 +559,32 @@ k_sel_rscan(const int32_t* __restrict__ offs, int32_t n_cells, int64_t capacity,
     if (threadIdx.x == blockDim.x - 1) round_off[DSMC_MAX_ROUNDS] = run;   // the total
     __syncthreads();
   }
-  int part = 0;
-  for (int q = threadIdx.x; q < (int)blockIdx.x; q += blockDim.x) part += round_count[q];
-  part = block_sum_256(part, red);
   const int chunks = (int)((total + kScatterChunk - 1) / kScatterChunk);
-  int32_t* row = cnt + (size_t)blockIdx.x * n_chunks;
-  if (threadIdx.x == 0) carry = part;
-  __syncthreads();
-  for (int c0 = 0; c0 < chunks; c0 += blockDim.x) {
-    const int c = c0 + threadIdx.x;
-    const int v = c < chunks ? row[c] : 0;
-    int x = v;  // inclusive scan in the warp
+  for (int r = blockIdx.x; r < R; r += gridDim.x) {
+    int part = 0;
+    for (int q = threadIdx.x; q < r; q += blockDim.x) part += round_count[q];
+    part = block_sum_256(part, red);
+    int32_t* row = cnt + (size_t)r * n_chunks;
+    if (threadIdx.x == 0) carry = part;
+    __syncthreads();
+    for (int c0 = 0; c0 < chunks; c0 += blockDim.x) {
+      const int c = c0 + threadIdx.x;
+      const int v = c < chunks ? row[c] : 0;
+      int x = v;  // inclusive scan in the warp
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+      }
+      if (lane == 31) warp_tot[w] = x;
+      __syncthreads();
+      int before = carry;
+      for (int q = 0; q < w; ++q) before += warp_tot[q];
+      if (c < chunks) row[c] = before + x - v;
+      __syncthreads();
+      if (threadIdx.x == blockDim.x - 1) carry = before + x;
+      __syncthreads();
     }
-    if (lane == 31) warp_tot[w] = x;
-    __syncthreads();
-    int before = carry;
-    for (int q = 0; q < w; ++q) before += warp_tot[q];
-    if (c < chunks) row[c] = before + x - v;
-    __syncthreads();
-    if (threadIdx.x == blockDim.x - 1) carry = before + x;
-    __syncthreads();
   }
 }
 
@@ -606,16 +669,6 @@ k_sel_scatter(const int4* __restrict__ tmp, const int32_t* __restrict__ tmp_roun
   }
 }
 
-__global__ void k_sel_finalize(const int32_t* offs, int32_t n_cells, int64_t capacity,
-                               const unsigned long long* n_cand, const int32_t* n_rounds,
-                               dsmc_select_info_t* info) {
-  const int64_t total = offs[n_cells];
-  info->n_pairs = total;
-  info->n_candidates = (int64_t)*n_cand;
-  info->n_rounds = total > capacity ? 0 : *n_rounds;
-  info->pad_ = 0;
-}
-
 // ---------------------------------------------------------------- workspace
 struct SelWs {
   int32_t *counts, *offs, *tmp_round, *last, *round_count, *round_fill, *n_rounds;
@@ -651,8 +704,8 @@ static size_t carve(SelWs* w, char* p, int32_t n, int32_t n_cells, int64_t capac
   w->bits = (uint32_t*)take(sizeof(uint32_t) * cap);
   w->chunk_cnt = (int32_t*)take(sizeof(int32_t) * (size_t)DSMC_MAX_ROUNDS * (size_t)w->n_chunks);
   w->last = (int32_t*)take(sizeof(int32_t) * (size_t)(n > 0 ? n : 1));
-  // the following four are zeroed together
-  w->round_count = (int32_t*)take(sizeof(int32_t) * DSMC_MAX_ROUNDS * 2 + 256);
+  // the following four are zeroed together (kTotalsWords)
+  w->round_count = (int32_t*)take(sizeof(int32_t) * kTotalsWords);
   w->round_fill = w->round_count + DSMC_MAX_ROUNDS;
   w->n_rounds = w->round_count + 2 * DSMC_MAX_ROUNDS;
   w->n_cand = (unsigned long long*)(w->round_count + 2 * DSMC_MAX_ROUNDS + 2);
@@ -692,42 +745,32 @@ int launch_select(Ctx* c, const dsmc_gas_t& gas, int32_t n, int32_t n_cells, con
   sel_model(a, gas);
   a.order = order;
   const int sms = sm_count(c);
-  if (cudaMemsetAsync(w.round_count, 0, sizeof(int32_t) * DSMC_MAX_ROUNDS * 2 + 256, s) != cudaSuccess)
-    return DSMC_ERR_CUDA;
-  if (cudaMemsetAsync(round_offsets, 0, sizeof(int32_t) * (DSMC_MAX_ROUNDS + 1), s) != cudaSuccess)
-    return DSMC_ERR_CUDA;
-  if (n_cells > 0) {
-    k_sel_nwords<<<blocks_for(n_cells, 256, sms * 4), 256, 0, s>>>(a);
+  if (n_cells <= kWordsOne) {
+    k_sel_nwords_one<<<1, kWordsThreads, 0, s>>>(a, round_offsets, w.wofs);
     count_launches(c, 1);
-    int rcw = launch_scan(c, w.wcnt, w.wofs, n_cells, w.scan, s);
-    if (rcw) return rcw;
-    const unsigned gb = blocks_for((n_cells + 1) / 2, kSelWarps, sms * 8);
-    k_sel_count<<<gb, kSelWarps * 32, 0, s>>>(a);
-    count_launches(c, 1);
-    int rc = launch_scan(c, w.counts, w.offs, n_cells, w.scan, s);
-    if (rc) return rc;
-    k_sel_emit<<<blocks_for((n_cells + 1) / 2, kEmitWarps, sms * 16), kEmitWarps * 32, 0, s>>>(a);
-    count_launches(c, 1);
-    // at least one block: the capacity-overflow commit of (sigma g)_max runs in k_sel_rcount
-    const unsigned sb = (unsigned)((capacity + kScatterChunk - 1) / kScatterChunk) + (capacity <= 0);
-    {
-      k_sel_rcount<<<sb, 256, 0, s>>>(w.tmp_round, w.offs, n_cells, capacity, w.n_rounds, w.n_chunks, w.chunk_cnt,
-                                      w.sgnew, sgmax, order, w.round_count);
-      k_sel_rscan<<<DSMC_MAX_ROUNDS, 256, 0, s>>>(w.offs, n_cells, capacity, w.n_rounds, w.round_count,
-                                                 round_offsets, w.n_chunks, w.chunk_cnt);
-      const int ssm = (int)(sizeof(int) * kScatterWarps * DSMC_MAX_ROUNDS);
-      if (cudaFuncSetAttribute(k_sel_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, ssm) != cudaSuccess)
-        return DSMC_ERR_CUDA;
-      k_sel_scatter<<<sb, kScatterWarps * 32, ssm, s>>>(w.tmp, w.tmp_round, w.tmp_dep, w.offs, n_cells, capacity,
-                                                       w.n_rounds, w.n_chunks, w.chunk_cnt, (int4*)pairs, deps,
-                                                       order);
-      count_launches(c, 3);
-    }
   } else {
-    if (cudaMemsetAsync(w.offs, 0, sizeof(int32_t), s) != cudaSuccess) return DSMC_ERR_CUDA;
+    k_sel_nwords<<<blocks_for(n_cells, 256, sms * 4), 256, 0, s>>>(a, round_offsets);
+    count_launches(c, 1);
+    if (int rc = launch_scan(c, w.wcnt, w.wofs, n_cells, w.scan, s)) return rc;
   }
-  k_sel_finalize<<<1, 1, 0, s>>>(w.offs, n_cells, capacity, w.n_cand, w.n_rounds, info);
+  const unsigned gb = blocks_for((n_cells + 1) / 2, kSelWarps, sms * 8);
+  k_sel_count<<<gb, kSelWarps * 32, 0, s>>>(a);
   count_launches(c, 1);
+  if (int rc = launch_scan(c, w.counts, w.offs, n_cells, w.scan, s)) return rc;
+  k_sel_emit<<<blocks_for((n_cells + 1) / 2, kEmitWarps, sms * 16), kEmitWarps * 32, 0, s>>>(a);
+  // at least one block: the capacity-overflow commit of (sigma g)_max runs in k_sel_rcount
+  const unsigned sb = (unsigned)((capacity + kScatterChunk - 1) / kScatterChunk) + (capacity <= 0);
+  k_sel_rcount<<<sb, 256, 0, s>>>(w.tmp_round, w.offs, n_cells, capacity, w.n_rounds, w.n_chunks, w.chunk_cnt,
+                                  w.sgnew, sgmax, order, w.round_count);
+  // (a gas needs a few tens of rounds; a block per possible round was mostly empty blocks)
+  k_sel_rscan<<<64, 256, 0, s>>>(w.offs, n_cells, capacity, w.n_rounds, w.round_count, round_offsets, w.n_chunks,
+                                 w.chunk_cnt, w.n_cand, info);
+  const int ssm = (int)(sizeof(int) * kScatterWarps * DSMC_MAX_ROUNDS);
+  if (cudaFuncSetAttribute(k_sel_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, ssm) != cudaSuccess)
+    return DSMC_ERR_CUDA;
+  k_sel_scatter<<<sb, kScatterWarps * 32, ssm, s>>>(w.tmp, w.tmp_round, w.tmp_dep, w.offs, n_cells, capacity,
+                                                   w.n_rounds, w.n_chunks, w.chunk_cnt, (int4*)pairs, deps, order);
+  count_launches(c, 4);
   return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
 }
 

@@ -79,3 +79,67 @@ def test_chi_does_not_depend_on_the_warp_it_runs_in(n_nodes):
     one = [float(host(C.jager_chi(gas, pot, cuda(b[q:q + 1]), cuda(g[q:q + 1]), n_nodes=n_nodes))[0])
            for q in range(0, len(g), 7)]
     assert np.array_equal(np.float32(one), whole[::7])
+
+
+@pytest.mark.parametrize("n", [4096, 65536, 65537, 2500000, 2500001])
+def test_sort_variants_by_particle_count(n):
+    """16 and 17 chunks of the radix sort (the scatter sums few chunks' counts itself) and both sides of
+    the gather's switch from one launch to one per component: the stable order, bit for bit."""
+    C = ctx()
+    rng = np.random.default_rng(n)
+    nc = 1000
+    cid = rng.integers(0, nc, n).astype(np.int32)
+    v = [rng.standard_normal(n) for _ in range(3)]
+    out = C.sort_cells(cuda(cid), *[cuda(c) for c in v], nc)
+    assert C.sync_status() == 0
+    perm = np.argsort(cid, kind="stable")
+    assert np.array_equal(host(out["perm"]), perm)
+    assert np.array_equal(host(out["cell_start"]), np.concatenate([[0], np.cumsum(np.bincount(cid, minlength=nc))]))
+    for k, c in zip(("svx", "svy", "svz"), v):
+        assert np.array_equal(host(out[k]), c[perm])
+
+
+@pytest.mark.parametrize("order", [0, 1])
+@pytest.mark.parametrize("pad", [4096, 4097, 8192, 8193])
+def test_selection_variants_by_cell_count(pad, order):
+    """One-block and two-launch word counts and scans: the same cells followed by empty ones give the same
+    selection, whatever the number of cells."""
+    from paper_2602_21244_gb300 import dsmc as D
+    from paper_2602_21244_gb300 import workloads as W
+    C = ctx()
+    w = W.hypersonic(scale=0.05)
+    gas = D.make_gas(w["gas"])
+    got = []
+    for nc in (w["n_cells"], pad):
+        o = C.sort_cells(cuda(w["cell_id"]), cuda(w["vx"]), cuda(w["vy"]), cuda(w["vz"]), nc)
+        sg = C.sigma_g_max_init(gas, cuda(np.concatenate([w["T_cell"], np.full(nc - w["n_cells"], 300.0)])))
+        sel = C.select_pairs(gas, o["cell_start"], o["svx"], o["svy"], o["svz"], sg, 5, 1 << 18, order=order)
+        assert C.sync_status() == 0
+        info = host(sel["info"])
+        n, R = int(info[0]), int(info[2])
+        assert n > 1000 and R > 3
+        got.append([info, host(sel["pairs"])[:n], host(sel["deps"])[:n], host(sel["round_offsets"])[:R + 1],
+                    host(sg)[:w["n_cells"]]])
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
+
+
+def test_collide_accepts_a_workspace_at_any_word():
+    """The done stamps are cleared 16 bytes at a time only from an aligned workspace."""
+    from paper_2602_21244_gb300 import dsmc as D
+    from paper_2602_21244_gb300 import workloads as W
+    C = ctx()
+    w = W.hypersonic(scale=0.05, model=0)
+    gas = D.make_gas(w["gas"])
+    o = C.sort_cells(cuda(w["cell_id"]), cuda(w["vx"]), cuda(w["vy"]), cuda(w["vz"]), w["n_cells"])
+    sg = C.sigma_g_max_init(gas, cuda(w["T_cell"]))
+    sel = C.select_pairs(gas, o["cell_start"], o["svx"], o["svy"], o["svz"], sg, 1, 1 << 18)
+    n = len(w["cell_id"])
+    got = []
+    for shift in (0, 4, 12):
+        ws = torch().full((4 * n + 1024,), 255, dtype=torch().uint8, device="cuda")[shift:]
+        v = [o[k].clone() for k in ("svx", "svy", "svz")]
+        C.collide_vhs(gas, 1, sel, *v, ws=ws)
+        assert C.sync_status() == 0
+        got.append(host(torch().stack(v)))
+    assert np.array_equal(got[0], got[1]) and np.array_equal(got[0], got[2])
