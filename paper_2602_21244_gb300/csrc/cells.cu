@@ -56,6 +56,7 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* total) {
 }
 
 __global__ void k_scan_reduce(const int32_t* __restrict__ in, int64_t n, int32_t* bsum) {
+  dep_wait();
   const int64_t base = (int64_t)blockIdx.x * kScanItems;
   int s = 0;
   for (int q = 0; q < kScanPer; ++q) {
@@ -68,6 +69,7 @@ __global__ void k_scan_reduce(const int32_t* __restrict__ in, int64_t n, int32_t
 }
 
 __global__ void k_scan_blocks(int32_t* bsum, int64_t nb) {
+  dep_wait();
   int carry = 0;
   for (int64_t b0 = 0; b0 < nb; b0 += kScanThreads) {
     const int64_t i = b0 + threadIdx.x;
@@ -82,6 +84,7 @@ __global__ void k_scan_blocks(int32_t* bsum, int64_t nb) {
 // bsum: the blocks' sums (scanned false) or their exclusive scan
 __global__ void k_scan_apply(const int32_t* __restrict__ in, int64_t n, const int32_t* bsum, int scanned,
                              int32_t* __restrict__ out) {
+  dep_wait();
   int first;
   if (scanned) {
     first = bsum[blockIdx.x];
@@ -110,6 +113,7 @@ __global__ void k_scan_apply(const int32_t* __restrict__ in, int64_t n, const in
 
 __global__ void __launch_bounds__(1024) k_scan_one(const int32_t* __restrict__ in, int64_t n,
                                                    int32_t* __restrict__ out) {
+  dep_wait();
   int run = 0;
   for (int64_t t0 = 0; t0 < n; t0 += 1024 * kScanOnePer) {
     const int64_t base = t0 + (int64_t)threadIdx.x * kScanOnePer;
@@ -138,16 +142,16 @@ int launch_scan(Ctx* c, const int32_t* in, int32_t* out, int64_t n, void* ws, cu
     return cudaMemsetAsync(out, 0, sizeof(int32_t), s) == cudaSuccess ? 0 : DSMC_ERR_CUDA;
   }
   if (n <= kScanOne) {
-    k_scan_one<<<1, 1024, 0, s>>>(in, n, out);
+    launch_dep(k_scan_one, 1, 1024, 0, s, in, n, out);
     if (c) count_launches(c, 1);
     return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
   }
   const int64_t nb = (n + kScanItems - 1) / kScanItems;
   int32_t* bsum = (int32_t*)ws;
   const bool scan_sums = nb > kScanBlocks;
-  k_scan_reduce<<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, bsum);
-  if (scan_sums) k_scan_blocks<<<1, kScanThreads, 0, s>>>(bsum, nb);
-  k_scan_apply<<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, bsum, scan_sums, out);
+  launch_dep(k_scan_reduce, (unsigned)nb, kScanThreads, 0, s, in, n, bsum);
+  if (scan_sums) launch_dep(k_scan_blocks, 1, kScanThreads, 0, s, bsum, nb);
+  launch_dep(k_scan_apply, (unsigned)nb, kScanThreads, 0, s, in, n, bsum, scan_sums, out);
   if (c) count_launches(c, 2 + scan_sums);
   return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
 }
@@ -309,6 +313,7 @@ __global__ void k_gather(int32_t n, const int32_t* __restrict__ cell_start, int3
                          const int32_t* __restrict__ perm, const double* __restrict__ vx,
                          const double* __restrict__ vy, const double* __restrict__ vz,
                          double* __restrict__ svx, double* __restrict__ svy, double* __restrict__ svz) {
+  dep_wait();
   const int32_t filled = min(n, cell_start[n_cells]);
   // four slots per thread per pass, their loads issued before any store, so
   // that twelve independent random reads per thread are in flight
@@ -342,6 +347,7 @@ __global__ void k_gather(int32_t n, const int32_t* __restrict__ cell_start, int3
 __global__ void k_gather1(int32_t n, const int32_t* __restrict__ cell_start, int32_t n_cells,
                           const int32_t* __restrict__ perm, const double* __restrict__ v,
                           double* __restrict__ sv) {
+  dep_wait();
   const int32_t filled = min(n, cell_start[n_cells]);
   constexpr int kIlp = 4;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -383,6 +389,7 @@ __device__ __forceinline__ uint32_t rs_key(const int32_t* cell_id, const uint32_
 __global__ void __launch_bounds__(256)
 k_rs_count(const int32_t* __restrict__ cell_id, const uint32_t* __restrict__ keys, int32_t n, int32_t n_cells,
            int shift, int32_t chunks, int32_t* __restrict__ cnt, int* status) {
+  dep_wait();
   __shared__ int hist[kRadix];
   for (int t = threadIdx.x; t < kRadix; t += blockDim.x) hist[t] = 0;
   __syncthreads();
@@ -397,6 +404,7 @@ k_rs_count(const int32_t* __restrict__ cell_id, const uint32_t* __restrict__ key
 // the digit-major table, in place into off) and the digit's total.
 __global__ void __launch_bounds__(256)
 k_rs_rowscan(const int32_t* __restrict__ cnt, int32_t chunks, int32_t* __restrict__ off, int32_t* __restrict__ tot) {
+  dep_wait();
   __shared__ int wt[8];
   __shared__ int carry;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -454,6 +462,7 @@ k_rs_scatter(const int32_t* __restrict__ cell_id, const uint32_t* __restrict__ k
              const int32_t* __restrict__ vals, int32_t n, int32_t n_cells, int shift, int32_t chunks,
              const int32_t* __restrict__ base, const int32_t* __restrict__ tot, uint32_t* __restrict__ keys_out,
              int32_t* __restrict__ vals_out) {
+  dep_wait();
   __shared__ union {
     int wh[kRsWarps][kRadix];                              // per-warp digit counters, then positions
     struct { uint32_t key[kRsChunk]; int32_t val[kRsChunk]; } st;  // the chunk in digit order
@@ -572,6 +581,7 @@ k_rs_scatter(const int32_t* __restrict__ cell_id, const uint32_t* __restrict__ k
 // (slot n closes the list with key n_cells).  Four slots per thread.
 __global__ void k_cell_start(const uint32_t* __restrict__ skeys, int32_t n, int32_t n_cells,
                              int32_t* __restrict__ cell_start) {
+  dep_wait();
   // 32-bit indices: slots 0..n (n < 2^31), keys 0..n_cells
   const uint32_t un = (uint32_t)n, stride = gridDim.x * blockDim.x * 4u;
   for (uint32_t s0 = (blockIdx.x * blockDim.x + threadIdx.x) * 4u; s0 <= un; s0 += stride) {
@@ -641,7 +651,7 @@ int launch_sort_keys(Ctx* c, int32_t n, int32_t n_cells, const int32_t* cell_id,
   int32_t* off = (int32_t*)take(4 * (tab + 1));
   int32_t* dtot = (int32_t*)take(sizeof(int32_t) * kRadix);   // digit totals
   if (n == 0) {
-    k_cell_start<<<1, 256, 0, s>>>(kb, 0, n_cells, cell_start);
+    launch_dep(k_cell_start, 1, 256, 0, s, kb, 0, n_cells, cell_start);
     count_launches(c, 1);
     return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
   }
@@ -652,17 +662,17 @@ int launch_sort_keys(Ctx* c, int32_t n, int32_t n_cells, const int32_t* cell_id,
     const bool last = q + 1 == passes;
     uint32_t* kout = (q & 1) ? kb : ka;
     int32_t* vout = last ? perm : ((q & 1) ? vb : va);
-    k_rs_count<<<chunks, 256, 0, s>>>(cell_id, kin, n, n_cells, q * kRadixBits, chunks, cnt,
+    launch_dep(k_rs_count, chunks, 256, 0, s, cell_id, kin, n, n_cells, q * kRadixBits, chunks, cnt,
                                       q == 0 ? status_ptr(c) : nullptr);
     const bool direct = chunks <= kRsDirect;
-    if (!direct) k_rs_rowscan<<<kRadix, 256, 0, s>>>(cnt, chunks, off, dtot);
-    k_rs_scatter<<<chunks, kRsWarps * 32, 0, s>>>(cell_id, kin, vin, n, n_cells, q * kRadixBits, chunks,
+    if (!direct) launch_dep(k_rs_rowscan, kRadix, 256, 0, s, cnt, chunks, off, dtot);
+    launch_dep(k_rs_scatter, chunks, kRsWarps * 32, 0, s, cell_id, kin, vin, n, n_cells, q * kRadixBits, chunks,
                                                   direct ? nullptr : off, direct ? cnt : dtot, kout, vout);
     count_launches(c, 3 - direct);
     kin = kout;
     vin = vout;
   }
-  k_cell_start<<<grid_for(((int64_t)n + 4) / 4, 256, sm_count(c) * 8), 256, 0, s>>>(kin, n, n_cells, cell_start);
+  launch_dep(k_cell_start, grid_for(((int64_t)n + 4) / 4, 256, sm_count(c) * 8), 256, 0, s, kin, n, n_cells, cell_start);
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
 }
@@ -673,7 +683,7 @@ int launch_gather_one(Ctx* c, int32_t n, int32_t n_cells, const int32_t* cell_st
   if (n <= 0) return 0;
   const Shape sh = shape_or_default(c, DSMC_TUNE_GATHER);
   const unsigned g = grid_for(n, sh.threads, sm_count(c) * sh.blocks_per_sm);
-  k_gather1<<<g, sh.threads, 0, s>>>(n, cell_start, n_cells, perm, v, sv);
+  launch_dep(k_gather1, g, sh.threads, 0, s, n, cell_start, n_cells, perm, v, sv);
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
 }
@@ -689,13 +699,15 @@ int launch_gather(Ctx* c, int32_t n, int32_t n_cells, const int32_t* cell_start,
   const Shape sh = shape_or_default(c, DSMC_TUNE_GATHER);
   const unsigned g = grid_for(n, sh.threads, sm_count(c) * sh.blocks_per_sm);
   if (n <= kGatherAll) {
-    k_gather<<<g, sh.threads, 0, s>>>(n, cell_start, n_cells, perm, vx, vy, vz, svx, svy, svz);
+    launch_dep(k_gather, g, sh.threads, 0, s, n, cell_start, n_cells, perm, vx, vy, vz, svx, svy, svz);
     count_launches(c, 1);
     return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
   }
+  // launched after the sort has ended, so that the split between L1 and shared
+  // memory is the gather's own (its random reads want the L1)
   k_gather1<<<g, sh.threads, 0, s>>>(n, cell_start, n_cells, perm, vx, svx);
-  k_gather1<<<g, sh.threads, 0, s>>>(n, cell_start, n_cells, perm, vy, svy);
-  k_gather1<<<g, sh.threads, 0, s>>>(n, cell_start, n_cells, perm, vz, svz);
+  launch_dep(k_gather1, g, sh.threads, 0, s, n, cell_start, n_cells, perm, vy, svy);
+  launch_dep(k_gather1, g, sh.threads, 0, s, n, cell_start, n_cells, perm, vz, svz);
   count_launches(c, 3);
   return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
 }
@@ -792,6 +804,7 @@ template <bool MATCH>
 __global__ void __launch_bounds__(kCwWarps * 32, MATCH ? 3 : 4)
 k_cells(int32_t n_cells, const int32_t* __restrict__ cs, double* vx, double* vy, double* vz, double* mom,
         int* status, unsigned* work) {
+  dep_wait();
   __shared__ CwWarp sw[kCwWarps];
   CwWarp& W = sw[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31, sl = lane & (kSeg - 1), seg = lane / kSeg;
@@ -865,6 +878,7 @@ template <bool MATCH, int SEG>
 __global__ void __launch_bounds__(kCwWarps * 32)
 k_cells_once(int32_t n_cells, const int32_t* __restrict__ cs, double* vx, double* vy, double* vz, double* mom,
              int* status) {
+  dep_wait();
   const int lane = threadIdx.x & 31, sl = lane & (SEG - 1);
   const int64_t k = ((int64_t)blockIdx.x * kCwWarps + (threadIdx.x >> 5)) * (32 / SEG) + lane / SEG;
   const bool act = k < n_cells;
@@ -934,11 +948,11 @@ static int launch_cells(Ctx* c, bool match, int32_t n_cells, const int32_t* cs, 
     const unsigned gb = grid_for(n_cells, kCwWarps * 32 / seg, INT_MAX);
     int* st = status_ptr(c);
     if (match) {
-      if (seg == 32) k_cells_once<true, 32><<<gb, kCwWarps * 32, 0, s>>>(n_cells, cs, vx, vy, vz, mom, st);
-      else k_cells_once<true, 8><<<gb, kCwWarps * 32, 0, s>>>(n_cells, cs, vx, vy, vz, mom, st);
+      if (seg == 32) launch_dep(k_cells_once<true, 32>, gb, kCwWarps * 32, 0, s, n_cells, cs, vx, vy, vz, mom, st);
+      else launch_dep(k_cells_once<true, 8>, gb, kCwWarps * 32, 0, s, n_cells, cs, vx, vy, vz, mom, st);
     } else {
-      if (seg == 32) k_cells_once<false, 32><<<gb, kCwWarps * 32, 0, s>>>(n_cells, cs, vx, vy, vz, mom, st);
-      else k_cells_once<false, 8><<<gb, kCwWarps * 32, 0, s>>>(n_cells, cs, vx, vy, vz, mom, st);
+      if (seg == 32) launch_dep(k_cells_once<false, 32>, gb, kCwWarps * 32, 0, s, n_cells, cs, vx, vy, vz, mom, st);
+      else launch_dep(k_cells_once<false, 8>, gb, kCwWarps * 32, 0, s, n_cells, cs, vx, vy, vz, mom, st);
     }
     count_launches(c, 1);
     return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
@@ -946,8 +960,8 @@ static int launch_cells(Ctx* c, bool match, int32_t n_cells, const int32_t* cs, 
   const Shape sh = shape_or_default(c, match ? DSMC_TUNE_MOMENT_MATCH : DSMC_TUNE_MOMENTS);
   const int64_t runs = ((int64_t)n_cells + kCwRun - 1) / kCwRun;
   const unsigned g = grid_for(runs, kCwWarps * kCwClaims, sm_count(c) * sh.blocks_per_sm);
-  if (match) k_cells<true><<<g, kCwWarps * 32, 0, s>>>(n_cells, cs, vx, vy, vz, mom, nullptr, work_ptr(c));
-  else k_cells<false><<<g, kCwWarps * 32, 0, s>>>(n_cells, cs, vx, vy, vz, mom, status_ptr(c), work_ptr(c));
+  if (match) launch_dep(k_cells<true>, g, kCwWarps * 32, 0, s, n_cells, cs, vx, vy, vz, mom, nullptr, work_ptr(c));
+  else launch_dep(k_cells<false>, g, kCwWarps * 32, 0, s, n_cells, cs, vx, vy, vz, mom, status_ptr(c), work_ptr(c));
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
 }
@@ -1047,7 +1061,7 @@ extern "C" int dsmc_sort_cells_static(int32_t n, int32_t n_cells, const int32_t*
     k_fix_gather<<<grid_for(n_cells, kFixWarps, d->sms * 4), kFixWarps * 32, 0, s>>>(n_cells, cell_start, slots,
                                                                                       perm);
     k_fix_large<<<grid_for(n_cells, 1, d->sms), kLgWarps * 32, 0, s>>>(n_cells, cell_start, slots, perm);
-    k_gather<<<grid_for(n, 256, d->sms * 16), 256, 0, s>>>(n, cell_start, n_cells, perm, vx, vy, vz, svx,
+    launch_dep(k_gather, grid_for(n, 256, d->sms * 16), 256, 0, s, n, cell_start, n_cells, perm, vx, vy, vz, svx,
                                                            svy, svz);
   }
   return cudaGetLastError() == cudaSuccess ? DSMC_OK : DSMC_ERR_CUDA;

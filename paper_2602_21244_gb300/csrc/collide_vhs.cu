@@ -25,6 +25,7 @@ struct VhsArgs {
 };
 
 __global__ void __launch_bounds__(256) k_collide_vhs(VhsArgs a) {
+  dep_wait();
   if (a.step_dev) a.step = *a.step_dev;
   const int R = a.info->n_rounds;
   const int lane = threadIdx.x & 31;
@@ -90,6 +91,7 @@ int occupancy_collide_vhs(int threads) {
 // The done stamps and the barrier words (abort, unit cursor) of a collide call
 // start at zero: one launch for both.
 __global__ void k_clear_stamps(unsigned* __restrict__ done, int32_t n, unsigned* bar) {
+  dep_wait();
   if (blockIdx.x == 0 && threadIdx.x < 4) bar[threadIdx.x] = 0u;
   const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
   // 16 bytes at a time from an aligned workspace, word by word otherwise and at the end
@@ -102,7 +104,7 @@ int launch_clear_stamps(Ctx* c, unsigned* done, int32_t n, unsigned* bar, cudaSt
   int64_t b = ((int64_t)n + 4095) / 4096;
   if (b < 1) b = 1;
   if (b > 8 * sm_count(c)) b = 8 * sm_count(c);
-  k_clear_stamps<<<(unsigned)b, 256, 0, s>>>(done, n, bar);
+  launch_dep(k_clear_stamps, (unsigned)b, 256, 0, s, done, n, bar);
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
 }
@@ -120,7 +122,7 @@ int launch_collide_vhs(Ctx* c, const dsmc_gas_t& gas, uint64_t step, int32_t n, 
   VhsArgs a{gas.seed, step, graph_step_ptr(c), (const int4*)pairs, deps, ro, info, vx, vy, vz,
             (unsigned*)ws, barrier_ptr(c), status_ptr(c)};
   if (int rc = launch_clear_stamps(c, a.done, n, a.bar, s)) return rc;
-  k_collide_vhs<<<blocks, sh.threads, 0, s>>>(a);
+  launch_dep(k_collide_vhs, blocks, sh.threads, 0, s, a);
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : record(c, DSMC_ERR_CUDA, "collide_vhs: launch failed");
 }

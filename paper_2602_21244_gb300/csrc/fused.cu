@@ -115,6 +115,7 @@ struct Mem {
 // first cell of the groups g with cs[k-1] < g G <= cs[k] (cs[-1] = -1).
 __global__ void k_group_starts(const int32_t* __restrict__ cs, int32_t n_cells, int32_t n_groups,
                                int32_t* __restrict__ gstart) {
+  dep_wait();
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k <= n_cells; k += gridDim.x * blockDim.x) {
     if (k == n_cells) {
       // groups past the last cell start: empty
@@ -377,6 +378,7 @@ __device__ __forceinline__ void run_batch(const FusedArgs& a, FusedShared& S, co
 
 template <int PATH>
 __global__ void __launch_bounds__(kFThreads, 3) k_step_fused(FusedArgs a) {
+  dep_wait();
   extern __shared__ __align__(16) char smem_raw[];
   FusedShared& S = *reinterpret_cast<FusedShared*>(smem_raw);
   const int tid = threadIdx.x;
@@ -514,9 +516,9 @@ int launch_step_fused(Ctx* c, const dsmc_gas_t& gas, int path, const dsmc_chi_ta
       cudaMemsetAsync(info, 0, sizeof(dsmc_select_info_t), s) != cudaSuccess)
     return DSMC_ERR_CUDA;
   const int64_t gb = (n_cells + 1 + 255) / 256;
-  k_group_starts<<<(unsigned)(gb < 4096 ? gb : 4096), 256, 0, s>>>(cs, n_cells, a.n_groups, gstart);
-  if (path == DSMC_PATH_TABLE) k_step_fused<DSMC_PATH_TABLE><<<(unsigned)blocks, kFThreads, smem, s>>>(a);
-  else k_step_fused<DSMC_PATH_VHS><<<(unsigned)blocks, kFThreads, smem, s>>>(a);
+  launch_dep(k_group_starts, (unsigned)(gb < 4096 ? gb : 4096), 256, 0, s, cs, n_cells, a.n_groups, gstart);
+  if (path == DSMC_PATH_TABLE) launch_dep(k_step_fused<DSMC_PATH_TABLE>, (unsigned)blocks, kFThreads, smem, s, a);
+  else launch_dep(k_step_fused<DSMC_PATH_VHS>, (unsigned)blocks, kFThreads, smem, s, a);
   count_launches(c, 2);
   return cudaGetLastError() == cudaSuccess ? 0 : record(c, DSMC_ERR_CUDA, "step_fused: launch failed");
 }

@@ -956,6 +956,7 @@ __device__ __forceinline__ void collide_pair(const PotDev& P, const ChiShared& S
 // pair does not change its result.
 template <int KIND>
 __global__ void __launch_bounds__(128, 4) k_collide_jager(PotDev P, JagerArgs a) {
+  dep_wait_alone();
   if (a.step_dev) a.step = *a.step_dev;
   extern __shared__ float4 chi_sm[];
   const ChiShared S = chi_shared(P, (float*)chi_sm);
@@ -1018,6 +1019,7 @@ struct TableArgs {
 // from tag 4, E~ = ln(m g^2 / (4 k_B))); work claimed and ordered as in
 // k_collide_jager.
 __global__ void __launch_bounds__(256) k_collide_table(TableArgs a) {
+  dep_wait();
   if (a.step_dev) a.step = *a.step_dev;
   const int R = a.info->n_rounds;
   const int lane = threadIdx.x & 31;
@@ -1135,7 +1137,7 @@ int launch_jager_chi(Ctx* c, const dsmc_gas_t& gas, const dsmc_potential_t& pot,
   if (sm > kDefaultSmem &&
       cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
     return record(c, DSMC_ERR_CUDA, "jager_chi: shared-memory attribute");
-  k<<<blocks_n(n, sh.threads, sm_count(c) * sh.blocks_per_sm), sh.threads, sm, s>>>(P, n, b, g, chi);
+  launch_dep(k, blocks_n(n, sh.threads, sm_count(c) * sh.blocks_per_sm), sh.threads, sm, s, P, n, b, g, chi);
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
 }
@@ -1168,7 +1170,7 @@ int launch_collide_jager(Ctx* c, const dsmc_gas_t& gas, const dsmc_potential_t& 
   JagerArgs a{gas.seed, step, graph_step_ptr(c), gas.b_max * 1e10, (const int4*)pairs, deps, ro, info, vx, vy, vz,
               chi_out, (unsigned*)ws, barrier_ptr(c), status_ptr(c)};
   if (int rc = launch_clear_stamps(c, a.done, n, a.bar, s)) return rc;
-  k<<<blocks, sh.threads, sm, s>>>(P, a);
+  launch_dep(k, blocks, sh.threads, sm, s, P, a);
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : record(c, DSMC_ERR_CUDA, "collide_jager: launch failed");
 }
@@ -1206,7 +1208,7 @@ int launch_collide_table(Ctx* c, const dsmc_gas_t& gas, const dsmc_chi_table_t& 
   a.vx = vx; a.vy = vy; a.vz = vz; a.chi_out = chi_out;
   a.done = (unsigned*)ws; a.bar = barrier_ptr(c); a.status = status_ptr(c);
   if (int rc = launch_clear_stamps(c, a.done, n, a.bar, s)) return rc;
-  k_collide_table<<<blocks, sh.threads, 0, s>>>(a);
+  launch_dep(k_collide_table, blocks, sh.threads, 0, s, a);
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : record(c, DSMC_ERR_CUDA, "collide_table: launch failed");
 }

@@ -783,6 +783,7 @@ __device__ __forceinline__ void role_sync(int id, int n) { asm volatile("bar.syn
 
 __global__ void __launch_bounds__(kPipeThreads, 1) k_collide_neural(MlpShape sh, const uint16_t* __restrict__ w,
                                                                  const float* __restrict__ bias, NeuralArgs a) {
+  dep_wait_alone();
   if (a.step_dev) a.step = *a.step_dev;
   extern __shared__ __align__(1024) char smem[];
   const PipeLayout P = pipe_layout(sh.n_hidden);
@@ -926,7 +927,7 @@ int launch_collide_neural(Ctx* c, const dsmc_gas_t& gas, const dsmc_mlp_t& mlp,
   a.mom = mom; a.u_out = u_out; a.pairs = (const int4*)pairs; a.deps = deps; a.ro = ro; a.info = info;
   a.vx = vx; a.vy = vy; a.vz = vz; a.done = (unsigned*)ws; a.bar = barrier_ptr(c); a.status = status_ptr(c);
   if (int rc = launch_clear_stamps(c, a.done, n, a.bar, s)) return rc;
-  k_collide_neural<<<sm_count(c) * per_sm, kPipeThreads, P.total, s>>>(sh, w, bias, a);
+  launch_dep(k_collide_neural, sm_count(c) * per_sm, kPipeThreads, P.total, s, sh, w, bias, a);
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : record(c, DSMC_ERR_CUDA, "collide_neural: launch failed");
 }

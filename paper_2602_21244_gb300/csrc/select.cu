@@ -52,6 +52,7 @@ __device__ __forceinline__ void clear_totals(const SelArgs& a, int32_t* round_of
 }
 
 __global__ void k_sel_nwords(SelArgs a, int32_t* round_off) {
+  dep_wait();
   if (a.step_dev) a.step = *a.step_dev;
   if (blockIdx.x == 0) clear_totals(a, round_off, threadIdx.x, blockDim.x);
   for (int32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < a.n_cells; k += gridDim.x * blockDim.x)
@@ -63,6 +64,7 @@ __global__ void k_sel_nwords(SelArgs a, int32_t* round_off) {
 constexpr int kWordsThreads = 1024;
 constexpr int32_t kWordsOne = 4 * kWordsThreads;
 __global__ void __launch_bounds__(kWordsThreads) k_sel_nwords_one(SelArgs a, int32_t* round_off, int32_t* wofs) {
+  dep_wait();
   if (a.step_dev) a.step = *a.step_dev;
   __shared__ int wsum[kWordsThreads / 32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -211,6 +213,7 @@ __device__ __forceinline__ void count_pair(const SelArgs& a, float4* stage, cons
 // most 16 candidates (and fits half the staging slice), else one after the
 // other by the whole warp.
 __global__ void __launch_bounds__(kSelWarps * 32, 4) k_sel_count(SelArgs a) {
+  dep_wait();
   if (a.step_dev) a.step = *a.step_dev;
   __shared__ float4 stage[kSelWarps][kStage];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -249,6 +252,7 @@ constexpr int kEmitWords = 16;    // accept-bit words expanded per step (512 can
 // from the FP64 velocities; a cell of more than kStage particles takes its
 // rounds on one lane from global memory.
 __global__ void __launch_bounds__(kEmitWarps * 32, 4) k_sel_emit(SelArgs a) {
+  dep_wait();
   if (a.step_dev) a.step = *a.step_dev;
   __shared__ uint32_t slist[kEmitWarps][kEmitWords * 32];  // accepted candidate indices
   __shared__ uint32_t smsk[kEmitWarps][kStage];            // per-particle lane masks (batch_rounds)
@@ -472,6 +476,7 @@ k_sel_rcount(const int32_t* __restrict__ tmp_round, const int32_t* __restrict__ 
              int64_t capacity, const int32_t* __restrict__ n_rounds, int32_t n_chunks, int32_t* __restrict__ cnt,
              const double* __restrict__ sgnew, double* __restrict__ sgmax, int order,
              int32_t* __restrict__ level_count) {
+  dep_wait();
   __shared__ int hist[DSMC_MAX_ROUNDS];
   const int64_t total = offs[n_cells];
   if (total > capacity) {
@@ -517,6 +522,7 @@ k_sel_rscan(const int32_t* __restrict__ offs, int32_t n_cells, int64_t capacity,
             const int32_t* __restrict__ n_rounds, const int32_t* __restrict__ round_count,
             int32_t* __restrict__ round_off, int32_t n_chunks, int32_t* __restrict__ cnt,
             const unsigned long long* __restrict__ n_cand, dsmc_select_info_t* info) {
+  dep_wait();
   __shared__ int warp_tot[8];
   __shared__ int red[8];
   __shared__ int carry;
@@ -605,6 +611,7 @@ k_sel_scatter(const int4* __restrict__ tmp, const int32_t* __restrict__ tmp_roun
               const uint32_t* __restrict__ tmp_dep, const int32_t* __restrict__ offs, int32_t n_cells,
               int64_t capacity, const int32_t* __restrict__ n_rounds, int32_t n_chunks,
               const int32_t* __restrict__ base, int4* __restrict__ out, uint32_t* __restrict__ deps, int order) {
+  dep_wait();
   extern __shared__ int swh[];   // [kScatterWarps][R]
   const int64_t total = offs[n_cells];
   if (total > capacity) return;
@@ -746,29 +753,29 @@ int launch_select(Ctx* c, const dsmc_gas_t& gas, int32_t n, int32_t n_cells, con
   a.order = order;
   const int sms = sm_count(c);
   if (n_cells <= kWordsOne) {
-    k_sel_nwords_one<<<1, kWordsThreads, 0, s>>>(a, round_offsets, w.wofs);
+    launch_dep(k_sel_nwords_one, 1, kWordsThreads, 0, s, a, round_offsets, w.wofs);
     count_launches(c, 1);
   } else {
-    k_sel_nwords<<<blocks_for(n_cells, 256, sms * 4), 256, 0, s>>>(a, round_offsets);
+    launch_dep(k_sel_nwords, blocks_for(n_cells, 256, sms * 4), 256, 0, s, a, round_offsets);
     count_launches(c, 1);
     if (int rc = launch_scan(c, w.wcnt, w.wofs, n_cells, w.scan, s)) return rc;
   }
   const unsigned gb = blocks_for((n_cells + 1) / 2, kSelWarps, sms * 8);
-  k_sel_count<<<gb, kSelWarps * 32, 0, s>>>(a);
+  launch_dep(k_sel_count, gb, kSelWarps * 32, 0, s, a);
   count_launches(c, 1);
   if (int rc = launch_scan(c, w.counts, w.offs, n_cells, w.scan, s)) return rc;
-  k_sel_emit<<<blocks_for((n_cells + 1) / 2, kEmitWarps, sms * 16), kEmitWarps * 32, 0, s>>>(a);
+  launch_dep(k_sel_emit, blocks_for((n_cells + 1) / 2, kEmitWarps, sms * 16), kEmitWarps * 32, 0, s, a);
   // at least one block: the capacity-overflow commit of (sigma g)_max runs in k_sel_rcount
   const unsigned sb = (unsigned)((capacity + kScatterChunk - 1) / kScatterChunk) + (capacity <= 0);
-  k_sel_rcount<<<sb, 256, 0, s>>>(w.tmp_round, w.offs, n_cells, capacity, w.n_rounds, w.n_chunks, w.chunk_cnt,
+  launch_dep(k_sel_rcount, sb, 256, 0, s, w.tmp_round, w.offs, n_cells, capacity, w.n_rounds, w.n_chunks, w.chunk_cnt,
                                   w.sgnew, sgmax, order, w.round_count);
   // (a gas needs a few tens of rounds; a block per possible round was mostly empty blocks)
-  k_sel_rscan<<<64, 256, 0, s>>>(w.offs, n_cells, capacity, w.n_rounds, w.round_count, round_offsets, w.n_chunks,
+  launch_dep(k_sel_rscan, 64, 256, 0, s, w.offs, n_cells, capacity, w.n_rounds, w.round_count, round_offsets, w.n_chunks,
                                  w.chunk_cnt, w.n_cand, info);
   const int ssm = (int)(sizeof(int) * kScatterWarps * DSMC_MAX_ROUNDS);
   if (cudaFuncSetAttribute(k_sel_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, ssm) != cudaSuccess)
     return DSMC_ERR_CUDA;
-  k_sel_scatter<<<sb, kScatterWarps * 32, ssm, s>>>(w.tmp, w.tmp_round, w.tmp_dep, w.offs, n_cells, capacity,
+  launch_dep(k_sel_scatter, sb, kScatterWarps * 32, ssm, s, w.tmp, w.tmp_round, w.tmp_dep, w.offs, n_cells, capacity,
                                                    w.n_rounds, w.n_chunks, w.chunk_cnt, (int4*)pairs, deps, order);
   count_launches(c, 4);
   return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;

@@ -167,6 +167,7 @@ __device__ __forceinline__ void half_sums(double* v) {
 }
 
 __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
+  dep_wait_alone();
   extern __shared__ __align__(1024) char sm[];
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const int row = ((warp & 3) << 5) | lane, cg = warp >> 2, c0 = cg * 32;
@@ -648,6 +649,7 @@ __device__ __forceinline__ float ordered_sum(float s, const float* __restrict__ 
 constexpr int kReduceThreads = 128;
 __global__ void __launch_bounds__(kReduceThreads) k_train_reduce(const float* __restrict__ partial, int nblk, int d_in,
                                                                  float* __restrict__ grad, double* loss) {
+  dep_wait();
   const int nw = kH * d_in + 2 * kH * kH + 3 * kH;
   const int nb = kNB;
   if (blockIdx.x == 0) {   // the loss: lane l the values l, l + 32, ... of [CTA][lane group], then a tree
@@ -700,6 +702,7 @@ __global__ void __launch_bounds__(kReduceThreads) k_train_reduce(const float* __
 __global__ void k_adam(int n_w, int n_b, const float* __restrict__ grad, float* __restrict__ master,
                        float* __restrict__ m, float* __restrict__ v, uint16_t* __restrict__ w_bf16,
                        float* __restrict__ bias, float lr, float b1, float b2, float eps, float c1, float c2) {
+  dep_wait();
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n_w + n_b; q += gridDim.x * blockDim.x) {
     const float g = grad[q];
     const float mq = b1 * m[q] + (1.f - b1) * g;
@@ -736,11 +739,11 @@ int launch_train(Ctx* c, const dsmc_mlp_t& mlp, int mode, uint64_t seed, uint64_
   a.oi = oi; a.oj = oj; a.zst = act; a.partial = (float*)ws; a.status = status_ptr(c);
   const int64_t tiles = (n + kT - 1) / kT;
   const int blocks = (int)(tiles < sms ? (tiles > 0 ? tiles : 1) : sms);
-  k_train<<<blocks, kNT, S_TOTAL, s>>>(a);
+  launch_dep(k_train, blocks, kNT, S_TOTAL, s, a);
   count_launches(c, 1);
   if (mode != 0) {
     const int outs = kH * mlp.d_in + 2 * kH * kH + 3 * kH + kNB;
-    k_train_reduce<<<1 + (outs + kReduceThreads - 1) / kReduceThreads, kReduceThreads, 0, s>>>(
+    launch_dep(k_train_reduce, 1 + (outs + kReduceThreads - 1) / kReduceThreads, kReduceThreads, 0, s, 
         (const float*)ws, blocks, mlp.d_in, grad, loss);
     count_launches(c, 1);
   }
@@ -751,7 +754,7 @@ int launch_adam(Ctx* c, int n_w, int n_b, const float* grad, float* master, floa
                 float* bias, float lr, double b1, double b2, double eps, int64_t step, cudaStream_t s) {
   const float c1 = (float)(1.0 / (1.0 - pow(b1, (double)step)));
   const float c2 = (float)(1.0 / (1.0 - pow(b2, (double)step)));
-  k_adam<<<64, 256, 0, s>>>(n_w, n_b, grad, master, m, v, w, bias, lr, (float)b1, (float)b2, (float)eps, c1, c2);
+  launch_dep(k_adam, 64, 256, 0, s, n_w, n_b, grad, master, m, v, w, bias, lr, (float)b1, (float)b2, (float)eps, c1, c2);
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
 }
