@@ -230,12 +230,21 @@ __device__ __forceinline__ bool unit_range(const int32_t* __restrict__ ro, int R
   return false;
 }
 
-// Release / acquire at GPU scope (PTX memory model): a relaxed load of a
-// stamp followed by fence.acq_rel is an acquire; fence.acq_rel followed by
-// a relaxed store of the stamp is a release.  Lighter than fence.sc.
+// Release / acquire at GPU scope (PTX memory model): fence.acq_rel followed by
+// a relaxed store of a stamp is a release (one fence for both particles'),
+// lighter than fence.sc.  The stamps are read by acquire loads: relaxed loads and
+// a fence on this side too made a warp wait for its other memory operations in
+// flight (look-up collide of 6.9 million pairs 594 against 564 us, neural
+// collide 1543 against 1531 us).
 __device__ __forceinline__ unsigned ld_relaxed(const unsigned* p) {
   unsigned v;
   asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+// (subsequent accesses of the thread are ordered after it)
+__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
 __device__ __forceinline__ void st_relaxed(unsigned* p, unsigned v) {
@@ -251,13 +260,13 @@ __device__ __forceinline__ bool wait_deps(const unsigned* done, int32_t i, int32
                                           uint64_t limit_ns = kBarrierLimitNs) {
   const unsigned ni = dep & 0xFFFFu, nj = dep >> 16;
   if (ni == 0 && nj == 0) return true;
-  if (ld_relaxed(done + i) >= ni && ld_relaxed(done + j) >= nj) { fence_acq_rel(); return true; }
+  if (ld_acquire(done + i) >= ni && ld_acquire(done + j) >= nj) return true;
   const uint64_t t0 = globaltimer_ns();
   unsigned sleep_ns = 32;   // doubling up to 1 us: a waiting lane costs few issue slots
   for (;;) {
     __nanosleep(sleep_ns);
     if (sleep_ns < 1024) sleep_ns <<= 1;
-    if (ld_relaxed(done + i) >= ni && ld_relaxed(done + j) >= nj) { fence_acq_rel(); return true; }
+    if (ld_acquire(done + i) >= ni && ld_acquire(done + j) >= nj) return true;
     if (ld_relaxed(abort_word) || globaltimer_ns() - t0 > limit_ns) {
       set_status(status, DSMC_ERR_TIMEOUT);
       atomicExch(abort_word, 1u);
