@@ -1,30 +1,29 @@
 // Neural collision operator (Sec. 2.2-2.3) on the tcgen05 tensor cores.
 //
-// A CTA of 512 threads runs two warp groups of 8 warps, each owning a tile
-// of 128 pairs and 256 TMEM columns (the FP32 accumulator, then the next
-// layer's A operand), so that one group's feature build, activation epilogue
-// and pair update run while the tensor core works on the other group's layer
-// (ping-pong; a single 16-warp group when two slots do not fit).  Within a
-// group: thread t < 128 builds row t of the bf16 input tile X (shared
-// memory), one elected thread issues the layer's tcgen05.mma chain (FP32
-// accumulator in TMEM, the bias added by the MMAs) and waits on the group's
-// mbarrier, the group's warps read their 32 TMEM lanes back (tcgen05.ld),
-// apply the activation and write the next layer's A operand into tensor memory
-// (tcgen05.st; row m in lane m, two bf16 per column) as two bf16 terms
-// (hi = bf16(a), lo = bf16(a - hi)) multiplied by the same bf16 weights:
-// bf16 operands, FP32 accumulation, about 16 significant bits kept for the
-// activations (single bf16 storage costs up to 6e-2 in the output direction
-// of badly conditioned pairs).  A hidden layer's MMA thus reads only its
-// weights from shared memory (with A there too its operand reads ran near
-// the SM's shared-memory bandwidth).  The weights of all layers stay in
-// shared memory for the life of the CTA.  After the last layer thread t
-// projects y onto the energy shell and applies the centre-of-mass update of
-// its pair in FP64.
+// The layers of a tile of 128 rows are tcgen05.mma chains issued by one thread
+// (FP32 accumulator in TMEM, the bias added by the MMAs); warps read their 32
+// TMEM lanes back (tcgen05.ld), apply the activation and write the next layer's
+// A operand into tensor memory (tcgen05.st; row m in lane m, two bf16 per
+// column) as two bf16 terms (hi = bf16(a), lo = bf16(a - hi)) multiplied by the
+// same bf16 weights: bf16 operands, FP32 accumulation, about 16 significant bits
+// kept for the activations (single bf16 storage costs up to 6e-2 in the output
+// direction of badly conditioned pairs).  A hidden layer's MMA thus reads only
+// its weights from shared memory (with A there too its operand reads ran near
+// the SM's shared-memory bandwidth).  The weights of all layers stay in shared
+// memory for the life of the CTA.
 //
-// The collide kernel is persistent: each group claims 128-pair tiles of one
-// round at a time from a global cursor, in round-major order, and a row
-// waits (bounded) until the previous pairs of its two particles are done
-// (per-particle done stamps), so no grid-wide barrier separates the rounds.
+// The standalone forward (k_mlp_forward): a CTA of 512 threads runs two warp
+// groups of 8 warps, each owning a tile and 256 TMEM columns (the accumulator,
+// then the next layer's A operand), so that one group's input rows and
+// epilogue run while the tensor core works on the other group's layer (a single
+// 16-warp group when two slots do not fit).
+//
+// The collide kernel (k_collide_neural, its roles described there) is
+// persistent: 128-pair tiles of one round are claimed from a global cursor, in
+// round-major order, and a row waits (bounded) until the previous pairs of its
+// two particles are done (per-particle done stamps), so no grid-wide barrier
+// separates the rounds; after the last layer a thread projects its row's y onto
+// the energy shell and applies the centre-of-mass update of its pair in FP64.
 #include <cstdio>
 
 #include "internal.cuh"
@@ -166,9 +165,12 @@ __device__ void load_weights(char* smem, const MlpLayout& L, const MlpShape& sh,
   const uint16_t* wl = w + kWidth * sh.d_in;
   for (int l = 0; l < sh.n_hidden - 1; ++l) {
     char* dst = smem + L.w_sq + (uint32_t)l * kWidth * kWidth * 2;
-    for (int e = t; e < kWidth * kWidth; e += nt) {
-      const int n = e >> 7, k = e & 127;
-      *(uint16_t*)(dst + tc::kmajor_offset(n, k, kWidth)) = wl[e];
+    if (((uintptr_t)wl & 15u) == 0) {   // eight columns, one 16-byte load and store, at a time
+      for (int e = t; e < kWidth * kWidth / 8; e += nt)
+        *(uint4*)(dst + tc::kmajor_offset(e >> 4, (e & 15) * 8, kWidth)) = ((const uint4*)wl)[e];
+    } else {
+      for (int e = t; e < kWidth * kWidth; e += nt)
+        *(uint16_t*)(dst + tc::kmajor_offset(e >> 7, e & 127, kWidth)) = wl[e];
     }
     wl += kWidth * kWidth;
   }
@@ -532,6 +534,7 @@ __global__ void __launch_bounds__(128) k_tc_selftest(int N, int K, int layout, c
 // ---------------------------------------------------------------- collide
 struct NeuralArgs {
   uint64_t seed, step;
+  PhiloxKey key;             // round keys of seed
   const uint64_t* step_dev;
   double sigma_v_inv, T_ref_inv, m_over_3k, eps;
   float sigma_v_inv_f, T_feat_f;  // 1/sigma_v and m/(3 k T_ref) in FP32 for the MLP inputs
@@ -562,9 +565,11 @@ __device__ __forceinline__ void box_muller_f(uint32_t w1, uint32_t w2, float* z0
 // Build the MLP input row of pair p (features in FP32, Sec. 2.2 Eq. (mlp_input))
 // into the group's X tile and stash what the pair update needs -- p, the
 // particle slots and the six velocity components -- in word w of the row at
-// stash[w * 128 + row] (shared memory).  p < 0 marks a padding row.
+// stash[w * 128 + row] (shared memory).  q, dep: the pair's record; p < 0
+// marks a padding row.
 __device__ __forceinline__ void build_row(char* smem, uint32_t xoff, volatile int* fail, const MlpShape& sh,
-                                          const NeuralArgs& a, int row, int32_t p, uint32_t* stash) {
+                                          const NeuralArgs& a, int row, int32_t p, int4 q, uint32_t dep,
+                                          uint32_t* stash) {
   float f[16];
 #pragma unroll
   for (int c = 0; c < 16; ++c) f[c] = 0.f;
@@ -572,11 +577,9 @@ __device__ __forceinline__ void build_row(char* smem, uint32_t xoff, volatile in
 #pragma unroll
   for (int c = 0; c < 16; ++c) st[c] = 0u;
   st[0] = (uint32_t)-1;
-  int4 q = make_int4(0, 0, 0, 0);
   if (p >= 0) {
-    q = a.pairs[p];
     // the previous pairs of both particles must be done (bounded wait)
-    if (!wait_deps(a.done, q.x, q.y, a.deps[p], a.bar + 2, a.status)) {
+    if (!wait_deps(a.done, q.x, q.y, dep, a.bar + 2, a.status)) {
       *fail = 1;
       p = -1;
     }
@@ -592,8 +595,8 @@ __device__ __forceinline__ void build_row(char* smem, uint32_t xoff, volatile in
     f[0] = (f64_to_f32(xi) - f64_to_f32(xj)) * a.sigma_v_inv_f;
     f[1] = (f64_to_f32(yi) - f64_to_f32(yj)) * a.sigma_v_inv_f;
     f[2] = (f64_to_f32(zi) - f64_to_f32(zj)) * a.sigma_v_inv_f;
-    const u32x4 wa = draw(a.seed, (uint32_t)q.w, (uint32_t)q.z, a.step, TAG_NOISE, 0);
-    const u32x4 wb = draw(a.seed, (uint32_t)q.w, (uint32_t)q.z, a.step, TAG_NOISE, 1);
+    const u32x4 wa = draw_k(a.key, (uint32_t)q.w, (uint32_t)q.z, a.step, TAG_NOISE, 0);
+    const u32x4 wb = draw_k(a.key, (uint32_t)q.w, (uint32_t)q.z, a.step, TAG_NOISE, 1);
     float z[4];
     box_muller_f(wa.x, wa.z, &z[0], &z[1]);
     box_muller_f(wb.x, wb.z, &z[2], &z[3]);
@@ -670,39 +673,73 @@ __device__ __forceinline__ void update_row(const NeuralArgs& a, const float y[3]
 }
 
 // ---------------------------------------------------------------- pipelined collide
-// A CTA of 768 threads: two MLP warp groups of 8 warps (threads 0..511, TMEM
-// columns and tile work as in mlp_tile), four builder warps (512..639) and
-// four updater warps (640..767).  Tiles of 128 pairs of one round are
-// claimed by the builders from a global cursor in round-major order and
-// handed to the two MLP groups alternately through three buffers per group
-// (the input tile X, the per-row pair data the update needs, the MLP output
-// y, the tile's pair range and round): builders build tile k + 2 (waiting,
-// bounded, until the previous pairs of its particles are done) while an MLP
-// group runs the layers of tile k + 1 and the updaters apply the pair updates
-// of tile k and stamp its particles done.  So the MLP groups never wait for
-// the latency-bound build or the FP64 update.  Hand-offs are mbarriers:
-// built (128 builder arrivals), ydone (the 128 threads that hold y), freed
-// (128 updater arrivals); each buffer is reused every third tile of its
-// group.  No wait can be circular: a build only waits on tiles claimed
-// earlier, whose MLP and update stages never wait on a later build.  Every
-// wait is bounded and ends early once any role of the CTA (or a dependency
-// wait of any CTA) has failed.
-constexpr int kPipeThreads = 768;
-constexpr int kPipeBufs = 3;
-constexpr int kBuildBase = 512, kUpdateBase = 640, kRoleThreads = 128;
+// A CTA of 960 threads: 16 epilogue warps, eight builder warps, four updater
+// warps and two warps of one working lane each, one claiming the work, one
+// issuing the MMAs.  Tiles of 128 pairs of one round are claimed from a global
+// cursor in round-major order into a ring of six buffers (the input tile X, the
+// per-row pair data the update needs, the MLP output y, the tile's pair range
+// and round): two groups of four builder warps build the coming tiles (waiting,
+// bounded, until the previous pairs of their particles are done) while up to
+// three tiles are in their layers and the updaters apply the pair updates of an
+// earlier one and stamp its particles done.
+//
+// The layers of the tiles in flight are separate steps: an MMA (the issuing
+// lane takes the oldest tile whose input is ready) and its epilogue, for which all
+// 16 epilogue warps take the accumulators together, 32 columns each, in the
+// order of the MMAs.  TMEM is four regions of 128 columns: an MMA writes its
+// FP32 accumulators into a free one, the epilogue turns them in place into the
+// next layer's A operand (every 16 columns become 8 of bf16 hi and 8 of lo
+// terms), and the operand's region is free again once the MMA that reads it is
+// done -- so three tiles and one MMA in flight fit.  With two tiles, each bound
+// to its own 8 epilogue warps, those waited out every MMA of their tile (0.9 of
+// 2.9 us per layer), and a tile alone took 2 us per epilogue.
+//
+// Measured on 6.9 million pairs (357 tiles per SM): 1660 us with two bound
+// tiles, 1531 us now; a 200 x 200 cavity (670,000 pairs, 18 levels) 291 -> 276
+// us.  Per tile and SM 8,850 cycles: the epilogue warps work 6,800 of them (three
+// steps of 2,250, twice their instructions' issue time: the other roles' warps
+// share the schedulers), the issuing lane 3,600; a builder group takes 9,000
+// (stamps 4,400, gather 2,200, arithmetic 1,750, stores 460) but there are two.
+// Not kept: two epilogue groups taking steps in turn (1698 us), partial sums
+// handed over by mbarriers instead of named barriers (1570), the next pair's
+// record and stamps read ahead (1660), two tiles in flight (1586).  The shared
+// memory counts: the same kernel with 20 KB more that it does not use takes 1684
+// us, with eight buffers 1700, with four 1619: the L1 that is left serves the
+// random loads in flight.
+//
+// Hand-offs are mbarriers: claimed, built (128 builder arrivals), dfull (an MMA step's
+// commit and its description), edone (its epilogue, 16 warps), ydone (the 128
+// threads that hold y), freed (128 updater arrivals).  No wait can be circular:
+// a build only waits on tiles claimed earlier, whose layers and update never
+// wait on a later build (the issuing lane admits a tile once it is built and
+// until then goes on with the others).  Every wait is bounded and ends early once
+// any role of the CTA (or a dependency wait of any CTA) has failed.
+constexpr int kEpiThreads = 512, kEpiWarpsN = kEpiThreads / 32;
+constexpr int kRoleThreads = 128, kBuilders = 2 * kRoleThreads;   // (two tiles built side by side)
+constexpr int kBuildBase = kEpiThreads, kUpdateBase = kBuildBase + kBuilders, kIssueBase = kUpdateBase + kRoleThreads;
+constexpr int kClaimBase = kIssueBase + 32, kPipeThreads = kClaimBase + 32;
+constexpr int kPipeBufs = 6;
+constexpr int kInFlight = 3, kRegions = 4;
+// named barriers: the epilogue warps, updaters, then the pairs of
+// epilogue warps that hand partial outputs on (one per row quadrant and half)
+constexpr int kBarEpi = 1, kBarUpdate = 2, kBarChain = 3, kBarHalves = 11;
 
 struct PipeLayout {
-  MlpLayout m;        // weights, biases, per-group MMA barriers, TMEM pointer, column-group partials
-  uint32_t x0, st0, y0, info0, bars, abort, bcast, total;
-  __host__ __device__ uint32_t buf(int g, int b) const { return (uint32_t)(g * kPipeBufs + b); }
-  __host__ __device__ uint32_t x(int g, int b) const { return x0 + buf(g, b) * (uint32_t)(kTileM * kKin * 2); }
-  __host__ __device__ uint32_t st(int g, int b) const { return st0 + buf(g, b) * (uint32_t)(kStashWords * kTileM * 4); }
-  __host__ __device__ uint32_t y(int g, int b) const { return y0 + buf(g, b) * (uint32_t)(kTileM * 3 * 4); }
-  __host__ __device__ uint32_t info(int g, int b) const { return info0 + buf(g, b) * 16u; }
-  // mbarriers: built[6], ydone[6], freed[6]
-  __host__ __device__ uint32_t built(int g, int b) const { return bars + buf(g, b) * 8u; }
-  __host__ __device__ uint32_t ydone(int g, int b) const { return bars + (6u + buf(g, b)) * 8u; }
-  __host__ __device__ uint32_t freed(int g, int b) const { return bars + (12u + buf(g, b)) * 8u; }
+  MlpLayout m;        // weights, biases, TMEM pointer
+  uint32_t x0, st0, y0, info0, ops, bars, abort, total;
+  __host__ __device__ uint32_t x(int b) const { return x0 + (uint32_t)b * (uint32_t)(kTileM * kKin * 2); }
+  __host__ __device__ uint32_t st(int b) const { return st0 + (uint32_t)b * (uint32_t)(kStashWords * kTileM * 4); }
+  __host__ __device__ uint32_t y(int b) const { return y0 + (uint32_t)b * (uint32_t)(kTileM * 3 * 4); }
+  __host__ __device__ uint32_t info(int b) const { return info0 + (uint32_t)b * 16u; }
+  __host__ __device__ uint32_t op(uint32_t n) const { return ops + (n & 3u) * 16u; }
+  // mbarriers: built[6], ydone[6], freed[6], dfull[4], edone[4], drain, claimed[6]
+  __host__ __device__ uint32_t built(int b) const { return bars + (uint32_t)b * 8u; }
+  __host__ __device__ uint32_t ydone(int b) const { return bars + (uint32_t)(kPipeBufs + b) * 8u; }
+  __host__ __device__ uint32_t freed(int b) const { return bars + (uint32_t)(2 * kPipeBufs + b) * 8u; }
+  __host__ __device__ uint32_t dfull(uint32_t n) const { return bars + (3u * kPipeBufs + (n & 3u)) * 8u; }
+  __host__ __device__ uint32_t edone(uint32_t n) const { return bars + (3u * kPipeBufs + 4u + (n & 3u)) * 8u; }
+  __host__ __device__ uint32_t drain() const { return bars + (3u * kPipeBufs + 8u) * 8u; }
+  __host__ __device__ uint32_t claimed(int b) const { return bars + (3u * kPipeBufs + 9u + (uint32_t)b) * 8u; }
 };
 
 __host__ __device__ inline PipeLayout pipe_layout(int n_hidden) {
@@ -717,22 +754,22 @@ __host__ __device__ inline PipeLayout pipe_layout(int n_hidden) {
   L.slot0 = 0;                                   // (the X tiles are per buffer below)
   L.slot_bytes = 0;
   L.bias = L.w_bias + (uint32_t)(n_hidden - 1) * kBiasTile;
-  L.ybuf = L.bias + (uint32_t)(n_hidden * kWidth + kNout) * 4;
-  L.ybuf_bytes = (uint32_t)(256 / kTileM - 1) * kTileM * 3 * 4;   // 8-warp groups: 2 column groups
-  L.mbar = (L.ybuf + 2 * L.ybuf_bytes + 15u) & ~15u;
+  L.ybuf = 0;                                    // (partial outputs pass through the X tiles)
+  L.ybuf_bytes = 0;
+  L.mbar = (L.bias + (uint32_t)(n_hidden * kWidth + kNout) * 4 + 15u) & ~15u;
   L.tptr = L.mbar + 16;
   L.flag = L.tptr + 4;
   L.claim = L.flag + 8;
   L.fail = L.claim + 8;
   L.stash = 0;
   P.x0 = (L.fail + 8 + 127u) & ~127u;            // X tiles: K-major core matrices
-  P.st0 = P.x0 + 2 * kPipeBufs * kTileM * kKin * 2;
-  P.y0 = P.st0 + 2 * kPipeBufs * kStashWords * kTileM * 4;
-  P.info0 = P.y0 + 2 * kPipeBufs * kTileM * 3 * 4;
-  P.bars = (P.info0 + 2 * kPipeBufs * 16 + 7u) & ~7u;
-  P.abort = P.bars + 18 * 8;
-  P.bcast = P.abort + 16;
-  P.total = P.bcast + 16 + 256;
+  P.st0 = P.x0 + kPipeBufs * kTileM * kKin * 2;
+  P.y0 = P.st0 + kPipeBufs * kStashWords * kTileM * 4;
+  P.info0 = P.y0 + kPipeBufs * kTileM * 3 * 4;
+  P.ops = P.info0 + kPipeBufs * 16;
+  P.bars = P.ops + 4 * 16;
+  P.abort = P.bars + (4 * kPipeBufs + 9) * 8;
+  P.total = P.abort + 16 + 256;
   L.total = P.total;
   return P;
 }
@@ -781,6 +818,259 @@ __device__ __forceinline__ bool role_all(int id, int n, bool pred) {
 }
 __device__ __forceinline__ void role_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 
+// The issuing lane: admits built tiles in order, up to kInFlight of them, and
+// issues the MMAs of the oldest tile whose input is ready into a free TMEM
+// region.  Step n: its description (buffer, layer, region) in ops[n & 3],
+// its accumulators announced on dfull[n & 3].
+__device__ __forceinline__ void issue_role(char* smem, const PipeLayout& P, const MlpShape& sh, const NeuralArgs& a,
+                                           uint32_t tmem) {
+  const MlpLayout& L = P.m;
+  const uint32_t sbase = tc::smem_u32(smem);
+  const uint32_t idesc = tc::idesc_bf16(kTileM, kWidth);
+  const uint64_t d_win = tc::sdesc(sbase + L.w_in, 128, kKin * 16);
+  const uint64_t d_sq = tc::sdesc(sbase + L.w_sq, 128, 2048);
+  const uint64_t d_x = tc::sdesc(sbase + P.x0, 128, kKin * 16);
+  constexpr uint32_t kXStep = kTileM * kKin * 2 >> 4, kSqStep = kWidth * kWidth * 2 >> 4;   // descriptor units
+  // the tiles in flight, oldest first: buffer, layer of its last step, that
+  // step, region (constant indices after unrolling: registers)
+  int buf[kInFlight] = {}, layer[kInFlight] = {}, region[kInFlight] = {};
+  uint32_t step[kInFlight] = {};
+  int active = 0, kb = 0;           // kb: buffer of the next tile to admit
+  uint32_t kph = 0, n = 0;          // its parity; steps issued
+  uint32_t used = 0;                // regions that hold accumulators or an operand
+  uint32_t reading = 0;             // of these, operands of MMAs not known to be done
+  bool ended = false;
+  uint64_t idle0 = 0;
+  auto issue = [&](int b, int l, int src) {   // returns the region written
+    int d = 0;
+    while ((used >> d) & 1u) ++d;
+    const uint32_t acc = tmem + (uint32_t)d * kWidth;
+    volatile int* op = (volatile int*)(smem + P.op(n));
+    op[0] = b; op[1] = l; op[2] = d; op[3] = 0;
+    tc::fence_after();
+    const uint64_t dx = d_x + (uint32_t)b * kXStep;
+    if (l == 0) {
+#pragma unroll
+      for (int s = 0; s < kKin / 16; ++s) tc::mma_bf16(acc, dx + 16u * s, d_win + 16u * s, idesc, s > 0);
+    } else {
+      // the bias: the input tile's first 16 columns (1.0 in 13..15) against
+      // [zeros | the layer's bias tile] (core-matrix rows 128 bytes apart)
+      tc::mma_bf16(acc, dx,
+                   tc::sdesc(sbase + L.w_zero, L.w_bias + (uint32_t)(l - 1) * kBiasTile - L.w_zero, 128), idesc, 0);
+      // activations enter as hi + lo bf16 terms against the same weights
+      const uint32_t op_a = tmem + (uint32_t)src * kWidth;
+      const uint64_t dw = d_sq + (uint32_t)(l - 1) * kSqStep;
+#pragma unroll
+      for (int s = 0; s < kWidth / 16; ++s) tc::mma_bf16_ta(acc, op_a + 16u * s, dw + 16u * s, idesc, 1);
+#pragma unroll
+      for (int s = 0; s < kWidth / 16; ++s) tc::mma_bf16_ta(acc, op_a + 16u * s + 8u, dw + 16u * s, idesc, 1);
+    }
+    tc::commit((uint64_t*)(smem + P.dfull(n)));
+    mbar_arrive(smem, P.dfull(n));   // (the description)
+    used |= 1u << d;
+    ++n;
+    return d;
+  };
+  for (;;) {
+    bool progress = false;
+    // regions read by MMAs up to the last step's are free once those are done
+    if (reading && tc::mbar_try_wait((uint64_t*)(smem + P.dfull(n - 1)), ((n - 1) >> 2) & 1u)) {
+      used &= ~reading;
+      reading = 0;
+    }
+#pragma unroll
+    for (int t = 0; t < kInFlight; ++t) {   // the oldest first
+      if (progress || t >= active) continue;
+      const bool last = layer[t] == sh.n_hidden - 1;
+      // a further step needs a free region, and the place of step n - 4
+      // in the ring of descriptions (another tile's, if it is not known done)
+      bool room = used != (1u << kRegions) - 1u;
+#pragma unroll
+      for (int q = 0; q < kInFlight; ++q) room = room && (q == t || q >= active || step[q] + 4u != n);
+      if (!last && !room) continue;
+      if (!tc::mbar_try_wait((uint64_t*)(smem + P.edone(step[t])), (step[t] >> 2) & 1u)) continue;
+      progress = true;
+      if (last) {   // its outputs are with the epilogue warps: the tile leaves
+        used &= ~(1u << region[t]);
+#pragma unroll
+        for (int q = t; q + 1 < kInFlight; ++q) {
+          buf[q] = buf[q + 1]; layer[q] = layer[q + 1]; region[q] = region[q + 1]; step[q] = step[q + 1];
+        }
+        --active;
+      } else {
+        const int src = region[t];
+        step[t] = n;
+        region[t] = issue(buf[t], ++layer[t], src);
+        reading |= 1u << src;
+      }
+    }
+    bool room = used != (1u << kRegions) - 1u;
+#pragma unroll
+    for (int q = 0; q < kInFlight; ++q) room = room && (q >= active || step[q] + 4u != n);
+    if (!progress && !ended && active < kInFlight && room &&
+        tc::mbar_try_wait((uint64_t*)(smem + P.built(kb)), kph)) {
+      progress = true;
+      if (((volatile int*)(smem + P.info(kb)))[3]) {
+        ended = true;
+      } else {
+        const uint32_t s0 = n;
+        const int d = issue(kb, 0, -1);
+#pragma unroll
+        for (int q = 0; q < kInFlight; ++q)
+          if (q == active) { buf[q] = kb; layer[q] = 0; step[q] = s0; region[q] = d; }
+        ++active;
+        if (++kb == kPipeBufs) { kb = 0; kph ^= 1u; }
+      }
+    }
+    if (ended && active == 0) break;
+    if (progress) { idle0 = 0; continue; }
+    if (idle0 == 0) idle0 = globaltimer_ns();
+    if (*(volatile int*)(smem + P.abort)) break;
+    if (globaltimer_ns() - idle0 > 100000u) {   // idle for long: look at the other CTAs too
+      if (pipe_aborted(smem, P, a)) break;
+      if (globaltimer_ns() - idle0 > kBarrierLimitNs) {
+        set_status(a.status, DSMC_ERR_TIMEOUT);
+        pipe_abort(smem, P, a);
+        break;
+      }
+      __nanosleep(200);
+    }
+  }
+  if (ended && active == 0) {   // the end, to the epilogue warps
+    ((volatile int*)(smem + P.op(n)))[3] = 1;
+    mbar_arrive(smem, P.dfull(n));
+    mbar_arrive(smem, P.dfull(n));
+  } else {                      // aborted: the MMAs in flight end (bounded) before TMEM is released
+    tc::commit((uint64_t*)(smem + P.drain()));
+    tc::mbar_wait((uint64_t*)(smem + P.drain()), 0, a.status, kBarrierLimitNs);
+  }
+}
+
+// The epilogue warps, step after step: warp w reads TMEM lanes 32 (w % 4) ..
+// (rows) and columns 32 (w / 4) .. of the step's region.
+__device__ __forceinline__ void epilogue_role(char* smem, const PipeLayout& P, const MlpShape& sh, const NeuralArgs& a,
+                                              uint32_t tmem) {
+  const MlpLayout& L = P.m;
+  const int t = threadIdx.x, w = t >> 5, lane = t & 31;
+  const int quad = w & 3, cq = w >> 2, half = cq >> 1;
+  const int row = (quad << 5) | lane, cb = 32 * cq;
+  const uint32_t lane_tm = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)cb;
+  const float* wo = (const float*)(smem + L.w_out) + cb;
+  const float* bo = (const float*)(smem + L.bias) + sh.n_hidden * kWidth;
+  for (uint32_t n = 0;; ++n) {
+    if (!role_all(kBarEpi, kEpiThreads, pipe_wait(smem, P, a, P.dfull(n), (n >> 2) & 1u))) break;
+    tc::fence_after();
+    const volatile int* op = (const volatile int*)(smem + P.op(n));
+    if (op[3]) break;
+    const int b = op[0];
+    const bool last = op[1] == sh.n_hidden - 1;
+    const uint32_t at = lane_tm + (uint32_t)op[2] * kWidth;
+    uint32_t ra[16], rb[16];
+    tc::ld16_async(at, ra);
+    tc::wait_ld16(ra);
+    tc::ld16_async(at + 16, rb);
+    if (!last) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        uint32_t* cur = h ? rb : ra;
+        if (h) tc::wait_ld16(rb);
+        // values in packed pairs (columns 2k, 2k + 1; the bias is already in
+        // them): activation products, residuals and output-layer FMAs run two
+        // per instruction
+        float2 v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = make_float2(__uint_as_float(cur[2 * k]), __uint_as_float(cur[2 * k + 1]));
+        if (sh.act == 0) {
+#pragma unroll
+          for (int k = 0; k < 8; k += 2) tc::silu2_4x2(v[k], v[k + 1]);
+        } else {
+#pragma unroll
+          for (int k = 0; k < 8; ++k) v[k] = make_float2(act_f(sh.act, v[k].x), act_f(sh.act, v[k].y));
+        }
+        uint32_t pk[8], lo[8];
+        const float2 m1 = make_float2(-1.f, -1.f);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          pk[k] = tc::pack_bf16x2(v[k].x, v[k].y);
+          // a - hi is exact (hi is a rounding of a); as an FMA with -1
+          const float2 r = __ffma2_rn(make_float2(__uint_as_float(pk[k] << 16), __uint_as_float(pk[k] & 0xFFFF0000u)),
+                                      m1, v[k]);
+          lo[k] = tc::pack_bf16x2(r.x, r.y);
+        }
+        // in place: these 16 columns, read above, become the hi and lo terms
+        tc::st8_async(at + 16u * h, pk);
+        tc::st8_async(at + 16u * h + 8u, lo);
+      }
+      // the A operand stores complete before the next MMA
+      tc::wait_st();
+      tc::fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem, P.edone(n));
+      continue;
+    }
+    // the last hidden layer: activations into the output layer's dot products,
+    // summed over 64 columns (a half) in column order by two warps one after
+    // the other, then the halves
+    float2 v[16];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = make_float2(__uint_as_float(ra[2 * k]), __uint_as_float(ra[2 * k + 1]));
+    tc::wait_ld16(rb);
+    tc::fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(smem, P.edone(n));   // the region is read
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[8 + k] = make_float2(__uint_as_float(rb[2 * k]), __uint_as_float(rb[2 * k + 1]));
+    if (sh.act == 0) {
+#pragma unroll
+      for (int k = 0; k < 16; k += 2) tc::silu2_4x2(v[k], v[k + 1]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 16; ++k) v[k] = make_float2(act_f(sh.act, v[k].x), act_f(sh.act, v[k].y));
+    }
+    // partial sums pass through the tile's input rows, which no MMA reads any
+    // more: [2 halves][6][128 rows], then [3][128 rows]
+    float* chain = (float*)(smem + P.x(b)) + half * 6 * kTileM + row;
+    float* hsum = (float*)(smem + P.x(b)) + 2 * 6 * kTileM + row;
+    static_assert((2 * 6 + 3) * kTileM * 4 <= kTileM * kKin * 2, "the partial sums fit an input tile");
+    float2 yq0 = make_float2(0.f, 0.f), yq1 = yq0, yq2 = yq0;   // even and odd columns apart
+    const int pair_bar = kBarChain + 2 * quad + half;
+    if (cq & 1) {
+      role_sync(pair_bar, 64);
+      yq0 = make_float2(chain[0], chain[kTileM]);
+      yq1 = make_float2(chain[2 * kTileM], chain[3 * kTileM]);
+      yq2 = make_float2(chain[4 * kTileM], chain[5 * kTileM]);
+    }
+    const float2 *w0 = (const float2*)wo, *w1 = (const float2*)(wo + kWidth), *w2 = (const float2*)(wo + 2 * kWidth);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      yq0 = __ffma2_rn(v[k], w0[k], yq0);
+      yq1 = __ffma2_rn(v[k], w1[k], yq1);
+      yq2 = __ffma2_rn(v[k], w2[k], yq2);
+    }
+    if (!(cq & 1)) {
+      chain[0] = yq0.x; chain[kTileM] = yq0.y;
+      chain[2 * kTileM] = yq1.x; chain[3 * kTileM] = yq1.y;
+      chain[4 * kTileM] = yq2.x; chain[5 * kTileM] = yq2.y;
+      role_sync(pair_bar, 64);
+      continue;
+    }
+    const float yp0 = yq0.x + yq0.y, yp1 = yq1.x + yq1.y, yp2 = yq2.x + yq2.y;
+    if (half) {
+      hsum[0] = yp0; hsum[kTileM] = yp1; hsum[2 * kTileM] = yp2;
+      role_sync(kBarHalves + quad, 64);
+    } else {
+      role_sync(kBarHalves + quad, 64);
+      float* yb = (float*)(smem + P.y(b)) + 3 * row;
+      yb[0] = yp0 + hsum[0] + bo[0];
+      yb[1] = yp1 + hsum[kTileM] + bo[1];
+      yb[2] = yp2 + hsum[2 * kTileM] + bo[2];
+      mbar_arrive(smem, P.ydone(b));
+    }
+    // (the input rows are written again only once the tile's update has freed
+    // its buffer)
+  }
+}
+
 __global__ void __launch_bounds__(kPipeThreads, 1) k_collide_neural(MlpShape sh, const uint16_t* __restrict__ w,
                                                                  const float* __restrict__ bias, NeuralArgs a) {
   dep_wait_alone();
@@ -790,92 +1080,88 @@ __global__ void __launch_bounds__(kPipeThreads, 1) k_collide_neural(MlpShape sh,
   const MlpLayout& L = P.m;
   load_weights(smem, L, sh, w, bias);
   if (threadIdx.x == 0) {
-    for (int q = 0; q < 6; ++q) {
-      tc::mbar_init((uint64_t*)(smem + P.bars) + q, kRoleThreads);        // built
-      tc::mbar_init((uint64_t*)(smem + P.bars) + 6 + q, kRoleThreads);    // ydone
-      tc::mbar_init((uint64_t*)(smem + P.bars) + 12 + q, kRoleThreads);   // freed
+    for (int b = 0; b < kPipeBufs; ++b) {
+      tc::mbar_init((uint64_t*)(smem + P.built(b)), kRoleThreads);
+      tc::mbar_init((uint64_t*)(smem + P.ydone(b)), kRoleThreads);
+      tc::mbar_init((uint64_t*)(smem + P.freed(b)), kRoleThreads);
+      tc::mbar_init((uint64_t*)(smem + P.claimed(b)), 1);
     }
+    for (uint32_t n = 0; n < 4; ++n) {
+      tc::mbar_init((uint64_t*)(smem + P.dfull(n)), 2);
+      tc::mbar_init((uint64_t*)(smem + P.edone(n)), kEpiWarpsN);
+    }
+    tc::mbar_init((uint64_t*)(smem + P.drain()), 1);
     *(volatile int*)(smem + P.abort) = 0;
   }
-  const uint32_t tmem = cta_setup(smem, L);   // TMEM (512 columns), per-group MMA barriers; CTA-wide barrier
+  const uint32_t tmem = cta_setup(smem, L);   // TMEM (512 columns); CTA-wide barrier
   const int R = a.info->n_rounds;
   const int t = threadIdx.x;
   if (t < kBuildBase) {
-    // ------------------------------------------------ MLP groups
-    const Group q{t / 256, 2, t % 256, 256};
-    uint32_t phase = 0;
-    const int row = (((q.t >> 5) & 3) << 5) | (q.t & 31);
-    const bool yrow = q.t < kTileM;   // column group 0: holds the row's output
-    for (int kk = 0;; ++kk) {
-      const int b = kk % kPipeBufs;
-      const bool ok = role_all(1 + q.g, 256, pipe_wait(smem, P, a, P.built(q.g, b), (uint32_t)(kk / kPipeBufs) & 1u));
-      if (!ok) break;
-      tc::fence_after();
-      const int end = ((volatile int*)(smem + P.info(q.g, b)))[3];
-      if (end) {
-        if (yrow) mbar_arrive(smem, P.ydone(q.g, b));
-        break;
-      }
-      float y[3];
-      if (!mlp_tile(smem, L, sh, q, tmem, phase, y, a.status, P.x(q.g, b))) {
-        pipe_abort(smem, P, a);
-        break;
-      }
-      if (yrow) {
-        float* yb = (float*)(smem + P.y(q.g, b)) + 3 * row;
-        yb[0] = y[0]; yb[1] = y[1]; yb[2] = y[2];
-        mbar_arrive(smem, P.ydone(q.g, b));
-      }
-    }
+    epilogue_role(smem, P, sh, a, tmem);
   } else if (t < kUpdateBase) {
     // ------------------------------------------------ builders
-    const int tb = t - kBuildBase;
-    int r = 0;
-    int64_t base = 0;
+    // two groups of four warps take the tiles in turn; a warp goes on to its
+    // next tile when its own 32 rows are built
+    const int tb = (t - kBuildBase) & (kRoleThreads - 1);
     volatile int* fail = (volatile int*)(smem + P.abort);
-    for (int k = 0;; ++k) {
-      const int g = k & 1, kk = k >> 1, b = kk % kPipeBufs;
-      bool ok = true;
-      if (kk >= kPipeBufs) ok = pipe_wait(smem, P, a, P.freed(g, b), (uint32_t)(kk / kPipeBufs - 1) & 1u);
-      if (!role_all(3, kRoleThreads, ok)) break;
-      volatile unsigned* bc = (volatile unsigned*)(smem + P.bcast) + (k & 1);
-      if (tb == 0) *bc = atomicAdd(a.bar + 3, 1u);
-      role_sync(3, kRoleThreads);
-      int32_t p0 = 0, p1 = 0;
-      const bool have = unit_range(a.ro, R, kTileM, r, base, *bc, &p0, &p1);
-      int* info = (int*)(smem + P.info(g, b));
-      if (tb == 0) { info[0] = p0; info[1] = p1; info[2] = r; info[3] = have ? 0 : 1; }
-      if (have) {
-        const int32_t p = p0 + tb;
-        build_row(smem, P.x(g, b), fail, sh, a, tb, p < p1 ? p : -1, (uint32_t*)(smem + P.st(g, b)));
-      }
-      mbar_arrive(smem, P.built(g, b));
-      if (!have) {
-        // the other group's next buffer carries the end too
-        const int k2 = k + 1, g2 = k2 & 1, kk2 = k2 >> 1, b2 = kk2 % kPipeBufs;
-        bool ok2 = true;
-        if (kk2 >= kPipeBufs) ok2 = pipe_wait(smem, P, a, P.freed(g2, b2), (uint32_t)(kk2 / kPipeBufs - 1) & 1u);
-        if (role_all(3, kRoleThreads, ok2)) {
-          if (tb == 0) ((volatile int*)(smem + P.info(g2, b2)))[3] = 1;
-          mbar_arrive(smem, P.built(g2, b2));
+    uint32_t ph = 0;
+    for (int b = (t - kBuildBase) / kRoleThreads;;) {
+      if (!__all_sync(0xffffffffu, pipe_wait(smem, P, a, P.claimed(b), ph))) break;
+      const volatile int* info = (const volatile int*)(smem + P.info(b));
+      const int32_t p = info[0] + tb, p1 = info[1];
+      if (const int end = info[3]) {
+        if (end == 1) {   // the first tile without a unit: the end, also to the updaters
+          mbar_arrive(smem, P.built(b));
+          mbar_arrive(smem, P.ydone(b));
         }
         break;
       }
+      int4 q = make_int4(0, 0, 0, 0);
+      uint32_t dep = 0u;
+      if (p < p1) { q = a.pairs[p]; dep = a.deps[p]; }
+      build_row(smem, P.x(b), fail, sh, a, tb, p < p1 ? p : -1, q, dep, (uint32_t*)(smem + P.st(b)));
+      mbar_arrive(smem, P.built(b));
       if (*fail) pipe_abort(smem, P, a);
+      if ((b += 2) >= kPipeBufs) { b -= kPipeBufs; ph ^= 1u; }
     }
-  } else {
+  } else if (t < kIssueBase) {
     // ------------------------------------------------ updaters
     const int tu = t - kUpdateBase;
-    for (int k = 0;; ++k) {
-      const int g = k & 1, kk = k >> 1, b = kk % kPipeBufs;
-      if (!role_all(4, kRoleThreads, pipe_wait(smem, P, a, P.ydone(g, b), (uint32_t)(kk / kPipeBufs) & 1u))) break;
-      const int* info = (const int*)(smem + P.info(g, b));
+    uint32_t ph = 0;
+    for (int b = 0;;) {
+      if (!role_all(kBarUpdate, kRoleThreads, pipe_wait(smem, P, a, P.ydone(b), ph))) break;
+      const int* info = (const int*)(smem + P.info(b));
       if (((volatile const int*)info)[3]) break;
-      const float* yb = (const float*)(smem + P.y(g, b)) + 3 * tu;
+      const float* yb = (const float*)(smem + P.y(b)) + 3 * tu;
       const float y[3] = {yb[0], yb[1], yb[2]};
-      update_row(a, y, (const uint32_t*)(smem + P.st(g, b)), tu, (unsigned)(info[2] + 1));
-      mbar_arrive(smem, P.freed(g, b));
+      update_row(a, y, (const uint32_t*)(smem + P.st(b)), tu, (unsigned)(info[2] + 1));
+      mbar_arrive(smem, P.freed(b));
+      if (++b == kPipeBufs) { b = 0; ph ^= 1u; }
     }
+  } else if (t < kClaimBase) {
+    if (t == kIssueBase) issue_role(smem, P, sh, a, tmem);
+    __syncwarp();
+  } else {
+    // ------------------------------------------------ claims
+    // the next unit into each buffer as it is freed: a tile's unit is never
+    // below that of an earlier tile of the CTA (tiles are admitted in order: an
+    // earlier tile must not wait on a later one).  Two ends, one per builder group.
+    if (t == kClaimBase) {
+      int r = 0, ends = 0;
+      int64_t base = 0;
+      uint32_t ph = 1;   // parity of the buffer's last release
+      for (int k = 0, b = 0; ends < 2; ++k) {
+        const unsigned unit = ends ? 0u : atomicAdd(a.bar + 3, 1u);
+        if (k >= kPipeBufs && !pipe_wait(smem, P, a, P.freed(b), ph)) break;
+        volatile int* info = (volatile int*)(smem + P.info(b));
+        int32_t p0 = 0, p1 = 0;
+        if (ends || !unit_range(a.ro, R, kTileM, r, base, unit, &p0, &p1)) ++ends;
+        info[0] = p0; info[1] = p1; info[2] = r; info[3] = ends;
+        mbar_arrive(smem, P.claimed(b));
+        if (++b == kPipeBufs) { b = 0; ph ^= 1u; }
+      }
+    }
+    __syncwarp();
   }
   cta_teardown(tmem, L);
 }
@@ -919,7 +1205,7 @@ int launch_collide_neural(Ctx* c, const dsmc_gas_t& gas, const dsmc_mlp_t& mlp,
           cudaSuccess || per_sm < 1)
     return record(c, DSMC_ERR_CUDA, "collide_neural: occupancy query failed");
   NeuralArgs a;
-  a.seed = gas.seed; a.step = step; a.step_dev = graph_step_ptr(c);
+  a.seed = gas.seed; a.key = philox_key(gas.seed); a.step = step; a.step_dev = graph_step_ptr(c);
   a.sigma_v_inv = 1.0 / mlp.sigma_v; a.T_ref_inv = 1.0 / mlp.T_ref;
   a.m_over_3k = gas.mass / (3.0 * DSMC_KB); a.eps = mlp.eps;
   a.sigma_v_inv_f = (float)a.sigma_v_inv;

@@ -143,3 +143,32 @@ def test_collide_accepts_a_workspace_at_any_word():
         assert C.sync_status() == 0
         got.append(host(torch().stack(v)))
     assert np.array_equal(got[0], got[1]) and np.array_equal(got[0], got[2])
+
+
+@pytest.mark.parametrize("n_hidden", [1, 3, 4])
+@pytest.mark.parametrize("cells,dt", [(1, 1e-9), (3, 1e-7), (40, 1e-7)])
+def test_neural_collide_does_not_depend_on_the_order_of_its_tiles(cells, dt, n_hidden):
+    """A single pair, fewer than a tile, and chains of many levels: the rounds' and the claim levels' lists hold
+    the same pairs in other tiles, and each pair's arithmetic is its own, so the velocities agree bit for bit."""
+    from paper_2602_21244_gb300 import dsmc as D
+    from paper_2602_21244_gb300 import workloads as W
+    T, C = torch(), ctx()
+    w = W.couette(seed=3, n_cells=cells, per_cell=150)
+    gas = D.make_gas(dict(w["gas"], fn_over_vc=4e19, dt=dt, model=1))
+    wts = W.mlp_weights(n_hidden=n_hidden)
+    mlp = D.make_mlp(8, 128, n_hidden, 3, 0, W.sigma_v(), 273.0, 1e-12)
+    bits, bias = cuda(wts["W_bits"].view(np.int16)), cuda(wts["bias"].astype(np.float32))
+    o = C.sort_cells(cuda(w["cell_id"]), cuda(w["vx"]), cuda(w["vy"]), cuda(w["vz"]), cells)
+    mom = C.cell_moments(o["cell_start"], o["svx"], o["svy"], o["svz"])
+    got, pairs = [], None
+    for order in (0, 1):
+        sg = C.sigma_g_max_init(gas, cuda(w["T_cell"]))
+        sel = C.select_pairs(gas, o["cell_start"], o["svx"], o["svy"], o["svz"], sg, 2, 1 << 18, order=order)
+        v = [o[k].clone() for k in ("svx", "svy", "svz")]
+        C.collide_neural(gas, mlp, bits, bias, 2, mom, sel, *v)
+        assert C.sync_status() == 0
+        got.append(host(T.stack(v)))
+        pairs = int(host(sel["info"])[0])
+    assert np.array_equal(got[0], got[1])
+    start = np.stack([host(o[k]) for k in ("svx", "svy", "svz")])
+    assert np.array_equal(got[0], start) == (pairs == 0)
