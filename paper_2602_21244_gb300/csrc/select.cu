@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(kSelWarps * 32, 4) k_sel_count(SelArgs a) {
   if (lane == 0 && cands) atomicAdd(a.n_cand, cands);   // the step's candidate count
 }
 
-constexpr int kEmitWarps = 8;
+constexpr int kEmitWarps = 4;
 constexpr int kEmitWords = 16;    // accept-bit words expanded per step (512 candidates)
 
 // Warp per cell.  The accepted candidates come from the count pass's accept
@@ -251,7 +251,7 @@ constexpr int kEmitWords = 16;    // accept-bit words expanded per step (512 can
 // is kept.  A cell whose bits were not kept re-evaluates its candidates
 // from the FP64 velocities; a cell of more than kStage particles takes its
 // rounds on one lane from global memory.
-__global__ void __launch_bounds__(kEmitWarps * 32, 4) k_sel_emit(SelArgs a) {
+__global__ void __launch_bounds__(kEmitWarps * 32, 8) k_sel_emit(SelArgs a) {
   dep_wait();
   if (a.step_dev) a.step = *a.step_dev;
   __shared__ uint32_t slist[kEmitWarps][kEmitWords * 32];  // accepted candidate indices
@@ -760,11 +760,14 @@ int launch_select(Ctx* c, const dsmc_gas_t& gas, int32_t n, int32_t n_cells, con
     count_launches(c, 1);
     if (int rc = launch_scan(c, w.wcnt, w.wofs, n_cells, w.scan, s)) return rc;
   }
-  const unsigned gb = blocks_for((n_cells + 1) / 2, kSelWarps, sms * 8);
+  // Many small blocks, so that the hardware evens out the cells' unequal numbers of candidates: selection
+  // of 6.9 million pairs in 150,000 cells 493 us with 8 blocks per SM, 469 with 64 (count), and 460 with
+  // blocks of 4 warps instead of 8 (emit: a block's warps wait for the slowest at its end)
+  const unsigned gb = blocks_for((n_cells + 1) / 2, kSelWarps, sms * 64);
   launch_dep(k_sel_count, gb, kSelWarps * 32, 0, s, a);
   count_launches(c, 1);
   if (int rc = launch_scan(c, w.counts, w.offs, n_cells, w.scan, s)) return rc;
-  launch_dep(k_sel_emit, blocks_for((n_cells + 1) / 2, kEmitWarps, sms * 16), kEmitWarps * 32, 0, s, a);
+  launch_dep(k_sel_emit, blocks_for((n_cells + 1) / 2, kEmitWarps, sms * 32), kEmitWarps * 32, 0, s, a);
   // at least one block: the capacity-overflow commit of (sigma g)_max runs in k_sel_rcount
   const unsigned sb = (unsigned)((capacity + kScatterChunk - 1) / kScatterChunk) + (capacity <= 0);
   launch_dep(k_sel_rcount, sb, 256, 0, s, w.tmp_round, w.offs, n_cells, capacity, w.n_rounds, w.n_chunks, w.chunk_cnt,
