@@ -575,7 +575,7 @@ constexpr int kLongShared = 28, kShortShared = 16;
 // long rule, 95 % of the warps did).  2^22 pairs of that batch: 4.00 -> 2.55
 // ms, and 1.90 ms with one copy of the node's code for both ways and the other
 // potentials' code compiled apart (a fifth of the warps' stalls were
-// instruction fetches), bit-identical; what is left is the FP64 refinement
+// instruction fetches), 1.79 ms with five blocks per SM, bit-identical; what is left is the FP64 refinement
 // (111 FP64 instructions per warp at 19 cycles: 0.9 ms) and the FP32 instructions.
 template <bool kWarp = false, int KIND = -1>
 __device__ float chi_device(const PotDev& P, float b_in, float E, ChiShared S = ChiShared{}, bool use = true) {
@@ -840,8 +840,10 @@ static PotDev make_pot(const dsmc_gas_t& gas, const dsmc_potential_t& p, int n_n
 // ---------------------------------------------------------------- kernels
 // Warp-uniform loop: every lane of a warp computes chi together (a lane past
 // the end, or with g = 0, on harmless inputs whose result is not kept).
+// Five blocks per SM: 2^22 pairs 1785 us, four 1896, six 1866 (the pair update,
+// with the rotation's registers besides, is faster with four: 1284 against 1331 us).
 template <int KIND>
-__global__ void __launch_bounds__(128, 4) k_jager_chi(PotDev P, int64_t n, const float* __restrict__ b,
+__global__ void __launch_bounds__(128, 5) k_jager_chi(PotDev P, int64_t n, const float* __restrict__ b,
                                                       const float* __restrict__ g, float* __restrict__ chi) {
   extern __shared__ float4 chi_sm[];
   const ChiShared S = chi_shared(P, (float*)chi_sm);
