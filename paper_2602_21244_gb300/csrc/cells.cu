@@ -479,8 +479,7 @@ k_rs_rowscan(const int32_t* __restrict__ cnt, int32_t chunks, int32_t* __restric
 // Ordered scatter of one chunk: warp w owns the chunk's w-th sixteenth, its
 // kRsPer elements per lane loaded into registers first.  Stable ranks in
 // two steps: (1) per element batch j (32 consecutive elements), the lanes
-// holding the same digit find each other from one ballot per digit bit; the lowest
-// of them adds the group's size to the warp's counter of that digit in
+// holding the same digit find each other (see kRsRuns); the lowest of them adds the group's size to the warp's counter of that digit in
 // shared memory and keeps the old value (the count of that digit in the
 // warp's earlier batches; the batches' atomics are ordered by __syncwarp),
 // the others their rank inside the group.  (2) After the counts are
@@ -498,6 +497,13 @@ k_rs_rowscan(const int32_t* __restrict__ cnt, int32_t chunks, int32_t* __restric
 // scan of that table is not launched.
 constexpr int32_t kRsDirect = 16;
 constexpr int kRsPer = kRsChunk / kRsWarps / 32;
+// Lanes with equal digits find each other by match.any, whose time grows with
+// the number of different digits, when the warp's first batch holds at most this
+// many runs of them (particles that have moved little since the last sort: both
+// passes of 9.15 million took 130 us, with ballots 162), else by nine ballots
+// (shuffled particles: the sort 376 us, with match.any 433).  6 runs as the
+// limit: sort of the moved particles 276 us, 12 to 20: 258 to 261.
+constexpr int kRsRuns = 16;
 static_assert(kRsWarps * 32 == kRadix, "one thread per digit in the offset step");
 
 __global__ void __launch_bounds__(kRsWarps * 32, 2)
@@ -531,19 +537,32 @@ k_rs_scatter(const int32_t* __restrict__ cell_id, const uint32_t* __restrict__ k
   const unsigned lt = (1u << lane) - 1u;
   int old[kRsPer];
   uint32_t pk[kRsPer];   // leader lane | rank in the group << 5
+  // the digit of batch j (lanes without an element share the digit kRadix)
+  auto digit = [&](int j) {
+    return s0 + j * 32 + lane < un ? (int)((key[j] >> shift) & (kRadix - 1)) : kRadix;
+  };
+  // runs of equal digits in batch j
+  auto runs = [&](int j) {
+    const int d = digit(j), up = __shfl_up_sync(0xffffffffu, d, 1);
+    return __popc(__ballot_sync(0xffffffffu, lane == 0 || d != up));
+  };
+  const bool few = runs(0) <= kRsRuns;
 #pragma unroll
   for (int j = 0; j < kRsPer; ++j) {
     const bool has = s0 + j * 32 + lane < un;
-    // lanes without an element share the digit kRadix (no counter)
-    const int d = has ? (int)((key[j] >> shift) & (kRadix - 1)) : kRadix;
-    // lanes holding the same digit: one ballot per digit bit (ALU pipe); the
-    // lanes without an element form their own set
-    unsigned peers = __ballot_sync(0xffffffffu, has);
-    if (!has) peers = ~peers;
+    const int d = digit(j);
+    // lanes holding the same digit (those without an element form their own set)
+    unsigned peers;
+    if (few) {
+      peers = __match_any_sync(0xffffffffu, d);
+    } else {
+      peers = __ballot_sync(0xffffffffu, has);
+      if (!has) peers = ~peers;
 #pragma unroll
-    for (int bit = 0; bit < kRadixBits; ++bit) {
-      const unsigned m = __ballot_sync(0xffffffffu, (d >> bit) & 1);
-      peers &= ((d >> bit) & 1) ? m : ~m;
+      for (int bit = 0; bit < kRadixBits; ++bit) {   // one ballot per digit bit (ALU pipe)
+        const unsigned m = __ballot_sync(0xffffffffu, (d >> bit) & 1);
+        peers &= ((d >> bit) & 1) ? m : ~m;
+      }
     }
     const int rank = __popc(peers & lt);
     old[j] = 0;

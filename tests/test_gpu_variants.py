@@ -172,3 +172,34 @@ def test_neural_collide_does_not_depend_on_the_order_of_its_tiles(cells, dt, n_h
     assert np.array_equal(got[0], got[1])
     start = np.stack([host(o[k]) for k in ("svx", "svy", "svz")])
     assert np.array_equal(got[0], start) == (pairs == 0)
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("runs", [1, 16, 17, 32, 0])
+@pytest.mark.parametrize("n", [4096, 4097, 12287, 17 * 4096 + 31])
+def test_sort_is_stable_for_every_run_length(n, runs, offset):
+    """Batches of 32 with 1, 16, 17 or 32 runs of equal cells (0: a mix, run lengths changing inside a
+    warp) take the ranks from match or from ballots; whole and partial chunks, ids at any word; ids out
+    of range in both.  Whole numbers: the order is the stable one."""
+    from paper_2602_21244_gb300 import dsmc as D
+    C, rng = ctx(), np.random.default_rng(n + runs)
+    n_cells = 70000
+    i = np.arange(n)
+    group = i * runs // 32 if runs else np.cumsum(rng.random(n) < np.repeat(rng.random(n // 64 + 1), 64)[:n])
+    ids = rng.integers(0, n_cells, int(group[-1]) + 1)[group].astype(np.int32)
+    ids[[0, n // 2, n - 1]] = [0, n_cells - 1, 0]
+    buf = cuda(np.concatenate([np.zeros(offset, np.int32), ids]))[offset:]
+    v = [cuda(rng.standard_normal(n)) for _ in range(3)]
+    o = C.sort_cells(buf, *v, n_cells)
+    assert C.sync_status() == 0
+    order = np.argsort(ids, kind="stable")
+    assert np.array_equal(host(o["perm"]), order)
+    assert np.array_equal(host(o["cell_start"]), np.concatenate([[0], np.cumsum(np.bincount(ids, minlength=n_cells))]))
+    assert np.array_equal(host(o["svx"]), host(v[0])[order])
+    buf[n // 3] = -1
+    buf[n // 5] = n_cells
+    o = C.sort_cells(buf, *v, n_cells)
+    assert C.sync_status() == D.DSMC_ERR_ARG
+    keep = host(buf)
+    keep = np.where((keep < 0) | (keep >= n_cells), n_cells, keep)
+    assert np.array_equal(host(o["perm"])[:n - 2], np.argsort(keep, kind="stable")[:n - 2])
