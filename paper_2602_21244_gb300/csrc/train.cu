@@ -68,6 +68,7 @@ struct TrainArgs {
   int64_t n;                 // pairs (multiple of 16)
   uint64_t seed, t;
   double sigma_v_inv, T_ref_inv, eps;
+  double grad_scale, loss_scale;   // 1 / (n sigma_v^2), 1 / (2 n sigma_v^2)
   const float* theta;        // FP32 parameters: weights (row-major per layer), then biases
   const double *vi, *vj, *T, *ti, *tj;   // [n x 3], [n], targets [n x 3]
   const double *gi, *gj;     // mode 1: dL/dv_new [n x 3]
@@ -107,10 +108,21 @@ __device__ __forceinline__ uint16_t to_bf16(float x) {
   return __bfloat16_as_ushort(__float2bfloat16_rn(x));
 }
 
-__device__ __forceinline__ void box_muller2(double u1, double u2, float* z0, float* z1) {
-  const float rho = sqrtf(-2.f * __logf((float)(1.0 - u1)));
+// FP64 -> FP32 as the hardware converts, on the integer pipe where the result is
+// a normal number (f64_to_f32), by the conversion instruction otherwise.
+__device__ __forceinline__ float to_f32(double v) {
+  const uint32_t e = ((uint32_t)__double2hiint(v) >> 20) & 0x7FFu;
+  return e - 897u < 254u ? f64_to_f32(v) : (float)v;
+}
+
+// Two normals from the 53-bit uniforms of (a0, a1) and (b0, b1): 1 - u1 is a
+// 53-bit integer over 2^53 too, rounded to FP32 from that integer.
+__device__ __forceinline__ void box_muller2(uint32_t a0, uint32_t a1, uint32_t b0, uint32_t b1, float* z0, float* z1) {
+  const uint64_t k = (((uint64_t)a0 << 32) | a1) >> 11;
+  const float v1 = __ull2float_rn((1ull << 53) - k) * 1.1102230246251565e-16f;   // 2^-53
+  const float rho = sqrtf(-2.f * __logf(v1));
   float s, c;
-  __sincosf((float)(2.0 * DSMC_PI * u2), &s, &c);
+  __sincosf(f64_to_f32(2.0 * DSMC_PI * u53_int(b0, b1)), &s, &c);
   *z0 = rho * c;
   *z1 = rho * s;
 }
@@ -122,24 +134,29 @@ __device__ __forceinline__ uint64_t mdesc(uint32_t a, int F) { return tc::sdesc(
 // ---- FP64 helpers of the row stage.  GB300's FP64 pipe (about 1/64 of the
 // FP32 rate; a warp instruction costs the same however few lanes need it)
 // bounds that stage, so square roots and reciprocals start from the
-// special-function unit's FP64 approximations (relative error below 2^-19
-// over the whole range) and take two Newton steps (2^-38, then FP64 rounding)
-// instead of the general routines: about 10 FP64 instructions against 20 to 30.
-__device__ __forceinline__ double rsqrt64(double x) {   // x > 0, normal
+// special-function unit's FP64 approximation r of 1/sqrt(x) (relative error below
+// 2^-19 over the whole range) and take one third-order step: with e = 1 - x r^2,
+// 1/sqrt(x) = r (1 - e)^(-1/2) = r (1 + e/2 + 3/8 e^2 + ...), cut after e^2
+// (relative error 5/16 e^3 < 2^-55): 5 FP64 instructions against 20 to 30.
+__device__ __forceinline__ double rsqrt_seed64(double x) {
   double r;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  const double h = 0.5 * x;
-  r = fma(r, fma(-h * r, r, 0.5), r);
-  return fma(r, fma(-h * r, r, 0.5), r);
+  return r;
 }
-// the smallest x that rsqrt64 takes (its products stay normal): below it the
-// general routines run
-constexpr double kTiny64 = 1e-280, kHuge64 = 1e280;
-__device__ __forceinline__ bool plain64(double x) { return x > kTiny64 && x < kHuge64; }
+__device__ __forceinline__ double rsqrt64(double x) {   // x > 0, normal
+  const double r = rsqrt_seed64(x), e = fma(-(x * r), r, 1.0);
+  return fma(r * e, fma(0.375, e, 0.5), r);
+}
+// x that rsqrt64 takes (its products stay normal): 2^-930 <= x < 2^930, from the
+// high word; outside it the general routines run
+__device__ __forceinline__ bool plain64(double x) {
+  constexpr uint32_t lo = (1023u - 930u) << 20, hi = (1023u + 930u) << 20;
+  return (uint32_t)__double2hiint(x) - lo < hi - lo;
+}
 __device__ __forceinline__ double sqrt64(double x) {
   if (!plain64(x)) return sqrt(x);
-  const double r = rsqrt64(x), y = x * r;
-  return fma(0.5 * r, fma(-y, y, x), y);
+  const double r = rsqrt_seed64(x), y = x * r, e = fma(-y, r, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
 // sums over the 16 lanes of this half-warp (groups are 16 consecutive rows)
@@ -181,7 +198,7 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
   // so the result does not depend on warp scheduling)
   float dbacc[3] = {0.f, 0.f, 0.f};  // layer l, column c0 + lane
   float dbo[3] = {0.f, 0.f, 0.f};    // output bias (lane 0 of warps 0..3)
-  double lossw = 0.0;                // loss of this warp's rows (lane 0 of warps 0..3)
+  double lossw = 0.0;                // sum of |v_new - v_target|^2 of this thread's rows (warps 0..3)
   float* dz4f = (float*)(sm + S_DZ4F);
   // ---- weights into K-major tiles (eight columns, one 16-byte store, at a
   // time: a mini-batch of one tile per CTA pays this once per step), biases
@@ -309,12 +326,12 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
     for (int q = 0; q < 8; ++q) f[q] = 0.f;
     if (p < a.n) {
 #pragma unroll
-      for (int c = 0; c < 3; ++c) f[c] = (float)((a.vi[3 * p + c] - a.vj[3 * p + c]) * a.sigma_v_inv);
-      f[3] = (float)(a.T[p] * a.T_ref_inv);
+      for (int c = 0; c < 3; ++c) f[c] = to_f32((a.vi[3 * p + c] - a.vj[3 * p + c]) * a.sigma_v_inv);
+      f[3] = to_f32(a.T[p] * a.T_ref_inv);
       const u32x4 wa = draw(a.seed, (uint32_t)p, 0u, a.t, TAG_NOISE, 0);
       const u32x4 wb = draw(a.seed, (uint32_t)p, 0u, a.t, TAG_NOISE, 1);
-      box_muller2(u53(wa.x, wa.y), u53(wa.z, wa.w), &f[4], &f[5]);
-      box_muller2(u53(wb.x, wb.y), u53(wb.z, wb.w), &f[6], &f[7]);
+      box_muller2(wa.x, wa.y, wa.z, wa.w, &f[4], &f[5]);
+      box_muller2(wb.x, wb.y, wb.z, wb.w, &f[6], &f[7]);
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -394,36 +411,38 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
       double vi[3] = {0, 0, 0}, vj[3] = {0, 0, 0};
       if (valid)
         for (int c = 0; c < 3; ++c) { vi[c] = a.vi[3 * p + c]; vj[c] = a.vj[3 * p + c]; }
-      double ur[3], g = 0.0, u[3], cm[3];
-      for (int c = 0; c < 3; ++c) { ur[c] = vi[c] - vj[c]; cm[c] = 0.5 * (vi[c] + vj[c]); }
-      g = sqrt64(ur[0] * ur[0] + ur[1] * ur[1] + ur[2] * ur[2]);
+      // The group moments over the 32 particles of the pseudo-cell, from the pairs'
+      // sums and differences: the pair update keeps vi + vj, so the mean velocity
+      // is the same before and after, and with d = (vi + vj)/2 - mean
+      //   |vi - mean|^2 + |vj - mean|^2 = 2 |d|^2 + |v_r|^2 / 2
+      // before it; after it the particles are at d +- v_r'/2.
+      double ur[3], u[3], d[4];
+      for (int c = 0; c < 3; ++c) { ur[c] = vi[c] - vj[c]; d[c] = vi[c] + vj[c]; }
+      const double sum[3] = {d[0], d[1], d[2]};
+      d[3] = 0.0;
+      half_sums<4>(d);
+      double upre[3], th[2] = {0.0, 0.0};
+      for (int c = 0; c < 3; ++c) {
+        upre[c] = d[c] * (1.0 / (2 * kGroup));
+        d[c] = fma(0.5, sum[c], -upre[c]);
+        th[0] = fma(d[c], d[c], th[0]);
+      }
+      const double g2 = ur[0] * ur[0] + ur[1] * ur[1] + ur[2] * ur[2], g = sqrt64(g2);
+      th[0] = fma(0.5, g2, th[0] + th[0]);
       wait_mma();
       float v[16];
       tc::ld16(lane_tm + TM_OUT, v);
-      const double yd[3] = {v[0] + bias[3 * kH], v[1] + bias[3 * kH + 1], v[2] + bias[3 * kH + 2]};
+      const double yd[3] = {f32_to_f64(v[0] + bias[3 * kH]), f32_to_f64(v[1] + bias[3 * kH + 1]),
+                            f32_to_f64(v[2] + bias[3 * kH + 2])};
       const double ny2 = yd[0] * yd[0] + yd[1] * yd[1] + yd[2] * yd[2];
       // 1/|y| (0 for y = 0)
       const double iny = !valid ? 0.0 : plain64(ny2) ? rsqrt64(ny2) : ny2 > 0.0 ? 1.0 / sqrt(ny2) : 0.0;
-      double pi[3], pj[3];
+      const double hg = 0.5 * g;
+      double dpi[3], dpj[3];
       for (int c = 0; c < 3; ++c) {
         u[c] = yd[c] * iny;
-        const double h = 0.5 * g * u[c];
-        pi[c] = cm[c] + h;
-        pj[c] = cm[c] - h;
-      }
-      // group moments over the 32 particles of the pseudo-cell (two passes)
-      double us[8];
-      for (int c = 0; c < 3; ++c) { us[c] = vi[c] + vj[c]; us[4 + c] = pi[c] + pj[c]; }
-      us[3] = us[7] = 0.0;
-      half_sums<8>(us);
-      double upre[3], dpi[3], dpj[3], th[2] = {0.0, 0.0};
-      for (int c = 0; c < 3; ++c) {
-        upre[c] = us[c] * (1.0 / (2 * kGroup));
-        const double upost = us[4 + c] * (1.0 / (2 * kGroup));
-        const double a1 = vi[c] - upre[c], a2 = vj[c] - upre[c];
-        th[0] = fma(a1, a1, fma(a2, a2, th[0]));
-        dpi[c] = pi[c] - upost;
-        dpj[c] = pj[c] - upost;
+        dpi[c] = fma(hg, u[c], d[c]);
+        dpj[c] = fma(-hg, u[c], d[c]);
         th[1] = fma(dpi[c], dpi[c], fma(dpj[c], dpj[c], th[1]));
       }
       half_sums<2>(th);
@@ -439,22 +458,16 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
         double l2 = 0.0;
         if (valid) {
           if (a.mode == 2) {
-            const double sc = a.sigma_v_inv * a.sigma_v_inv / (double)a.n;
             for (int c = 0; c < 3; ++c) {
               const double ri = ni[c] - a.ti[3 * p + c], rj = nj[c] - a.tj[3 * p + c];
               l2 = fma(ri, ri, fma(rj, rj, l2));
-              Gd[c] = (ri - rj) * sc;
+              Gd[c] = (ri - rj) * a.grad_scale;
             }
           } else {
             for (int c = 0; c < 3; ++c) Gd[c] = a.gi[3 * p + c] - a.gj[3 * p + c];
           }
         }
-        if (a.mode == 2) {  // loss = sum |v_new - v_target|^2 / sigma_v^2 / (2 n)
-          double lw = l2 * a.sigma_v_inv * a.sigma_v_inv / (2.0 * (double)a.n);
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) lw += __shfl_xor_sync(0xffffffffu, lw, o);
-          lossw += lw;
-        }
+        lossw += l2;   // (summed over the lanes and scaled at the end)
         // Backward of moment matching, dL/dv = alpha (G - Gbar) - (alpha S /
         // Theta_post) (v - u_post), then of the centre-of-mass update (v_r'
         // enters as +1/2 for i, -1/2 for j) and of the projection, dy =
@@ -468,10 +481,10 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
         }
         const double s = valid ? g * iny : 0.0;
         for (int c = 0; c < 3; ++c) {
-          const float d = valid ? (float)(s * fma(-u[c], ud, dvr[c])) : 0.f;
-          dz4f[4 * row + c] = d;
+          const float dy = valid ? to_f32(s * fma(-u[c], ud, dvr[c])) : 0.f;
+          dz4f[4 * row + c] = dy;
           // bias gradient of the output layer
-          float s3 = d;
+          float s3 = dy;
 #pragma unroll
           for (int o = 16; o > 0; o >>= 1) s3 += __shfl_xor_sync(0xffffffffu, s3, o);
           dbo[c] += s3;
@@ -611,10 +624,12 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
         put(P + kH * kXin + 2 * kH * kH + row * 16, 16);
       }
       const int g = warp & 3;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) lossw += __shfl_xor_sync(0xffffffffu, lossw, o);
       for (int l = 0; l < 3; ++l) P[kPDB + g * 400 + l * kH + c0 + lane] = dbacc[l];
       if (cg == 0 && lane == 0) {
         for (int c = 0; c < 3; ++c) P[kPDB + g * 400 + 3 * kH + c] = dbo[c];
-        P[kPLOSS + g] = (float)lossw;
+        P[kPLOSS + g] = (float)(lossw * a.loss_scale);
       }
     }
   } else if (a.mode != 0 && t == 0 && !alive) {
@@ -735,6 +750,8 @@ int launch_train(Ctx* c, const dsmc_mlp_t& mlp, int mode, uint64_t seed, uint64_
   TrainArgs a;
   a.mode = mode; a.act = mlp.act; a.n = n; a.seed = seed; a.t = t;
   a.sigma_v_inv = 1.0 / mlp.sigma_v; a.T_ref_inv = 1.0 / mlp.T_ref; a.eps = mlp.eps;
+  a.grad_scale = n > 0 ? a.sigma_v_inv * a.sigma_v_inv / (double)n : 0.0;
+  a.loss_scale = 0.5 * a.grad_scale;
   a.theta = theta; a.vi = vi; a.vj = vj; a.T = T; a.ti = ti; a.tj = tj; a.gi = gi; a.gj = gj;
   a.oi = oi; a.oj = oj; a.zst = act; a.partial = (float*)ws; a.status = status_ptr(c);
   const int64_t tiles = (n + kT - 1) / kT;
