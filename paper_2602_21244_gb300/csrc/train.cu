@@ -608,8 +608,18 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
       for (int q = t; q < kPartial; q += kNT) P[q] = 0.f;
     } else {
       float v[32];
-      auto put = [&](float* dst, int k) {   // k consecutive values of this thread (16-byte aligned)
-        for (int q = 0; q < k; q += 4) *(float4*)(dst + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
+      // k consecutive values of this thread (16 bytes at a time where the workspace allows it)
+      const bool wide = ((uintptr_t)a.partial & 15u) == 0;
+      auto put = [&](float* dst, int k) {
+        if (wide) {
+#pragma unroll
+          for (int q = 0; q < 32; q += 4)
+            if (q < k) *(float4*)(dst + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
+        } else {
+#pragma unroll
+          for (int q = 0; q < 32; ++q)
+            if (q < k) dst[q] = v[q];
+        }
       };
       // dW2, dW3: [128 out x 128 in]
       tc::ld32(lane_tm + TM_DW2 + (uint32_t)c0, v);
