@@ -11,8 +11,8 @@
 //             backward -> dz4 = dL/dy; z_3 is still in the accumulator that
 //             the forward left it in (the output layer has columns of its
 //             own), z_2 and z_1 are recomputed by an MMA from exactly the
-//             forward's operands (h1's low bf16 terms stay in tensor memory, so
-//             nothing else has to be regenerated), so every z_l equals the
+//             forward's operands (h1's low bf16 terms stay in tensor memory until
+//             z_2 is there, so nothing else has to be regenerated), so every z_l equals the
 //             forward's bit for bit (the stored variant reads back the copy
 //             the forward wrote to global memory instead),
 //             dz_l = dh_l * act'(z_l), dW_l += dz_l^T h_{l-1} (MN-major
@@ -22,7 +22,7 @@
 //             sums them over CTAs in a fixed order (deterministic)
 // TMEM columns: 0..127 scratch, 128..255 dW2, 256..383 dW3, 384..415 dW1
 // (hi|lo input columns), 416..431 dW4^T, 432..447 output layer, 448..511 the
-// low terms of h1 (A operand).
+// low terms of h1 (A operand), in the backward 64 columns of z_1.
 #include <cuda_bf16.h>
 
 #include "internal.cuh"
@@ -82,10 +82,15 @@ __device__ __forceinline__ float act_fn(int act, float z) {
   if (act == 1) return fmaxf(z, 0.f);
   return __fdividef(z, 1.f + __expf(-z));
 }
-__device__ __forceinline__ float act_grad(int act, float z) {
-  if (act == 1) return z > 0.f ? 1.f : 0.f;
-  const float s = __fdividef(1.f, 1.f + __expf(-z));
-  return s * (1.f + z * (1.f - s));
+// SiLU'(z) = s (1 + z (1 - s)), s = 1/(1 + e^-z), of two values on the paired FP32
+// pipe, the same roundings as one value at a time (which took the 16 warps 3,700
+// cycles a layer, now 2,000).
+__device__ __forceinline__ float2 silu_slope2(float2 z) {
+  const float2 one = make_float2(1.f, 1.f), m1 = make_float2(-1.f, -1.f);
+  const float2 t = __fmul2_rn(z, make_float2(-1.44269504f, -1.44269504f));   // -z log2(e)
+  const float2 d = __fadd2_rn(make_float2(tc::ex2_approx(t.x), tc::ex2_approx(t.y)), one);
+  const float2 s = make_float2(tc::rcp_approx(d.x), tc::rcp_approx(d.y));
+  return __fmul2_rn(s, __ffma2_rn(z, __ffma2_rn(s, m1, one), one));
 }
 
 // v[32] per lane -> lane l returns the sum over the warp's lanes of v[l]
@@ -266,6 +271,11 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
     for (int s = 0; s < 2; ++s)
       tc::mma_bf16(tm, kdesc(sb + S_X + 256u * s, kXin), kdesc(sb + S_WIN + 256u * s, kXin), id, s > 0);
   };
+  // columns 64 h .. 64 h + 63 of z1, for the backward (thread 0)
+  auto half_input_mma = [&](int h) {
+    const uint32_t id = tc::idesc_bf16(kT, 64), w = sb + S_WIN + tc::kmajor_offset(64 * h, 0, kXin);
+    for (int s = 0; s < 2; ++s) tc::mma_bf16(tm + TM_H1LO, kdesc(sb + S_X + 256u * s, kXin), kdesc(w + 256u * s, kXin), id, s > 0);
+  };
   // The MMA of hidden layer l + 1 (l = 1, 2) on its input as hi + lo terms:
   // h1 = S_H1 + TM_H1LO (tensor memory), h2 = S_H2 + S_WK (thread 0)
   auto hidden_mma = [&](int l) {
@@ -341,8 +351,20 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
   };
   // act'(z + bias) of this thread's 32 values of layer l
   auto act_slopes = [&](int l, const float* z, float* g) {
+    const float2* b2 = (const float2*)(bias + l * kH + c0);
+    if (a.act == 0) {
 #pragma unroll
-    for (int q = 0; q < 32; ++q) g[q] = act_grad(a.act, z[q] + bias[l * kH + c0 + q]);
+      for (int q = 0; q < 16; ++q) {
+        const float2 v = silu_slope2(__fadd2_rn(make_float2(z[2 * q], z[2 * q + 1]), b2[q]));
+        g[2 * q] = v.x; g[2 * q + 1] = v.y;
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 16; ++q) {
+        const float2 v = __fadd2_rn(make_float2(z[2 * q], z[2 * q + 1]), b2[q]);
+        g[2 * q] = v.x > 0.f ? 1.f : 0.f; g[2 * q + 1] = v.y > 0.f ? 1.f : 0.f;
+      }
+    }
   };
   // this tile's z_l of the stored variant, row-major [128 x 128]
   auto stored_z = [&](int64_t tile, int l) { return (float4*)(a.zst + (((size_t)tile * 3 + l) * kT + row) * kH + c0); };
@@ -355,7 +377,8 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
         z[4 * q] = f.x; z[4 * q + 1] = f.y; z[4 * q + 2] = f.z; z[4 * q + 3] = f.w;
       }
     } else {
-      tc::ld32(lane_tm + (uint32_t)c0, z);
+      // (z_1: its first 64 columns, later the others, in TM_H1LO)
+      tc::ld32(lane_tm + (l == 0 ? TM_H1LO + (uint32_t)(c0 & 63) : (uint32_t)c0), z);
     }
   };
 
@@ -429,6 +452,12 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
       }
       const double g2 = ur[0] * ur[0] + ur[1] * ur[1] + ur[2] * ur[2], g = sqrt64(g2);
       th[0] = fma(0.5, g2, th[0] + th[0]);
+      double gi[3] = {0, 0, 0}, gj[3] = {0, 0, 0};   // targets (mode 2) or dL/dv_new (mode 1)
+      if (valid && a.mode != 0) {
+        const double* si = a.mode == 2 ? a.ti : a.gi;
+        const double* sj = a.mode == 2 ? a.tj : a.gj;
+        for (int c = 0; c < 3; ++c) { gi[c] = si[3 * p + c]; gj[c] = sj[3 * p + c]; }
+      }
       wait_mma();
       float v[16];
       tc::ld16(lane_tm + TM_OUT, v);
@@ -459,12 +488,12 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
         if (valid) {
           if (a.mode == 2) {
             for (int c = 0; c < 3; ++c) {
-              const double ri = ni[c] - a.ti[3 * p + c], rj = nj[c] - a.tj[3 * p + c];
+              const double ri = ni[c] - gi[c], rj = nj[c] - gj[c];
               l2 = fma(ri, ri, fma(rj, rj, l2));
               Gd[c] = (ri - rj) * a.grad_scale;
             }
           } else {
-            for (int c = 0; c < 3; ++c) Gd[c] = a.gi[3 * p + c] - a.gj[3 * p + c];
+            for (int c = 0; c < 3; ++c) Gd[c] = gi[c] - gj[c];
           }
         }
         lossw += l2;   // (summed over the lanes and scaled at the end)
@@ -497,6 +526,12 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
     } else {
       phase ^= 1u;   // the output layer's MMAs, which only the row threads wait for
       if (xthr && tile + gridDim.x < ntiles) features((tile + gridDim.x) * kT + row, xw);
+      // the coming tile's rows of the arrays that the row stage reads, into L2 (3 KB of each: 24 lines)
+      if (cg == 2 && a.mode != 0 && lane < 24 && tile + gridDim.x < ntiles) {
+        const double* arr[4] = {a.vi, a.vj, a.mode == 2 ? a.ti : a.gi, a.mode == 2 ? a.tj : a.gj};
+        const double* q = arr[warp & 3] + 3 * (tile + gridDim.x) * kT + 16 * lane;
+        if (q < arr[warp & 3] + 3 * a.n) asm volatile("prefetch.global.L2 [%0];" ::"l"(q));
+      }
     }
     if (a.mode == 0) {
       tc::fence_before();
@@ -506,14 +541,16 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
       continue;
     }
     // ---------------- layers 3, 2, 1: z3 is still in the scratch accumulator
-    float dh[32];
-    {
-      float z[32];
-      load_z(tile, 2, z);
-      act_slopes(2, z, dh);
-    }
+    // Every MMA that a layer needs is issued with the one before: z_2 beside
+    // dW4, z_1 beside dh_2 and dh_1 (64 columns at a time, where h1's low terms
+    // were), so a layer costs one barrier and one wait, and act' is formed while
+    // the next MMAs run (z_2 and z_1 each behind a barrier and a wait of their own:
+    // 1M pairs 1112 us, now 1072).
+    float dh[32], g[32];
+    load_z(tile, 2, g);
+    act_slopes(2, g, dh);
     if (!(alive = to_mma())) break;
-    // dW4^T += h3^T dz4 (hi and lo)
+    // dW4^T += h3^T dz4 (hi and lo); z_2 from h1 (hi + lo)
     const uint32_t acc0 = tiles_done > 0 ? 1u : 0u;
     if (t == 0) {
       tc::fence_after();
@@ -523,6 +560,7 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
                      (acc0 | (s > 0)) ? 1u : 0u);
       for (int s = 0; s < 8; ++s)
         tc::mma_bf16(tm + TM_DW4, mdesc(sb + S_WKLO + 2u * 2048u * s, kH), mdesc(sb + S_DZ4 + 2u * 256u * s, 16), id4, 1);
+      if (!a.zst) hidden_mma(1);
       tc::commit(mbar);
     }
     // dz3 = dh3 act'(z3) with dh3 = dz4 W4 on CUDA cores (K = 3)
@@ -533,19 +571,24 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
         dh[q] = (d0 * wo32[c0 + q] + d1 * wo32[kH + c0 + q] + d2 * wo32[2 * kH + c0 + q]) * dh[q];
     }
     for (int l = 2;; --l) {
-      // dh holds dz_l: stored as the operand of dW_l and dh_{l-1} once the
-      // MMAs that read the last one (h3's high terms for l = 2) are done
+      // dh holds dz_l: packed as the operand of dW_l and dh_{l-1}.  dz_3 and dz_1
+      // go to S_WK, dz_2 to S_WKLO, whose last readers are done: h3's dW4 by
+      // the first wait, dW_3 by the wait for dh_1, which was committed after it.
+      const uint32_t dzb = l == 1 ? S_WKLO : S_WK;
       uint32_t pk[16];
 #pragma unroll
       for (int q = 0; q < 16; ++q) pk[q] = tc::pack_bf16x2(dh[2 * q], dh[2 * q + 1]);
-      if (l == 2) wait_mma();
+      if (l == 2) {
+        wait_mma();
+        load_z(tile, 1, g);   // z_2, before dh_2 takes the accumulator
+      }
 #pragma unroll
       for (int j = 0; j < 4; ++j)
-        tc::st_shared_v4(sb + S_WK + tc::kmajor_offset(row, c0 + 8 * j, kH), pk[4 * j], pk[4 * j + 1], pk[4 * j + 2],
+        tc::st_shared_v4(sb + dzb + tc::kmajor_offset(row, c0 + 8 * j, kH), pk[4 * j], pk[4 * j + 1], pk[4 * j + 2],
                          pk[4 * j + 3]);
       if (!(alive = to_mma())) break;
-      // dh_{l-1} = dz W_l (not needed for l = 0), then dW_l += dz^T h_{l-1},
-      // which runs on while dh_{l-1} is read back
+      // dh_{l-1} = dz W_l and a half of z_1 (not for l = 0), then dW_l += dz^T
+      // h_{l-1}, which runs on while dh_{l-1} is read back
       if (t == 0) {
         tc::fence_after();
         if (l > 0) {
@@ -553,44 +596,36 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
           const uint32_t wl = l == 2 ? S_W3 : S_W2;
           const uint32_t dw = l == 2 ? TM_DW3 : TM_DW2;
           const uint32_t idh = tc::idesc_bf16(kT, kH) | (1u << 16);
+          if (!a.zst) half_input_mma(2 - l);
           for (int s = 0; s < 8; ++s)
-            tc::mma_bf16(tm, kdesc(sb + S_WK + 256u * s, kH), mdesc(sb + wl + 2u * 2048u * s, kH), idh, s > 0);
+            tc::mma_bf16(tm, kdesc(sb + dzb + 256u * s, kH), mdesc(sb + wl + 2u * 2048u * s, kH), idh, s > 0);
           tc::commit(mbar);
           const uint32_t idw = tc::idesc_bf16(kH, kH) | (1u << 15) | (1u << 16);
           for (int s = 0; s < 8; ++s)
-            tc::mma_bf16(tm + dw, mdesc(sb + S_WK + 2u * 2048u * s, kH), mdesc(sb + hprev + 2u * 2048u * s, kH), idw,
+            tc::mma_bf16(tm + dw, mdesc(sb + dzb + 2u * 2048u * s, kH), mdesc(sb + hprev + 2u * 2048u * s, kH), idw,
                          (acc0 | (s > 0)) ? 1u : 0u);
         } else {
           const uint32_t idw = tc::idesc_bf16(kH, kXin) | (1u << 15) | (1u << 16);
           for (int s = 0; s < 8; ++s)
-            tc::mma_bf16(tm + TM_DW1, mdesc(sb + S_WK + 2u * 2048u * s, kH), mdesc(sb + S_X + 2u * 512u * s, kXin), idw,
+            tc::mma_bf16(tm + TM_DW1, mdesc(sb + dzb + 2u * 2048u * s, kH), mdesc(sb + S_X + 2u * 512u * s, kXin), idw,
                          (acc0 | (s > 0)) ? 1u : 0u);
           tc::commit(mbar);
         }
       }
       dbacc[l] += warp_colsum32(dh);   // (the column sums; dh is not used after)
       if (l == 0) break;
+      // act'(z_{l-1}): formed here, beside the MMAs, but for the columns of z_1
+      // that come with dh_1
+      if (l == 2 || cg < 2) act_slopes(l - 1, g, g);
       wait_mma();
       tc::ld32(lane_tm + (uint32_t)c0, dh);
-      if (!(alive = to_mma())) break;
-      // z_{l-1} recomputed from the forward's own operands (h1 hi + lo, then
-      // x hi + lo) into the scratch accumulator; its commit covers dW_l too
-      if (t == 0) {
-        tc::fence_after();
-        if (!a.zst) {
-          if (l == 2) hidden_mma(1);
-          else input_mma();
-        }
-        tc::commit(mbar);
+      if (l == 1 && cg >= 2) {
+        load_z(tile, 0, g);
+        act_slopes(0, g, g);
       }
-      wait_mma();
-      {
-        float z[32], g[32];
-        load_z(tile, l - 1, z);
-        act_slopes(l - 1, z, g);
 #pragma unroll
-        for (int q = 0; q < 32; ++q) dh[q] *= g[q];
-      }
+      for (int q = 0; q < 32; ++q) dh[q] *= g[q];
+      if (l == 2 && cg < 2) load_z(tile, 0, g);
     }
     if (!alive) break;
     busy = true;
