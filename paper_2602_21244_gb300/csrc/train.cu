@@ -51,7 +51,11 @@ constexpr uint32_t S_DZ4F = S_DZ4 + kT * 16 * 2;       // [128 x 3] FP32
 constexpr uint32_t S_BIAS = S_DZ4F + kT * 4 * 4;       // 3*128 + 16 floats
 constexpr uint32_t S_WO32 = S_BIAS + (3 * kH + 16) * 4;  // output weights in FP32 [3 x 128]
 constexpr uint32_t S_MISC = S_WO32 + 3 * kH * 4;       // mbarrier, tmem ptr, flag
-constexpr uint32_t S_TOTAL = S_MISC + 64;
+constexpr uint32_t S_PRE = S_MISC + 64;                // [5 x 128] FP64: d, |v_r|, Theta_pre term of each row
+constexpr uint32_t S_MEAN = S_PRE + 5 * kT * 8;        // [8 x 4] FP64: mean velocity of each group
+constexpr uint32_t S_TOTAL = S_MEAN + (kT / kGroup) * 4 * 8;
+static_assert(S_PRE % 8 == 0 && S_TOTAL <= 227 * 1024, "shared memory");
+constexpr int kIssuer = 256;     // thread that issues the MMAs (of a warp without rows)
 // per-CTA partial: dW1 [128 x 32], dW2, dW3 [128 x 128], dW4^T [128 x 16], then the bias
 // gradients of each of the 4 TMEM lane groups [4 x 400], then the loss of each lane group
 constexpr int kPDB = kH * kXin + 2 * kH * kH + kH * 16;
@@ -265,19 +269,19 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
     return *flag != 0;
   };
 
-  // z1 from x (hi + lo): two K steps (thread 0)
+  // z1 from x (hi + lo): two K steps (thread kIssuer)
   auto input_mma = [&]() {
     const uint32_t id = tc::idesc_bf16(kT, kH);
     for (int s = 0; s < 2; ++s)
       tc::mma_bf16(tm, kdesc(sb + S_X + 256u * s, kXin), kdesc(sb + S_WIN + 256u * s, kXin), id, s > 0);
   };
-  // columns 64 h .. 64 h + 63 of z1, for the backward (thread 0)
+  // columns 64 h .. 64 h + 63 of z1, for the backward (thread kIssuer)
   auto half_input_mma = [&](int h) {
     const uint32_t id = tc::idesc_bf16(kT, 64), w = sb + S_WIN + tc::kmajor_offset(64 * h, 0, kXin);
     for (int s = 0; s < 2; ++s) tc::mma_bf16(tm + TM_H1LO, kdesc(sb + S_X + 256u * s, kXin), kdesc(w + 256u * s, kXin), id, s > 0);
   };
   // The MMA of hidden layer l + 1 (l = 1, 2) on its input as hi + lo terms:
-  // h1 = S_H1 + TM_H1LO (tensor memory), h2 = S_H2 + S_WK (thread 0)
+  // h1 = S_H1 + TM_H1LO (tensor memory), h2 = S_H2 + S_WK (thread kIssuer)
   auto hidden_mma = [&](int l) {
     const uint32_t id = tc::idesc_bf16(kT, kH);
     const uint32_t wl = l == 1 ? S_W2 : S_W3, hhi = l == 1 ? S_H1 : S_H2;
@@ -349,6 +353,44 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
       x[4 + q] = tc::pack_bf16x2(f[2 * q] - __uint_as_float(x[q] << 16), f[2 * q + 1] - __uint_as_float(x[q] & 0xFFFF0000u));
     }
   };
+  // The row stage's part that needs no network, one row per thread of warps 0..3
+  // in two halves of about an MMA wait each, handed to the row stage in shared
+  // memory: the group moments over the 32 particles of the pseudo-cell, from the pairs'
+  // sums and differences: the pair update keeps vi + vj, so the mean velocity
+  // is the same before and after, and with d = (vi + vj)/2 - mean
+  //   |vi - mean|^2 + |vj - mean|^2 = 2 |d|^2 + |v_r|^2 / 2
+  // before it; after it the particles are at d +- v_r'/2.  (At the head of the
+  // row stage it took 4,000 of a tile's 36,600 cycles: 1M pairs 1072 us, now 1010.)
+  double* pre = (double*)(sm + S_PRE);
+  double* mean = (double*)(sm + S_MEAN);
+  auto row_pairs = [&](int64_t p, bool valid) {
+    double g2 = 0.0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double vi = valid ? a.vi[3 * p + c] : 0.0, vj = valid ? a.vj[3 * p + c] : 0.0, ur = vi - vj;
+      g2 = fma(ur, ur, g2);
+      pre[c * kT + row] = vi + vj;
+    }
+    pre[3 * kT + row] = g2;
+  };
+  auto row_groups = [&]() {
+    double d[4], sum[3], th = 0.0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) d[c] = sum[c] = pre[c * kT + row];
+    d[3] = 0.0;
+    half_sums<4>(d);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double u = d[c] * (1.0 / (2 * kGroup));
+      if ((lane & (kGroup - 1)) == c) mean[4 * (row / kGroup) + c] = u;
+      d[c] = fma(0.5, sum[c], -u);
+      th = fma(d[c], d[c], th);
+      pre[c * kT + row] = d[c];
+    }
+    const double g2 = pre[3 * kT + row];
+    pre[3 * kT + row] = sqrt64(g2);
+    pre[4 * kT + row] = fma(0.5, g2, th + th);
+  };
   // act'(z + bias) of this thread's 32 values of layer l
   auto act_slopes = [&](int l, const float* z, float* g) {
     const float2* b2 = (const float2*)(bias + l * kH + c0);
@@ -400,12 +442,15 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
     if (!(alive = to_mma())) break;
     // ---------------- forward, layers 1..3 (scratch accumulator at TMEM column 0)
     for (int l = 0; l < 3; ++l) {
-      if (t == 0) {
+      if (t == kIssuer) {
         tc::fence_after();
         if (l == 0) input_mma();
         else hidden_mma(l);
         tc::commit(mbar);
       }
+      // beside the MMAs of layers 2 and 3, what the row stage needs of the pairs alone
+      if (rowthr && l == 1) row_pairs(p, valid);
+      if (rowthr && l == 2) row_groups();
       wait_mma();
       float v[32];
       tc::ld32(lane_tm + (uint32_t)c0, v);
@@ -420,7 +465,7 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
     if (!alive) break;
     // ---------------- output layer, into columns of its own: z3 stays in the
     // scratch accumulator for the backward
-    if (t == 0) {
+    if (t == kIssuer) {
       tc::fence_after();
       const uint32_t id = tc::idesc_bf16(kT, 16);
       for (int s = 0; s < 8; ++s)
@@ -431,27 +476,10 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
     }
     // ---------------- shell projection, pair update, moment matching, loss (rows)
     if (rowthr) {
-      double vi[3] = {0, 0, 0}, vj[3] = {0, 0, 0};
-      if (valid)
-        for (int c = 0; c < 3; ++c) { vi[c] = a.vi[3 * p + c]; vj[c] = a.vj[3 * p + c]; }
-      // The group moments over the 32 particles of the pseudo-cell, from the pairs'
-      // sums and differences: the pair update keeps vi + vj, so the mean velocity
-      // is the same before and after, and with d = (vi + vj)/2 - mean
-      //   |vi - mean|^2 + |vj - mean|^2 = 2 |d|^2 + |v_r|^2 / 2
-      // before it; after it the particles are at d +- v_r'/2.
-      double ur[3], u[3], d[4];
-      for (int c = 0; c < 3; ++c) { ur[c] = vi[c] - vj[c]; d[c] = vi[c] + vj[c]; }
-      const double sum[3] = {d[0], d[1], d[2]};
-      d[3] = 0.0;
-      half_sums<4>(d);
-      double upre[3], th[2] = {0.0, 0.0};
-      for (int c = 0; c < 3; ++c) {
-        upre[c] = d[c] * (1.0 / (2 * kGroup));
-        d[c] = fma(0.5, sum[c], -upre[c]);
-        th[0] = fma(d[c], d[c], th[0]);
-      }
-      const double g2 = ur[0] * ur[0] + ur[1] * ur[1] + ur[2] * ur[2], g = sqrt64(g2);
-      th[0] = fma(0.5, g2, th[0] + th[0]);
+      double u[3], d[3], upre[3], th[2] = {0.0, 0.0};
+      for (int c = 0; c < 3; ++c) { d[c] = pre[c * kT + row]; upre[c] = mean[4 * (row / kGroup) + c]; }
+      const double g = pre[3 * kT + row];
+      th[0] = pre[4 * kT + row];
       double gi[3] = {0, 0, 0}, gj[3] = {0, 0, 0};   // targets (mode 2) or dL/dv_new (mode 1)
       if (valid && a.mode != 0) {
         const double* si = a.mode == 2 ? a.ti : a.gi;
@@ -552,7 +580,7 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
     if (!(alive = to_mma())) break;
     // dW4^T += h3^T dz4 (hi and lo); z_2 from h1 (hi + lo)
     const uint32_t acc0 = tiles_done > 0 ? 1u : 0u;
-    if (t == 0) {
+    if (t == kIssuer) {
       tc::fence_after();
       const uint32_t id4 = tc::idesc_bf16(kT, 16) | (1u << 15) | (1u << 16);
       for (int s = 0; s < 8; ++s)
@@ -589,7 +617,7 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
       if (!(alive = to_mma())) break;
       // dh_{l-1} = dz W_l and a half of z_1 (not for l = 0), then dW_l += dz^T
       // h_{l-1}, which runs on while dh_{l-1} is read back
-      if (t == 0) {
+      if (t == kIssuer) {
         tc::fence_after();
         if (l > 0) {
           const uint32_t hprev = l == 2 ? S_H2 : S_H1;
