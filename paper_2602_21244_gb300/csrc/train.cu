@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
   // is the same before and after, and with d = (vi + vj)/2 - mean
   //   |vi - mean|^2 + |vj - mean|^2 = 2 |d|^2 + |v_r|^2 / 2
   // before it; after it the particles are at d +- v_r'/2.  (At the head of the
-  // row stage it took 4,000 of a tile's 36,600 cycles: 1M pairs 1072 us, now 1010.)
+  // row stage it took 4,000 of a tile's 36,600 cycles: 1M pairs 1072 us, then 1010.)
   double* pre = (double*)(sm + S_PRE);
   double* mean = (double*)(sm + S_MEAN);
   auto row_pairs = [&](int64_t p, bool valid) {
@@ -540,11 +540,6 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
         for (int c = 0; c < 3; ++c) {
           const float dy = valid ? to_f32(s * fma(-u[c], ud, dvr[c])) : 0.f;
           dz4f[4 * row + c] = dy;
-          // bias gradient of the output layer
-          float s3 = dy;
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) s3 += __shfl_xor_sync(0xffffffffu, s3, o);
-          dbo[c] += s3;
         }
         uint32_t d0 = tc::pack_bf16x2(dz4f[4 * row], dz4f[4 * row + 1]);
         uint32_t d1 = tc::pack_bf16x2(dz4f[4 * row + 2], 0.f);
@@ -597,6 +592,13 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
 #pragma unroll
       for (int q = 0; q < 32; ++q)
         dh[q] = (d0 * wo32[c0 + q] + d1 * wo32[kH + c0 + q] + d2 * wo32[2 * kH + c0 + q]) * dh[q];
+      if (rowthr) {   // bias gradient of the output layer
+        float s3[3] = {d0, d1, d2};
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+          for (int c = 0; c < 3; ++c) s3[c] += __shfl_xor_sync(0xffffffffu, s3[c], o);
+        for (int c = 0; c < 3; ++c) dbo[c] += s3[c];
+      }
     }
     for (int l = 2;; --l) {
       // dh holds dz_l: packed as the operand of dW_l and dh_{l-1}.  dz_3 and dz_1
