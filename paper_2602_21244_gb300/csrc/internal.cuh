@@ -198,6 +198,28 @@ __device__ __forceinline__ double f32_to_f64(float f) {
   return __hiloint2double((int)hi, (int)(m << 29));
 }
 
+// 1/sqrt(x) where GB300's FP64 pipe (about 1/64 of the FP32 rate; a warp
+// instruction costs the same however few lanes need it) bounds the code: the
+// special-function unit's FP64 approximation r (relative error below 2^-19 over
+// the whole range) and one third-order step: with e = 1 - x r^2,
+// 1/sqrt(x) = r (1 - e)^(-1/2) = r (1 + e/2 + 3/8 e^2 + ...), cut after e^2
+// (relative error 5/16 e^3 < 2^-55): 5 FP64 instructions.
+__device__ __forceinline__ double rsqrt_seed64(double x) {
+  double r;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  return r;
+}
+__device__ __forceinline__ double rsqrt64(double x) {   // x > 0, normal
+  const double r = rsqrt_seed64(x), e = fma(-(x * r), r, 1.0);
+  return fma(r * e, fma(0.375, e, 0.5), r);
+}
+// x that rsqrt64 takes (its products stay normal): 2^-930 <= x < 2^930, from the
+// high word; outside it the general routines run
+__device__ __forceinline__ bool plain64(double x) {
+  constexpr uint32_t lo = (1023u - 930u) << 20, hi = (1023u + 930u) << 20;
+  return (uint32_t)__double2hiint(x) - lo < hi - lo;
+}
+
 // ---------------------------------------------------------------- pair dependencies
 // The collide kernels walk the pairs of a step in round-major order without
 // grid-wide barriers.  Work units (a warp's 32 pairs, a 128-pair MLP tile)

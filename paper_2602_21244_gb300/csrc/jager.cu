@@ -841,7 +841,7 @@ static PotDev make_pot(const dsmc_gas_t& gas, const dsmc_potential_t& p, int n_n
 // Warp-uniform loop: every lane of a warp computes chi together (a lane past
 // the end, or with g = 0, on harmless inputs whose result is not kept).
 // Five blocks per SM: 2^22 pairs 1785 us, four 1896, six 1866 (the pair update,
-// with the rotation's registers besides, is faster with four: 1284 against 1331 us).
+// with the rotation's registers besides, is faster with four: 1230 against 1272 us, three 1249).
 template <int KIND>
 __global__ void __launch_bounds__(128, 5) k_jager_chi(PotDev P, int64_t n, const float* __restrict__ b,
                                                       const float* __restrict__ g, float* __restrict__ chi) {
@@ -893,6 +893,78 @@ __device__ __forceinline__ void deflect(double u, double v, double w, double g, 
   o[2] = cc * w + g * sc * (ce * cz + se * az);
 }
 
+// ---- The pair update's rotation with fewer FP64 instructions than the general
+// functions take.  Sine and cosine of an angle 2 pi k / 256 + d, |d| <= pi/256,
+// from those of 2 pi k / 256 (the first quarter comes with the launch, the circle
+// is laid out in shared memory) by the angle-sum formulas, with the Taylor series of
+// sin d to d^7 and of cos d - 1 to d^6 (truncation below 2e-21 and 2e-20): 13 FP64
+// instructions for both, errors of an FP64 rounding or two as sincos has.
+constexpr int kTurnSteps = 256;
+struct TurnTable {
+  double quarter[kTurnSteps / 4 + 1];   // sin(2 pi k / 256), k = 0..64
+};
+__host__ inline TurnTable make_turn_table() {
+  TurnTable t;
+  for (int k = 0; k <= kTurnSteps / 4; ++k) t.quarter[k] = sin(2.0 * DSMC_PI * k / kTurnSteps);
+  t.quarter[kTurnSteps / 4] = 1.0;
+  return t;
+}
+__device__ __forceinline__ void lay_turn_table(const TurnTable& t, double2* turn) {
+  auto sine = [&](int k) {
+    const int r = k & (kTurnSteps / 4 - 1), q = (k / (kTurnSteps / 4)) & 3;
+    const double v = t.quarter[q & 1 ? kTurnSteps / 4 - r : r];
+    return q & 2 ? -v : v;
+  };
+  for (int k = threadIdx.x; k < kTurnSteps; k += blockDim.x) turn[k] = make_double2(sine(k), sine(k + kTurnSteps / 4));
+}
+__device__ __forceinline__ void turn_sincos(const double2* turn, int k, double d, double* s, double* c) {
+  const double2 t = turn[k & (kTurnSteps - 1)];
+  const double d2 = d * d;
+  const double sd = fma(d * d2, fma(fma(-1.0 / 5040, d2, 1.0 / 120), d2, -1.0 / 6), d);
+  const double cm = d2 * fma(fma(-1.0 / 720, d2, 1.0 / 24), d2, -0.5);   // cos d - 1
+  *s = t.x + fma(t.x, cm, t.y * sd);
+  *c = t.y + fma(t.y, cm, -(t.x * sd));
+}
+// of an FP32 angle: less k steps of 2 pi / 256 (as an FP64 value and the rest)
+__device__ __forceinline__ void sincos_of(const double2* turn, float x, double* s, double* c) {
+  if (!(fabsf(x) < 4096.f)) { sincos((double)x, s, c); return; }
+  const float kf = rintf(x * (float)(kTurnSteps / (2.0 * DSMC_PI)));
+  const double kd = f32_to_f64(kf);
+  const double d = fma(-kd, 9.567553118338697e-19, fma(-kd, 2.0 * DSMC_PI / kTurnSteps, f32_to_f64(x)));
+  turn_sincos(turn, (int)kf, d, s, c);
+}
+// of 2 pi U, U the 53-bit uniform of (a, b): the nearest of 256 steps from its
+// top bits, the signed remainder made a double by its bits
+__device__ __forceinline__ void sincos_turn(const double2* turn, uint32_t a, uint32_t b, double* s, double* c) {
+  const int64_t x = (int64_t)(((((uint64_t)a) << 32) | b) >> 11);
+  const int k = (int)((x + (1ll << 44)) >> 45);
+  const int64_t rem = x - ((int64_t)k << 45);   // |rem| <= 2^44
+  const double r = __longlong_as_double(0x4338000000000000ll + rem) - 6755399441055744.0;   // 1.5 2^52 + rem, less it
+  turn_sincos(turn, k, r * (2.0 * DSMC_PI / 9007199254740992.0), s, c);
+}
+
+// Deflect v_r = (u, v, w), |v_r|^2 = g2 > 0, by chi with azimuth eps as deflect does,
+// collected so that each product is formed once: with q^2 = v^2 + w^2,
+//   u' = cos(chi) u + sin(chi) sin(eps) q
+//   v' = cos(chi) v + (sin(chi)/q) (cos(eps) g w - sin(eps) u v)
+//   w' = cos(chi) w - (sin(chi)/q) (cos(eps) g v + sin(eps) u w)
+__device__ __forceinline__ void deflect_pair(double u, double v, double w, double g2, double cc, double sc, double ce,
+                                             double se, double* o) {
+  const double q2 = fma(v, v, w * w);
+  const double g = g2 * (plain64(g2) ? rsqrt64(g2) : rsqrt(g2));
+  const double B = ce * g;
+  if (q2 > 1e-24 * g2) {   // q > 1e-12 g
+    const double iq = plain64(q2) ? rsqrt64(q2) : rsqrt(q2), q = q2 * iq, A = se * u, si = sc * iq;
+    o[0] = fma(sc * se, q, cc * u);
+    o[1] = fma(si, fma(B, w, -(A * v)), cc * v);
+    o[2] = fma(-si, fma(B, v, A * w), cc * w);
+  } else {
+    o[0] = cc * u;
+    o[1] = fma(sc, B, cc * v);
+    o[2] = fma(sc, u >= 0.0 ? -se * g : se * g, cc * w);
+  }
+}
+
 struct JagerArgs {
   uint64_t seed, step;
   const uint64_t* step_dev;
@@ -912,13 +984,17 @@ struct JagerArgs {
 // (Bird 1994, Eq. 2.22) in FP64 -- cos and sin of the FP32 chi and of the
 // azimuth eps = 2 pi U2 in FP64, so that the post-collision velocities are
 // the exact deflection by that chi to FP64 rounding -- then the
-// centre-of-mass update; velocities through L2.  Every lane of the warp runs
+// centre-of-mass update, v_i' = v_i + (v_r' - v_r)/2 and v_j' = v_j - that (the pair
+// keeps its sum); velocities through L2.  Rotation and update take about 80 FP64
+// instructions, with sincos, sincospi, rsqrt and the frame written out 110: with
+// chi's 111 the FP64 pipe, 57 % busy, bounds the kernel (1.7 million pairs 1284
+// us, now 1230).  Every lane of the warp runs
 // it together (live false: a lane with no pair, or whose dependency wait
 // failed, computes on harmless inputs and stores nothing), so that chi's FP64
 // refinement and the FP64 rotation run with the warp converged.
 template <int KIND>
-__device__ __forceinline__ void collide_pair(const PotDev& P, const ChiShared& S, const JagerArgs& a, int64_t p,
-                                             int4 q, bool live) {
+__device__ __forceinline__ void collide_pair(const PotDev& P, const ChiShared& S, const double2* turn,
+                                             const JagerArgs& a, int64_t p, int4 q, bool live) {
   double xi = 0.0, yi = 0.0, zi = 0.0, xj = 0.0, yj = 0.0, zj = 0.0;
   if (live) {
     xi = __ldcg(a.vx + q.x); yi = __ldcg(a.vy + q.x); zi = __ldcg(a.vz + q.x);
@@ -935,17 +1011,15 @@ __device__ __forceinline__ void collide_pair(const PotDev& P, const ChiShared& S
   if (live && a.chi_out) a.chi_out[p] = chi;
   __syncwarp();
   double sc, cc, se, ce;
-  sincos(f32_to_f64(chi), &sc, &cc);
-  sincospi(2.0 * u53_int(w.z, w.w), &se, &ce);
-  const double g2s = use ? g2 : 1.0;
-  const double ig = rsqrt(g2s);
+  sincos_of(turn, chi, &sc, &cc);
+  sincos_turn(turn, w.z, w.w, &se, &ce);
   double o[3];
-  deflect(use ? ux : 1.0, use ? uy : 0.0, use ? uz : 0.0, g2s * ig, ig, cc, sc, ce, se, o);
+  deflect_pair(use ? ux : 1.0, use ? uy : 0.0, use ? uz : 0.0, use ? g2 : 1.0, cc, sc, ce, se, o);
   if (!use) o[0] = o[1] = o[2] = 0.0;
   if (live) {
-    const double cx = 0.5 * (xi + xj), cy = 0.5 * (yi + yj), cz = 0.5 * (zi + zj);
-    __stcg(a.vx + q.x, cx + 0.5 * o[0]); __stcg(a.vy + q.x, cy + 0.5 * o[1]); __stcg(a.vz + q.x, cz + 0.5 * o[2]);
-    __stcg(a.vx + q.y, cx - 0.5 * o[0]); __stcg(a.vy + q.y, cy - 0.5 * o[1]); __stcg(a.vz + q.y, cz - 0.5 * o[2]);
+    const double dx = o[0] - ux, dy = o[1] - uy, dz = o[2] - uz;
+    __stcg(a.vx + q.x, fma(0.5, dx, xi)); __stcg(a.vy + q.x, fma(0.5, dy, yi)); __stcg(a.vz + q.x, fma(0.5, dz, zi));
+    __stcg(a.vx + q.y, fma(-0.5, dx, xj)); __stcg(a.vy + q.y, fma(-0.5, dy, yj)); __stcg(a.vz + q.y, fma(-0.5, dz, zj));
   }
 }
 
@@ -957,11 +1031,13 @@ __device__ __forceinline__ void collide_pair(const PotDev& P, const ChiShared& S
 // to end: only true dependencies order the work.  Which thread handles a
 // pair does not change its result.
 template <int KIND>
-__global__ void __launch_bounds__(128, 4) k_collide_jager(PotDev P, JagerArgs a) {
+__global__ void __launch_bounds__(128, 4) k_collide_jager(PotDev P, TurnTable turn_table, JagerArgs a) {
   dep_wait_alone();
   if (a.step_dev) a.step = *a.step_dev;
   extern __shared__ float4 chi_sm[];
-  const ChiShared S = chi_shared(P, (float*)chi_sm);
+  __shared__ double2 turn[kTurnSteps];
+  lay_turn_table(turn_table, turn);
+  const ChiShared S = chi_shared(P, (float*)chi_sm);   // (ends with a barrier)
   const int R = a.info->n_rounds;
   const int lane = threadIdx.x & 31;
   int r = 0;
@@ -981,7 +1057,7 @@ __global__ void __launch_bounds__(128, 4) k_collide_jager(PotDev P, JagerArgs a)
       ok = wait_deps(a.done, q.x, q.y, a.deps[p], a.bar + 2, a.status);
     }
     __syncwarp();
-    collide_pair<KIND>(P, S, a, p, q, valid && ok);
+    collide_pair<KIND>(P, S, turn, a, p, q, valid && ok);
     if (valid && ok) release_pair(a.done, q.x, q.y, (unsigned)(r + 1));
     if (!__all_sync(0xffffffffu, ok)) break;
   }
@@ -1113,7 +1189,14 @@ __global__ void k_selftest_math(Exp64 E, int which, int64_t n, const double* __r
   }
 }
 
-constexpr size_t kDefaultSmem = 48 * 1024;   // dynamic shared memory a kernel may have without asking
+// dynamic shared memory that these kernels may have without asking (48 KB less their static arrays), and
+// what they ask for beyond it: the most that any node count takes, so that calls of other threads agree
+constexpr size_t kDefaultSmem = 48 * 1024 - sizeof(double2) * kTurnSteps;
+constexpr size_t kMostSmem = chi_smem(128);
+static bool allow_smem(const void* k, size_t sm) {
+  return sm <= kDefaultSmem || cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                    (int)(sm > kMostSmem ? sm : kMostSmem)) == cudaSuccess;
+}
 
 static unsigned blocks_n(int64_t n, int threads, int cap) {
   int64_t b = (n + threads - 1) / threads;
@@ -1136,9 +1219,7 @@ int launch_jager_chi(Ctx* c, const dsmc_gas_t& gas, const dsmc_potential_t& pot,
   const Shape sh = shape_or_default(c, DSMC_TUNE_JAGER_CHI);
   const size_t sm = chi_smem(sh.threads, P.n_nodes + P.n_low);
   const auto k = P.kind == 0 ? k_jager_chi<0> : k_jager_chi<-1>;
-  if (sm > kDefaultSmem &&
-      cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
-    return record(c, DSMC_ERR_CUDA, "jager_chi: shared-memory attribute");
+  if (!allow_smem((const void*)k, sm)) return record(c, DSMC_ERR_CUDA, "jager_chi: shared-memory attribute");
   launch_dep(k, blocks_n(n, sh.threads, sm_count(c) * sh.blocks_per_sm), sh.threads, sm, s, P, n, b, g, chi);
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
@@ -1147,9 +1228,7 @@ int launch_jager_chi(Ctx* c, const dsmc_gas_t& gas, const dsmc_potential_t& pot,
 // resident blocks per SM of the Jager collide at a block size (0 on failure)
 static int occupancy_jager(const void* k, int threads, size_t sm) {
   int per_sm = 0;
-  if (sm > kDefaultSmem &&
-      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
-    return 0;
+  if (!allow_smem(k, sm)) return 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, sm) != cudaSuccess) return 0;
   return per_sm;
 }
@@ -1172,7 +1251,8 @@ int launch_collide_jager(Ctx* c, const dsmc_gas_t& gas, const dsmc_potential_t& 
   JagerArgs a{gas.seed, step, graph_step_ptr(c), gas.b_max * 1e10, (const int4*)pairs, deps, ro, info, vx, vy, vz,
               chi_out, (unsigned*)ws, barrier_ptr(c), status_ptr(c)};
   if (int rc = launch_clear_stamps(c, a.done, n, a.bar, s)) return rc;
-  launch_dep(k, blocks, sh.threads, sm, s, P, a);
+  static const TurnTable turn_table = make_turn_table();
+  launch_dep(k, blocks, sh.threads, sm, s, P, turn_table, a);
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : record(c, DSMC_ERR_CUDA, "collide_jager: launch failed");
 }

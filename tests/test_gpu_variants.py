@@ -203,3 +203,33 @@ def test_sort_is_stable_for_every_run_length(n, runs, offset):
     keep = host(buf)
     keep = np.where((keep < 0) | (keep >= n_cells), n_cells, keep)
     assert np.array_equal(host(o["perm"])[:n - 2], np.argsort(keep, kind="stable")[:n - 2])
+
+
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_jager_rotation_along_an_axis(axis):
+    """Relative velocities along one axis: along x the rotation's frame is the degenerate one.  Velocities
+    within 1e-12 of max(|v|, c_ref) of the oracle's rotation by the kernel's own chi, as for the random gas."""
+    from gpu_util import c_ref
+    import test_gpu_parity as P
+    W = P.W
+    from paper_2602_21244_gb300 import dsmc as D
+    w = W.hypersonic(scale=0.04)
+    for c in range(3):
+        if c != axis:
+            w[("vx", "vy", "vz")[c]][:] = 0.0
+    gas = P.O.make_gas(**w["gas"])
+    sg0 = P._sgmax0(w, gas)
+    perm, cs, *x = P.oracle_sorted(w)
+    pr = P.O.select_pairs(gas, cs, *x, sg0, 4, capacity=1 << 22)
+    Dg, srt, mom, sg, sel = P.gpu_step_pieces(w, sg0, step=4)
+    C = ctx()
+    n = int(host(sel["info"])[0])
+    assert n == pr["n_pairs"] > 0
+    chi = torch().zeros(n, dtype=torch().float32, device="cuda")
+    C.collide_jager(Dg, D.make_potential(P.JP), 4, sel, srt["svx"], srt["svy"], srt["svz"], n_nodes=32, chi_out=chi)
+    assert C.sync_status() == 0
+    p = P.sel_host(sel)["pairs"]
+    order = np.lexsort((p[:, 3], p[:, 2]))
+    want = P.O.collide_given_chi(gas, pr, 4, host(chi)[order].astype(np.float64), *x)
+    for a, r in zip(("svx", "svy", "svz"), want):
+        assert (np.abs(host(srt[a]) - r) / np.maximum(np.abs(r), c_ref(W.M_AR))).max() <= 1e-12
