@@ -778,7 +778,11 @@ int launch_gather(Ctx* c, int32_t n, int32_t n_cells, const int32_t* cell_start,
 // Cell moments and moment matching without block-wide synchronisation: each
 // warp claims runs of kCwRun consecutive cells from a counter (so that the
 // warps given cheap runs, such as empty cells or the free stream, take more
-// of them) and collects kCwClaims runs before finishing their cells.
+// of them) and collects kCwClaims runs before finishing their cells.  A warp
+// claims only a few times, so short claims even out the end: four of 4 cells
+// instead of two of 8 took matching at 37,500 cells of 61 particles from 71 to 50
+// us, at 73,500 from 103 to 93, moments at 150,000 from 98 to 85 us (matching there
+// 172 both ways; two of 4: 57 us at 37,500, eight of 4: 182 us at 150,000).
 // Segments of 8 lanes take four cells at a time through the two passes of
 // the exact integer moments (the largest exponent, then the split sums of
 // moments.cuh); the per-cell remainder (means, centred sum of squares,
@@ -787,8 +791,8 @@ int launch_gather(Ctx* c, int32_t n, int32_t n_cells, const int32_t* cell_start,
 // particles one lane per particle, four at a time (three FP64 FMAs each,
 // every lane busy, coalesced reads and writes).
 constexpr int kCwWarps = 8;
-constexpr int kCwRun = 8;                    // cells per claim
-constexpr int kCwClaims = 2;                 // claims per batch
+constexpr int kCwRun = 4;                    // cells per claim (one per segment)
+constexpr int kCwClaims = 4;                 // claims per batch
 constexpr int kCwCells = kCwRun * kCwClaims; // cells per batch (one lane each in the remainder)
 
 struct CwWarp {
@@ -997,10 +1001,10 @@ k_cells_once(int32_t n_cells, const int32_t* __restrict__ cs, double* vx, double
 // memory and the batched remainder takes 18 us (moments) and 25 to 29 us
 // (matching) however few cells there are; one group per warp takes 9 and 9 to
 // 10 us (launch overhead included) at 100 to 2,867 cells, 22.7 against 26.2 us
-// (moments) at 40,000 cells of 20 particles and 40.5 against 46.4 us at 37,500 of 61, but from then on its FP64
+// (moments) at 40,000 cells of 20 particles (with claims of 4 cells 20.0 against 21.0), but from then on its FP64
 // remainder, paid per group of 4 cells instead of 16, costs more (matching
-// 18.5 against 25.2 us at 10,000 cells, 43.2 against 39.1 us at 40,000; at
-// 150,000 cells 113 against 100 us and 240 against 175 us).  32 lanes per
+// 18.5 against 25.2 us at 10,000 cells, 43.2 against 33.7 us at 40,000; at
+// 150,000 cells 113 against 85 us and 240 against 172 us).  32 lanes per
 // cell for up to 8 cells per SM (1,000 cells of 50: 9.5 against 12.3 us).
 static int launch_cells(Ctx* c, bool match, int32_t n_cells, const int32_t* cs, double* vx, double* vy,
                         double* vz, double* mom, cudaStream_t s) {
