@@ -580,6 +580,13 @@ static int collide_step(dsmc_ctx_t* c, const dsmc_gas_t* gas, const dsmc_path_t*
   int rc = 0;
   switch (path->path) {
     case DSMC_PATH_VHS:
+      if (dsmc::groups_suit(c, B->n_cells, false)) {
+        REQUIRE(c, B->round_offsets && B->info && B->svx && B->svy && B->svz && B->ws && B->n >= 0,
+                "collide_vhs: null pointer");
+        rc = dsmc::launch_groups_vhs(c, *gas, step, B->n_cells, B->pairs, B->round_offsets, B->info, B->svx, B->svy,
+                                     B->svz, S(stream));
+        break;
+      }
       rc = dsmc_collide_vhs(c, gas, step, B->n, B->pairs, B->deps, B->round_offsets, B->info, B->svx, B->svy,
                             B->svz, B->ws, B->ws_bytes, stream);
       break;
@@ -593,6 +600,14 @@ static int collide_step(dsmc_ctx_t* c, const dsmc_gas_t* gas, const dsmc_path_t*
                                nullptr, B->ws, B->ws_bytes, stream);
       break;
     case DSMC_PATH_TABLE:
+      if (dsmc::groups_suit(c, B->n_cells, true)) {
+        if ((rc = check_table(c, path->table))) return rc;
+        REQUIRE(c, B->round_offsets && B->info && B->svx && B->svy && B->svz && B->ws && B->n >= 0,
+                "collide_table: null pointer");
+        rc = dsmc::launch_groups_table(c, *gas, *path->table, step, B->n_cells, B->pairs, B->round_offsets, B->info,
+                                       B->svx, B->svy, B->svz, S(stream));
+        break;
+      }
       rc = dsmc_collide_table(c, gas, path->table, step, B->n, B->pairs, B->deps, B->round_offsets, B->info,
                               B->svx, B->svy, B->svz, nullptr, B->ws, B->ws_bytes, stream);
       break;

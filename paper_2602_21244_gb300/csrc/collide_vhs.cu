@@ -127,6 +127,164 @@ int launch_collide_vhs(Ctx* c, const dsmc_gas_t& gas, uint64_t step, int32_t n, 
   return cudaGetLastError() == cudaSuccess ? 0 : record(c, DSMC_ERR_CUDA, "collide_vhs: launch failed");
 }
 
+// ---------------------------------------------------------------- pair updates of the step
+// In a step the pair list is the selection's own: inside a round the pairs are
+// in cell order, and a cell's pairs touch that cell's particles only.  So a warp
+// can take a group of consecutive cells through all rounds by itself, 32 pairs at a
+// time, with a __syncwarp between rounds where the collide calls (which take
+// any list) wait on done stamps, release fences and a claim per 32 pairs.  Lane r
+// finds the group's pairs of round r by two binary searches on the cell index.
+// A group has about kGroupPairs pairs (fewer cells than that to a group leave a
+// round's lanes empty, and the FP64 pipe costs a warp instruction however few
+// lanes are active; more make the chain of one warp long), at most kGroupCells cells,
+// and there are a thousand groups if there are as many cells.  Step of 2,867 cells
+// and 47,580 pairs on the look-up path 152 -> 120 us.  Larger gases fill the
+// chip without this, and the groups' partly filled warps and searches cost more than
+// the waits they save: see groups_suit.
+struct GroupArgs {
+  uint64_t seed, step;
+  const uint64_t* step_dev;
+  const int4* pairs;
+  const int32_t* ro;
+  const dsmc_select_info_t* info;
+  double *vx, *vy, *vz;
+  unsigned* work;   // groups claimed, finished blocks (zero between launches)
+  int32_t n_cells;
+};
+
+struct VhsUpdate {
+  __device__ __forceinline__ void operator()(const GroupArgs& a, int4 q, double* v) const {
+    vhs_pair(a.seed, a.step, (uint32_t)q.w, (uint32_t)q.z, v);
+  }
+};
+struct TableUpdate {
+  TableLook look;
+  __device__ __forceinline__ void operator()(const GroupArgs& a, int4 q, double* v) const {
+    table_pair(look, a.seed, a.step, (uint32_t)q.w, (uint32_t)q.z, v);
+  }
+};
+
+constexpr int kGroupThreads = 128;
+constexpr int kGroupPairs = 128, kGroupCells = 8;
+
+template <class Update>
+__global__ void __launch_bounds__(kGroupThreads, 8) k_collide_groups(GroupArgs a, Update update) {
+  dep_wait();
+  if (a.step_dev) a.step = *a.step_dev;
+  const int R = a.info->n_rounds;
+  const int64_t pairs = a.info->n_pairs;
+  // cells per group
+  const int cells = (int)min((int64_t)(a.n_cells / 1024 + 1),
+                             max((int64_t)1, pairs > 0 ? min((int64_t)kGroupCells, kGroupPairs * (int64_t)a.n_cells / pairs)
+                                                       : (int64_t)kGroupCells));
+  const int lane = threadIdx.x & 31;
+  // every warp's first group is its own index; further ones, if there are more groups
+  // than warps, are claimed (dense cells lie together: 37,500 cells of the
+  // hypersonic gas 577 us, by stride 685; claims from one counter by warps that have
+  // only one group to take cost 20 us)
+  const unsigned warps = gridDim.x * (kGroupThreads / 32);
+  const bool claims = (int64_t)warps * cells < a.n_cells;
+  unsigned g = blockIdx.x * (kGroupThreads / 32) + (threadIdx.x >> 5);
+  for (int64_t first; (first = (int64_t)g * cells) < a.n_cells;) {
+    const int32_t k0 = (int32_t)first, k1 = (int32_t)min((int64_t)a.n_cells, first + cells);
+    for (int rb = 0; rb < R; rb += 32) {
+      // the pairs of cells [k0, k1) in round rb + lane: [lo, hi)
+      int32_t lo = 0, hi = 0;
+      if (rb + lane < R) {
+        int32_t l0 = a.ro[rb + lane], l1 = a.ro[rb + lane + 1], h0 = l0, h1 = l1;
+        while (l0 < l1 || h0 < h1) {
+          const int32_t ml = (l0 + l1) >> 1, mh = (h0 + h1) >> 1;
+          const int32_t zl = l0 < l1 ? a.pairs[ml].z : k0, zh = h0 < h1 ? a.pairs[mh].z : k1;
+          if (l0 < l1) { if (zl < k0) l0 = ml + 1; else l1 = ml; }
+          if (h0 < h1) { if (zh < k1) h0 = mh + 1; else h1 = mh; }
+        }
+        lo = l0; hi = h0;
+      }
+      __syncwarp();
+      const int nr = min(32, R - rb);
+      int r = -1;
+      int32_t p0 = 0, end = 0;
+      auto next = [&]() {
+        p0 += 32;
+        while (p0 >= end) {
+          if (++r >= nr) return false;
+          p0 = __shfl_sync(0xffffffffu, lo, r);
+          end = __shfl_sync(0xffffffffu, hi, r);
+        }
+        return true;
+      };
+      bool have = next();
+      int4 qn = make_int4(0, 0, 0, 0);
+      bool actn = have && p0 + lane < end;
+      if (actn) qn = a.pairs[p0 + lane];
+      while (have) {
+        const int4 q = qn;
+        const bool act = actn;
+        // the next pairs' records load while these update
+        have = next();
+        actn = have && p0 + lane < end;
+        if (actn) qn = a.pairs[p0 + lane];
+        double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+        if (act) {
+          v[0] = a.vx[q.x]; v[1] = a.vy[q.x]; v[2] = a.vz[q.x];
+          v[3] = a.vx[q.y]; v[4] = a.vy[q.y]; v[5] = a.vz[q.y];
+        }
+        update(a, q, v);
+        if (act) {
+          a.vx[q.x] = v[0]; a.vy[q.x] = v[1]; a.vz[q.x] = v[2];
+          a.vx[q.y] = v[3]; a.vy[q.y] = v[4]; a.vz[q.y] = v[5];
+        }
+        __syncwarp();   // the next round's loads see these stores
+      }
+    }
+    if (!claims) break;
+    if (lane == 0) g = warps + atomicAdd(a.work, 1u);
+    g = __shfl_sync(0xffffffffu, g, 0);
+  }
+  // the last block to finish leaves the counters zero for the next launch
+  if (claims) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      __threadfence();
+      if (atomicAdd(a.work + 1, 1u) == gridDim.x - 1) {
+        __threadfence();
+        a.work[0] = 0u;
+        a.work[1] = 0u;
+      }
+    }
+  }
+}
+
+template <class Update>
+static int launch_groups(Ctx* c, const Update& u, const dsmc_gas_t& gas, uint64_t step, int32_t n_cells,
+                         const int32_t* pairs, const int32_t* ro, const dsmc_select_info_t* info, double* vx,
+                         double* vy, double* vz, cudaStream_t s) {
+  GroupArgs a{gas.seed, step, graph_step_ptr(c), (const int4*)pairs, ro, info, vx, vy, vz, work_ptr(c), n_cells};
+  const int warps = kGroupThreads / 32;
+  const int64_t want = ((int64_t)n_cells + warps - 1) / warps, most = (int64_t)sm_count(c) * 8;
+  launch_dep(k_collide_groups<Update>, (unsigned)(want < most ? want : most), kGroupThreads, 0, s, a, u);
+  count_launches(c, 1);
+  return cudaGetLastError() == cudaSuccess ? 0 : record(c, DSMC_ERR_CUDA, "step: pair update launch failed");
+}
+
+// Up to how many cells a step takes its pairs in groups (step, by stamps against groups,
+// us): look-up path 138 / 107 at 1,600 cells of 20 particles, 268 / 226 at 25,600, 324 /
+// 298 at 40,000, 494 / 503 at 57,600; 638 / 569 at 37,500 cells of the hypersonic gas, 926
+// / 926 at 73,500.  VHS, with fewer pairs and no table: 91 / 83 at 1,600, 115 / 103 at
+// 6,400, 134 / 130 at 14,400; hypersonic 147 / 136 at 6,000, 227 / 236 at 18,375.
+bool groups_suit(Ctx* c, int32_t n_cells, bool table) { return n_cells <= (table ? 288 : 64) * sm_count(c); }
+
+int launch_groups_vhs(Ctx* c, const dsmc_gas_t& gas, uint64_t step, int32_t n_cells, const int32_t* pairs,
+                    const int32_t* ro, const dsmc_select_info_t* info, double* vx, double* vy, double* vz,
+                    cudaStream_t s) {
+  return launch_groups(c, VhsUpdate{}, gas, step, n_cells, pairs, ro, info, vx, vy, vz, s);
+}
+int launch_groups_table(Ctx* c, const dsmc_gas_t& gas, const dsmc_chi_table_t& tab, uint64_t step, int32_t n_cells,
+                      const int32_t* pairs, const int32_t* ro, const dsmc_select_info_t* info, double* vx, double* vy,
+                      double* vz, cudaStream_t s) {
+  return launch_groups(c, TableUpdate{table_look(gas, tab)}, gas, step, n_cells, pairs, ro, info, vx, vy, vz, s);
+}
+
 // Failure-detection self test: every block but block 0 enters the grid
 // barrier; block 0 never arrives, so the others' bounded waits run out and
 // record DSMC_ERR_TIMEOUT.  No trap, no unbounded spin.

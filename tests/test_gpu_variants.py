@@ -233,3 +233,50 @@ def test_jager_rotation_along_an_axis(axis):
     want = P.O.collide_given_chi(gas, pr, 4, host(chi)[order].astype(np.float64), *x)
     for a, r in zip(("svx", "svy", "svz"), want):
         assert (np.abs(host(srt[a]) - r) / np.maximum(np.abs(r), c_ref(W.M_AR))).max() <= 1e-12
+
+
+@pytest.mark.parametrize("path", ["vhs", "table"])
+@pytest.mark.parametrize("nx,ny,per,scale", [(1, 1, 300, 2000.0), (3, 1, 200, 5000.0), (33, 31, 20, 300.0),
+                                             (-64, 1, 20, 7000.0), (-64, 1, 4, 2000.0), (-64, 1, 4, 0.0)])
+def test_step_by_cell_groups_equals_the_collide_calls(path, nx, ny, per, scale):
+    """The step's pair update by groups of cells against the collide call that takes any pair list: more
+    rounds than a warp has lanes, one cell, more groups than warps, the last size that goes by groups
+    (VHS: 64 cells per SM, nx = -64), fewer pairs than cells and none at all.  The same functions on the same pairs in the
+    same order of each particle's pairs: the same bits."""
+    from paper_2602_21244_gb300 import dsmc as D
+    from paper_2602_21244_gb300 import workloads as W
+    T, C = torch(), ctx()
+    nx = nx if nx > 0 else -nx * _sms()
+    nc, rng = nx * ny, np.random.default_rng(nx + per)
+    counts = rng.poisson(per, nc)
+    cid = rng.permutation(np.repeat(np.arange(nc, dtype=np.int32), counts))
+    n = len(cid)
+    v = [cuda(c) for c in 400.0 * rng.standard_normal((3, n))]
+    gas = D.make_gas(dict(W.couette()["gas"], b_max=4.17e-10, fn_over_vc=max(scale, 1e-6) * 2e18, dt=1e-7,
+                          model=1 if path == "table" else 0))
+    cells = cuda(cid)
+    sg0 = C.sigma_g_max_init(gas, cuda(np.full(nc, 300.0)))
+    o = C.sort_cells(cells, *v, nc)
+    x = [o[k] for k in ("svx", "svy", "svz")]
+    mom = C.cell_moments(o["cell_start"], *x)
+    cap = 1 << 22
+    sel = C.select_pairs(gas, o["cell_start"], *x, sg0.clone(), 7, cap)
+    chi = cuda(np.linspace(0.1, 3.0, 64 * 64).astype(np.float32).reshape(64, 64))
+    tab = D.ChiTable(chi, 2.0, 12.0)
+    if path == "vhs":
+        C.collide_vhs(gas, 7, sel, *x)
+    else:
+        C.collide_table(gas, tab, 7, sel, *x)
+    C.moment_match(o["cell_start"], mom, *x)
+    info = host(sel["info"])
+    st = D.StepState(C, n, nc, cap)
+    for a, b in zip((st.vx, st.vy, st.vz), v):
+        a.copy_(b)
+    st.cell_id.copy_(cells)
+    st.sigma_g_max.copy_(sg0)
+    C.step(gas, D.make_path(D.PATH_VHS) if path == "vhs" else D.make_path(D.PATH_TABLE, table=tab), st, 7)
+    assert C.sync_status() == 0
+    assert np.array_equal(host(st.info), info)
+    assert (info[0] > 0) == (scale > 0) and (per < 200 or (info[2] & 0xFFFFFFFF) > 32)
+    for a, b in zip((st.svx, st.svy, st.svz), x):
+        assert np.array_equal(host(a), host(b))
