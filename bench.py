@@ -40,10 +40,10 @@ MLP_FLOP_PER_PAIR = 2 * (8 * 128 + 128 * 128 * 2 + 128 * 3)   # 68,352 (unpadded
 CHI_MLP_FLOP_PER_QUERY = 2 * (2 * 512 + 512 * 512 * 2 + 512 * 256 + 256 * 128 + 128)
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per pair of
 # k_collide_neural, from one ncu capture of a full-size launch on the
-# hypersonic gas: 1000.1 + 941.5 MB for about 6.885 million pairs
+# hypersonic gas: 894.4 + 855.5 MB for about 6.885 million pairs
 # (the committed ncu summary of this kernel); the roofline's traffic is this
 # times the pairs of the timed launch.
-NEURAL_DRAM_BYTES_PER_PAIR = (1000.14e6 + 941.49e6) / 6.885e6
+NEURAL_DRAM_BYTES_PER_PAIR = (894.41e6 + 855.47e6) / 6.885e6
 CANDIDATE_BYTES = 48                                             # two FP64 3-vectors read
 PAIR_BYTES = 104                                                 # 2x24 read + 2x24 write + 8 index
 # special-function operations per pair of the neural collide: 3 hidden layers
@@ -58,10 +58,10 @@ MLP_MUFU_PER_PAIR = 3 * 128 * 1.25
 # until captured for the current kernels.  FP64 and FP32 in FLOPs (an FMA is
 # two), MUFU in thread operations.
 KERNEL_OPS = {
-    "k_collide_vhs": {"fp64_flop": 99.2, "fp32_flop": 0.0, "mufu": 25.4},
-    "k_collide_table": {"fp64_flop": 37.0, "fp32_flop": 180.0, "mufu": 18.0},
-    "k_collide_jager": {"fp64_flop": 340.3, "fp32_flop": 7560.6, "mufu": 661.7},
-    "k_jager_chi": {"fp64_flop": 179.3, "fp32_flop": 9008.9, "mufu": 1915.1},
+    "k_collide_vhs": {"fp64_flop": 99.2, "fp32_flop": 0.0, "mufu": 21.4},
+    "k_collide_table": {"fp64_flop": 37.0, "fp32_flop": 180.0, "mufu": 17.8},
+    "k_collide_jager": {"fp64_flop": 301.7, "fp32_flop": 6402.6, "mufu": 534.1},
+    "k_jager_chi": {"fp64_flop": 180.0, "fp32_flop": 7971.9, "mufu": 652.8},
 }
 
 # the kernels of each phase of the step (for the per-phase rooflines)
@@ -73,14 +73,14 @@ KERNEL_OPS = {
 # phases' instruction-issue roof (only at that size).
 ISSUE_REF_PARTICLES = 9144283
 PHASE_WARP_INSTR = {
-    1: {"sort": 151.11e6, "moments": 60.94e6, "select": 249.49e6, "moment_match": 77.84e6},
-    0: {"sort": 151.12e6, "moments": 60.95e6, "select": 77.67e6, "moment_match": 77.84e6},
+    1: {"sort": 148.67e6, "moments": 61.47e6, "select": 256.82e6, "moment_match": 79.12e6},
+    0: {"sort": 148.67e6, "moments": 61.47e6, "select": 83.82e6, "moment_match": 79.12e6},
 }
 PHASE_KERNELS = {
     "sort": ["k_rs_count", "k_rs_rowscan", "k_rs_scatter", "k_cell_start", "k_gather1"],
     "moments": ["k_cells<false>"],
     "select": ["k_sel_nwords", "k_scan_*", "k_sel_count", "k_sel_emit", "k_sel_rcount", "k_sel_rscan",
-               "k_sel_scatter", "k_sel_finalize"],
+               "k_sel_scatter"],
     "moment_match": ["k_cells<true>"],
 }
 COLLIDE_KERNEL = {"vhs": "k_collide_vhs", "table": "k_collide_table", "jager": "k_collide_jager",

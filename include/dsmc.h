@@ -334,7 +334,8 @@ int dsmc_transport_viscosity(dsmc_ctx_t* ctx, const dsmc_gas_t* gas, const dsmc_
  *
  * dsmc_chi_mlp_pack writes the weights once into `packed` (device memory of
  * dsmc_chi_mlp_packed_size() bytes, 16-byte aligned) in the operand layout
- * the kernel streams.  dsmc_chi_mlp_forward: n rows x [2] (FP32, device) ->
+ * the kernel streams (a form of this library version: pack again after an
+ * update).  dsmc_chi_mlp_forward: n rows x [2] (FP32, device) ->
  * y (Softplus output) and/or chi (e^y - 1), either may be NULL.
  * dsmc_chi_mlp_table: the nE x nb table of Sec. 3.4.4 (row j: ln(E_r)* =
  * j/(nE-1); column i: b/b_max = i/(nb-1)), chi = e^y - 1, FP32 device memory. */
@@ -477,7 +478,10 @@ size_t dsmc_step_workspace_size(int32_t n, int32_t n_cells, int64_t capacity);
 /* One collision step: sort, pre moments, selection, pair updates of the
  * chosen path, moment matching (Sec. 2.1-2.6).  The pair list in `buf` is
  * bucketed by claim level (DSMC_ORDER_LEVELS) on DSMC_PATH_NEURAL and by
- * round on the other paths. */
+ * round on the other paths.  On DSMC_PATH_VHS and DSMC_PATH_TABLE a small gas
+ * (up to 64 or 288 cells per SM) is updated by groups of cells, with the
+ * results of the collide calls bit for bit; the shapes set for those calls
+ * (dsmc_tune_set) then have no part in it. */
 int dsmc_step(dsmc_ctx_t* ctx, const dsmc_gas_t* gas, const dsmc_path_t* path,
               const dsmc_step_buffers_t* buf, uint64_t step, void* stream);
 
@@ -624,11 +628,11 @@ int dsmc_neural_operator_forward(dsmc_ctx_t* ctx, const dsmc_mlp_t* mlp, const f
  * ([n x 3] FP64), writes dL/dtheta (FP32, theta layout) to grad.  The
  * moment-matching and projection backward are closed forms; the MLP
  * backward recomputes each layer's pre-activation from the saved input of
- * that layer from exactly the forward's operands (the low bf16 terms of
- * the hidden activations regenerated by running the first layers again), so
- * the recomputed pre-activations equal the forward's bit for bit, and no
- * activations are stored in HBM; dW accumulates per SM in TMEM and the
- * per-SM partials are summed in a fixed order. */
+ * that layer from exactly the forward's operands (the low bf16 terms of the
+ * first hidden activation are kept in tensor memory), so the recomputed
+ * pre-activations equal the forward's bit for bit, and no activations are
+ * stored in HBM; dW accumulates per SM in TMEM and the per-SM partials are
+ * summed in a fixed order. */
 int dsmc_neural_operator_backward(dsmc_ctx_t* ctx, const dsmc_mlp_t* mlp, const float* theta, uint64_t seed,
                                   uint64_t t, int64_t n, const double* vi, const double* vj, const double* T,
                                   const double* g_vi, const double* g_vj, float* grad, void* ws,
