@@ -29,7 +29,7 @@
 
 namespace dsmc {
 
-constexpr int kSelWarps = 8;
+constexpr int kSelWarps = 4;
 constexpr int kTotalsWords = 2 * DSMC_MAX_ROUNDS + 64;   // round counts, round count, candidate count (SelWs)
 
 // The NTC candidate count M of a cell, and its words of accept bits: ceil(M/32).
@@ -212,7 +212,7 @@ __device__ __forceinline__ void count_pair(const SelArgs& a, float4* stage, cons
 // Warp per pair of consecutive cells: both by half-warps when each draws at
 // most 16 candidates (and fits half the staging slice), else one after the
 // other by the whole warp.
-__global__ void __launch_bounds__(kSelWarps * 32, 4) k_sel_count(SelArgs a) {
+__global__ void __launch_bounds__(kSelWarps * 32, 8) k_sel_count(SelArgs a) {
   dep_wait();
   if (a.step_dev) a.step = *a.step_dev;
   __shared__ float4 stage[kSelWarps][kStage];
@@ -760,10 +760,11 @@ int launch_select(Ctx* c, const dsmc_gas_t& gas, int32_t n, int32_t n_cells, con
     count_launches(c, 1);
     if (int rc = launch_scan(c, w.wcnt, w.wofs, n_cells, w.scan, s)) return rc;
   }
-  // Many small blocks, so that the hardware evens out the cells' unequal numbers of candidates: selection
-  // of 6.9 million pairs in 150,000 cells 493 us with 8 blocks per SM, 469 with 64 (count), and 460 with
-  // blocks of 4 warps instead of 8 (emit: a block's warps wait for the slowest at its end)
-  const unsigned gb = blocks_for((n_cells + 1) / 2, kSelWarps, sms * 64);
+  // Many small blocks (of 4 warps: a block's warps wait for the slowest at its end), so that the hardware evens
+  // out the cells' unequal numbers of candidates: selection of 6.9 million pairs in 150,000 cells 493 us with 8
+  // blocks of 8 warps per SM for both passes, 460 with 64 (count) and 32 blocks of 4 (emit), 446 with 128 of 4
+  // (blocks of 2 and 1 warps: count 450 and 449, emit 468 and 514)
+  const unsigned gb = blocks_for((n_cells + 1) / 2, kSelWarps, sms * 128);
   launch_dep(k_sel_count, gb, kSelWarps * 32, 0, s, a);
   count_launches(c, 1);
   if (int rc = launch_scan(c, w.counts, w.offs, n_cells, w.scan, s)) return rc;
