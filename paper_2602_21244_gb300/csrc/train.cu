@@ -56,11 +56,19 @@ constexpr uint32_t S_MEAN = S_PRE + 5 * kT * 8;        // [8 x 4] FP64: mean vel
 constexpr uint32_t S_TOTAL = S_MEAN + (kT / kGroup) * 4 * 8;
 static_assert(S_PRE % 8 == 0 && S_TOTAL <= 227 * 1024, "shared memory");
 constexpr int kIssuer = 256;     // thread that issues the MMAs (of a warp without rows)
-// per-CTA partial: dW1 [128 x 32], dW2, dW3 [128 x 128], dW4^T [128 x 16], then the bias
-// gradients of each of the 4 TMEM lane groups [4 x 400], then the loss of each lane group
+// per-CTA partial: dW1 (128 x 32), dW2, dW3 (128 x 128), dW4^T (128 x 16), then the bias
+// gradients of each of the 4 TMEM lane groups [4 x 400], then the loss of each lane group.
+// The matrices lie as the threads hold them, four consecutive columns per thread and
+// the threads side by side (wpos), so that a warp's stores fill whole lines: row-major,
+// every store of a warp touched 32 lines, 16 bytes of each, and the flush of a
+// mini-batch's one tile took 17,000 of its 64,000 cycles, now 7,000 (2^14 pairs 51 us, now 48).
 constexpr int kPDB = kH * kXin + 2 * kH * kH + kH * 16;
 constexpr int kPLOSS = kPDB + 4 * 400;
 constexpr int kPartial = kPLOSS + 16;
+// position of (row, column) in a matrix of `rows` rows held 4 columns at a time; of
+// dW2 and dW3 with 32 columns per group of 128 threads
+__host__ __device__ constexpr int wpos(int row, int col, int rows) { return ((col >> 2) * rows + row) * 4 + (col & 3); }
+__host__ __device__ constexpr int wpos32(int row, int col) { return wpos((col >> 5) * kH + row, col & 31, 4 * kH); }
 constexpr int kNW = kH * 8 + 2 * kH * kH + 3 * kH;   // weights (d_in 8)
 constexpr int kNB = 3 * kH + 3;                      // biases
 constexpr uint32_t TM_DW2 = 128, TM_DW3 = 256, TM_DW1 = 384, TM_DW4 = 416, TM_OUT = 432, TM_H1LO = 448;
@@ -196,10 +204,18 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
     const float* bsrc = a.theta + kNW;
     for (int q = t; q < 3 * kH + 16; q += kNT) bias[q] = q < 3 * kH + 3 ? bsrc[q] : 0.f;
     __syncthreads();
+    // (every row of eight then starts at 16 bytes; word by word the prologue took 2 us more of 2^14 pairs' 53)
+    const bool wide = ((uintptr_t)a.theta & 15u) == 0;
     auto put8 = [&](uint32_t dst, const float* w8) {
       uint32_t r[4];
+      if (wide) {
+        const float4 x = ((const float4*)w8)[0], y = ((const float4*)w8)[1];
+        r[0] = tc::pack_bf16x2(x.x, x.y); r[1] = tc::pack_bf16x2(x.z, x.w);
+        r[2] = tc::pack_bf16x2(y.x, y.y); r[3] = tc::pack_bf16x2(y.z, y.w);
+      } else {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) r[q] = tc::pack_bf16x2(w8[2 * q], w8[2 * q + 1]);
+        for (int q = 0; q < 4; ++q) r[q] = tc::pack_bf16x2(w8[2 * q], w8[2 * q + 1]);
+      }
       tc::st_shared_v4(sb + dst, r[0], r[1], r[2], r[3]);
     };
     if (t < kH) {   // W1's eight columns, in columns 0..7 (hi) and 16..23 (lo) of its tile
@@ -652,30 +668,33 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
       for (int q = t; q < kPartial; q += kNT) P[q] = 0.f;
     } else {
       float v[32];
-      // k consecutive values of this thread (16 bytes at a time where the workspace allows it)
+      // k values of this thread, its 4 q-th to (4 q + 3)-th `stride` floats after the ones
+      // before (16 bytes at a time where the workspace allows it)
       const bool wide = ((uintptr_t)a.partial & 15u) == 0;
-      auto put = [&](float* dst, int k) {
-        if (wide) {
+      auto put = [&](float* dst, int k, int stride) {
 #pragma unroll
-          for (int q = 0; q < 32; q += 4)
-            if (q < k) *(float4*)(dst + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
-        } else {
+        for (int q = 0; q < 8; ++q) {
+          if (4 * q >= k) break;
+          float* d = dst + q * stride;
+          if (wide) {
+            *(float4*)d = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+          } else {
 #pragma unroll
-          for (int q = 0; q < 32; ++q)
-            if (q < k) dst[q] = v[q];
+            for (int e = 0; e < 4; ++e) d[e] = v[4 * q + e];
+          }
         }
       };
       // dW2, dW3: [128 out x 128 in]
       tc::ld32(lane_tm + TM_DW2 + (uint32_t)c0, v);
-      put(P + kH * kXin + row * kH + c0, 32);
+      put(P + kH * kXin + wpos32(row, c0), 32, 4 * kNT);
       tc::ld32(lane_tm + TM_DW3 + (uint32_t)c0, v);
-      put(P + kH * kXin + kH * kH + row * kH + c0, 32);
+      put(P + kH * kXin + kH * kH + wpos32(row, c0), 32, 4 * kNT);
       if (cg == 0) {
         tc::ld32(lane_tm + TM_DW1, v);  // [128 out x 32 (hi | lo)]
-        put(P + row * kXin, 32);
+        put(P + wpos(row, 0, kH), 32, 4 * kH);
       } else if (cg == 1) {
         tc::ld16(lane_tm + TM_DW4, v);  // [128 in x 16 out]
-        put(P + kH * kXin + 2 * kH * kH + row * 16, 16);
+        put(P + kH * kXin + 2 * kH * kH + wpos(row, 0, kH), 16, 4 * kH);
       }
       const int g = warp & 3;
 #pragma unroll
@@ -716,10 +735,10 @@ __device__ __forceinline__ float ordered_sum(float s, const float* __restrict__ 
 // warp for the loss; 16,384 threads with one load in flight each took 81 us
 // for 34,563 outputs of 128 CTAs.
 constexpr int kReduceThreads = 128;
-__global__ void __launch_bounds__(kReduceThreads) k_train_reduce(const float* __restrict__ partial, int nblk, int d_in,
+__global__ void __launch_bounds__(kReduceThreads) k_train_reduce(const float* __restrict__ partial, int nblk,
                                                                  float* __restrict__ grad, double* loss) {
   dep_wait();
-  const int nw = kH * d_in + 2 * kH * kH + 3 * kH;
+  const int nw = kNW;
   const int nb = kNB;
   if (blockIdx.x == 0) {   // the loss: lane l the values l, l + 32, ... of [CTA][lane group], then a tree
     if (threadIdx.x < 32) {
@@ -731,27 +750,36 @@ __global__ void __launch_bounds__(kReduceThreads) k_train_reduce(const float* __
     }
     return;
   }
+  // thread q: the q-th value of the partials (neighbouring threads read
+  // neighbouring words), out: where its sum goes in the weight layout
   const int q = (blockIdx.x - 1) * kReduceThreads + threadIdx.x;
   if (q >= nw + nb) return;
+  int out = q;
   float s = 0.f;
-  if (q < kH * d_in) {                       // W1[o][k] = hi column k + lo column 16 + k
-    const float* p = partial + (q / d_in) * kXin + q % d_in;
+  if (q < kH * 8) {                          // W1[o][k] = hi column k + lo column 16 + k
+    const int o = (q >> 2) & (kH - 1), k = (q >> 9) * 4 + (q & 3);
+    out = o * 8 + k;
+    const float* p = partial + wpos(o, k, kH);
+    constexpr int lo = wpos(0, 16, kH);
     for (int b = 0; b < nblk; b += 8) {
       float v[16];
 #pragma unroll
       for (int r = 0; r < 8; ++r) {
         v[2 * r] = b + r < nblk ? p[(size_t)(b + r) * kPartial] : 0.f;
-        v[2 * r + 1] = b + r < nblk ? p[(size_t)(b + r) * kPartial + 16] : 0.f;
+        v[2 * r + 1] = b + r < nblk ? p[(size_t)(b + r) * kPartial + lo] : 0.f;
       }
 #pragma unroll
       for (int r = 0; r < 8; ++r)
         if (b + r < nblk) s += v[2 * r] + v[2 * r + 1];
     }
-  } else if (q < kH * d_in + 2 * kH * kH) {  // W2, W3
-    s = ordered_sum(s, partial + kH * kXin + (q - kH * d_in), nblk, kPartial);
+  } else if (q < kH * 8 + 2 * kH * kH) {     // W2, W3
+    const int j = q - kH * 8, m = j / (kH * kH), w = j % (kH * kH);
+    const int t = (w >> 2) & (kNT - 1), o = t & (kH - 1), k = (t / kH) * 32 + (w / (4 * kNT)) * 4 + (w & 3);
+    out = kH * 8 + m * kH * kH + o * kH + k;
+    s = ordered_sum(s, partial + kH * kXin + j, nblk, kPartial);
   } else if (q < nw) {                       // W4[o][k] = dW4^T[k][o]
-    const int r = q - kH * d_in - 2 * kH * kH, o = r / kH, k = r % kH;
-    s = ordered_sum(s, partial + kH * kXin + 2 * kH * kH + k * 16 + o, nblk, kPartial);
+    const int r = q - kH * 8 - 2 * kH * kH, o = r / kH, k = r % kH;
+    s = ordered_sum(s, partial + kH * kXin + 2 * kH * kH + wpos(k, o, kH), nblk, kPartial);
   } else {                                   // biases: lane groups 0..3 of every CTA, in order
     const float* p = partial + kPDB + (q - nw);
     for (int b = 0; b < nblk; b += 4) {
@@ -763,7 +791,7 @@ __global__ void __launch_bounds__(kReduceThreads) k_train_reduce(const float* __
         if (b + r / 4 < nblk) s += v[r];
     }
   }
-  grad[q] = s;
+  grad[out] = s;
 }
 
 // Adam (Kingma & Ba 2015, Algorithm 1) on FP32 parameters theta = [weights, biases];
@@ -813,9 +841,9 @@ int launch_train(Ctx* c, const dsmc_mlp_t& mlp, int mode, uint64_t seed, uint64_
   launch_dep(k_train, blocks, kNT, S_TOTAL, s, a);
   count_launches(c, 1);
   if (mode != 0) {
-    const int outs = kH * mlp.d_in + 2 * kH * kH + 3 * kH + kNB;
+    const int outs = kNW + kNB;
     launch_dep(k_train_reduce, 1 + (outs + kReduceThreads - 1) / kReduceThreads, kReduceThreads, 0, s, 
-        (const float*)ws, blocks, mlp.d_in, grad, loss);
+        (const float*)ws, blocks, grad, loss);
     count_launches(c, 1);
   }
   return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
