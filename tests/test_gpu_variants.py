@@ -280,3 +280,32 @@ def test_step_by_cell_groups_equals_the_collide_calls(path, nx, ny, per, scale):
     assert (info[0] > 0) == (scale > 0) and (per < 200 or (info[2] & 0xFFFFFFFF) > 32)
     for a, b in zip((st.svx, st.svy, st.svz), x):
         assert np.array_equal(host(a), host(b))
+
+
+@pytest.mark.parametrize("n", [16, 128, 144, 4096])
+@pytest.mark.parametrize("act", [0, 1])
+def test_training_takes_parameters_and_workspace_at_any_word(n, act):
+    """Weights read 16 bytes or a word at a time, partial gradients written 16 bytes or a word at a time: the
+    same values, so loss and gradient agree bit for bit; part of a tile, one, more than one, many."""
+    from paper_2602_21244_gb300 import dsmc as D
+    from paper_2602_21244_gb300 import workloads as W
+    T, C, rng = torch(), ctx(), np.random.default_rng(n)
+    mlp = D.make_mlp(8, 128, 3, 3, act, W.sigma_v(), 273.0, 1e-12)
+    theta = (0.1 * rng.standard_normal(D_PARAMS)).astype(np.float32)
+    pairs = [cuda(400.0 * rng.standard_normal((n, 3))) for _ in range(4)]
+    temp = cuda(rng.uniform(200.0, 400.0, n))
+    nb = C.train_workspace("cuda").numel()
+    got = []
+    for off in (0, 1, 2):
+        th = T.zeros(D_PARAMS + off, device="cuda")[off:]
+        th.copy_(cuda(theta))
+        ws = T.zeros(nb + 4 * off, dtype=T.uint8, device="cuda")[4 * off:]
+        g, l = C.train_loss_grad(mlp, th, 5, 1, pairs[0], pairs[1], temp, pairs[2], pairs[3], ws=ws)
+        assert C.sync_status() == 0
+        got.append((host(g), host(l)))
+    assert np.isfinite(got[0][0]).all() and np.abs(got[0][0]).max() > 0
+    for g, l in got[1:]:
+        assert np.array_equal(g, got[0][0]) and np.array_equal(l, got[0][1])
+
+
+D_PARAMS = 34563   # weights and biases of the operator (d_in 8, width 128, 3 hidden layers, 3 outputs)
