@@ -547,19 +547,28 @@ int dsmc_adam_step(dsmc_ctx_t* c, int32_t n_params, int32_t n_weights, const flo
   CHECK_CTX(c);
   REQUIRE(c, n_params > 0 && n_weights >= 0 && n_weights <= n_params && step >= 1, "adam: bad sizes");
   REQUIRE(c, grad && theta && m && v, "adam: null pointer");
-  return dsmc::launch_adam(c, n_weights, n_params - n_weights, grad, theta, m, v, weights_bf16, biases, lr, beta1,
-                           beta2, eps, step, S(stream));
+  return dsmc::launch_adam(
+      c, n_params, grad, dsmc::AdamStep{theta, m, v, weights_bf16, biases, n_weights, lr, beta1, beta2, eps, step}, S(stream));
 }
 
 int dsmc_train_step(dsmc_ctx_t* c, const dsmc_mlp_t* mlp, float* theta, float* m, float* v, int64_t step,
                     float lr, uint64_t seed, int64_t n, const double* vi, const double* vj, const double* T,
                     const double* vi_target, const double* vj_target, float* grad, double* loss,
                     uint16_t* weights_bf16, float* biases, void* ws, size_t ws_bytes, void* stream) {
+  const int32_t np = mlp ? dsmc_mlp_param_count(mlp) : 0;
+  const int32_t nw = mlp ? np - (mlp->n_hidden * mlp->width + mlp->d_out) : 0;
+  // the reduction of the gradient applies Adam to each sum it has formed; arguments that Adam refuses go the
+  // long way round, to its own check
+  if (c && mlp && theta && m && v && grad && loss && ws && step >= 1 && n > 0 && vi && vj && T && vi_target && vj_target) {
+    CHECK_CTX(c);
+    if (int rc = check_train(c, mlp, n)) return rc;
+    const dsmc::AdamStep adam{theta, m, v, weights_bf16, biases, nw, lr, 0.9f, 0.999f, 1e-8f, step};
+    return dsmc::launch_train(c, *mlp, 2, seed, (uint64_t)step, n, theta, vi, vj, T, vi_target, vj_target, nullptr,
+                              nullptr, nullptr, nullptr, grad, loss, ws, ws_bytes, S(stream), nullptr, &adam);
+  }
   int rc = dsmc_train_loss_grad(c, mlp, theta, seed, (uint64_t)step, n, vi, vj, T, vi_target, vj_target, grad,
                                 loss, ws, ws_bytes, stream);
   if (rc) return rc;
-  const int32_t np = dsmc_mlp_param_count(mlp);
-  const int32_t nw = np - (mlp->n_hidden * mlp->width + mlp->d_out);
   return dsmc_adam_step(c, np, nw, grad, theta, m, v, step, lr, 0.9f, 0.999f, 1e-8f, weights_bf16, biases,
                         stream);
 }

@@ -462,13 +462,24 @@ int launch_selftest_deps(Ctx* c, uint64_t limit_ns, cudaStream_t s);
 int launch_selftest_mbar(Ctx* c, uint64_t limit_ns, cudaStream_t s);
 
 size_t train_ws(int sms);
+// One Adam step on the parameters `master` (the first n_w of them weights).
+struct AdamStep {
+  float *master, *m, *v;
+  uint16_t* w_bf16;
+  float* bias;
+  int n_w;
+  float lr;
+  double b1, b2;
+  float eps;
+  int64_t step;
+};
 int launch_train(Ctx* c, const dsmc_mlp_t& mlp, int mode, uint64_t seed, uint64_t t, int64_t n,
                  const float* theta, const double* vi, const double* vj, const double* T,
                  const double* ti, const double* tj, const double* gi, const double* gj, double* oi, double* oj,
-                 float* grad, double* loss, void* ws, size_t ws_bytes, cudaStream_t s, float* act = nullptr);
+                 float* grad, double* loss, void* ws, size_t ws_bytes, cudaStream_t s, float* act = nullptr,
+                 const AdamStep* adam = nullptr);   // adam: the update with the gradient just formed
 size_t train_act_bytes(int64_t n);
-int launch_adam(Ctx* c, int n_w, int n_b, const float* grad, float* master, float* m, float* v, uint16_t* w,
-                float* bias, float lr, double b1, double b2, double eps, int64_t step, cudaStream_t s);
+int launch_adam(Ctx* c, int n, const float* grad, const AdamStep& adam, cudaStream_t s);
 
 // the fused step (cell groups staged in shared memory), after the sort's keys
 size_t fused_ws(int32_t n);

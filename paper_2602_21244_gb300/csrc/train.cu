@@ -714,6 +714,29 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
   if (warp == 0) tc::tmem_dealloc(tm, 512);
 }
 
+// Adam (Kingma & Ba 2015, Algorithm 1) on FP32 parameters [weights, biases];
+// optionally writes the bf16 weights and FP32 biases the collide kernel takes.
+struct AdamArgs {
+  float *master, *m, *v;    // master null: no update
+  uint16_t* w_bf16;
+  float* bias;
+  int n_w;
+  float lr, b1, b2, eps, c1, c2;
+};
+__device__ __forceinline__ void adam_one(const AdamArgs& A, int q, float g) {
+  const float mq = A.b1 * A.m[q] + (1.f - A.b1) * g;
+  const float vq = A.b2 * A.v[q] + (1.f - A.b2) * g * g;
+  A.m[q] = mq;
+  A.v[q] = vq;
+  const float th = A.master[q] - A.lr * (mq * A.c1) / (sqrtf(vq * A.c2) + A.eps);
+  A.master[q] = th;
+  if (q < A.n_w) {
+    if (A.w_bf16) A.w_bf16[q] = to_bf16(th);
+  } else if (A.bias) {
+    A.bias[q - A.n_w] = th;
+  }
+}
+
 // s plus n values `stride` floats apart, added in order; sixteen loads are
 // in flight at a time (the sum is a chain of FP32 additions, the loads are not:
 // one at a time, the 152 partials cost as many round trips to L2).
@@ -736,7 +759,7 @@ __device__ __forceinline__ float ordered_sum(float s, const float* __restrict__ 
 // for 34,563 outputs of 128 CTAs.
 constexpr int kReduceThreads = 128;
 __global__ void __launch_bounds__(kReduceThreads) k_train_reduce(const float* __restrict__ partial, int nblk,
-                                                                 float* __restrict__ grad, double* loss) {
+                                                                 float* __restrict__ grad, double* loss, AdamArgs A) {
   dep_wait();
   const int nw = kNW;
   const int nb = kNB;
@@ -792,38 +815,31 @@ __global__ void __launch_bounds__(kReduceThreads) k_train_reduce(const float* __
     }
   }
   grad[out] = s;
+  if (A.master) adam_one(A, out, s);   // (a training step: a launch less than Adam by itself, 2^14 pairs 48 us, now 45)
 }
 
-// Adam (Kingma & Ba 2015, Algorithm 1) on FP32 parameters theta = [weights, biases];
-// optionally writes the bf16 weights and FP32 biases the collide kernel takes.
-__global__ void k_adam(int n_w, int n_b, const float* __restrict__ grad, float* __restrict__ master,
-                       float* __restrict__ m, float* __restrict__ v, uint16_t* __restrict__ w_bf16,
-                       float* __restrict__ bias, float lr, float b1, float b2, float eps, float c1, float c2) {
+__global__ void k_adam(int n, const float* __restrict__ grad, AdamArgs A) {
   dep_wait();
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n_w + n_b; q += gridDim.x * blockDim.x) {
-    const float g = grad[q];
-    const float mq = b1 * m[q] + (1.f - b1) * g;
-    const float vq = b2 * v[q] + (1.f - b2) * g * g;
-    m[q] = mq;
-    v[q] = vq;
-    const float th = master[q] - lr * (mq * c1) / (sqrtf(vq * c2) + eps);
-    master[q] = th;
-    if (q < n_w) {
-      if (w_bf16) w_bf16[q] = to_bf16(th);
-    } else if (bias) {
-      bias[q - n_w] = th;
-    }
-  }
+  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) adam_one(A, q, grad[q]);
 }
 
 size_t train_act_bytes(int64_t n) { return sizeof(float) * 3 * (size_t)kT * kH * (size_t)((n + kT - 1) / kT); }
 
 size_t train_ws(int sms) { return align256(sizeof(float) * (size_t)kPartial * (size_t)(sms > 0 ? sms : 1)); }
 
+static AdamArgs adam_args(const AdamStep& a) {
+  AdamArgs A;
+  A.master = a.master; A.m = a.m; A.v = a.v; A.w_bf16 = a.w_bf16; A.bias = a.bias; A.n_w = a.n_w;
+  A.lr = a.lr; A.b1 = (float)a.b1; A.b2 = (float)a.b2; A.eps = a.eps;
+  A.c1 = (float)(1.0 / (1.0 - pow(a.b1, (double)a.step)));
+  A.c2 = (float)(1.0 / (1.0 - pow(a.b2, (double)a.step)));
+  return A;
+}
+
 int launch_train(Ctx* c, const dsmc_mlp_t& mlp, int mode, uint64_t seed, uint64_t t, int64_t n,
                  const float* theta, const double* vi, const double* vj, const double* T,
                  const double* ti, const double* tj, const double* gi, const double* gj, double* oi, double* oj,
-                 float* grad, double* loss, void* ws, size_t ws_bytes, cudaStream_t s, float* act) {
+                 float* grad, double* loss, void* ws, size_t ws_bytes, cudaStream_t s, float* act, const AdamStep* adam) {
   const int sms = sm_count(c);
   if (mode != 0 && ws_bytes < train_ws(sms)) return record(c, DSMC_ERR_ARG, "train: workspace too small");
   if (cudaFuncSetAttribute((const void*)k_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S_TOTAL) !=
@@ -843,17 +859,14 @@ int launch_train(Ctx* c, const dsmc_mlp_t& mlp, int mode, uint64_t seed, uint64_
   if (mode != 0) {
     const int outs = kNW + kNB;
     launch_dep(k_train_reduce, 1 + (outs + kReduceThreads - 1) / kReduceThreads, kReduceThreads, 0, s, 
-        (const float*)ws, blocks, grad, loss);
+        (const float*)ws, blocks, grad, loss, adam ? adam_args(*adam) : AdamArgs{});
     count_launches(c, 1);
   }
   return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
 }
 
-int launch_adam(Ctx* c, int n_w, int n_b, const float* grad, float* master, float* m, float* v, uint16_t* w,
-                float* bias, float lr, double b1, double b2, double eps, int64_t step, cudaStream_t s) {
-  const float c1 = (float)(1.0 / (1.0 - pow(b1, (double)step)));
-  const float c2 = (float)(1.0 / (1.0 - pow(b2, (double)step)));
-  launch_dep(k_adam, 64, 256, 0, s, n_w, n_b, grad, master, m, v, w, bias, lr, (float)b1, (float)b2, (float)eps, c1, c2);
+int launch_adam(Ctx* c, int n, const float* grad, const AdamStep& adam, cudaStream_t s) {
+  launch_dep(k_adam, 64, 256, 0, s, n, grad, adam_args(adam));
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
 }

@@ -309,3 +309,38 @@ def test_training_takes_parameters_and_workspace_at_any_word(n, act):
 
 
 D_PARAMS = 34563   # weights and biases of the operator (d_in 8, width 128, 3 hidden layers, 3 outputs)
+
+
+@pytest.mark.parametrize("copies", [False, True])
+@pytest.mark.parametrize("n", [16, 144])
+def test_training_step_is_gradient_then_adam(n, copies):
+    """The step applies Adam where the gradient is summed: the same formulas on the same sums in FP32, whose
+    multiply-adds either kernel may contract: within four roundings (4 x 2^-24) of the larger term."""
+    from paper_2602_21244_gb300 import dsmc as D
+    from paper_2602_21244_gb300 import workloads as W
+    T, C, rng = torch(), ctx(), np.random.default_rng(n)
+    mlp = D.make_mlp(8, 128, 3, 3, 0, W.sigma_v(), 273.0, 1e-12)
+    pairs = [cuda(400.0 * rng.standard_normal((n, 3))) for _ in range(4)]
+    temp = cuda(rng.uniform(200.0, 400.0, n))
+    start = [cuda((s * np.abs(rng.standard_normal(D_PARAMS))).astype(np.float32)) for s in (0.1, 1e-3, 1e-6)]
+    weights, ws, res = D_PARAMS - 387, C.train_workspace("cuda"), []
+    for fused in (True, False):
+        th, m, v = (t.clone() for t in start)
+        wb = T.zeros(weights, dtype=T.int16, device="cuda") if copies else None
+        bias = T.zeros(387, device="cuda") if copies else None
+        grad, loss = T.zeros(D_PARAMS, device="cuda"), T.zeros(1, dtype=T.float64, device="cuda")
+        if fused:
+            C.train_step(mlp, th, m, v, 3, 1e-3, 9, pairs[0], pairs[1], temp, pairs[2], pairs[3], grad, loss, ws, wb, bias)
+        else:
+            grad, loss = C.train_loss_grad(mlp, th, 9, 3, pairs[0], pairs[1], temp, pairs[2], pairs[3], ws=ws)
+            C.adam_step(weights, grad, th, m, v, 3, w_bits=wb, bias=bias)
+        assert C.sync_status() == 0
+        res.append([host(t) for t in (grad, loss, th, m, v)])
+        if copies:
+            assert np.array_equal(host(bias), res[-1][2][weights:])
+            bits = host(wb).view(np.uint16).astype(np.uint32) << 16
+            assert np.abs(bits.view(np.float32) - res[-1][2][:weights]).max() <= np.abs(res[-1][2]).max() * 2.0 ** -8
+    (g0, l0, *a), (g1, l1, *b) = res
+    assert np.array_equal(g0, g1) and np.array_equal(l0, l1)
+    for x, y, s in zip(a, b, start):
+        assert np.abs(x - y).max() <= 4 * 2.0 ** -24 * max(np.abs(y).max(), float(s.abs().max()))
