@@ -60,9 +60,10 @@ __global__ void k_sel_nwords(SelArgs a, int32_t* round_off) {
 }
 
 // The same and the exclusive scan of the words in one block, for few cells:
-// one launch instead of two.
+// one launch instead of two (a step of 2,025 cells the same either way, of 2,867 cells
+// 114.6 us in one block and 111 in two launches, of 4,096 127 and 123).
 constexpr int kWordsThreads = 1024;
-constexpr int32_t kWordsOne = 4 * kWordsThreads;
+constexpr int32_t kWordsOne = 2 * kWordsThreads;
 __global__ void __launch_bounds__(kWordsThreads) k_sel_nwords_one(SelArgs a, int32_t* round_off, int32_t* wofs) {
   dep_wait();
   if (a.step_dev) a.step = *a.step_dev;

@@ -55,16 +55,27 @@ __device__ __forceinline__ double sigma_g(const SelArgs& a, double g) {
   return __dmul_rn(s, g);
 }
 
+// M = floor(N (N - 1) / 2 fn (sigma g)_max dt + U).  N (N - 1) / 2 and U are formed
+// on the integer pipe (both exact) and the floor is the conversion's: 6 FP64
+// instructions instead of 13, which bound the one-block selection start of a small gas
+// (2,867 cells on one SM).
 __device__ __forceinline__ int32_t ntc_count(const SelArgs& a, int32_t k, int32_t N, int* bad) {
   const u32x4 w = draw_k(a.key, 0, (uint32_t)k, a.step, TAG_NTC);
-  double mt = __dmul_rn(0.5, (double)N);
-  mt = __dmul_rn(mt, (double)(N - 1));
+  const uint64_t half = (uint64_t)((uint32_t)N) * (uint32_t)(N - 1) / 2;
+  double mt;
+  if (half < (1ull << 53)) {
+    // half 2^-53 as a uniform's double, times 2^53 through the exponent (half > 0: N >= 2)
+    const double x = u53_int((uint32_t)((half << 11) >> 32), (uint32_t)(half << 11));
+    mt = __hiloint2double(__double2hiint(x) + (53 << 20), __double2loint(x));
+  } else {
+    mt = __dmul_rn(__dmul_rn(0.5, (double)N), (double)(N - 1));
+  }
   mt = __dmul_rn(mt, a.fn);
   mt = __dmul_rn(mt, a.sgmax[k]);
   mt = __dmul_rn(mt, a.dt);
-  const double mf = floor(__dadd_rn(mt, u53(w.x, w.y)));
-  if (!(mf < 2147483647.0)) { *bad = 1; return 0; }
-  return (int32_t)mf;
+  const double m = __dadd_rn(mt, u53_int(w.x, w.y));
+  if (!(m < 2147483647.0)) { *bad = 1; return 0; }   // (as for its floor)
+  return __double2int_rd(m);
 }
 
 // A cell's FP64 velocities: particle i of the cell is vx[base + i] (any
