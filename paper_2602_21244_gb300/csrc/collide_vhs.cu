@@ -138,7 +138,9 @@ int launch_collide_vhs(Ctx* c, const dsmc_gas_t& gas, uint64_t step, int32_t n, 
 // round's lanes empty, and the FP64 pipe costs a warp instruction however few
 // lanes are active; more make the chain of one warp long), at most kGroupCells cells,
 // and there are a thousand groups if there are as many cells.  Step of 2,867 cells
-// and 47,580 pairs on the look-up path 152 -> 120 us.  Larger gases fill the
+// and 47,580 pairs on the look-up path 152 -> 120 us.  Blocks of one warp, so that few
+// groups spread evenly over the SMs' four sub-partitions, each with an FP64 pipe of its
+// own: 105 us where blocks of four took 110 (of two: 106).  Larger gases fill the
 // chip without this, and the groups' partly filled warps and searches cost more than
 // the waits they save: see groups_suit.
 struct GroupArgs {
@@ -164,11 +166,12 @@ struct TableUpdate {
   }
 };
 
-constexpr int kGroupThreads = 128;
+constexpr int kGroupThreads = 32;   // a warp: see above
+constexpr int kGroupBlocks = 32;    // per SM
 constexpr int kGroupPairs = 128, kGroupCells = 8;
 
 template <class Update>
-__global__ void __launch_bounds__(kGroupThreads, 8) k_collide_groups(GroupArgs a, Update update) {
+__global__ void __launch_bounds__(kGroupThreads, kGroupBlocks) k_collide_groups(GroupArgs a, Update update) {
   dep_wait();
   if (a.step_dev) a.step = *a.step_dev;
   const int R = a.info->n_rounds;
@@ -261,7 +264,7 @@ static int launch_groups(Ctx* c, const Update& u, const dsmc_gas_t& gas, uint64_
                          double* vy, double* vz, cudaStream_t s) {
   GroupArgs a{gas.seed, step, graph_step_ptr(c), (const int4*)pairs, ro, info, vx, vy, vz, work_ptr(c), n_cells};
   const int warps = kGroupThreads / 32;
-  const int64_t want = ((int64_t)n_cells + warps - 1) / warps, most = (int64_t)sm_count(c) * 8;
+  const int64_t want = ((int64_t)n_cells + warps - 1) / warps, most = (int64_t)sm_count(c) * kGroupBlocks;
   launch_dep(k_collide_groups<Update>, (unsigned)(want < most ? want : most), kGroupThreads, 0, s, a, u);
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : record(c, DSMC_ERR_CUDA, "step: pair update launch failed");
