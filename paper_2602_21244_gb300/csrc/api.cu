@@ -206,12 +206,23 @@ int dsmc_sort_cells(dsmc_ctx_t* c, int32_t n, int32_t n_cells, const int32_t* ce
                            ws, ws_bytes, S(stream));
 }
 
+// (n: the number of particles if known, or 0)
+static int cell_moments(Ctx* c, int32_t n_cells, const int32_t* cell_start, const double* vx, const double* vy,
+                        const double* vz, double* mom, void* stream, int64_t n) {
+  REQUIRE(c, n_cells >= 0 && cell_start && mom, "moments: bad arguments");
+  return dsmc::launch_moments(c, n_cells, cell_start, vx, vy, vz, mom, S(stream), n);
+}
+static int moment_match(Ctx* c, int32_t n_cells, const int32_t* cell_start, const double* mom_pre, double* vx,
+                        double* vy, double* vz, void* stream, int64_t n) {
+  REQUIRE(c, n_cells >= 0 && cell_start && mom_pre, "moment_match: bad arguments");
+  return dsmc::launch_moment_match(c, n_cells, cell_start, mom_pre, vx, vy, vz, S(stream), n);
+}
+
 int dsmc_cell_moments(dsmc_ctx_t* c, int32_t n_cells, const int32_t* cell_start,
                       const double* vx, const double* vy, const double* vz, double* mom,
                       void* stream) {
   CHECK_CTX(c);
-  REQUIRE(c, n_cells >= 0 && cell_start && mom, "moments: bad arguments");
-  return dsmc::launch_moments(c, n_cells, cell_start, vx, vy, vz, mom, S(stream));
+  return cell_moments(c, n_cells, cell_start, vx, vy, vz, mom, stream, 0);
 }
 
 int dsmc_sigma_g_max_init(dsmc_ctx_t* c, const dsmc_gas_t* gas, int32_t n_cells,
@@ -461,8 +472,7 @@ int dsmc_selftest_peak(dsmc_ctx_t* c, int32_t which, int32_t blocks, int32_t thr
 int dsmc_moment_match(dsmc_ctx_t* c, int32_t n_cells, const int32_t* cell_start,
                       const double* mom_pre, double* vx, double* vy, double* vz, void* stream) {
   CHECK_CTX(c);
-  REQUIRE(c, n_cells >= 0 && cell_start && mom_pre, "moment_match: bad arguments");
-  return dsmc::launch_moment_match(c, n_cells, cell_start, mom_pre, vx, vy, vz, S(stream));
+  return moment_match(c, n_cells, cell_start, mom_pre, vx, vy, vz, stream, 0);
 }
 
 int dsmc_harvest_jager(dsmc_ctx_t* c, const dsmc_gas_t* gas, const dsmc_potential_t* pot,
@@ -661,7 +671,7 @@ static int step_after_sort(dsmc_ctx_t* c, const dsmc_gas_t* gas, const dsmc_path
   cudaStream_t s = S(stream);
   if (cudaEventRecord(c->f_ev[0], s) != cudaSuccess || cudaStreamWaitEvent(c->f_side, c->f_ev[0], 0) != cudaSuccess)
     return dsmc::record(c, DSMC_ERR_CUDA, "step: fork of the moments stream failed");
-  int rc = dsmc_cell_moments(c, B->n_cells, B->cell_start, B->svx, B->svy, B->svz, B->mom, c->f_side);
+  int rc = cell_moments(c, B->n_cells, B->cell_start, B->svx, B->svy, B->svz, B->mom, c->f_side, B->n);
   // the side stream joins the caller's stream whatever happens next
   const bool joined_ev = cudaEventRecord(c->f_ev[1], c->f_side) == cudaSuccess;
   if (!rc)
@@ -672,7 +682,7 @@ static int step_after_sort(dsmc_ctx_t* c, const dsmc_gas_t* gas, const dsmc_path
   if (rc) return rc;
   if (!joined) return dsmc::record(c, DSMC_ERR_CUDA, "step: join of the moments stream failed");
   if ((rc = collide_step(c, gas, path, B, step, stream))) return rc;
-  return dsmc_moment_match(c, B->n_cells, B->cell_start, B->mom, B->svx, B->svy, B->svz, stream);
+  return moment_match(c, B->n_cells, B->cell_start, B->mom, B->svx, B->svy, B->svz, stream, B->n);
 }
 
 int dsmc_step_fused(dsmc_ctx_t* c, const dsmc_gas_t* gas, const dsmc_path_t* path,
@@ -947,7 +957,7 @@ int dsmc_autotune_step(dsmc_ctx_t* c, const dsmc_gas_t* gas, const dsmc_path_t* 
                                B->svy, B->svz, s);
   }, trials, cap, &nt);
   if (!rc) rc = tune_kernel(c, DSMC_TUNE_MOMENTS, reps, s, [&] {
-    return dsmc::launch_moments(c, B->n_cells, B->cell_start, B->svx, B->svy, B->svz, B->mom, s);
+    return dsmc::launch_moments(c, B->n_cells, B->cell_start, B->svx, B->svy, B->svz, B->mom, s, B->n);
   }, trials, cap, &nt);
   if (!rc && path->path == DSMC_PATH_VHS)
     rc = tune_kernel(c, DSMC_TUNE_COLLIDE_VHS, reps, s, [&] {
@@ -965,7 +975,7 @@ int dsmc_autotune_step(dsmc_ctx_t* c, const dsmc_gas_t* gas, const dsmc_path_t* 
                                 B->info, B->svx, B->svy, B->svz, nullptr, B->ws, B->ws_bytes, stream);
     }, trials, cap, &nt);
   if (!rc) rc = tune_kernel(c, DSMC_TUNE_MOMENT_MATCH, reps, s, [&] {
-    return dsmc::launch_moment_match(c, B->n_cells, B->cell_start, B->mom, B->svx, B->svy, B->svz, s);
+    return dsmc::launch_moment_match(c, B->n_cells, B->cell_start, B->mom, B->svx, B->svy, B->svz, s, B->n);
   }, trials, cap, &nt);
   *n_trials = nt;
   return rc;

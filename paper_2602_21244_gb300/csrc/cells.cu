@@ -976,14 +976,17 @@ k_cells(int32_t n_cells, const int32_t* __restrict__ cs, double* vx, double* vy,
 // particles held in registers from the one read that serves the exponent, the
 // sums and the update.
 constexpr int kOnceHold = 4;
+// warps per block: few, so that few groups spread over all SMs (matching at 6,000 cells
+// of 61 particles 34.8 us with eight, 29.9 with two)
+constexpr int kOnceWarps = 2;
 
 template <bool MATCH, int SEG>
-__global__ void __launch_bounds__(kCwWarps * 32)
+__global__ void __launch_bounds__(kOnceWarps * 32)
 k_cells_once(int32_t n_cells, const int32_t* __restrict__ cs, double* vx, double* vy, double* vz, double* mom,
              int* status) {
   dep_wait();
   const int lane = threadIdx.x & 31, sl = lane & (SEG - 1);
-  const int64_t k = ((int64_t)blockIdx.x * kCwWarps + (threadIdx.x >> 5)) * (32 / SEG) + lane / SEG;
+  const int64_t k = ((int64_t)blockIdx.x * kOnceWarps + (threadIdx.x >> 5)) * (32 / SEG) + lane / SEG;
   const bool act = k < n_cells;
   const int32_t a = act ? cs[k] : 0, b = act ? cs[k + 1] : 0, n = b - a;
   double* mk = mom + 5 * (act ? k : 0);
@@ -1041,21 +1044,26 @@ k_cells_once(int32_t n_cells, const int32_t* __restrict__ cs, double* vx, double
 // (moments) at 40,000 cells of 20 particles (with claims of 4 cells 20.0 against 21.0), but from then on its FP64
 // remainder, paid per group of 4 cells instead of 16, costs more (matching
 // 18.5 against 25.2 us at 10,000 cells, 43.2 against 33.7 us at 40,000; at
-// 150,000 cells 113 against 85 us and 240 against 172 us).  32 lanes per
+// 150,000 cells 113 against 85 us and 240 against 172 us).  And it costs more with many
+// particles per cell, 8 lanes each: where their number n is known (in a step), up to
+// 2,500 per SM for matching (6,000 cells of 61: 30 against 32 us, 18,375: 71 against 39;
+// 14,400 of 20: 16 against 22) and 10,000 for the moments (18,375 of 61: 26 against 28 us,
+// 37,500: 38 against 34).  32 lanes per
 // cell for up to 8 cells per SM (1,000 cells of 50: 9.5 against 12.3 us).
 static int launch_cells(Ctx* c, bool match, int32_t n_cells, const int32_t* cs, double* vx, double* vy,
-                        double* vz, double* mom, cudaStream_t s) {
+                        double* vz, double* mom, cudaStream_t s, int64_t n) {
   if (n_cells <= 0) return 0;
-  if (n_cells <= (match ? 128 : 320) * sm_count(c)) {
-    const int seg = n_cells <= 8 * sm_count(c) ? 32 : 8;
-    const unsigned gb = grid_for(n_cells, kCwWarps * 32 / seg, INT_MAX);
+  const int64_t sms = sm_count(c);
+  if (n_cells <= (match ? 128 : 320) * sms && n <= (match ? 2500 : 10000) * sms) {
+    const int seg = n_cells <= 8 * sms ? 32 : 8;
+    const unsigned gb = grid_for(n_cells, kOnceWarps * 32 / seg, INT_MAX);
     int* st = status_ptr(c);
     if (match) {
-      if (seg == 32) launch_dep(k_cells_once<true, 32>, gb, kCwWarps * 32, 0, s, n_cells, cs, vx, vy, vz, mom, st);
-      else launch_dep(k_cells_once<true, 8>, gb, kCwWarps * 32, 0, s, n_cells, cs, vx, vy, vz, mom, st);
+      if (seg == 32) launch_dep(k_cells_once<true, 32>, gb, kOnceWarps * 32, 0, s, n_cells, cs, vx, vy, vz, mom, st);
+      else launch_dep(k_cells_once<true, 8>, gb, kOnceWarps * 32, 0, s, n_cells, cs, vx, vy, vz, mom, st);
     } else {
-      if (seg == 32) launch_dep(k_cells_once<false, 32>, gb, kCwWarps * 32, 0, s, n_cells, cs, vx, vy, vz, mom, st);
-      else launch_dep(k_cells_once<false, 8>, gb, kCwWarps * 32, 0, s, n_cells, cs, vx, vy, vz, mom, st);
+      if (seg == 32) launch_dep(k_cells_once<false, 32>, gb, kOnceWarps * 32, 0, s, n_cells, cs, vx, vy, vz, mom, st);
+      else launch_dep(k_cells_once<false, 8>, gb, kOnceWarps * 32, 0, s, n_cells, cs, vx, vy, vz, mom, st);
     }
     count_launches(c, 1);
     return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
@@ -1072,8 +1080,8 @@ static int launch_cells(Ctx* c, bool match, int32_t n_cells, const int32_t* cs, 
 }
 
 int launch_moments(Ctx* c, int32_t n_cells, const int32_t* cs, const double* vx, const double* vy,
-                   const double* vz, double* mom, cudaStream_t s) {
-  return launch_cells(c, false, n_cells, cs, (double*)vx, (double*)vy, (double*)vz, mom, s);
+                   const double* vz, double* mom, cudaStream_t s, int64_t n) {
+  return launch_cells(c, false, n_cells, cs, (double*)vx, (double*)vy, (double*)vz, mom, s, n);
 }
 
 // ---------------------------------------------------------------- moment matching
@@ -1081,8 +1089,8 @@ int launch_moments(Ctx* c, int32_t n_cells, const int32_t* cs, const double* vx,
 // applied as v <- alpha v + (u_pre - alpha u_post) (FP64); u_post and Th_post
 // from the exact integer moments above (k_cells<true>).
 int launch_moment_match(Ctx* c, int32_t n_cells, const int32_t* cs, const double* mom,
-                        double* vx, double* vy, double* vz, cudaStream_t s) {
-  return launch_cells(c, true, n_cells, cs, vx, vy, vz, (double*)mom, s);
+                        double* vx, double* vy, double* vz, cudaStream_t s, int64_t n) {
+  return launch_cells(c, true, n_cells, cs, vx, vy, vz, (double*)mom, s, n);
 }
 
 }  // namespace dsmc
