@@ -845,6 +845,7 @@ static PotDev make_pot(const dsmc_gas_t& gas, const dsmc_potential_t& p, int n_n
 template <int KIND>
 __global__ void __launch_bounds__(128, 5) k_jager_chi(PotDev P, int64_t n, const float* __restrict__ b,
                                                       const float* __restrict__ g, float* __restrict__ chi) {
+  dep_wait_alone();
   extern __shared__ float4 chi_sm[];
   const ChiShared S = chi_shared(P, (float*)chi_sm);
   const int lane = threadIdx.x & 31;

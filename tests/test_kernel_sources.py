@@ -1,0 +1,43 @@
+"""Rules that hold for every kernel of the library, read from its source: a violation may show as wrong results
+only now and then on a GPU, so they are checked where they stand."""
+import glob
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2602_21244_gb300", "csrc")
+
+
+def _source(path):
+    """Text without comments."""
+    with open(path) as f:
+        text = f.read()
+    return re.sub(r"//[^\n]*", "", re.sub(r"/\*.*?\*/", "", text, flags=re.S))
+
+
+SOURCES = {os.path.basename(p): _source(p) for p in sorted(glob.glob(os.path.join(CSRC, "*.cu")))}
+
+
+def _dependent_kernels():
+    """(file, kernel) of every kernel that a launch_dep call names, directly or through a variable."""
+    found = set()
+    for name, text in SOURCES.items():
+        for call in re.finditer(r"\blaunch_dep\(\s*(\w+)", text):
+            arg = call.group(1)
+            kernels = {arg} if arg.startswith("k_") else set()
+            if not kernels:   # a variable: the kernels in its last assignment before the call
+                values = re.findall(r"\b%s\s*=([^;]*);" % arg, text[:call.start()])
+                kernels = set(re.findall(r"\bk_\w+", values[-1])) if values else set()
+            assert kernels, f"{name}: launch_dep({arg}): kernel not found"
+            found |= {(name, k) for k in kernels}
+    return sorted(found)
+
+
+@pytest.mark.parametrize("where,kernel", _dependent_kernels())
+def test_kernel_placed_early_waits_for_the_one_before(where, kernel):
+    """A kernel launched by launch_dep may be placed while the kernel before it runs: it has to wait for that
+    one's end, and so for all before it, ahead of everything else."""
+    m = re.search(r"__global__[^;{}]*\b%s\s*\([^{;]*\)\s*\{\s*([^;]*;)" % kernel, SOURCES[where])
+    assert m, "definition not found"
+    assert re.fullmatch(r"dep_wait(_alone)?\(\);", m.group(1)), m.group(1)
