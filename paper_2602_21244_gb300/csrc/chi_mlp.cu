@@ -218,11 +218,10 @@ __global__ void __launch_bounds__(kThr, 1) k_chi_mlp(ChiArgs a) {
         if (++at == kPerTile) at = 0;
         if (++b == kNbuf) { b = 0; ph ^= 1u; }
       }
-      // after a failure: let the copies in flight land (bounded) before the
-      // shared memory is released
-      if (m < total)
-        for (int q = m > kNbuf ? m - kNbuf : 0; q < m; ++q)
-          tc::mbar_wait(full + q % kNbuf, (uint32_t)(q / kNbuf) & 1u, a.status, kBarrierLimitNs);
+      // the copies in flight land (bounded) before the shared memory is released,
+      // those of the last chunks too: another role may fail after they are issued
+      for (int q = m > kNbuf ? m - kNbuf : 0; q < m; ++q)
+        tc::mbar_wait(full + q % kNbuf, (uint32_t)(q / kNbuf) & 1u, a.status, kBarrierLimitNs);
     }
     __syncwarp();
   } else if (w == kMmaWarp) {

@@ -41,3 +41,24 @@ def test_kernel_placed_early_waits_for_the_one_before(where, kernel):
     m = re.search(r"__global__[^;{}]*\b%s\s*\([^{;]*\)\s*\{\s*([^;]*;)" % kernel, SOURCES[where])
     assert m, "definition not found"
     assert re.fullmatch(r"dep_wait(_alone)?\(\);", m.group(1)), m.group(1)
+
+
+def _body(text, start):
+    """The braced block that opens first after `start`, and what follows it up to the next __syncwarp()."""
+    at = text.index("{", start)
+    depth, end = 0, at
+    while True:
+        depth += {"{": 1, "}": -1}.get(text[end], 0)
+        end += 1
+        if depth == 0:
+            break
+    return text[at:end], text[end:text.index("__syncwarp();", end)]
+
+
+def test_chi_mlp_copy_lane_leaves_no_copy_in_flight():
+    """However its loop ends (all chunks issued, or another role's failure), the lane that issues the weight
+    copies waits for the last one into each buffer before the CTA can release its shared memory."""
+    text = SOURCES["chi_mlp.cu"]
+    body, rest = _body(text, text.index("for (; m < total; ++m)"))
+    assert "bulk_g2s" in body
+    assert re.match(r"\s*for \(int q = m > kNbuf \? m - kNbuf : 0; q < m; \+\+q\)\s*tc::mbar_wait\(full \+ q % kNbuf", rest), rest
