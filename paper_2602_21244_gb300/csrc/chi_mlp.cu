@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(kThr, 1) k_chi_mlp(ChiArgs a) {
   uint64_t* alast = aearly + 1;                   // all of them
   uint64_t* xfull = alast + 1;                    // the tile's input rows are in shared memory
   uint64_t* yfull = xfull + 1;                    // the column groups' partial outputs are
-  uint64_t* drain = yfull + 1;                    // after a failure: the MMAs in flight are done
+  uint64_t* drain = yfull + 1;                    // at the end: the MMAs in flight are done
   volatile int* fail = (volatile int*)(smem + kFlagOff);
   const uint32_t sbase = tc::smem_u32(smem);
   float* bias = (float*)(smem + kBiasOff);
@@ -278,11 +278,10 @@ __global__ void __launch_bounds__(kThr, 1) k_chi_mlp(ChiArgs a) {
           }
         }
       }
-      // after a failure: MMAs in flight end (bounded) before TMEM and shared memory are released
-      if (!ok) {
-        tc::commit(drain);
-        tc::mbar_wait(drain, 0, a.status, kBarrierLimitNs);
-      }
+      // MMAs in flight end (bounded) before TMEM and shared memory are released,
+      // those of the last pass too: its epilogue may fail after they are issued
+      tc::commit(drain);
+      tc::mbar_wait(drain, 0, a.status, kBarrierLimitNs);
     }
     __syncwarp();
   } else {

@@ -62,3 +62,12 @@ def test_chi_mlp_copy_lane_leaves_no_copy_in_flight():
     body, rest = _body(text, text.index("for (; m < total; ++m)"))
     assert "bulk_g2s" in body
     assert re.match(r"\s*for \(int q = m > kNbuf \? m - kNbuf : 0; q < m; \+\+q\)\s*tc::mbar_wait\(full \+ q % kNbuf", rest), rest
+
+
+def test_chi_mlp_issuing_lane_leaves_no_mma_in_flight():
+    """The lane that issues the MMAs waits for all of them before the CTA can release its tensor memory, also
+    when it has issued its last one and the epilogue of that pass fails."""
+    text = SOURCES["chi_mlp.cu"]
+    body, rest = _body(text, text.index("for (int it = 0; it < my_its && ok; ++it)"))
+    assert "mma_bf16_ta" in body
+    assert re.match(r"\s*tc::commit\(drain\);\s*tc::mbar_wait\(drain, 0,", rest), rest
