@@ -50,7 +50,7 @@ constexpr uint32_t S_DZ4 = S_WKLO + kT * kH * 2;       // [128 x 16] dz of the o
 constexpr uint32_t S_DZ4F = S_DZ4 + kT * 16 * 2;       // [128 x 3] FP32
 constexpr uint32_t S_BIAS = S_DZ4F + kT * 4 * 4;       // 3*128 + 16 floats
 constexpr uint32_t S_WO32 = S_BIAS + (3 * kH + 16) * 4;  // output weights in FP32 [3 x 128]
-constexpr uint32_t S_MISC = S_WO32 + 3 * kH * 4;       // mbarrier, tmem ptr, flag
+constexpr uint32_t S_MISC = S_WO32 + 3 * kH * 4;       // mbarrier, tmem ptr, flag, drain mbarrier
 constexpr uint32_t S_PRE = S_MISC + 64;                // [5 x 128] FP64: d, |v_r|, Theta_pre term of each row
 constexpr uint32_t S_MEAN = S_PRE + 5 * kT * 8;        // [8 x 4] FP64: mean velocity of each group
 constexpr uint32_t S_TOTAL = S_MEAN + (kT / kGroup) * 4 * 8;
@@ -188,6 +188,7 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
   uint64_t* mbar = (uint64_t*)(sm + S_MISC);
   uint32_t* tptr = (uint32_t*)(sm + S_MISC + 8);
   volatile int* flag = (volatile int*)(sm + S_MISC + 12);
+  uint64_t* drain = (uint64_t*)(sm + S_MISC + 16);   // after a wait that ran out: the MMAs in flight are done
   float* bias = (float*)(sm + S_BIAS);
   const float* wo32 = (const float*)(sm + S_WO32);
   // bias gradients and loss accumulate in registers of fixed threads (no atomics,
@@ -238,7 +239,7 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
     }
   }
   if (warp == 0) { tc::tmem_alloc(tptr, 512); tc::tmem_relinquish(); }
-  if (t == 0) { tc::mbar_init(mbar, 1); tc::mbar_fence_init(); *flag = 1; }
+  if (t == 0) { tc::mbar_init(mbar, 1); tc::mbar_init(drain, 1); tc::mbar_fence_init(); *flag = 1; }
   tc::fence_async_smem();
   tc::fence_before();
   __syncthreads();
@@ -657,6 +658,12 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
     ++tiles_done;
   }
   if (busy && alive) wait_mma();
+  // the tiles' loop was left early: MMAs that not every thread has waited for (a
+  // layer's dW runs on beside the next one) end (bounded) before TMEM is released
+  if (!alive && t == kIssuer) {
+    tc::commit(drain);
+    tc::mbar_wait(drain, 0, a.status, kBarrierLimitNs);
+  }
   tc::fence_before();
   __syncthreads();
   tc::fence_after();

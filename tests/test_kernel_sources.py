@@ -71,3 +71,14 @@ def test_chi_mlp_issuing_lane_leaves_no_mma_in_flight():
     body, rest = _body(text, text.index("for (int it = 0; it < my_its && ok; ++it)"))
     assert "mma_bf16_ta" in body
     assert re.match(r"\s*tc::commit\(drain\);\s*tc::mbar_wait\(drain, 0,", rest), rest
+
+
+def test_training_leaves_no_mma_in_flight():
+    """When a wait of the training kernel runs out, the MMAs that are committed but not waited for by every thread
+    end before the tensor memory is released: the issuing thread waits for them after the loop over tiles."""
+    text = SOURCES["train.cu"]
+    start = text.index("for (int64_t tile = blockIdx.x; tile < ntiles && alive;")
+    _, rest = _body(text + "__syncwarp();", text.index("{", start) - 1)
+    rest = rest[:rest.index("tmem_dealloc")]
+    assert re.search(r"if \(!alive && t == kIssuer\) \{\s*tc::commit\(drain\);\s*tc::mbar_wait\(drain, 0,[^;]*;\s*\}"
+                     r".*__syncthreads\(\);", rest, flags=re.S), rest
