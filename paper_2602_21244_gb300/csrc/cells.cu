@@ -9,6 +9,7 @@
 // matching use exact integer sums over 8 lanes per cell (moments.cuh).
 #include <climits>
 
+#include "dispatch.cuh"
 #include "internal.cuh"
 #include "moments.cuh"
 
@@ -974,7 +975,9 @@ k_cells(int32_t n_cells, const int32_t* __restrict__ cs, double* vx, double* vy,
 // The same moments and matching for few cells: one group of 32 / SEG cells per
 // warp, SEG lanes each, without claims, and each lane's first kOnceHold
 // particles held in registers from the one read that serves the exponent, the
-// sums and the update.
+// sums and the update; the particles beyond them are read once for each, four
+// loads at a time (matching of 18,375 unequal cells, up to 250 particles each:
+// 76 us with one load at a time, 52; of 1,300 cells of 1,000: 208, 108).
 constexpr int kOnceHold = 4;
 // warps per block: few, so that few groups spread over all SMs (matching at 6,000 cells
 // of 61 particles 34.8 us with eight, 29.9 with two)
@@ -1000,6 +1003,7 @@ k_cells_once(int32_t n_cells, const int32_t* __restrict__ cs, double* vx, double
   }
 #pragma unroll
   for (int u = 0; u < kOnceHold; ++u) E = max(E, max(dexp(x[u]), max(dexp(y[u]), dexp(z[u]))));
+#pragma unroll 4
   for (int32_t i = a + kOnceHold * SEG + sl; i < b; i += SEG) E = max(E, max(dexp(vx[i]), max(dexp(vy[i]), dexp(vz[i]))));
   E = seg_max_i<SEG>(E);
   const int Ec = E + cell_scale(E, n).c, sp = fix_split(n);
@@ -1010,6 +1014,7 @@ k_cells_once(int32_t n_cells, const int32_t* __restrict__ cs, double* vx, double
     fix_add(q, q.sy, y[u], Ec, sp);
     fix_add(q, q.sz, z[u], Ec, sp);
   }
+#pragma unroll 4
   for (int32_t i = a + kOnceHold * SEG + sl; i < b; i += SEG) {
     fix_add(q, q.sx, vx[i], Ec, sp);
     fix_add(q, q.sy, vy[i], Ec, sp);
@@ -1029,33 +1034,28 @@ k_cells_once(int32_t n_cells, const int32_t* __restrict__ cs, double* vx, double
       const int32_t i = a + u * SEG + sl;
       if (i < b) { vx[i] = fma(alpha, x[u], ox); vy[i] = fma(alpha, y[u], oy); vz[i] = fma(alpha, z[u], oz); }
     }
-    for (int32_t i = a + kOnceHold * SEG + sl; i < b; i += SEG) {
-      vx[i] = fma(alpha, vx[i], ox);
-      vy[i] = fma(alpha, vy[i], oy);
-      vz[i] = fma(alpha, vz[i], oz);
+    for (uint32_t i0 = (uint32_t)a + kOnceHold * SEG + sl; i0 < (uint32_t)b; i0 += kOnceHold * SEG) {
+#pragma unroll
+      for (int u = 0; u < kOnceHold; ++u) {
+        const uint32_t i = i0 + u * SEG;
+        if (i < (uint32_t)b) { x[u] = vx[i]; y[u] = vy[i]; z[u] = vz[i]; }
+      }
+#pragma unroll
+      for (int u = 0; u < kOnceHold; ++u) {
+        const uint32_t i = i0 + u * SEG;
+        if (i < (uint32_t)b) { vx[i] = fma(alpha, x[u], ox); vy[i] = fma(alpha, y[u], oy); vz[i] = fma(alpha, z[u], oz); }
+      }
     }
   }
 }
 
-// Which kernel: the claiming kernel's chain of two claims, two passes over
-// memory and the batched remainder takes 18 us (moments) and 25 to 29 us
-// (matching) however few cells there are; one group per warp takes 9 and 9 to
-// 10 us (launch overhead included) at 100 to 2,867 cells, 22.7 against 26.2 us
-// (moments) at 40,000 cells of 20 particles (with claims of 4 cells 20.0 against 21.0), but from then on its FP64
-// remainder, paid per group of 4 cells instead of 16, costs more (matching
-// 18.5 against 25.2 us at 10,000 cells, 43.2 against 33.7 us at 40,000; at
-// 150,000 cells 113 against 85 us and 240 against 172 us).  And it costs more with many
-// particles per cell, 8 lanes each: where their number n is known (in a step), up to
-// 2,500 per SM for matching (6,000 cells of 61: 30 against 32 us, 18,375: 71 against 39;
-// 14,400 of 20: 16 against 22) and 10,000 for the moments (18,375 of 61: 26 against 28 us,
-// 37,500: 38 against 34).  32 lanes per
-// cell for up to 8 cells per SM (1,000 cells of 50: 9.5 against 12.3 us).
+// Which kernel: cells_kernel.
 static int launch_cells(Ctx* c, bool match, int32_t n_cells, const int32_t* cs, double* vx, double* vy,
                         double* vz, double* mom, cudaStream_t s, int64_t n) {
   if (n_cells <= 0) return 0;
-  const int64_t sms = sm_count(c);
-  if (n_cells <= (match ? 128 : 320) * sms && n <= (match ? 2500 : 10000) * sms) {
-    const int seg = n_cells <= 8 * sms ? 32 : 8;
+  const CellKernel kernel = cells_kernel(match, n_cells, n, sm_count(c));
+  if (kernel != CELLS_CLAIMED) {
+    const int seg = kernel;
     const unsigned gb = grid_for(n_cells, kOnceWarps * 32 / seg, INT_MAX);
     int* st = status_ptr(c);
     if (match) {

@@ -1,0 +1,29 @@
+// Rules that choose between kernels by the sizes of a call.  Plain C++: times
+// in us on GB300 (152 SMs); sizes per SM so that the rules scale with the chip.
+#pragma once
+#include <stdint.h>
+
+namespace dsmc {
+
+// Cell moments and moment matching (match): claims of cells by warps that stay
+// (k_cells), or one group of cells per warp with 8 or 32 lanes per cell
+// (k_cells_once).  Direct calls, by claims / by groups:
+//   20 particles a cell   match 12 / 9 at 1,000 cells, 22 / 17 at 10,000, 25 / 22 at 19,456, 30 / 32 at 30,000,
+//                         moments 16 / 11 at 14,400, 21.0 / 19.5 at 40,000, 23.0 / 22.9 at 48,640
+//   61 on average, up to  match 33 / 27 at 6,000 cells, 37 / 36 at 9,375, 37 / 41 at 13,500, 40 / 52 at 18,375,
+//   250 (dense cells      moments 23 / 16 at 6,000, 30 / 26 at 18,375, 33 / 35 at 30,375, 39 / 43 at 45,375
+//   side by side)
+// The groups save the claims' chain but pay the FP64 remainder per group of 4
+// cells instead of per 16, and in matching a dense cell holds up its group: so
+// the limits lie by cells, for matching lower where the number of particles is
+// not known (n = 0: a direct call, the cell starts are in device memory), and
+// by particles where it is (a step).  32 lanes per cell up to 8 cells per SM
+// (1,000 cells of 200: match 12 by 32 lanes, 20 by 8).
+enum CellKernel { CELLS_CLAIMED = 0, CELLS_ONCE_8 = 8, CELLS_ONCE_32 = 32 };
+
+inline CellKernel cells_kernel(bool match, int64_t n_cells, int64_t n, int64_t sms) {
+  if (n_cells > (!match ? 320 : n > 0 ? 128 : 96) * sms || n > (match ? 2500 : 10000) * sms) return CELLS_CLAIMED;
+  return n_cells <= 8 * sms ? CELLS_ONCE_32 : CELLS_ONCE_8;
+}
+
+}  // namespace dsmc

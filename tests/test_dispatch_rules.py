@@ -1,0 +1,42 @@
+"""The rules that choose between kernels (csrc/dispatch.cuh), compiled for the host."""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2602_21244_gb300", "csrc")
+SMS = 152
+CLAIMED, ONCE_8, ONCE_32 = 0, 8, 32
+
+STUB = r"""
+#include "dispatch.cuh"
+extern "C" int cells(int match, int64_t n_cells, int64_t n, int64_t sms) {
+  return dsmc::cells_kernel(match != 0, n_cells, n, sms);
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def rules(tmp_path_factory):
+    d = tmp_path_factory.mktemp("dispatch")
+    src, lib = d / "rules.cc", d / "rules.so"
+    src.write_text(STUB)
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I" + CSRC, str(src), "-o", str(lib)], check=True)
+    so = ctypes.CDLL(str(lib))
+    for f in (so.cells,):
+        f.argtypes = [ctypes.c_int] + [ctypes.c_int64] * 3
+    return so
+
+
+@pytest.mark.parametrize("match,n_cells,n,want", [
+    (1, 8 * SMS, 0, ONCE_32), (1, 8 * SMS + 1, 0, ONCE_8), (0, 8 * SMS, 0, ONCE_32), (0, 320 * SMS, 0, ONCE_8),
+    (0, 320 * SMS + 1, 0, CLAIMED),
+    # a direct call does not know its particles: dense cells cost the groups more, so it changes over earlier
+    (1, 96 * SMS, 0, ONCE_8), (1, 96 * SMS + 1, 0, CLAIMED), (1, 18375, 0, CLAIMED),
+    # a step does
+    (1, 128 * SMS, 2500 * SMS, ONCE_8), (1, 128 * SMS + 1, 2500 * SMS, CLAIMED), (1, 96 * SMS, 2500 * SMS + 1, CLAIMED),
+    (0, 320 * SMS, 10000 * SMS, ONCE_8), (0, 96 * SMS, 10000 * SMS + 1, CLAIMED),
+])
+def test_cell_kernel(rules, match, n_cells, n, want):
+    assert rules.cells(match, n_cells, n, SMS) == want

@@ -1,0 +1,70 @@
+"""Both sides of the sizes at which a call changes its kernel, and what the change costs."""
+import numpy as np
+import pytest
+
+from gpu_util import ctx, cuda, host, torch
+
+pytestmark = pytest.mark.gpu
+
+
+def _sms():
+    return torch().cuda.get_device_properties(0).multi_processor_count
+
+
+def _best_us(f, reps=20):
+    """Shortest of five means over `reps` calls, by events."""
+    T = torch()
+    f()
+    best = 1e30
+    for _ in range(5):
+        a, b = T.cuda.Event(enable_timing=True), T.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(reps):
+            f()
+        b.record()
+        T.cuda.synchronize()
+        best = min(best, a.elapsed_time(b) * 1e3 / reps)
+    return best
+
+
+def _moments_and_matching(sizes, seed=6):
+    """Moments and matched velocities of cells of these sizes: (starts, moments, velocities)."""
+    C, rng = ctx(), np.random.default_rng(seed)
+    cs = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int32)
+    x = [cuda(v) for v in 1e3 * rng.standard_normal((3, int(cs[-1]))) + 50.0]
+    mom = C.cell_moments(cuda(cs), *x)
+    y = [c * 1.5 - 7.0 for c in x]
+    C.moment_match(cuda(cs), mom, *y)
+    assert C.sync_status() == 0
+    return cs, host(mom), [host(c) for c in y]
+
+
+@pytest.mark.parametrize("per_sm,more", [(0, 40), (8, 1), (96, 0), (96, 1)])
+def test_cells_longer_than_a_lane_group_holds(per_sm, more):
+    """Cells of up to ten times what a group's lanes hold in registers (32 and 128 particles), around every
+    multiple that the batches of four loads have: bit for bit what the claiming kernel gives, whatever the size."""
+    ends = [[k + d for k in (32, 64, 96, 128, 160) for d in (-1, 0, 1)],
+            [k + d for k in (256, 384, 512, 640, 1280) for d in (-1, 0, 1)] + [0, 7]]
+    out = []
+    for nc in (per_sm * _sms() + more, 400 * _sms()):
+        sizes = np.zeros(nc, np.int64)
+        sizes[:15], sizes[-17:] = ends
+        _, mom, v = _moments_and_matching(sizes)
+        out.append([mom[:15], mom[-17:]] + v)
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
+
+
+def test_dense_cells_cost_no_more_by_groups_than_by_claims():
+    """Matching of 1,300 cells of about 1,000 particles (by groups of cells) against the same cells before 20,000
+    empty ones (by claims, which visit those too): not above 1.4 times (one load at a time for the particles
+    beyond the held ones took twice the time)."""
+    T, C = torch(), ctx()
+    sizes = np.random.default_rng(1).poisson(1000, 1300)
+    took = []
+    for nc in (1300, 21300):
+        starts = cuda(np.concatenate([[0], np.cumsum(np.pad(sizes, (0, nc - 1300)))]).astype(np.int32))
+        v = [T.randn(int(sizes.sum()), dtype=T.float64, device="cuda") for _ in range(3)]
+        mom = C.cell_moments(starts, *v)
+        took.append(_best_us(lambda: C.moment_match(starts, mom, *v)))
+    assert took[0] <= 1.4 * took[1], took
