@@ -17,13 +17,15 @@ namespace dsmc {
 // cells instead of per 16, and in matching a dense cell holds up its group: so
 // the limits lie by cells, for matching lower where the number of particles is
 // not known (n = 0: a direct call, the cell starts are in device memory), and
-// by particles where it is (a step).  32 lanes per cell up to 8 cells per SM
-// (1,000 cells of 200: match 12 by 32 lanes, 20 by 8).
+// by particles where it is (a step).  Up to 8 cells per SM 32 lanes per cell,
+// however many particles (1,000 cells of 200: match 12 by 32 lanes, 20 by 8, 28 by
+// claims; of 1,000: 31, 103, 98).
 enum CellKernel { CELLS_CLAIMED = 0, CELLS_ONCE_8 = 8, CELLS_ONCE_32 = 32 };
 
 inline CellKernel cells_kernel(bool match, int64_t n_cells, int64_t n, int64_t sms) {
+  if (n_cells <= 8 * sms) return CELLS_ONCE_32;
   if (n_cells > (!match ? 320 : n > 0 ? 128 : 96) * sms || n > (match ? 2500 : 10000) * sms) return CELLS_CLAIMED;
-  return n_cells <= 8 * sms ? CELLS_ONCE_32 : CELLS_ONCE_8;
+  return CELLS_ONCE_8;
 }
 
 }  // namespace dsmc
