@@ -479,9 +479,10 @@ size_t dsmc_step_workspace_size(int32_t n, int32_t n_cells, int64_t capacity);
  * chosen path, moment matching (Sec. 2.1-2.6).  The pair list in `buf` is
  * bucketed by claim level (DSMC_ORDER_LEVELS) on DSMC_PATH_NEURAL and by
  * round on the other paths.  On DSMC_PATH_VHS and DSMC_PATH_TABLE a small gas
- * (up to 64 or 288 cells per SM) is updated by groups of cells, with the
- * results of the collide calls bit for bit; the shapes set for those calls
- * (dsmc_tune_set) then have no part in it. */
+ * (up to 64 or 288 cells and 4,000 or 16,000 particles per SM, 512 particles
+ * per cell on average) is updated by groups of cells, with the results of the
+ * collide calls bit for bit; the shapes set for those calls (dsmc_tune_set)
+ * then have no part in it. */
 int dsmc_step(dsmc_ctx_t* ctx, const dsmc_gas_t* gas, const dsmc_path_t* path,
               const dsmc_step_buffers_t* buf, uint64_t step, void* stream);
 

@@ -4,6 +4,7 @@
 #include <cstring>
 #include <mutex>
 
+#include "dispatch.cuh"
 #include "internal.cuh"
 
 namespace dsmc {
@@ -599,7 +600,7 @@ static int collide_step(dsmc_ctx_t* c, const dsmc_gas_t* gas, const dsmc_path_t*
   int rc = 0;
   switch (path->path) {
     case DSMC_PATH_VHS:
-      if (dsmc::groups_suit(c, B->n_cells, false)) {
+      if (dsmc::groups_suit(false, B->n_cells, B->n, dsmc::sm_count(c))) {
         REQUIRE(c, B->round_offsets && B->info && B->svx && B->svy && B->svz && B->ws && B->n >= 0,
                 "collide_vhs: null pointer");
         rc = dsmc::launch_groups_vhs(c, *gas, step, B->n_cells, B->pairs, B->round_offsets, B->info, B->svx, B->svy,
@@ -619,7 +620,7 @@ static int collide_step(dsmc_ctx_t* c, const dsmc_gas_t* gas, const dsmc_path_t*
                                nullptr, B->ws, B->ws_bytes, stream);
       break;
     case DSMC_PATH_TABLE:
-      if (dsmc::groups_suit(c, B->n_cells, true)) {
+      if (dsmc::groups_suit(true, B->n_cells, B->n, dsmc::sm_count(c))) {
         if ((rc = check_table(c, path->table))) return rc;
         REQUIRE(c, B->round_offsets && B->info && B->svx && B->svy && B->svz && B->ws && B->n >= 0,
                 "collide_table: null pointer");

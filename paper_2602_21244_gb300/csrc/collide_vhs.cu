@@ -142,7 +142,7 @@ int launch_collide_vhs(Ctx* c, const dsmc_gas_t& gas, uint64_t step, int32_t n, 
 // groups spread evenly over the SMs' four sub-partitions, each with an FP64 pipe of its
 // own: 105 us where blocks of four took 110 (of two: 106).  Larger gases fill the
 // chip without this, and the groups' partly filled warps and searches cost more than
-// the waits they save: see groups_suit.
+// the waits they save, as does the one warp that takes a dense cell's pairs: see groups_suit.
 struct GroupArgs {
   uint64_t seed, step;
   const uint64_t* step_dev;
@@ -269,13 +269,6 @@ static int launch_groups(Ctx* c, const Update& u, const dsmc_gas_t& gas, uint64_
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : record(c, DSMC_ERR_CUDA, "step: pair update launch failed");
 }
-
-// Up to how many cells a step takes its pairs in groups (step, by stamps against groups,
-// us): look-up path 138 / 107 at 1,600 cells of 20 particles, 268 / 226 at 25,600, 324 /
-// 298 at 40,000, 494 / 503 at 57,600; 638 / 569 at 37,500 cells of the hypersonic gas, 926
-// / 926 at 73,500.  VHS, with fewer pairs and no table: 91 / 83 at 1,600, 115 / 103 at
-// 6,400, 134 / 130 at 14,400; hypersonic 147 / 136 at 6,000, 227 / 236 at 18,375.
-bool groups_suit(Ctx* c, int32_t n_cells, bool table) { return n_cells <= (table ? 288 : 64) * sm_count(c); }
 
 int launch_groups_vhs(Ctx* c, const dsmc_gas_t& gas, uint64_t step, int32_t n_cells, const int32_t* pairs,
                     const int32_t* ro, const dsmc_select_info_t* info, double* vx, double* vy, double* vz,

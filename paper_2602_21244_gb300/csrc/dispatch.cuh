@@ -28,4 +28,21 @@ inline CellKernel cells_kernel(bool match, int64_t n_cells, int64_t n, int64_t s
   return CELLS_ONCE_8;
 }
 
+// The pair update of a step on the VHS (table false) and look-up paths: by
+// groups of cells (k_collide_groups, one warp per group), or by stamps
+// (k_collide_vhs, k_collide_table, every SM on every cell's pairs).  Whole
+// step, by stamps / by groups, pairs a particle in brackets:
+//   VHS       1,024 cells of 60 [0.6] 120 / 96, of 400 269 / 255, of 1,000 540 / 528; 6,000 of 60 177 / 164, of 120
+//             221 / 246; 9,700 of 20 159 / 148, of 60 [0.15] 159 / 151, [0.6] 210 / 211, of 120 268 / 311
+//   look-up   1,024 cells of 60 [0.8] 137 / 101, of 400 393 / 343; 9,000 of 60 250 / 216; 30,000 of 20 281 / 243, of
+//             60 394 / 457, of 120 637 / 807; 43,000 of 20 325 / 305; of the hypersonic gas (61 a cell, up to
+//             250) 37,500 638 / 569, 73,500 926 / 926
+//   few cells, very dense: 16 cells of 400 [0.6] VHS 137 / 130, of 1,000 264 / 278, of 4,000 1536 / 1585; look-up
+//             220 / 214, 540 / 564, 3182 / 3305; 64 of 4,000 1587 / 1634, 3309 / 3418; one of 4,000 [1.3] VHS 603 / 781
+// Groups save the stamps and the waits between a cell's rounds; larger gases
+// fill the chip without that, and a very dense cell is one warp's work.
+inline bool groups_suit(bool table, int64_t n_cells, int64_t n, int64_t sms) {
+  return n_cells <= (table ? 288 : 64) * sms && n <= (table ? 16000 : 4000) * sms && n <= 512 * n_cells;
+}
+
 }  // namespace dsmc

@@ -385,9 +385,8 @@ int launch_collide_jager(Ctx* c, const dsmc_gas_t& gas, const dsmc_potential_t& 
                          double* vz, float* chi_out, void* ws, size_t ws_bytes, cudaStream_t s);
 int launch_chi_table(Ctx* c, const dsmc_gas_t& gas, const dsmc_potential_t& pot, int n_nodes, int32_t nb,
                      int32_t nE, double lnE_min, double lnE_max, float* T, cudaStream_t s);
-// the same updates on the selection's own list (pairs in cell order inside a round), for the step, and
-// whether they are the faster ones at a number of cells
-bool groups_suit(Ctx* c, int32_t n_cells, bool table);
+// the same updates on the selection's own list (pairs in cell order inside a round), for the step where
+// they are the faster ones (groups_suit)
 int launch_groups_vhs(Ctx* c, const dsmc_gas_t& gas, uint64_t step, int32_t n_cells, const int32_t* pairs,
                       const int32_t* ro, const dsmc_select_info_t* info, double* vx, double* vy, double* vz,
                       cudaStream_t s);

@@ -14,6 +14,9 @@ STUB = r"""
 extern "C" int cells(int match, int64_t n_cells, int64_t n, int64_t sms) {
   return dsmc::cells_kernel(match != 0, n_cells, n, sms);
 }
+extern "C" int groups(int table, int64_t n_cells, int64_t n, int64_t sms) {
+  return dsmc::groups_suit(table != 0, n_cells, n, sms);
+}
 """
 
 
@@ -24,7 +27,7 @@ def rules(tmp_path_factory):
     src.write_text(STUB)
     subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I" + CSRC, str(src), "-o", str(lib)], check=True)
     so = ctypes.CDLL(str(lib))
-    for f in (so.cells,):
+    for f in (so.cells, so.groups):
         f.argtypes = [ctypes.c_int] + [ctypes.c_int64] * 3
     return so
 
@@ -42,3 +45,16 @@ def rules(tmp_path_factory):
 ])
 def test_cell_kernel(rules, match, n_cells, n, want):
     assert rules.cells(match, n_cells, n, SMS) == want
+
+
+@pytest.mark.parametrize("table,n_cells,n,want", [
+    (0, 64 * SMS, 20 * 64 * SMS, 1), (0, 64 * SMS + 1, 20 * 64 * SMS, 0), (1, 288 * SMS, 20 * 288 * SMS, 1),
+    (1, 288 * SMS + 1, 20 * 288 * SMS, 0), (0, 100, 0, 1),
+    # few cells with many particles are many pairs for one warp each
+    (0, 1, 512, 1), (0, 1, 513, 0), (1, 1, 1000000, 0), (1, 100, 51200, 1), (1, 100, 51201, 0),
+    # a gas that fills the chip
+    (0, 64 * SMS, 4000 * SMS, 1), (0, 64 * SMS, 4000 * SMS + 1, 0), (1, 288 * SMS, 16000 * SMS, 1),
+    (1, 288 * SMS, 16000 * SMS + 1, 0),
+])
+def test_pair_update_by_groups(rules, table, n_cells, n, want):
+    assert rules.groups(table, n_cells, n, SMS) == want

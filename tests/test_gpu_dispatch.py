@@ -68,3 +68,46 @@ def test_dense_cells_cost_no_more_by_groups_than_by_claims():
         mom = C.cell_moments(starts, *v)
         took.append(_best_us(lambda: C.moment_match(starts, mom, *v)))
     assert took[0] <= 1.4 * took[1], took
+
+
+@pytest.mark.parametrize("path,nx,per,scale", [("vhs", 64, 20, 2000.0), ("vhs", 65, 20, 2000.0), ("table", 288, 20, 1000.0),
+                                               ("table", 289, 20, 1000.0), ("vhs", 0, 470, 1500.0), ("vhs", 0, 600, 1500.0),
+                                               ("table", 0, 470, 1500.0), ("table", 0, 600, 1500.0), ("vhs", 64, 75, 300.0),
+                                               ("table", 288, 65, 300.0)])
+def test_step_on_both_sides_of_the_cell_groups(path, nx, per, scale):
+    """A step on each side of every limit of the update by groups of cells (cells per SM; particles per cell, three
+    cells; particles per SM) against the collide call: the same bits."""
+    import test_gpu_variants as V
+    V.test_step_by_cell_groups_equals_the_collide_calls(path, nx * _sms() if nx else 3, 1, per, scale)
+
+
+def test_pair_update_of_few_dense_cells():
+    """The step of one cell of 4,000 particles takes at most a tenth more than its phases called one by one, whose
+    pair update puts every SM on that cell's pairs (one warp for all of them: a third more)."""
+    from paper_2602_21244_gb300 import dsmc as D
+    from paper_2602_21244_gb300 import workloads as W
+    T, C = torch(), ctx()
+    nc, per = 1, 4000
+    n = nc * per
+    gas = D.make_gas(dict(W.couette()["gas"], b_max=4.17e-10, fn_over_vc=2e18 * 300 * 60.0 / per, dt=1e-7, model=0))
+    st = D.StepState(C, n, nc, 8 * n)
+    for c in (st.vx, st.vy, st.vz):
+        c.copy_(T.randn(n, dtype=T.float64, device="cuda") * 400)
+    st.cell_id.zero_()
+    st.sigma_g_max.copy_(C.sigma_g_max_init(gas, T.full((nc,), 300.0, dtype=T.float64, device="cuda")))
+    path = D.make_path(D.PATH_VHS)
+    C.step(gas, path, st, 0)
+    sel = dict(pairs=st.pairs, deps=st.deps, round_offsets=st.round_offsets, info=st.info)
+    cs, sg = st.cell_start, st.sigma_g_max.clone()
+
+    def phases():
+        o = C.sort_cells(st.cell_id, st.vx, st.vy, st.vz, nc)
+        x = [o[k] for k in ("svx", "svy", "svz")]
+        mom = C.cell_moments(o["cell_start"], *x)
+        C.select_pairs(gas, cs, *x, sg, 0, 8 * n, out=sel)
+        C.collide_vhs(gas, 0, sel, *x)
+        C.moment_match(o["cell_start"], mom, *x)
+
+    assert C.sync_status() == 0
+    took = _best_us(lambda: C.step(gas, path, st, 0)), _best_us(phases)
+    assert took[0] <= 1.1 * took[1], took
