@@ -521,7 +521,11 @@ int dsmc_step_graph_launch(dsmc_ctx_t* ctx, uint64_t step, void* stream);
  * set directly.  No setting changes a result: each of these kernels gives a
  * thread whole work items (a sorted slot, a group of cells, a pair of a
  * round, one chi) through a grid-stride loop, so every item is computed by
- * the same arithmetic in the same order whatever the shape.  (The paper
+ * the same arithmetic in the same order whatever the shape.  Kernels that a
+ * small gas takes in their place have no shape to set: the moments and
+ * matching of one group of cells per warp (up to 320 and 128 cells per SM,
+ * 10,000 and 2,500 particles per SM in a step), the pair update by groups of
+ * cells (dsmc_step).  (The paper
  * fixes no launch configuration; the tuned kernels are those of Sec. 2.1,
  * 2.3 and 2.5 and of the scattering integral, Sec. 3.4.) */
 enum {
@@ -565,7 +569,10 @@ int dsmc_tune_candidates(dsmc_ctx_t* ctx, int32_t kernel, dsmc_tune_entry_t* out
  * the context.  Synchronises `stream`.  The buffers are left holding the
  * state after an unspecified number of collide and moment-matching passes
  * over that step's pairs (each pass conserves momentum and energy), so tune
- * on a copy or before loading the state to be advanced.  trials (may be
+ * on a copy or before loading the state to be advanced.  The kernels timed
+ * are those that the shapes are for, also where the step of a small gas takes
+ * others.  Shapes that launch alike on a small gas share one time, and of them
+ * the first candidate (the built-in shape or the nearest to it) is kept.  trials (may be
  * NULL) receives up to `cap` measured entries; *n_trials their count. */
 int dsmc_autotune_step(dsmc_ctx_t* ctx, const dsmc_gas_t* gas, const dsmc_path_t* path,
                        const dsmc_step_buffers_t* buf, uint64_t step, int32_t reps,

@@ -1,5 +1,6 @@
 // C ABI of the DSMC library: context, status word, argument checks, the
 // whole collision step and its host-buffer variant.
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -78,7 +79,9 @@ ShapeInfo shape_info(int k) {
 // Candidate shapes of one kernel: block sizes up to the kernel's limit with
 // at most 2048 threads and 32 blocks per SM (the chi batch grid-strides over up to
 // 64 blocks per SM); for the persistent collides
-// the full occupancy at each block size and half of it.
+// the full occupancy at each block size and half of it.  The built-in shape
+// or the nearest to it first, and more blocks before fewer: of shapes that a
+// small gas cannot tell apart the first is kept.
 static int tune_candidates(int k, dsmc_tune_entry_t* out, int cap) {
   int n = 0;
   auto push = [&](int t, int b) {
@@ -87,14 +90,16 @@ static int tune_candidates(int k, dsmc_tune_entry_t* out, int cap) {
   };
   switch (k) {
     case DSMC_TUNE_GATHER:
-      for (int t : {128, 256, 512})
-        for (int b : {2, 4, 8, 16})
+      for (int t : {256, 128, 512})
+        for (int b : {16, 8, 4, 2})
           if (t * b <= 2048) push(t, b);
       break;
     case DSMC_TUNE_MOMENTS:
-    case DSMC_TUNE_MOMENT_MATCH:
       // block size fixed (256 threads); up to four blocks resident per SM
-      for (int b : {1, 2, 3, 4}) push(256, b);
+      for (int b : {4, 3, 2, 1}) push(256, b);
+      break;
+    case DSMC_TUNE_MOMENT_MATCH:
+      for (int b : {3, 4, 2, 1}) push(256, b);
       break;
     case DSMC_TUNE_COLLIDE_VHS:
     case DSMC_TUNE_COLLIDE_JAGER:
@@ -111,8 +116,8 @@ static int tune_candidates(int k, dsmc_tune_entry_t* out, int cap) {
       break;
     }
     case DSMC_TUNE_JAGER_CHI:
-      for (int t : {64, 128})
-        for (int b : {8, 16, 32, 64}) push(t, b);
+      for (int t : {128, 64})
+        for (int b : {64, 32, 16, 8}) push(t, b);
       break;
     default: break;
   }
@@ -895,10 +900,15 @@ int dsmc_tune_candidates(dsmc_ctx_t* c, int32_t kernel, dsmc_tune_entry_t* out, 
 
 namespace {
 
+// Blocks of a persistent kernel, whatever the work.
+const auto full_grid = [](int, int bps) { return (int64_t)bps; };
+
 // Time every candidate shape of `kernel` with `launch` (one untimed launch,
-// then `reps` between events), keep the fastest; entries go to trials.
-template <class F>
-int tune_kernel(dsmc_ctx* c, int kernel, int reps, cudaStream_t s, F&& launch, dsmc_tune_entry_t* trials,
+// then `reps` between events), keep the fastest; entries go to trials.  Shapes
+// with the same block size and the same `blocks` (few of either on small work)
+// are one launch and share one time: of these the first listed is kept.
+template <class G, class F>
+int tune_kernel(dsmc_ctx* c, int kernel, int reps, cudaStream_t s, G&& blocks, F&& launch, dsmc_tune_entry_t* trials,
                 int cap, int* nt) {
   dsmc_tune_entry_t cand[64];
   const int nc = dsmc::tune_candidates(kernel, cand, 64);
@@ -909,17 +919,25 @@ int tune_kernel(dsmc_ctx* c, int kernel, int reps, cudaStream_t s, F&& launch, d
   const int t0 = c->tune_threads[kernel], b0 = c->tune_bps[kernel];
   int best = -1, rc = DSMC_OK;
   for (int q = 0; q < nc && q < 64; ++q) {
-    c->tune_threads[kernel] = cand[q].threads;
-    c->tune_bps[kernel] = cand[q].blocks_per_sm;
-    rc = launch();
-    if (!rc && cudaEventRecord(e0, s) != cudaSuccess) rc = DSMC_ERR_CUDA;
-    for (int r = 0; r < reps && !rc; ++r) rc = launch();
-    if (!rc && cudaEventRecord(e1, s) != cudaSuccess) rc = DSMC_ERR_CUDA;
-    if (!rc) rc = dsmc_ctx_sync_status(c, s);
-    if (rc) break;
-    float el = 0.f;
-    cudaEventElapsedTime(&el, e0, e1);
-    cand[q].ms = el / (float)reps;
+    int same = 0;
+    while (same < q && !(cand[same].threads == cand[q].threads && blocks(cand[q].threads, cand[same].blocks_per_sm) ==
+                                                                      blocks(cand[q].threads, cand[q].blocks_per_sm)))
+      ++same;
+    if (same < q) {
+      cand[q].ms = cand[same].ms;
+    } else {
+      c->tune_threads[kernel] = cand[q].threads;
+      c->tune_bps[kernel] = cand[q].blocks_per_sm;
+      rc = launch();
+      if (!rc && cudaEventRecord(e0, s) != cudaSuccess) rc = DSMC_ERR_CUDA;
+      for (int r = 0; r < reps && !rc; ++r) rc = launch();
+      if (!rc && cudaEventRecord(e1, s) != cudaSuccess) rc = DSMC_ERR_CUDA;
+      if (!rc) rc = dsmc_ctx_sync_status(c, s);
+      if (rc) break;
+      float el = 0.f;
+      cudaEventElapsedTime(&el, e0, e1);
+      cand[q].ms = el / (float)reps;
+    }
     if (trials && *nt < cap) trials[*nt] = cand[q];
     ++*nt;
     if (best < 0 || cand[q].ms < cand[best].ms) best = q;
@@ -952,31 +970,39 @@ int dsmc_autotune_step(dsmc_ctx_t* c, const dsmc_gas_t* gas, const dsmc_path_t* 
   if (!rc) rc = dsmc_ctx_sync_status(c, stream);
   if (rc) return rc;
   if (B->n == 0 || B->n_cells == 0) return DSMC_OK;
+  // Each trial runs the kernel that the shape is for, although the step of a
+  // small gas takes others (cell groups, one group of cells per warp): the shapes
+  // stay with the context for its direct calls and its larger gases.
+  const int64_t sms = dsmc::sm_count(c);
+  auto cell_blocks = [&](int, int bps) {
+    return std::min((B->n_cells + dsmc::kCellsPerBlock - 1) / (int64_t)dsmc::kCellsPerBlock, sms * bps);
+  };
+  auto gather_blocks = [&](int threads, int bps) { return std::min(((int64_t)B->n + threads - 1) / threads, sms * bps); };
   int nt = 0;
-  rc = tune_kernel(c, DSMC_TUNE_GATHER, reps, s, [&] {
+  rc = tune_kernel(c, DSMC_TUNE_GATHER, reps, s, gather_blocks, [&] {
     return dsmc::launch_gather(c, B->n, B->n_cells, B->cell_start, B->perm, B->vx, B->vy, B->vz, B->svx,
                                B->svy, B->svz, s);
   }, trials, cap, &nt);
-  if (!rc) rc = tune_kernel(c, DSMC_TUNE_MOMENTS, reps, s, [&] {
-    return dsmc::launch_moments(c, B->n_cells, B->cell_start, B->svx, B->svy, B->svz, B->mom, s, B->n);
+  if (!rc) rc = tune_kernel(c, DSMC_TUNE_MOMENTS, reps, s, cell_blocks, [&] {
+    return dsmc::launch_moments(c, B->n_cells, B->cell_start, B->svx, B->svy, B->svz, B->mom, s, dsmc::kByClaims);
   }, trials, cap, &nt);
   if (!rc && path->path == DSMC_PATH_VHS)
-    rc = tune_kernel(c, DSMC_TUNE_COLLIDE_VHS, reps, s, [&] {
+    rc = tune_kernel(c, DSMC_TUNE_COLLIDE_VHS, reps, s, full_grid, [&] {
       return dsmc_collide_vhs(c, gas, step, B->n, B->pairs, B->deps, B->round_offsets, B->info, B->svx, B->svy,
                               B->svz, B->ws, B->ws_bytes, stream);
     }, trials, cap, &nt);
   if (!rc && path->path == DSMC_PATH_TABLE)
-    rc = tune_kernel(c, DSMC_TUNE_COLLIDE_TABLE, reps, s, [&] {
+    rc = tune_kernel(c, DSMC_TUNE_COLLIDE_TABLE, reps, s, full_grid, [&] {
       return dsmc_collide_table(c, gas, path->table, step, B->n, B->pairs, B->deps, B->round_offsets, B->info,
                                 B->svx, B->svy, B->svz, nullptr, B->ws, B->ws_bytes, stream);
     }, trials, cap, &nt);
   if (!rc && path->path == DSMC_PATH_JAGER)
-    rc = tune_kernel(c, DSMC_TUNE_COLLIDE_JAGER, reps, s, [&] {
+    rc = tune_kernel(c, DSMC_TUNE_COLLIDE_JAGER, reps, s, full_grid, [&] {
       return dsmc_collide_jager(c, gas, path->pot, path->n_nodes, step, B->n, B->pairs, B->deps, B->round_offsets,
                                 B->info, B->svx, B->svy, B->svz, nullptr, B->ws, B->ws_bytes, stream);
     }, trials, cap, &nt);
-  if (!rc) rc = tune_kernel(c, DSMC_TUNE_MOMENT_MATCH, reps, s, [&] {
-    return dsmc::launch_moment_match(c, B->n_cells, B->cell_start, B->mom, B->svx, B->svy, B->svz, s, B->n);
+  if (!rc) rc = tune_kernel(c, DSMC_TUNE_MOMENT_MATCH, reps, s, cell_blocks, [&] {
+    return dsmc::launch_moment_match(c, B->n_cells, B->cell_start, B->mom, B->svx, B->svy, B->svz, s, dsmc::kByClaims);
   }, trials, cap, &nt);
   *n_trials = nt;
   return rc;
@@ -990,7 +1016,10 @@ int dsmc_autotune_chi(dsmc_ctx_t* c, const dsmc_gas_t* gas, const dsmc_potential
   *n_trials = 0;
   if (n == 0) return DSMC_OK;
   int nt = 0;
-  const int rc = tune_kernel(c, DSMC_TUNE_JAGER_CHI, reps, S(stream), [&] {
+  const auto blocks = [&](int threads, int bps) {
+    return std::min((n + threads - 1) / threads, (int64_t)dsmc::sm_count(c) * bps);
+  };
+  const int rc = tune_kernel(c, DSMC_TUNE_JAGER_CHI, reps, S(stream), blocks, [&] {
     return dsmc_jager_chi(c, gas, pot, n_nodes, n, b, g, chi, stream);
   }, trials, cap, &nt);
   *n_trials = nt;

@@ -832,6 +832,7 @@ constexpr int kCwWarps = 8;
 constexpr int kCwRun = 4;                    // cells per claim (one per segment)
 constexpr int kCwClaims = 4;                 // claims per batch
 constexpr int kCwCells = kCwRun * kCwClaims; // cells per batch (one lane each in the remainder)
+static_assert(kCwRun * kCwWarps == kCellsPerBlock, "a run per warp");
 
 struct CwWarp {
   FixAcc acc[kCwCells];

@@ -21,8 +21,13 @@ namespace dsmc {
 // however many particles (1,000 cells of 200: match 12 by 32 lanes, 20 by 8, 28 by
 // claims; of 1,000: 31, 103, 98).
 enum CellKernel { CELLS_CLAIMED = 0, CELLS_ONCE_8 = 8, CELLS_ONCE_32 = 32 };
+constexpr int64_t kByClaims = -1;   // in the place of n: k_cells, the kernel that the tuned shapes are for
+
+// Cells that k_cells gives to a block at least.
+constexpr int kCellsPerBlock = 32;
 
 inline CellKernel cells_kernel(bool match, int64_t n_cells, int64_t n, int64_t sms) {
+  if (n == kByClaims) return CELLS_CLAIMED;
   if (n_cells <= 8 * sms) return CELLS_ONCE_32;
   if (n_cells > (!match ? 320 : n > 0 ? 128 : 96) * sms || n > (match ? 2500 : 10000) * sms) return CELLS_CLAIMED;
   return CELLS_ONCE_8;

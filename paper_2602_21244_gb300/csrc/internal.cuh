@@ -359,7 +359,7 @@ int launch_sort(Ctx* c, int32_t n, int32_t n_cells, const int32_t* cell_id, cons
 int launch_sort_keys(Ctx* c, int32_t n, int32_t n_cells, const int32_t* cell_id, int32_t* perm,
                      int32_t* cell_start, void* ws, size_t ws_bytes, cudaStream_t s);
 size_t sort_ws(int32_t n, int32_t n_cells);
-// n: the number of particles where the caller knows it (it decides which kernel is the faster one), or 0
+// n: the number of particles where the caller knows it (it decides which kernel is the faster one), 0 or kByClaims
 int launch_moments(Ctx* c, int32_t n_cells, const int32_t* cs, const double* vx,
                    const double* vy, const double* vz, double* mom, cudaStream_t s, int64_t n = 0);
 int launch_moment_match(Ctx* c, int32_t n_cells, const int32_t* cs, const double* mom,

@@ -40,6 +40,8 @@ def rules(tmp_path_factory):
     # a step does
     (1, 128 * SMS, 2500 * SMS, ONCE_8), (1, 128 * SMS + 1, 2500 * SMS, CLAIMED), (1, 96 * SMS, 2500 * SMS + 1, CLAIMED),
     (0, 320 * SMS, 10000 * SMS, ONCE_8), (0, 96 * SMS, 10000 * SMS + 1, CLAIMED),
+    # what the tuned shapes are for
+    (1, 10, -1, CLAIMED), (0, 10, -1, CLAIMED),
     # few cells: most lanes per cell, however dense
     (1, 1000, 500000, ONCE_32), (0, 1000, 8000000, ONCE_32), (1, 8 * SMS, 2**31 - 1, ONCE_32),
 ])

@@ -81,33 +81,50 @@ def test_step_on_both_sides_of_the_cell_groups(path, nx, per, scale):
     V.test_step_by_cell_groups_equals_the_collide_calls(path, nx * _sms() if nx else 3, 1, per, scale)
 
 
-def test_pair_update_of_few_dense_cells():
-    """The step of one cell of 4,000 particles takes at most a tenth more than its phases called one by one, whose
-    pair update puts every SM on that cell's pairs (one warp for all of them: a third more)."""
+def _uniform_gas(n_cells, per):
     from paper_2602_21244_gb300 import dsmc as D
     from paper_2602_21244_gb300 import workloads as W
     T, C = torch(), ctx()
-    nc, per = 1, 4000
-    n = nc * per
-    gas = D.make_gas(dict(W.couette()["gas"], b_max=4.17e-10, fn_over_vc=2e18 * 300 * 60.0 / per, dt=1e-7, model=0))
-    st = D.StepState(C, n, nc, 8 * n)
+    n = n_cells * per
+    gas = D.make_gas(dict(W.couette()["gas"], b_max=4.17e-10, fn_over_vc=3e20, dt=1e-7, model=0))
+    st = D.StepState(C, n, n_cells, 4 * n)
     for c in (st.vx, st.vy, st.vz):
         c.copy_(T.randn(n, dtype=T.float64, device="cuda") * 400)
-    st.cell_id.zero_()
-    st.sigma_g_max.copy_(C.sigma_g_max_init(gas, T.full((nc,), 300.0, dtype=T.float64, device="cuda")))
-    path = D.make_path(D.PATH_VHS)
-    C.step(gas, path, st, 0)
-    sel = dict(pairs=st.pairs, deps=st.deps, round_offsets=st.round_offsets, info=st.info)
-    cs, sg = st.cell_start, st.sigma_g_max.clone()
+    st.cell_id.copy_(T.arange(n, device="cuda", dtype=T.int32) % n_cells)
+    st.sigma_g_max.copy_(C.sigma_g_max_init(gas, T.full((n_cells,), 300.0, dtype=T.float64, device="cuda")))
+    return gas, D.make_path(D.PATH_VHS), st
 
-    def phases():
-        o = C.sort_cells(st.cell_id, st.vx, st.vy, st.vz, nc)
-        x = [o[k] for k in ("svx", "svy", "svz")]
-        mom = C.cell_moments(o["cell_start"], *x)
-        C.select_pairs(gas, cs, *x, sg, 0, 8 * n, out=sel)
-        C.collide_vhs(gas, 0, sel, *x)
-        C.moment_match(o["cell_start"], mom, *x)
 
-    assert C.sync_status() == 0
-    took = _best_us(lambda: C.step(gas, path, st, 0)), _best_us(phases)
-    assert took[0] <= 1.1 * took[1], took
+def test_autotune_times_the_kernels_that_take_the_shapes():
+    """A gas whose step takes the moments one group of cells per warp, without a shape: the trials are of the
+    claiming kernel, which a quarter of the blocks slows down by more than a quarter; by the other kernel all
+    would take the same time."""
+    from paper_2602_21244_gb300 import dsmc as D
+    C = ctx()
+    gas, path, st = _uniform_gas(250 * _sms(), 20)
+    try:
+        trials = C.autotune_step(gas, path, st, step=0, reps=20)
+        ms = {t["blocks_per_sm"]: t["ms"] for t in trials if t["kernel"] == "moments"}
+        assert sorted(ms) == [1, 2, 3, 4] and ms[1] > 1.25 * ms[4], ms
+    finally:
+        for k in range(len(D.TUNE_KERNELS)):
+            C.tune_set(k)
+
+
+def test_autotune_keeps_the_builtin_shape_where_all_launch_alike():
+    """A gas of fewer cells than a block per SM: one launch, one time, and no shape chosen by noise."""
+    from paper_2602_21244_gb300 import dsmc as D
+    C = ctx()
+    gas, path, st = _uniform_gas(8 * _sms(), 20)
+    kernels = [D.TUNE_KERNELS.index(k) for k in ("moments", "moment_match")]
+    for k in kernels:
+        C.tune_set(k)
+    default = [C.tune_get(k) for k in kernels]
+    try:
+        trials = C.autotune_step(gas, path, st, step=0, reps=2)
+        for k in ("moments", "moment_match"):
+            assert len({t["ms"] for t in trials if t["kernel"] == k}) == 1
+        assert [C.tune_get(k) for k in kernels] == default
+    finally:
+        for k in range(len(D.TUNE_KERNELS)):
+            C.tune_set(k)
