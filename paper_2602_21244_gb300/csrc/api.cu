@@ -979,8 +979,11 @@ int dsmc_autotune_step(dsmc_ctx_t* c, const dsmc_gas_t* gas, const dsmc_path_t* 
   };
   auto gather_blocks = [&](int threads, int bps) { return std::min(((int64_t)B->n + threads - 1) / threads, sms * bps); };
   int nt = 0;
-  rc = tune_kernel(c, DSMC_TUNE_GATHER, reps, s, gather_blocks, [&] {
-    return dsmc::launch_gather(c, B->n, B->n_cells, B->cell_start, B->perm, B->vx, B->vy, B->vz, B->svx,
+  const uint32_t* skeys = nullptr;
+  rc = dsmc::launch_sort_for_gather(c, B->n, B->n_cells, B->cell_id, B->perm, B->cell_start, B->ws, B->ws_bytes, s,
+                                    &skeys);
+  if (!rc) rc = tune_kernel(c, DSMC_TUNE_GATHER, reps, s, gather_blocks, [&] {
+    return dsmc::launch_gather(c, B->n, B->n_cells, skeys, B->cell_start, B->perm, B->vx, B->vy, B->vz, B->svx,
                                B->svy, B->svz, s);
   }, trials, cap, &nt);
   if (!rc) rc = tune_kernel(c, DSMC_TUNE_MOMENTS, reps, s, cell_blocks, [&] {

@@ -713,17 +713,18 @@ int launch_sort(Ctx* c, int32_t n, int32_t n_cells, const int32_t* cell_id, cons
                 const double* vy, const double* vz, int32_t* perm, int32_t* cell_start,
                 double* svx, double* svy, double* svz, void* ws, size_t ws_bytes,
                 cudaStream_t s) {
-  if (n > 0 && n <= kGatherAll) {
-    const uint32_t* skeys = nullptr;
-    if (int rc = sort_passes(c, n, n_cells, cell_id, perm, cell_start, ws, ws_bytes, s, &skeys)) return rc;
-    const Shape sh = shape_or_default(c, DSMC_TUNE_GATHER);
-    const unsigned g = grid_for(n, sh.threads, sm_count(c) * sh.blocks_per_sm);
-    launch_dep(k_gather<true>, g, sh.threads, 0, s, n, cell_start, n_cells, skeys, perm, vx, vy, vz, svx, svy, svz);
-    count_launches(c, 1);
-    return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
-  }
-  if (int rc = launch_sort_keys(c, n, n_cells, cell_id, perm, cell_start, ws, ws_bytes, s)) return rc;
-  return launch_gather(c, n, n_cells, cell_start, perm, vx, vy, vz, svx, svy, svz, s);
+  const uint32_t* skeys = nullptr;
+  if (int rc = launch_sort_for_gather(c, n, n_cells, cell_id, perm, cell_start, ws, ws_bytes, s, &skeys)) return rc;
+  return launch_gather(c, n, n_cells, skeys, cell_start, perm, vx, vy, vz, svx, svy, svz, s);
+}
+
+// What the gather starts from: perm, with *skeys the sorted keys (in the
+// workspace) where it forms cell_start from them, else null and cell_start.
+int launch_sort_for_gather(Ctx* c, int32_t n, int32_t n_cells, const int32_t* cell_id, int32_t* perm,
+                           int32_t* cell_start, void* ws, size_t ws_bytes, cudaStream_t s, const uint32_t** skeys) {
+  if (n > 0 && n <= kGatherAll) return sort_passes(c, n, n_cells, cell_id, perm, cell_start, ws, ws_bytes, s, skeys);
+  *skeys = nullptr;
+  return launch_sort_keys(c, n, n_cells, cell_id, perm, cell_start, ws, ws_bytes, s);
 }
 
 // The radix passes on the cell ids alone: perm and cell_start (the velocities
@@ -791,15 +792,14 @@ int launch_gather_one(Ctx* c, int32_t n, int32_t n_cells, const int32_t* cell_st
   return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
 }
 
-int launch_gather(Ctx* c, int32_t n, int32_t n_cells, const int32_t* cell_start, const int32_t* perm,
+int launch_gather(Ctx* c, int32_t n, int32_t n_cells, const uint32_t* skeys, int32_t* cell_start, const int32_t* perm,
                   const double* vx, const double* vy, const double* vz, double* svx, double* svy,
                   double* svz, cudaStream_t s) {
   if (n <= 0) return 0;
   const Shape sh = shape_or_default(c, DSMC_TUNE_GATHER);
   const unsigned g = grid_for(n, sh.threads, sm_count(c) * sh.blocks_per_sm);
-  if (n <= kGatherAll) {
-    launch_dep(k_gather<false>, g, sh.threads, 0, s, n, const_cast<int32_t*>(cell_start), n_cells, nullptr, perm, vx, vy, vz,
-               svx, svy, svz);   // (cell_start is only read)
+  if (skeys) {
+    launch_dep(k_gather<true>, g, sh.threads, 0, s, n, cell_start, n_cells, skeys, perm, vx, vy, vz, svx, svy, svz);
     count_launches(c, 1);
     return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
   }

@@ -451,7 +451,9 @@ int occupancy_collide_jager(int threads);
 // the gather step of the cell sort alone (autotuning)
 int launch_gather_one(Ctx* c, int32_t n, int32_t n_cells, const int32_t* cell_start, const int32_t* perm,
                       const double* v, double* sv, cudaStream_t s);
-int launch_gather(Ctx* c, int32_t n, int32_t n_cells, const int32_t* cell_start, const int32_t* perm,
+int launch_sort_for_gather(Ctx* c, int32_t n, int32_t n_cells, const int32_t* cell_id, int32_t* perm,
+                           int32_t* cell_start, void* ws, size_t ws_bytes, cudaStream_t s, const uint32_t** skeys);
+int launch_gather(Ctx* c, int32_t n, int32_t n_cells, const uint32_t* skeys, int32_t* cell_start, const int32_t* perm,
                   const double* vx, const double* vy, const double* vz, double* svx, double* svy,
                   double* svz, cudaStream_t s);
 int launch_selftest_barrier(Ctx* c, uint64_t limit_ns, cudaStream_t s);

@@ -82,3 +82,11 @@ def test_training_leaves_no_mma_in_flight():
     rest = rest[:rest.index("tmem_dealloc")]
     assert re.search(r"if \(!alive && t == kIssuer\) \{\s*tc::commit\(drain\);\s*tc::mbar_wait\(drain, 0,[^;]*;\s*\}"
                      r".*__syncthreads\(\);", rest, flags=re.S), rest
+
+
+def test_autotuner_times_the_gather_of_the_step():
+    """The step's sort and the autotuner's trials share the gather, which for up to kGatherAll particles forms the
+    cell starts; the form that reads them is the static sort's alone."""
+    text = SOURCES["cells.cu"]
+    calls = [m.start() for m in re.finditer(r"k_gather<false>", text)]
+    assert len(calls) == 1 and calls[0] > text.index("int dsmc_sort_cells_static(")
