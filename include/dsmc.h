@@ -415,12 +415,17 @@ int dsmc_selftest_timeout(dsmc_ctx_t* ctx, int32_t which, uint64_t limit_ns, voi
  * is optimised away.  dsmc_selftest_peak_ops gives the operations one thread
  * performs (FLOPs for the FMA kinds, 2 per FMA and 4 per paired FMA;
  * results for ex2; -1 for bad arguments); the caller times the launch. */
-/* Diagnostic with no counterpart in the paper: the FP64 helpers of the
- * turning-point refinement against CUDA's own routines, y[i] = f(x[i]) for
+/* Diagnostic with no counterpart in the paper: the kernels' FP64 helpers
+ * against CUDA's own routines, y[i] = f(x[i]) for
  * n values (device memory) -- which 0: the refinement's exponential (Cody-
  * Waite reduction by ln 2, Taylor polynomial to degree 12; |x| < 700),
  * 1: CUDA's exp, 2: the refinement's reciprocal (FP32 seed and two Newton
- * steps; x positive, inside the FP32 normal range), 3: 1.0 / x. */
+ * steps; x positive, inside the FP32 normal range), 3: 1.0 / x, 4: the
+ * reciprocal square root of the rotation and the training, 5: CUDA's rsqrt,
+ * 6: the training's square root, 7: CUDA's sqrt, 8 and 10: sine and cosine of
+ * the FP32 angle x by the rotation's table, 9 and 11: by CUDA's sincos, 12
+ * and 14: sine and cosine of 2 pi x, x a multiple of 2^-53 in [0, 1), by the
+ * table, 13 and 15: by CUDA's sincospi. */
 int dsmc_selftest_math(dsmc_ctx_t* ctx, int32_t which, int64_t n, const double* x, double* y, void* stream);
 
 int64_t dsmc_selftest_peak_ops(int32_t which, int32_t iters);

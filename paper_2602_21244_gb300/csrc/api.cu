@@ -457,7 +457,7 @@ int dsmc_selftest_timeout(dsmc_ctx_t* c, int32_t which, uint64_t limit_ns, void*
 
 int dsmc_selftest_math(dsmc_ctx_t* c, int32_t which, int64_t n, const double* x, double* y, void* stream) {
   CHECK_CTX(c);
-  REQUIRE(c, which >= 0 && which <= 3 && n >= 0 && (n == 0 || (x && y)), "selftest_math: which 0..3, n >= 0, x, y");
+  REQUIRE(c, which >= 0 && which <= 15 && n >= 0 && (n == 0 || (x && y)), "selftest_math: which 0..15, n >= 0, x, y");
   return dsmc::launch_selftest_math(c, which, n, x, y, S(stream));
 }
 

@@ -202,8 +202,11 @@ __device__ __forceinline__ double f32_to_f64(float f) {
 // instruction costs the same however few lanes need it) bounds the code: the
 // special-function unit's FP64 approximation r (relative error below 2^-19 over
 // the whole range) and one third-order step: with e = 1 - x r^2,
-// 1/sqrt(x) = r (1 - e)^(-1/2) = r (1 + e/2 + 3/8 e^2 + ...), cut after e^2
-// (relative error 5/16 e^3 < 2^-55): 5 FP64 instructions.
+// 1/sqrt(x) = r (1 - e)^(-1/2) = r (1 + e/2 + 3/8 e^2 + ...), the binomial series
+// cut after e^2 (the third-order step of Householder 1970, The Numerical Treatment
+// of a Single Nonlinear Equation; relative error 5/16 e^3 < 2^-55): 5 FP64
+// instructions, the result within 2^-52 (measured 2^-52.7 at most and 2^-54.3 on
+// average, CUDA's rsqrt 2^-53.0 and 2^-54.5: dsmc_selftest_math).
 __device__ __forceinline__ double rsqrt_seed64(double x) {
   double r;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
@@ -218,6 +221,12 @@ __device__ __forceinline__ double rsqrt64(double x) {   // x > 0, normal
 __device__ __forceinline__ bool plain64(double x) {
   constexpr uint32_t lo = (1023u - 930u) << 20, hi = (1023u + 930u) << 20;
   return (uint32_t)__double2hiint(x) - lo < hi - lo;
+}
+// sqrt(x) = x r (1 - e)^(-1/2), as rsqrt64 (measured 2^-52.4 at most and 2^-54.4 on average, sqrt 2^-53 and 2^-54.5)
+__device__ __forceinline__ double root64(double x) {
+  if (!plain64(x)) return sqrt(x);
+  const double r = rsqrt_seed64(x), y = x * r, e = fma(-y, r, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
 // ---------------------------------------------------------------- pair dependencies

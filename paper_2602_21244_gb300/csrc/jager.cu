@@ -897,9 +897,11 @@ __device__ __forceinline__ void deflect(double u, double v, double w, double g, 
 // ---- The pair update's rotation with fewer FP64 instructions than the general
 // functions take.  Sine and cosine of an angle 2 pi k / 256 + d, |d| <= pi/256,
 // from those of 2 pi k / 256 (the first quarter comes with the launch, the circle
-// is laid out in shared memory) by the angle-sum formulas, with the Taylor series of
-// sin d to d^7 and of cos d - 1 to d^6 (truncation below 2e-21 and 2e-20): 13 FP64
-// instructions for both, errors of an FP64 rounding or two as sincos has.
+// is laid out in shared memory) by the angle-sum formulas (the table method of Tang
+// 1991), with the Taylor series of sin d to d^7 and of cos d - 1 to d^6 (truncation
+// below 2e-21 and 2e-20): 13 FP64 instructions for both, errors of at most two FP64
+// roundings (measured 2^-52.5 at most, sincos 2^-52.8: dsmc_selftest_math; the
+// whole rotation is within 3.7e-16 |v_r|, with sincos and the frame written out 5.1e-16).
 constexpr int kTurnSteps = 256;
 struct TurnTable {
   double quarter[kTurnSteps / 4 + 1];   // sin(2 pi k / 256), k = 0..64
@@ -1181,12 +1183,33 @@ __global__ void __launch_bounds__(128) k_harvest(PotDev P, int64_t n, const doub
 }
 
 
-// Self test of the refinement's FP64 helpers against CUDA's own routines:
-// which 0: exp64, 1: exp, 2: rcp64, 3: 1.0 / x.
-__global__ void k_selftest_math(Exp64 E, int which, int64_t n, const double* __restrict__ x, double* __restrict__ y) {
+// Self test of the FP64 helpers (even `which`, in pairs) against CUDA's own
+// routines: 0, 1: exp64, exp; 2, 3: rcp64, 1.0 / x; 4, 5: rsqrt64 as it is used,
+// rsqrt; 6, 7: root64, sqrt; 8, 9 and 10, 11: sin and cos of an FP32 angle by the
+// turn table, by sincos; 12, 13 and 14, 15: sin and cos of 2 pi x by the turn
+// table, by sincospi.
+__global__ void k_selftest_math(Exp64 E, TurnTable turn_table, int which, int64_t n, const double* __restrict__ x,
+                                double* __restrict__ y) {
+  __shared__ double2 turn[kTurnSteps];
+  lay_turn_table(turn_table, turn);
+  __syncthreads();
+  auto angle = [&](double v) {
+    double s, c;
+    if (which < 12) {
+      if (which & 1) sincos(f32_to_f64((float)v), &s, &c); else sincos_of(turn, (float)v, &s, &c);
+    } else if (which & 1) {
+      sincospi(2.0 * v, &s, &c);
+    } else {   // v = k 2^-53: the uniform of k's bits
+      const uint64_t k = (uint64_t)(v * 9007199254740992.0) << 11;
+      sincos_turn(turn, (uint32_t)(k >> 32), (uint32_t)k, &s, &c);
+    }
+    return which & 2 ? c : s;
+  };
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
     const double v = x[q];
-    y[q] = which == 0 ? exp64(E, v) : which == 1 ? exp(v) : which == 2 ? rcp64(v) : 1.0 / v;
+    y[q] = which == 0 ? exp64(E, v) : which == 1 ? exp(v) : which == 2 ? rcp64(v) : which == 3 ? 1.0 / v
+         : which == 4 ? (plain64(v) ? rsqrt64(v) : rsqrt(v)) : which == 5 ? rsqrt(v)
+         : which == 6 ? root64(v) : which == 7 ? sqrt(v) : angle(v);
   }
 }
 
@@ -1208,7 +1231,7 @@ static unsigned blocks_n(int64_t n, int threads, int cap) {
 
 int launch_selftest_math(Ctx* c, int which, int64_t n, const double* x, double* y, cudaStream_t s) {
   if (n == 0) return 0;
-  k_selftest_math<<<blocks_n(n, 256, sm_count(c) * 8), 256, 0, s>>>(make_exp64(), which, n, x, y);
+  k_selftest_math<<<blocks_n(n, 256, sm_count(c) * 8), 256, 0, s>>>(make_exp64(), make_turn_table(), which, n, x, y);
   count_launches(c, 1);
   return cudaGetLastError() == cudaSuccess ? 0 : DSMC_ERR_CUDA;
 }

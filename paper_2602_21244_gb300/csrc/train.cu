@@ -148,13 +148,6 @@ __device__ __forceinline__ uint64_t kdesc(uint32_t a, int K) { return tc::sdesc(
 // MN-major view of a [rows x F] tile: MN = F (features), K = rows
 __device__ __forceinline__ uint64_t mdesc(uint32_t a, int F) { return tc::sdesc(a, (uint32_t)(F / 8) * 128, 128); }
 
-// (the square roots of the FP64-bound row stage: see rsqrt64)
-__device__ __forceinline__ double sqrt64(double x) {
-  if (!plain64(x)) return sqrt(x);
-  const double r = rsqrt_seed64(x), y = x * r, e = fma(-y, r, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
-}
-
 // sums over the 16 lanes of this half-warp (groups are 16 consecutive rows)
 // of K values at once, K a power of two up to 8: each step halves the values a lane still adds (the
 // other half goes to its partner), so K values take K + log2(16/K) - 1 or so FP64
@@ -384,7 +377,7 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
       pre[c * kT + row] = d[c];
     }
     const double g2 = pre[3 * kT + row];
-    pre[3 * kT + row] = sqrt64(g2);
+    pre[3 * kT + row] = root64(g2);
     pre[4 * kT + row] = fma(0.5, g2, th + th);
   };
   // act'(z + bias) of this thread's 32 values of layer l
