@@ -128,3 +128,12 @@ def test_autotune_keeps_the_builtin_shape_where_all_launch_alike():
     finally:
         for k in range(len(D.TUNE_KERNELS)):
             C.tune_set(k)
+
+
+@pytest.mark.parametrize("order", [0, 1])
+@pytest.mark.parametrize("pad", [1024, 1025, 2048, 2049, 8192, 8193, 2048 * 4096, 2048 * 4096 + 1])
+def test_selection_on_both_sides_of_its_launches(pad, order):
+    """One tile and two of the one-block word counts, their last size (2,048 cells) and the first of two launches, the
+    last one-block scan (8,192 counts), the last scan whose blocks sum the ones before them (2,048 blocks)."""
+    import test_gpu_variants as V
+    V.test_selection_variants_by_cell_count(pad, order)
