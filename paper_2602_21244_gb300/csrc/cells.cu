@@ -2,11 +2,12 @@
 //
 // Sort (Sec. 2.6 (1)): a stable LSD radix sort of (cell id, input index) on
 // 9-bit digits (two passes for up to 2^18 cells), each pass a per-chunk
-// digit count, one exclusive scan over (digit, chunk) and an ordered
-// per-chunk scatter; cell_start from the sorted ids; then the gather of the
-// velocities.  (The allocation-free variant keeps an atomic histogram +
-// cursor scatter + per-cell sort of the slots.)  Moments and moment
-// matching use exact integer sums over 8 lanes per cell (moments.cuh).
+// digit count, a scan of every digit's counts along the chunks (left to the
+// scatter for few chunks) and an ordered per-chunk scatter; then the gather of
+// the velocities, which up to 2.5 million particles forms cell_start from the
+// sorted ids too.  (The allocation-free variant keeps an atomic histogram +
+// cursor scatter + per-cell sort of the slots.)  Moments and moment matching
+// use exact integer sums over 8 or 32 lanes per cell (moments.cuh).
 #include <climits>
 
 #include "dispatch.cuh"
@@ -312,7 +313,7 @@ k_fix_large(int32_t n_cells, const int32_t* __restrict__ cell_start, int32_t* sl
 // slot, and the perm entries past the filled ones are never written.
 // START: cell_start is formed here from the sorted keys, as k_cell_start does
 // (slot s starts every cell in (key[s-1], key[s]]; a key n_cells has no cell): a
-// launch less (look-up step of 2,867 cells 112.1 -> 109.8 us, Couette VHS step 47.3 -> 45.0).
+// launch less (2.3 us of a small step).
 template <bool START>
 __global__ void k_gather(int32_t n, int32_t* __restrict__ cell_start, int32_t n_cells, const uint32_t* __restrict__ skeys,
                          const int32_t* __restrict__ perm, const double* __restrict__ vx,
@@ -817,10 +818,9 @@ int launch_gather(Ctx* c, int32_t n, int32_t n_cells, const uint32_t* skeys, int
 // warp claims runs of kCwRun consecutive cells from a counter (so that the
 // warps given cheap runs, such as empty cells or the free stream, take more
 // of them) and collects kCwClaims runs before finishing their cells.  A warp
-// claims only a few times, so short claims even out the end: four of 4 cells
-// instead of two of 8 took matching at 37,500 cells of 61 particles from 71 to 50
-// us, at 73,500 from 103 to 93, moments at 150,000 from 98 to 85 us (matching there
-// 172 both ways; two of 4: 57 us at 37,500, eight of 4: 182 us at 150,000).
+// claims only a few times, so short claims even out the end (matching of 37,500
+// unequal cells 50 us with four claims of 4 cells, 71 with two of 8, 57 with two
+// of 4; moments of 150,000 cells 85 and 98 with the first two).
 // Segments of 8 lanes take four cells at a time through the two passes of
 // the exact integer moments (the largest exponent, then the split sums of
 // moments.cuh); the per-cell remainder (means, centred sum of squares,
@@ -1072,7 +1072,7 @@ static int launch_cells(Ctx* c, bool match, int32_t n_cells, const int32_t* cs, 
   const Shape sh = shape_or_default(c, match ? DSMC_TUNE_MOMENT_MATCH : DSMC_TUNE_MOMENTS);
   const int64_t runs = ((int64_t)n_cells + kCwRun - 1) / kCwRun;
   // a warp per run as long as they fit, so that a mid-size gas keeps one run
-  // per warp (40,000 cells: matching 38 -> 33 us)
+  // per warp (matching of 40,000 cells 33 us, with two per warp 38)
   const unsigned g = grid_for(runs, kCwWarps, sm_count(c) * sh.blocks_per_sm);
   if (match) launch_dep(k_cells<true>, g, kCwWarps * 32, 0, s, n_cells, cs, vx, vy, vz, mom, nullptr, work_ptr(c));
   else launch_dep(k_cells<false>, g, kCwWarps * 32, 0, s, n_cells, cs, vx, vy, vz, mom, status_ptr(c), work_ptr(c));

@@ -567,16 +567,15 @@ __device__ __forceinline__ float node_term(const PotDev& P, const PairCoef& c, c
 constexpr int kLongShared = 28, kShortShared = 16;
 
 // kWarp: see rmin_device (every lane of the warp calls it together, with the
-// block's ChiShared).  Then the pairs with the short rule run side by side,
-// and the nodes of a pair with the long rule (below orbit_E) are spread over
-// the warp's lanes, four each, the integrand summed by the pair's own lane in
-// the order of the nodes: one such pair in a warp used to hold the other lanes
-// for the long rule's 128 nodes (of the chi batch's pairs, a twelfth of them with the
-// long rule, 95 % of the warps did).  2^22 pairs of that batch: 4.00 -> 2.55
-// ms, and 1.90 ms with one copy of the node's code for both ways and the other
-// potentials' code compiled apart (a fifth of the warps' stalls were
-// instruction fetches), 1.79 ms with five blocks per SM, bit-identical; what is left is the FP64 refinement
-// (111 FP64 instructions per warp at 19 cycles: 0.9 ms) and the FP32 instructions.
+// block's ChiShared).  Then the nodes of the pairs with the long rule (below
+// orbit_E), and of those with the short one where few lanes have it, are spread
+// over the warp's lanes, the integrand summed by the pair's own lane in the order
+// of the nodes; the other pairs run side by side.  So one pair with the long rule
+// does not hold its warp for 128 nodes (in the chi batch a twelfth of the pairs, in
+// 95 % of the warps: 2^22 pairs 1.79 ms, every pair side by side 4.00).  What is
+// left is the FP64 refinement (111 FP64 instructions per warp at 19 cycles: 0.9
+// ms) and the FP32 instructions; both ways share one copy of the node's code, since
+// instruction fetches stall the warps.
 template <bool kWarp = false, int KIND = -1>
 __device__ float chi_device(const PotDev& P, float b_in, float E, ChiShared S = ChiShared{}, bool use = true) {
   const int kind = KIND >= 0 ? KIND : P.kind;
@@ -811,7 +810,8 @@ static PotDev build_pot(double mass, const dsmc_potential_t& p, int n_nodes) {
 
 // The constants above of a (mass, potential, node count).  Building them (the
 // Gauss-Legendre rules, the zero and the depth of V) takes the host about 0.4
-// ms, so the last few are kept, found by the values they were built from.
+// ms, so the last few are kept, found by the values they were built from (a caller
+// with another potential on every call pays it every time).
 static PotDev make_pot(const dsmc_gas_t& gas, const dsmc_potential_t& p, int n_nodes) {
   struct Kept {
     double mass;
@@ -989,10 +989,11 @@ struct JagerArgs {
 // the exact deflection by that chi to FP64 rounding -- then the
 // centre-of-mass update, v_i' = v_i + (v_r' - v_r)/2 and v_j' = v_j - that (the pair
 // keeps its sum); velocities through L2.  Rotation and update take about 80 FP64
-// instructions, with sincos, sincospi, rsqrt and the frame written out 110: with
-// chi's 111 the FP64 pipe, 57 % busy, bounds the kernel (1.7 million pairs 1284
-// us, now 1230).  Every lane of the warp runs
-// it together (live false: a lane with no pair, or whose dependency wait
+// instructions, with sincos, sincospi, rsqrt and the frame written out 110, and chi's
+// refinement 111: the FP64 pipe is the busiest (64 % of 6.9 million pairs' 3.56 ms,
+// 35 % of 0.6 million's), the rest is latency: a quarter of the warp slots, and one
+// warp's chi per round and link (1.7 million pairs 1230 us, with 110 1284).  Every
+// lane of the warp runs it together (live false: a lane with no pair, or whose dependency wait
 // failed, computes on harmless inputs and stores nothing), so that chi's FP64
 // refinement and the FP64 rotation run with the warp converged.
 template <int KIND>

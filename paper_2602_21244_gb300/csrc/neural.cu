@@ -690,22 +690,18 @@ __device__ __forceinline__ void update_row(const NeuralArgs& a, const float y[3]
 // FP32 accumulators into a free one, the epilogue turns them in place into the
 // next layer's A operand (every 16 columns become 8 of bf16 hi and 8 of lo
 // terms), and the operand's region is free again once the MMA that reads it is
-// done -- so three tiles and one MMA in flight fit.  With two tiles, each bound
-// to its own 8 epilogue warps, those waited out every MMA of their tile (0.9 of
-// 2.9 us per layer), and a tile alone took 2 us per epilogue.
+// done -- so three tiles and one MMA in flight fit (6.9 million pairs, 357 tiles
+// per SM: 1531 us; with two in flight 1586).
 //
-// Measured on 6.9 million pairs (357 tiles per SM): 1660 us with two bound
-// tiles, 1531 us now; a 200 x 200 cavity (670,000 pairs, 18 levels) 291 -> 276
-// us.  Per tile and SM 8,850 cycles: the epilogue warps work 6,800 of them (three
-// steps of 2,250, twice their instructions' issue time: the other roles' warps
-// share the schedulers), the issuing lane 3,600; a builder group takes 9,000
-// (stamps 4,400, gather 2,200, arithmetic 1,750, stores 460) but there are two.
-// Not kept: two epilogue groups taking steps in turn (1698 us), partial sums
-// handed over by mbarriers instead of named barriers (1570), the next pair's
-// record and stamps read ahead (1660), two tiles in flight (1586).  The shared
-// memory counts: the same kernel with 20 KB more that it does not use takes 1684
-// us, with eight buffers 1700, with four 1619: the L1 that is left serves the
-// random loads in flight.
+// What bounds it: per tile and SM 8,850 cycles, of which the epilogue warps work
+// 6,800 (three steps of 2,250, twice their instructions' issue time: the other
+// roles' warps share the schedulers, and each step ends with the slowest of the 16
+// warps) and the issuing lane 3,600; a builder group takes 9,000 (stamps 4,400,
+// gather 2,200, arithmetic 1,750, stores 460) but there are two.  A gas of few
+// tiles per SM is bound by its claim levels instead, one tile's latency each (a
+// 200 x 200 cavity, 670,000 pairs in 18 levels: 276 us, its tiles' throughput 150).
+// Six buffers, because the L1 that they leave serves the random loads in flight
+// (with eight 1700 us, with four 1619).
 //
 // Hand-offs are mbarriers: claimed, built (128 builder arrivals), dfull (an MMA step's
 // commit and its description), edone (its epilogue, 16 warps), ydone (the 128

@@ -17,9 +17,8 @@
 //                 each with the rounds of the previous pairs of its particles
 //
 // A gas of a few thousand particles is bound by its launches, about 3 us each:
-// the zeroing, *info and the scans' middle pass ride on other kernels (a
-// 100-cell gas's selection took 13 launches and two memsets, now 8; its whole
-// step 128 -> 82 us).
+// the zeroing, *info and the scans' middle pass ride on other kernels (8
+// launches for a 100-cell gas; with 13 and two memsets its step took 46 us more).
 //
 // The accept decision and M are taken in FP64 with explicitly rounded
 // operations (no contraction into FMA), in the operation order of the

@@ -59,9 +59,8 @@ constexpr int kIssuer = 256;     // thread that issues the MMAs (of a warp witho
 // per-CTA partial: dW1 (128 x 32), dW2, dW3 (128 x 128), dW4^T (128 x 16), then the bias
 // gradients of each of the 4 TMEM lane groups [4 x 400], then the loss of each lane group.
 // The matrices lie as the threads hold them, four consecutive columns per thread and
-// the threads side by side (wpos), so that a warp's stores fill whole lines: row-major,
-// every store of a warp touched 32 lines, 16 bytes of each, and the flush of a
-// mini-batch's one tile took 17,000 of its 64,000 cycles, now 7,000 (2^14 pairs 51 us, now 48).
+// the threads side by side (wpos), so that a warp's stores fill whole lines (2^14 pairs, one
+// tile per CTA: 48 us; row-major, 32 lines per store of a warp, 51).
 constexpr int kPDB = kH * kXin + 2 * kH * kH + kH * 16;
 constexpr int kPLOSS = kPDB + 4 * 400;
 constexpr int kPartial = kPLOSS + 16;
@@ -349,7 +348,7 @@ __global__ void __launch_bounds__(kNT, 1) k_train(TrainArgs a) {
   // is the same before and after, and with d = (vi + vj)/2 - mean
   //   |vi - mean|^2 + |vj - mean|^2 = 2 |d|^2 + |v_r|^2 / 2
   // before it; after it the particles are at d +- v_r'/2.  (At the head of the
-  // row stage it took 4,000 of a tile's 36,600 cycles: 1M pairs 1072 us, then 1010.)
+  // row stage 1M pairs take 1072 us, here 1010.)
   double* pre = (double*)(sm + S_PRE);
   double* mean = (double*)(sm + S_MEAN);
   auto row_pairs = [&](int64_t p, bool valid) {
