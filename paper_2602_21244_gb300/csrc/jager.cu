@@ -329,7 +329,8 @@ constexpr int kScanShared = 20;    // fine scans a warp shares (more run side by
 
 // KIND: the potential's kind when the kernel is compiled for it (the other
 // kinds' code, FP64 pow among it, then does not spread the hot loops over the
-// instruction cache), or -1.
+// instruction cache or take registers), or -1 (the table, the harvest and the
+// transport integrals).
 template <bool kWarp, int KIND>
 __device__ Turn rmin_device(const PotDev& P, float b, float E) {
   Turn T = {};
@@ -493,8 +494,14 @@ struct ChiShared {
   float *par, *term;   // this warp's
 };
 
-// Called by the whole block (with a barrier) before the first chi_device<true>.
+// Called by the whole block (with a barrier) before the first chi_device<true>;
+// the potentials without shared nodes have no such memory.
+template <int KIND>
 __device__ __forceinline__ ChiShared chi_shared(const PotDev& P, float* sm) {
+  if (KIND != 0) {
+    __syncthreads();
+    return ChiShared{};
+  }
   for (int i = threadIdx.x; i < P.n_nodes + P.n_low; i += blockDim.x) {
     const int q = i < P.n_nodes ? i : kMaxNodes + i - P.n_nodes;
     const float s = P.s_node[q];
@@ -842,12 +849,15 @@ static PotDev make_pot(const dsmc_gas_t& gas, const dsmc_potential_t& p, int n_n
 // the end, or with g = 0, on harmless inputs whose result is not kept).
 // Five blocks per SM: 2^22 pairs 1785 us, four 1896, six 1866 (the pair update,
 // with the rotation's registers besides, is faster with four: 1230 against 1272 us, three 1249).
+// A kernel per kind: 2^22 pairs with 128 nodes take 1056 us for hard spheres, 2076 for
+// an inverse power; one kernel for both, with the Jager form's code and shared memory,
+// took 2041 and 2934.
 template <int KIND>
 __global__ void __launch_bounds__(128, 5) k_jager_chi(PotDev P, int64_t n, const float* __restrict__ b,
                                                       const float* __restrict__ g, float* __restrict__ chi) {
   dep_wait_alone();
   extern __shared__ float4 chi_sm[];
-  const ChiShared S = chi_shared(P, (float*)chi_sm);
+  const ChiShared S = chi_shared<KIND>(P, (float*)chi_sm);
   const int lane = threadIdx.x & 31;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
@@ -1041,7 +1051,7 @@ __global__ void __launch_bounds__(128, 4) k_collide_jager(PotDev P, TurnTable tu
   extern __shared__ float4 chi_sm[];
   __shared__ double2 turn[kTurnSteps];
   lay_turn_table(turn_table, turn);
-  const ChiShared S = chi_shared(P, (float*)chi_sm);   // (ends with a barrier)
+  const ChiShared S = chi_shared<KIND>(P, (float*)chi_sm);   // (ends with a barrier)
   const int R = a.info->n_rounds;
   const int lane = threadIdx.x & 31;
   int r = 0;
@@ -1242,8 +1252,8 @@ int launch_jager_chi(Ctx* c, const dsmc_gas_t& gas, const dsmc_potential_t& pot,
   if (n == 0) return 0;
   const PotDev P = make_pot(gas, pot, n_nodes);
   const Shape sh = shape_or_default(c, DSMC_TUNE_JAGER_CHI);
-  const size_t sm = chi_smem(sh.threads, P.n_nodes + P.n_low);
-  const auto k = P.kind == 0 ? k_jager_chi<0> : k_jager_chi<-1>;
+  const size_t sm = P.kind == 0 ? chi_smem(sh.threads, P.n_nodes + P.n_low) : 0;
+  const auto k = P.kind == 0 ? k_jager_chi<0> : P.kind == 1 ? k_jager_chi<1> : k_jager_chi<2>;
   if (!allow_smem((const void*)k, sm)) return record(c, DSMC_ERR_CUDA, "jager_chi: shared-memory attribute");
   launch_dep(k, blocks_n(n, sh.threads, sm_count(c) * sh.blocks_per_sm), sh.threads, sm, s, P, n, b, g, chi);
   count_launches(c, 1);
@@ -1268,8 +1278,8 @@ int launch_collide_jager(Ctx* c, const dsmc_gas_t& gas, const dsmc_potential_t& 
   if (ws_bytes < collide_ws(n)) return record(c, DSMC_ERR_ARG, "collide_jager: workspace too small");
   const Shape sh = shape_or_default(c, DSMC_TUNE_COLLIDE_JAGER);
   const PotDev P = make_pot(gas, pot, n_nodes);
-  const size_t sm = chi_smem(sh.threads, P.n_nodes + P.n_low);
-  const auto k = P.kind == 0 ? k_collide_jager<0> : k_collide_jager<-1>;
+  const size_t sm = P.kind == 0 ? chi_smem(sh.threads, P.n_nodes + P.n_low) : 0;
+  const auto k = P.kind == 0 ? k_collide_jager<0> : P.kind == 1 ? k_collide_jager<1> : k_collide_jager<2>;
   const int occ = occupancy_jager((const void*)k, sh.threads, sm);
   if (occ < 1) return record(c, DSMC_ERR_CUDA, "collide_jager: occupancy query failed");
   const int blocks = sm_count(c) * (sh.blocks_per_sm > 0 && sh.blocks_per_sm < occ ? sh.blocks_per_sm : occ);
