@@ -103,7 +103,27 @@ def parse():
                     help="which standalone measurements to run (comma list)")
     ap.add_argument("--no-autotune", dest="autotune", action="store_false",
                     help="keep the built-in launch shapes")
+    ap.add_argument("--details", metavar="FILE",
+                    help="also write every measurement (phases, rooflines, standalone kernels) to FILE as JSON")
     return ap.parse_args()
+
+
+def short_line(line):
+    """The one line printed: the whole record less what --details is for, so that it stays short enough (about
+    1,400 characters) for a log that keeps only the end of the output.  Of each path its rate and time; numbers
+    below the top level to five significant digits."""
+    def brief(v):
+        if isinstance(v, dict):
+            return {k: brief(x) for k, x in v.items()}
+        return float(f"{v:.5g}") if isinstance(v, float) else v
+
+    out = {k: (v if isinstance(v, (int, float)) else brief(v)) for k, v in line.items() if k not in ("paths", "standalone")}
+    out["paths"] = {name: brief({k: r[k] for k in ("collisions_per_s", "ms_per_step") if k in r})
+                    for name, r in line["paths"].items()}
+    for key, left_out in (("cpu_baseline", ("single_thread", "nproc")), ("roofline", ("peak_source",))):
+        if out.get(key):
+            out[key] = {k: v for k, v in out[key].items() if k not in left_out}
+    return out
 
 
 def phase_bytes(n, nc, pairs):
@@ -820,7 +840,10 @@ def main():
                 "paths": results, "standalone": extra, "roofline": roof, "cpu_baseline": cb, "e2e": e2e,
                 "gpu_launches": int(sum(r["gpu_launches"] for r in results.values())),
                 "clocks": clocks}
-        print(json.dumps(line), flush=True)
+        if args.details:
+            with open(args.details, "w") as f:
+                json.dump(line, f, indent=1)
+        print(json.dumps(short_line(line)), flush=True)
     if dist is not None:
         dist.destroy_process_group()
 
